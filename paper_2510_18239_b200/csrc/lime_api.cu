@@ -668,6 +668,7 @@ lime_status lime_score_candidates(lime_ctx* ctx, const void* link_states, int32_
   a.LS = link_states; a.W = cand_w; a.T = cand_emb; a.dtype = c->cfg.dtype; a.B = B; a.ell = c->ell_c; a.d = c->cfg.d;
   a.cand_off = cand_off; a.C = C; a.total = total_cands; a.cand_ids = cand_ids; a.logits = logits;
   a.corpus_rows = cand_ids ? corpus_rows : 0; a.dev_flag = cand_ids ? dev_flag : nullptr;
+  if (score_rows_preferred(a)) return launch_score_rows(a, static_cast<cudaStream_t>(stream));
   if (score_tc_supported(a)) return launch_score_tc(a, c->dev_err, static_cast<cudaStream_t>(stream));
   if (score_gather_tc_supported(a)) return launch_score_gather_tc(a, c->dev_err, static_cast<cudaStream_t>(stream));
   return launch_score_simt(a, static_cast<cudaStream_t>(stream));
@@ -829,6 +830,7 @@ lime_status lime_score_candidates_packed(lime_ctx* ctx, const void* link_states,
   a.dtype = c->cfg.dtype; a.B = B; a.ell = c->ell_c; a.d = c->cfg.d;
   a.cand_off = cand_off; a.C = C; a.total = total_cands; a.cand_ids = cand_ids; a.logits = logits;
   a.corpus_rows = corpus_rows; a.dev_flag = dev_flag;
+  if (score_rows_preferred(a)) return launch_score_rows(a, static_cast<cudaStream_t>(stream));
   if (score_gather_tc_supported(a)) return launch_score_gather_tc(a, c->dev_err, static_cast<cudaStream_t>(stream));
   return launch_score_simt(a, static_cast<cudaStream_t>(stream));
 }

@@ -232,6 +232,10 @@ lime_status launch_score_tc(const ScoreArgs& a, int* err, cudaStream_t st);
 bool score_gather_tc_supported(const ScoreArgs& a);
 lime_status launch_score_gather_tc(const ScoreArgs& a, int* err, cudaStream_t st);
 
+// warp-level scorer: by id, ragged lists, small widths (bf16, d in {32, 64, 128, 256}, ell in {8, 16, 32, 64}), k_score_rows.cu
+bool score_rows_preferred(const ScoreArgs& a);
+lime_status launch_score_rows(const ScoreArgs& a, cudaStream_t st);
+
 // one-thread kernel whose only wait can never be satisfied (self-test of the bounded waits, tc_host.cu)
 lime_status launch_wait_expiry(int* err, uint64_t limit_ns, int code, cudaStream_t st);
 
