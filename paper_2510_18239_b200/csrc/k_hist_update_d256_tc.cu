@@ -1,5 +1,5 @@
-// History update of one XOR layer on tcgen05 at d = d_ff = 256 with ell = 64 links and H in {2, 4, 8} heads (bf16 storage,
-// rows LayerNorm-ed already):
+// History update of one XOR layer on tcgen05 at d = d_ff = 256 with 64 links and 2, 4 or 8 heads or 32 links and 4 or 8
+// heads (bf16 storage, rows LayerNorm-ed already):
 //
 //   S'[t,:] = GatedMLP( O[S]_t ),   O[S]_t = concat_h phi( Q[S]_{t,h} K[T]_{l,h}^T * scale ) V[T]_{l,h}          (Eq. 7, Eq. 5)
 //   GatedMLP(A) = ( SiLU(A W_g) * (A W_u) ) W_o
@@ -8,9 +8,9 @@
 // (k_link_prep.cu: Q[S] is never formed), the value mix is done head by head against the plain link values V[T], and
 // the GatedMLP weights follow unfolded - at this width folding W_V W_g into the link side (as the d = 128 kernels do)
 // would cost twice the tensor work and twice the operand traffic:
-//   scores [128 x H*64] = X . K2^T, 256 stacked (head, link) rows = four heads per contraction
-//   per group c of two heads: per-head softmax over the 64 links, unnormalised (or SiLU(s) / 64) -> P_c (bf16);
-//                             O[:, head] = P_head [128 x 64] . V_head [64 x d_h]
+//   scores [128 x H*ell] = X . K2^T, 256 stacked (head, link) rows per contraction
+//   per group c of 128 stacked rows (two heads of 64 links, four of 32): per-head softmax over the links, unnormalised (or
+//                             SiLU(s) / ell) -> P_c (bf16);  O[:, head] = P_head [128 x ell] . V_head [ell x d_h]
 //   O * 1 / (row sum of the head) -> bf16
 //   per half hf of the hidden columns:   [gate | up] = O . [W_g | W_u][:, hf]  ->  U = SiLU(gate) * up (bf16)
 //                                        S' (+)= U . W_o[hf rows, :]
@@ -27,14 +27,15 @@
 // 16 KB slabs of 32 of the contraction index, 64-byte swizzle - half again as many bytes in flight - were measured:
 // 8.3 against 7.4 ms per production_ragged step; what limits the stream is not its depth but the 64-byte pieces.)
 // Warp 0 TMA producer, warp 1 MMA issuer, warps 2-17 token rows.  For the softmax the row warps form two groups that
-// take alternate groups of two heads, one thread per (token, head): no exchange between threads, and one group's
-// exponentials overlap the other group's value mix.  Elsewhere four threads share a token, a quarter of the columns each.
+// take alternate groups of 128 stacked rows, one thread per token and 64 of them (one head of 64 links, or two of 32, whose
+// maxima and sums are the two halves' own): no exchange between threads, and one group's exponentials overlap the other
+// group's value mix.  Elsewhere four threads share a token, a quarter of the columns each.
 #include "lime_common.cuh"
 #include "tc_common.cuh"
 
 namespace lime {
 
-constexpr int HC_D = 256, HC_F = 256, HC_TILE = 128, HC_ELL = 64;
+constexpr int HC_D = 256, HC_F = 256, HC_TILE = 128;
 constexpr int HC_PARTS = 4, HC_ROW_WARPS = 4 * HC_PARTS, HC_THREADS = 64 + 32 * HC_ROW_WARPS;
 constexpr int HC_RING = 3;
 constexpr uint32_t HC_SUB = 128 * 128;                          // bytes of one [128 rows x 64 bf16] swizzled sub-tile
@@ -54,7 +55,7 @@ struct HistUpdate256Params {
   __nv_bfloat16* out;            // [total x d]
   const int32_t* off;            // [B+1]
   const int32_t* tile_start;     // [B+1] prefix of per-user tile counts (tile = 128 tokens)
-  int B, H, HL, NG, shared, out_ln;   // NG = HL / 128 groups of two heads
+  int B, H, HL, NG, shared, out_ln;   // NG = HL / 128 groups of 128 stacked rows
   int silu;                      // 1: P = SiLU(scores) / ell (Algorithm 2) instead of the per-head softmax
   float ln_eps;
   int* err;
@@ -96,6 +97,7 @@ struct HcTileUser {
   }
 };
 
+template <int ELL>
 __global__ void __launch_bounds__(HC_THREADS, 1)
 k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmK2,
                       const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmWgu,
@@ -131,7 +133,10 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   const int t_begin = (int)(((int64_t)blockIdx.x * n_tiles_all) / gridDim.x);
   const int t_end = (int)(((int64_t)(blockIdx.x + 1) * n_tiles_all) / gridDim.x);
   const int n = t_end - t_begin;
-  const int NG = p.NG;                                       // groups of two heads
+  constexpr int HPG = 128 / ELL;                             // heads per group of 128 stacked rows
+  constexpr uint32_t V_ROW = ELL * 2;                        // bytes of a V[T]^T row (its swizzle span)
+  constexpr uint32_t V_BYTES = HC_D * V_ROW;
+  const int NG = p.NG;                                       // groups of 128 stacked rows
   const int d_h = HC_D / p.H;
   const int n_sg = (p.HL + 255) / 256;                       // score contractions per tile (four heads each)
   const int sc_boxes = p.HL >= 256 ? 2 : 1;                  // 128-row boxes of K2 per score slab
@@ -201,7 +206,7 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         if (!ok) break;
         // the user's link values go where U of the previous tile was and where its rows left through
         if (g > 0 && !mbar_wait(pu_free, (uint32_t)(g - 1) & 1u, p.err, 13)) { ok = false; break; }
-        mbar_arrive_expect_tx(v_full, 2 * HC_SUB);
+        mbar_arrive_expect_tx(v_full, V_BYTES);
         tma_load_2d_hint(smem + HC_OFF_PU, &tmV, 0, urow * HC_D, v_full, pol_keep);
         v_sent = true;
         // then per half of the hidden columns the gate and up columns of W_g / W_u (contraction over d) and that half's
@@ -268,11 +273,12 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
           if (!mbar_wait(&p_ready[rg], p_uses[rg] & 1u, p.err, 24)) { ok = false; break; }
           ++p_uses[rg];
           tc_fence_after();
-          for (int hl = 0; hl < 2; ++hl) {
-            const int h = c * 2 + hl;
-            for (int kk = 0; kk < 4; ++kk)
-              mma_bf16_ss(tmem_base + R0 + (uint32_t)(h * d_h), make_sdesc_k_sw128(xo + (uint32_t)(rg * 2 + hl) * HC_SUB + kk * 32),
-                          make_sdesc_k_sw128(pu + (uint32_t)(h * d_h) * 128 + kk * 32), idesc_v, kk != 0);
+          for (int hl = 0; hl < HPG; ++hl) {
+            const int h = c * HPG + hl;
+            const uint32_t a0 = xo + (uint32_t)(rg * 2) * HC_SUB + (uint32_t)(hl * ELL / 64) * HC_SUB + (uint32_t)(hl * ELL % 64) * 2;
+            for (int kk = 0; kk < ELL / 16; ++kk)
+              mma_bf16_ss(tmem_base + R0 + (uint32_t)(h * d_h), make_sdesc_k_sw128(a0 + kk * 32),
+                          make_sdesc_k_sw(pu + (uint32_t)(h * d_h) * V_ROW + kk * 32, V_ROW), idesc_v, kk != 0);
           }
           mma_commit(&pv_done[rg]);
           if (c == NG - 1) mma_commit(o_full);
@@ -304,12 +310,12 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     const int rw = warp - 2;                                 // 0..15
     const int q4 = warp & 3;                                 // TMEM lane quarter of this warp
     const int part = rw >> 2;                                // which quarter of the columns of every step
-    const int rg = part >> 1, hh = part & 1;                 // softmax: row-warp group, head within a group of two
+    const int rg = part >> 1, hh = part & 1;                 // softmax: row-warp group, half (64 columns) of a group of 128 stacked rows
     const uint32_t r = (uint32_t)(q4 * 32 + lane);           // token row of the tile == TMEM lane
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q4 * 32) << 16);
     float2* exch = reinterpret_cast<float2*>(smem + HC_OFF_EXCH);         // [2][PARTS][128]
     float* inv_sum = reinterpret_cast<float*>(smem + HC_OFF_INV);         // [8][128]
-    uint8_t* p_head = smem + HC_OFF_XO + (uint32_t)(rg * 2 + hh) * HC_SUB;   // P of this thread's head: one K-block
+    uint8_t* p_head = smem + HC_OFF_XO + (uint32_t)(rg * 2 + hh) * HC_SUB;   // P of this thread's 64 columns: one K-block
     uint8_t* pu_part = smem + HC_OFF_PU + (part >> 1) * HC_SUB;           // U: K-block part / 2, chunks (part % 2) * 4 ..
     const uint32_t pu_chunk0 = (uint32_t)(part & 1) * 4;
     uint32_t row_uses = 0, my_p = 0;
@@ -320,24 +326,26 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
       const int b = tu.of(tile_start, p.B, t);
       const int row0 = off[b] + (t - tu.lo) * HC_TILE;
       const uint32_t R0 = (uint32_t)(g & 1) * 256u, R1 = 256u - R0;
-      // ---- this row-warp group's groups of two heads: softmax over the 64 links of this thread's head, P_c -> smem
+      // ---- this row-warp group's groups: softmax over the links of this thread's head (or two heads of 32), P_c -> smem
       for (int c = rg; c < NG && ok; c += 2, ++my_p) {
         const int sg = c >> 1;
         if (!mbar_wait(&s_full[sg], (uint32_t)g & 1u, p.err, 32)) { ok = false; break; }
         tc_fence_after();
         const uint32_t col = lane_addr + (sg ? R1 : R0) + (uint32_t)(c & 1) * 128u + (uint32_t)hh * 64u;
         float v[32];
-        float mx = 0.f, sum = 0.f;
+        float mx[64 / ELL] = {}, sum[64 / ELL] = {};       // by head; with ELL = 32 the two halves are heads of their own
         if (!p.silu) {
           tmem_ld_32x32(col, v);
           tmem_wait_ld();
-          mx = v[0];
+          mx[0] = v[0];
 #pragma unroll
-          for (int j = 1; j < 32; ++j) mx = fmaxf(mx, v[j]);
+          for (int j = 1; j < 32; ++j) mx[0] = fmaxf(mx[0], v[j]);
           tmem_ld_32x32(col + 32, v);
           tmem_wait_ld();
+          float& m1 = mx[64 / ELL - 1];
+          if (ELL == 32) m1 = v[0];
 #pragma unroll
-          for (int j = 0; j < 32; ++j) mx = fmaxf(mx, v[j]);
+          for (int j = 0; j < 32; ++j) m1 = fmaxf(m1, v[j]);
         }
         // the P buffers lie over the token tile: every score contraction of the tile must have read it, and the value mix
         // that read this buffer last must have run
@@ -350,17 +358,18 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
           if (p.silu) {
             // SiLU(s) / ell: every history query attends to the ell links of the head (Algorithm 1)
 #pragma unroll
-            for (int j = 0; j < 32; ++j) { const float hx = 0.5f * v[j]; v[j] = fmaf(hx, hc_tanh(hx), hx) * (1.0f / HC_ELL); }
+            for (int j = 0; j < 32; ++j) { const float hx = 0.5f * v[j]; v[j] = fmaf(hx, hc_tanh(hx), hx) * (1.0f / ELL); }
           } else {
             float s0 = 0.f, s1 = 0.f;
+            const float m = mx[hv * (64 / ELL - 1)];
 #pragma unroll
             for (int j = 0; j < 32; j += 2) {
-              v[j] = hc_ex2(v[j] - mx);
-              v[j + 1] = hc_ex2(v[j + 1] - mx);
+              v[j] = hc_ex2(v[j] - m);
+              v[j + 1] = hc_ex2(v[j + 1] - m);
               s0 += v[j];
               s1 += v[j + 1];
             }
-            sum += s0 + s1;
+            sum[hv * (64 / ELL - 1)] += s0 + s1;
           }
 #pragma unroll
           for (int c8 = 0; c8 < 4; ++c8) {
@@ -371,7 +380,9 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
           }
         }
         // the exponentials go to the value mix unnormalised; O is divided by the row sum of its head afterwards
-        inv_sum[(c * 2 + hh) * 128 + (int)r] = p.silu ? 1.0f : __fdividef(1.0f, sum);
+#pragma unroll
+        for (int i = 0; i < 64 / ELL; ++i)
+          inv_sum[(c * HPG + hh * (64 / ELL) + i) * 128 + (int)r] = p.silu ? 1.0f : __fdividef(1.0f, sum[i]);
         tc_fence_before();
         fence_proxy_async_smem();
         __syncwarp();
@@ -508,18 +519,19 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
 }
 
 bool hist_update_d256_tc_supported(int dtype, int d, int f, int H, int ell, int phi, int gated_mlp) {
-  return dtype == LIME_BF16 && d == HC_D && f == HC_F && ell == HC_ELL && (H == 2 || H == 4 || H == 8) &&
+  return dtype == LIME_BF16 && d == HC_D && f == HC_F && ((ell == 64 && H == 2) || ((ell == 64 || ell == 32) && (H == 4 || H == 8))) &&
          (phi == LIME_PHI_SOFTMAX || phi == LIME_PHI_SILU) && gated_mlp != 0;
 }
 
-lime_status launch_hist_update_d256_tc(const HistUpdate256Args& a, cudaStream_t st) {
+template <int ELL>
+static lime_status launch_hist_update_d256_t(const HistUpdate256Args& a, cudaStream_t st) {
   if (a.total == 0) return LIME_OK;
-  const int HL = a.H * HC_ELL;
+  const int HL = a.H * ELL;
   CUtensorMap tmX, tmK2, tmV, tmWgu, tmWo;
   const uint64_t users = a.shared ? 1 : (uint64_t)a.B;
   if (!make_tmap_bf16_sw128(&tmX, a.hist_in, (uint64_t)a.total, HC_D, HC_D, HC_TILE) ||
       !make_tmap_bf16_sw128(&tmK2, a.K2, users * HL, HC_D, HC_D, 128) ||
-      !make_tmap_bf16_sw128(&tmV, a.V2t, users * HC_D, HC_ELL, HC_ELL, 256) ||
+      !make_tmap_bf16_kmajor(&tmV, a.V2t, users * HC_D, ELL, ELL, 256, ELL) ||
       !make_tmap_bf16_sw128(&tmWgu, a.WguT, 2 * HC_F, HC_D, HC_D, 128) ||
       !make_tmap_bf16_sw128(&tmWo, a.WoT, HC_D, HC_F, HC_F, 128))
     return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
@@ -529,12 +541,16 @@ lime_status launch_hist_update_d256_tc(const HistUpdate256Args& a, cudaStream_t 
   int grid = a.n_tile_upper < kSMs ? a.n_tile_upper : kSMs;
   if (grid < 1) return LIME_OK;
   static bool smem_set[kMaxDeviceOrdinals] = {};
-  lime_status es = ensure_dynamic_smem((const void*)k_hist_update_d256_tc, (int)HC_SMEM, smem_set);
+  lime_status es = ensure_dynamic_smem((const void*)k_hist_update_d256_tc<ELL>, (int)HC_SMEM, smem_set);
   if (es != LIME_OK) return es;
   ProfScope _p("k_hist_update_d256_tc", st);
-  k_hist_update_d256_tc<<<grid, HC_THREADS, HC_SMEM, st>>>(tmX, tmK2, tmV, tmWgu, tmWo, p);
+  k_hist_update_d256_tc<ELL><<<grid, HC_THREADS, HC_SMEM, st>>>(tmX, tmK2, tmV, tmWgu, tmWo, p);
   LIME_LAUNCH_CHECK("k_hist_update_d256_tc");
   return LIME_OK;
+}
+
+lime_status launch_hist_update_d256_tc(const HistUpdate256Args& a, cudaStream_t st) {
+  return a.ell == 32 ? launch_hist_update_d256_t<32>(a, st) : launch_hist_update_d256_t<64>(a, st);
 }
 
 }  // namespace lime

@@ -11,6 +11,10 @@
 // Same streaming structure as k_score_tc.cu: warp 0 TMA producer (candidate tile + weight rows into a ring of stages,
 // the user's LSW into its own one or two buffers), warp 1 MMA issuer, warps 2-5 epilogue (thread r = candidate row r =
 // TMEM lane r: bias, ReLU and the n1-term dot with w_2 in registers).
+// With GATHER the candidates are rows of the corpus caches named by cand_ids: the whole of warp 0 produces, lane g fetching
+// rows 4 g .. 4 g + 3 of the tile by the gather form of the copy (one row high box, four row indices), both operands in the
+// swizzle their MMA expects.  An id outside the caches fetches row 0 and its slot scores 0.  (64 users x 500 candidates by id,
+// d = 256, ell = 32, n1 = 96: 308 us on the CUDA-core scorer before.)
 #include "lime_common.cuh"
 #include "tc_common.cuh"
 
@@ -20,6 +24,9 @@ constexpr int SH_TILE = 128, SH_THREADS = 192, SH_MAX_STAGES = 6;
 
 struct ScoreHeadParams {
   float* logits;
+  const int32_t* ids;    // GATHER: [B x C] rows of the caches
+  int32_t* flag;         // nullable: smallest slot whose id was outside [0, V)
+  int V;
   const float* b1;       // [n1] or NULL
   const float* w2;       // [n1]
   const float* b2;       // [1] or NULL
@@ -29,7 +36,7 @@ struct ScoreHeadParams {
   int* err;
 };
 
-template <int ELL>
+template <int ELL, bool GATHER>
 __global__ void __launch_bounds__(SH_THREADS, 1)
 k_score_head_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmW,
                 const __grid_constant__ CUtensorMap tmLSW, const __grid_constant__ CUtensorMap tmW1b, const ScoreHeadParams p) {
@@ -90,31 +97,63 @@ k_score_head_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0 && t_begin < t_end) {
+    if ((GATHER || lane == 0) && t_begin < t_end) {
       const uint64_t pol_stream = policy_evict_first(), pol_keep = policy_evict_last();
-      mbar_arrive_expect_tx(w1b_full, w1b_bytes);
-      for (int kb = 0; kb < KB; ++kb) tma_load_2d_hint(w1b_base + (size_t)kb * n1 * 128, &tmW1b, kb * 64, 0, w1b_full, pol_keep);
+      if (lane == 0) {
+        mbar_arrive_expect_tx(w1b_full, w1b_bytes);
+        for (int kb = 0; kb < KB; ++kb) tma_load_2d_hint(w1b_base + (size_t)kb * n1 * 128, &tmW1b, kb * 64, 0, w1b_full, pol_keep);
+      }
+      // GATHER: this lane's four rows of a tile (row 0 stands in past the user's last candidate and for a bad id)
+      auto read_ids = [&](int t, int (&id)[4]) {
+        const int b = t / p.tiles_per_user, c = (t % p.tiles_per_user) * SH_TILE + 4 * lane;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          id[i] = (t < t_end && c + i < p.C) ? __ldg(p.ids + (int64_t)b * p.C + c + i) : 0;
+          if (id[i] < 0 || id[i] >= p.V) id[i] = 0;
+        }
+      };
+      // the lanes of a gathering warp go on or give up together
+      auto all = [](bool w) { return GATHER ? __all_sync(0xffffffffu, w) != 0 : w; };
+      int id_now[4] = {0, 0, 0, 0}, id_next[4] = {0, 0, 0, 0};
+      if constexpr (GATHER) read_ids(t_begin, id_next);
       int it = 0, un = 0, prev_user = -1;
       bool ok = true;
       for (int t = t_begin; t < t_end && ok; ++t, ++it) {
         const int b = t / p.tiles_per_user;
+        if constexpr (GATHER) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) id_now[i] = id_next[i];
+          read_ids(t + 1, id_next);
+        }
         if (b != prev_user) {
           const int lb = un % LB;
-          if (!mbar_wait(&lsw_empty[lb], ((uint32_t)(un / LB) & 1u) ^ 1u, p.err, 101)) { ok = false; break; }
-          mbar_arrive_expect_tx(&lsw_full[lb], (uint32_t)n1 * ELL * 2);
-          for (int kb = 0; kb < WKB; ++kb)
-            tma_load_2d_hint(lsw_base + (size_t)lb * lsw_bytes + (size_t)kb * n1 * W_ROW, &tmLSW, kb * WK, b * n1, &lsw_full[lb], pol_keep);
+          if (!all(mbar_wait(&lsw_empty[lb], ((uint32_t)(un / LB) & 1u) ^ 1u, p.err, 101))) { ok = false; break; }
+          if (lane == 0) {
+            mbar_arrive_expect_tx(&lsw_full[lb], (uint32_t)n1 * ELL * 2);
+            for (int kb = 0; kb < WKB; ++kb)
+              tma_load_2d_hint(lsw_base + (size_t)lb * lsw_bytes + (size_t)kb * n1 * W_ROW, &tmLSW, kb * WK, b * n1, &lsw_full[lb], pol_keep);
+          }
           ++un;
           prev_user = b;
         }
         const int s = it % S;
-        if (!mbar_wait(&empty[s], ((uint32_t)(it / S) & 1u) ^ 1u, p.err, 102)) { ok = false; break; }
-        const int row0 = b * p.C + (t % p.tiles_per_user) * SH_TILE;
+        if (!all(mbar_wait(&empty[s], ((uint32_t)(it / S) & 1u) ^ 1u, p.err, 102))) { ok = false; break; }
         uint8_t* st = smem + (size_t)s * stage_bytes;
-        mbar_arrive_expect_tx(&full[s], stage_bytes);
-        for (int kb = 0; kb < KB; ++kb) tma_load_2d_hint(st + (size_t)kb * SH_TILE * 128, &tmT, kb * 64, row0, &full[s], pol_stream);
-        for (int kb = 0; kb < WKB; ++kb)
-          tma_load_2d_hint(st + t_bytes + (size_t)kb * SH_TILE * W_ROW, &tmW, kb * WK, row0, &full[s], pol_stream);
+        if (lane == 0) mbar_arrive_expect_tx(&full[s], stage_bytes);
+        if constexpr (GATHER) {
+          __syncwarp();                            // the stage's bytes are announced before any lane's copy can land
+          for (int kb = 0; kb < KB; ++kb)
+            tma_gather4_2d_hint(st + (size_t)kb * SH_TILE * 128 + (size_t)lane * 512, &tmT, kb * 64, id_now[0], id_now[1], id_now[2],
+                                id_now[3], &full[s], pol_stream);
+          for (int kb = 0; kb < WKB; ++kb)
+            tma_gather4_2d_hint(st + t_bytes + (size_t)kb * SH_TILE * W_ROW + (size_t)lane * (4 * W_ROW), &tmW, kb * WK, id_now[0],
+                                id_now[1], id_now[2], id_now[3], &full[s], pol_stream);
+        } else {
+          const int row0 = b * p.C + (t % p.tiles_per_user) * SH_TILE;
+          for (int kb = 0; kb < KB; ++kb) tma_load_2d_hint(st + (size_t)kb * SH_TILE * 128, &tmT, kb * 64, row0, &full[s], pol_stream);
+          for (int kb = 0; kb < WKB; ++kb)
+            tma_load_2d_hint(st + t_bytes + (size_t)kb * SH_TILE * W_ROW, &tmW, kb * WK, row0, &full[s], pol_stream);
+        }
       }
       if (!ok || *(volatile int*)p.err != 0) {
         // giving up: let the copies already issued land (bounded) before this CTA's shared memory goes away
@@ -193,7 +232,18 @@ k_score_head_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tmem_empty[buf]);
-      if (c0 + r < p.C) p.logits[(int64_t)b * p.C + c0 + r] = (acc4[0] + acc4[1]) + (acc4[2] + acc4[3]) + b2;
+      if (c0 + r < p.C) {
+        const int64_t slot = (int64_t)b * p.C + c0 + r;
+        float logit = (acc4[0] + acc4[1]) + (acc4[2] + acc4[3]) + b2;
+        if constexpr (GATHER) {
+          const int32_t id = __ldg(p.ids + slot);
+          if (id < 0 || id >= p.V) {
+            logit = 0.f;
+            if (p.flag != nullptr) atomicMin(p.flag, (int32_t)slot);
+          }
+        }
+        p.logits[slot] = logit;
+      }
     }
   }
 
@@ -223,7 +273,7 @@ static bool score_head_plan(int ell, int d, int n1, int* stages, int* lsw_bufs, 
 }
 
 bool score_head_tc_supported(const ScoreArgs& a, int n1) {
-  if (a.dtype != LIME_BF16 || a.cand_off != nullptr || a.cand_ids != nullptr) return false;
+  if (a.dtype != LIME_BF16 || a.cand_off != nullptr) return false;
   if (!(a.ell == 32 || a.ell == 64 || a.ell == 128)) return false;
   if (a.d % 64 != 0 || a.d > 512) return false;
   if (n1 % 16 != 0 || n1 < 16 || n1 > 256) return false;
@@ -233,36 +283,39 @@ bool score_head_tc_supported(const ScoreArgs& a, int n1) {
   return score_head_plan(a.ell, a.d, n1, &S, &lb, &smem);
 }
 
-template <int ELL>
+template <int ELL, bool GATHER>
 static lime_status launch_score_head_tc_t(const ScoreArgs& a, const ScoreHeadArgs& h, int* err, cudaStream_t st) {
   int S, lb;
   size_t smem;
   if (!score_head_plan(ELL, a.d, h.n1, &S, &lb, &smem)) return LIME_UNSUPPORTED_SHAPE;
   constexpr int WK = ELL > 64 ? 64 : ELL;
   CUtensorMap tmT, tmW, tmLSW, tmW1b;
-  if (!make_tmap_bf16_sw128(&tmT, a.T, (uint64_t)a.total, (uint64_t)a.d, (uint64_t)a.d, SH_TILE) ||
-      !make_tmap_bf16_kmajor(&tmW, a.W, (uint64_t)a.total, ELL, ELL, SH_TILE, WK) ||
+  const uint64_t rows = (uint64_t)(GATHER ? a.corpus_rows : a.total);
+  const uint32_t box = GATHER ? 1 : SH_TILE;
+  if (!make_tmap_bf16_sw128(&tmT, a.T, rows, (uint64_t)a.d, (uint64_t)a.d, box) ||
+      !make_tmap_bf16_kmajor(&tmW, a.W, rows, ELL, ELL, box, WK) ||
       !make_tmap_bf16_kmajor(&tmLSW, h.LSWt, (uint64_t)a.B * h.n1, ELL, ELL, (uint32_t)h.n1, WK) ||
       !make_tmap_bf16_sw128(&tmW1b, h.W1bT, (uint64_t)h.n1, (uint64_t)a.d, (uint64_t)a.d, (uint32_t)h.n1))
     return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
   ScoreHeadParams p;
+  p.ids = a.cand_ids; p.flag = a.dev_flag; p.V = (int)a.corpus_rows;
   p.logits = a.logits; p.b1 = h.b1; p.w2 = h.w2; p.b2 = h.b2; p.B = a.B; p.C = a.C; p.d = a.d; p.n1 = h.n1;
   p.tiles_per_user = (a.C + SH_TILE - 1) / SH_TILE;
   p.n_tiles = p.tiles_per_user * a.B;
   p.stages = S; p.lsw_bufs = lb; p.err = err;
   const int grid = p.n_tiles < kSMs ? p.n_tiles : kSMs;
-  LIME_CUDA(cudaFuncSetAttribute(k_score_head_tc<ELL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  LIME_CUDA(cudaFuncSetAttribute(k_score_head_tc<ELL, GATHER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   ProfScope _p("k_score_head_tc", st);
-  k_score_head_tc<ELL><<<grid, SH_THREADS, smem, st>>>(tmT, tmW, tmLSW, tmW1b, p);
+  k_score_head_tc<ELL, GATHER><<<grid, SH_THREADS, smem, st>>>(tmT, tmW, tmLSW, tmW1b, p);
   LIME_LAUNCH_CHECK("k_score_head_tc");
   return LIME_OK;
 }
 
 lime_status launch_score_head_tc(const ScoreArgs& a, const ScoreHeadArgs& h, int* err, cudaStream_t st) {
   switch (a.ell) {
-    case 32: return launch_score_head_tc_t<32>(a, h, err, st);
-    case 64: return launch_score_head_tc_t<64>(a, h, err, st);
-    case 128: return launch_score_head_tc_t<128>(a, h, err, st);
+    case 32: return a.cand_ids ? launch_score_head_tc_t<32, true>(a, h, err, st) : launch_score_head_tc_t<32, false>(a, h, err, st);
+    case 64: return a.cand_ids ? launch_score_head_tc_t<64, true>(a, h, err, st) : launch_score_head_tc_t<64, false>(a, h, err, st);
+    case 128: return a.cand_ids ? launch_score_head_tc_t<128, true>(a, h, err, st) : launch_score_head_tc_t<128, false>(a, h, err, st);
   }
   return LIME_UNSUPPORTED_SHAPE;
 }

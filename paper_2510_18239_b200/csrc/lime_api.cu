@@ -188,7 +188,7 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
   if (hist_out && c->tc_mode == 2) {
     HistUpdate256Args hu{};
     hu.hist_in = hist_in; hu.hist_out = hist_out; hu.total = total; hu.K2 = ops.K2; hu.V2t = ops.V2t; hu.WguT = c->WguT[layer];
-    hu.WoT = c->WoT[layer]; hu.off = off; hu.tile_start = w.tile_start; hu.B = B; hu.n_tile_upper = w.n_tile_upper; hu.H = g.H;
+    hu.WoT = c->WoT[layer]; hu.off = off; hu.tile_start = w.tile_start; hu.B = B; hu.n_tile_upper = w.n_tile_upper; hu.H = g.H; hu.ell = g.ell;
     hu.shared = ops.shared; hu.out_ln = out_ln; hu.silu = g.phi == LIME_PHI_SILU; hu.ln_eps = c->ln_eps; hu.err = c->dev_err;
     if ((s = launch_hist_update_d256_tc(hu, st)) != LIME_OK) return s;
   } else if (hist_out) {

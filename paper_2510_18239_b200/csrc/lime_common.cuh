@@ -331,7 +331,7 @@ lime_status launch_hist_update_tc(const HistUpdateArgs& a, cudaStream_t st);
 bool hist_update2_tc_supported(int dtype, int d, int f, int H, int ell, int phi, int gated_mlp);
 lime_status launch_hist_update2_tc(const HistUpdateArgs& a, int H, cudaStream_t st);
 
-// ---- tensor-core XOR layer at d = d_ff = 256 (bf16, ell = 64, H in {2, 4, 8}; history rows LayerNorm-ed already) ----
+// ---- tensor-core XOR layer at d = d_ff = 256 (bf16; ell = 64 with H in {2, 4, 8}, ell = 32 with H in {4, 8}; history rows LayerNorm-ed already) ----
 bool link_attn_d256_tc_supported(int dtype, int d, int H, int ell, int phi);
 lime_status launch_link_attn_d256_tc(const LinkAttnArgs& a, cudaStream_t st);   // a.ln must be 0
 
@@ -341,7 +341,7 @@ struct HistUpdate256Args {
   const void* V2t;                      // link values, transposed [users x d x ell] bf16
   const void* WguT; const void* WoT;    // [W_g | W_u]^T [2f x d] and W_o^T [d x f], bf16
   const int32_t* off; const int32_t* tile_start; int B, n_tile_upper;
-  int H, shared;
+  int H, ell, shared;
   int out_ln;                           // 1: store LayerNorm(S') instead of S'
   int silu;                             // 1: SiLU(s) / ell instead of the per-head softmax (Algorithm 2)
   float ln_eps;

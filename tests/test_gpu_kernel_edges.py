@@ -46,3 +46,77 @@ def test_score_lists_by_warp(d, ell, counts, by_id):
     assert np.abs(got - want).max() <= 1e-4 * max(1.0, np.abs(want).max())
     if by_id:
         assert np.all(got[~ok] == 0.0) and int(flag.item()) == total // 2
+
+
+def _layer_against_oracle(dtype, d, H, ell, lengths, shared, phi, tol_max, tol_mean):
+    """One XOR layer with a history update, per user against the oracle."""
+    Bd = _lib()
+    B, total = len(lengths), int(sum(lengths))
+    wl = synth.Workload("edge", B=B, n_min=0, n_max=1, d=d, H=H, ell=ell, n_layers=1, C=1, dtype=dtype, V=3000, zipf_s=1.1,
+                        table_std=0.05, link_std=1.0)
+    inp = synth.make_inputs(wl, seed=H + B)
+    inp["lengths"] = np.asarray(lengths, dtype=np.int32)
+    inp["hist_ids"] = synth.zipf_ids(3, "h", total, wl.V, 1.1)
+    dev = Hh.DeviceBatch(wl, inp, phi=Bd.LIME_PHI_SILU if phi == "silu" else Bd.LIME_PHI_SOFTMAX)
+    L = dev.lime
+    off = L.lengths_to_offsets(dev.lengths)
+    hist = L.gather_history(dev.table, dev.hist_ids)
+    if shared:
+        links_np = synth.storage_to_f64(inp["links"], dtype)[None].repeat(B, axis=0)
+        links32 = dev.links.float().contiguous()
+    else:
+        links_np = np.random.default_rng(9).normal(size=(B, ell, d)).astype(np.float32).astype(np.float64)
+        links32 = torch.from_numpy(links_np.astype(np.float32)).cuda()
+    hist_out = torch.zeros_like(hist)
+    links_out = torch.empty((B, ell, d), dtype=torch.float32, device="cuda")
+    Bd.lime_xor_layer(L.ctx, 0, hist, off, B, links32, shared, hist_out if total else None, links_out, L.workspace(B, total))
+    assert Bd.lime_device_status(L.ctx) == 0
+    cfg = Hh.oracle_config(wl, phi=O.SILU if phi == "silu" else O.SOFTMAX)
+    lw = Hh.oracle_layers(inp, wl)[0]
+    table64 = synth.storage_to_f64(inp["table"], dtype)
+    offh = O.lengths_to_offsets(lengths)
+    for b in range(B):
+        E = O.gather_history(table64, inp["hist_ids"][offh[b]:offh[b + 1]])
+        S_next, T_next = O.xor_layer(E, links_np[b], lw, cfg)
+        pairs = [(Hh.to_f64(links_out[b]), T_next)]
+        if lengths[b]:
+            pairs.append((Hh.to_f64(hist_out[offh[b]:offh[b + 1]]), S_next))
+        for got, want in pairs:
+            assert np.abs(got - want).max() <= tol_max * max(1.0, np.abs(want).max()), (b, np.abs(got - want).max())
+            assert np.abs(got - want).mean() <= tol_mean * max(want.std(), 1e-6) + 1e-5, (b, np.abs(got - want).mean())
+
+
+@pytest.mark.parametrize("H", [4, 8])
+@pytest.mark.parametrize("lengths", [[1], [0, 63, 65, 127, 129, 300], [256] * 40])
+@pytest.mark.parametrize("shared,phi", [(True, "softmax"), (False, "softmax"), (False, "silu")])
+def test_xor_layer_d256_with_32_links(H, lengths, shared, phi):
+    _layer_against_oracle(synth.BF16, 256, H, 32, lengths, shared, phi, 4e-2, 1e-2)
+
+
+@pytest.mark.parametrize("d,ell,n1,B,C", [(256, 32, 96, 3, 129), (128, 64, 128, 2, 1), (64, 128, 16, 40, 260)])
+def test_interaction_head_by_id_on_tensor_cores(d, ell, n1, B, C):
+    Bd = _lib()
+    dtype, V = synth.BF16, 300
+    r = np.random.default_rng(d + C)
+    LS, W, T = (synth.to_storage(x, dtype) for x in (r.normal(size=(B, ell, d)) * 0.5, O.softmax_rows(r.normal(size=(V, ell))),
+                                                     r.normal(size=(V, d)) * 0.5))
+    lime = Bd.Lime(d, 4, ell, 1, dtype=Bd.LIME_BF16)
+    layers = synth.ffn_weights(5, "head", (2 * d, n1, 1), dtype)
+    lime.set_head([(Bd.to_device(w, dtype), torch.from_numpy(b).cuda()) for w, b in layers])
+    ids = r.integers(0, V, size=B * C).astype(np.int32)
+    ids[B * C // 2], ids[-1] = V, -1
+    flag = torch.full((1,), 2 ** 31 - 1, dtype=torch.int32, device="cuda")
+    got = Hh.to_f64(lime.score_candidates_head(Bd.to_device(LS, dtype), Bd.to_device(W, dtype), Bd.to_device(T, dtype), C=C,
+                                               cand_ids=torch.from_numpy(ids).cuda(), dev_flag=flag))
+    Bd.lime_device_status(lime.ctx)
+    L64 = [(synth.storage_to_f64(w, dtype), b.astype(np.float64)) for w, b in layers]
+    W64, T64, LS64 = (synth.storage_to_f64(x, dtype) for x in (W, T, LS))
+    ok = (ids >= 0) & (ids < V)
+    want = np.zeros(B * C)
+    for b in range(B):
+        s = np.arange(b * C, (b + 1) * C)
+        s = s[ok[s]]
+        if s.size:
+            want[s] = O.score_candidates_head(W64[ids[s]], LS64[b], T64[ids[s]], L64)
+    assert np.abs(got - want).max() <= 2e-2 and np.abs(got - want).max() <= 3e-2 * want.std() + 1e-3
+    assert np.all(got[~ok] == 0.0) and int(flag.item()) == B * C // 2
