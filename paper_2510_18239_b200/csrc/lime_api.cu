@@ -60,6 +60,12 @@ static int tensor_core_mode(const lime_config& g, int d_ff) {
     return 2;
   return 0;
 }
+// One block per user serves histories of ordinary length; a few very long ones leave most SMs idle and take the generic
+// kernels, which split them.
+static bool encode_small_wanted(const Ctx* c, int32_t B, int64_t total) {
+  const lime_config& g = c->cfg;
+  return encode_small_supported(g.dtype, g.d, c->d_ff, g.H, g.ell, g.gated_mlp) && total <= 2048ll * B;
+}
 constexpr int kHistTile = 128;  // tokens per block of the history<-links attention
 
 struct Workspace {
@@ -613,9 +619,20 @@ static lime_status encode_user_impl(lime_ctx* ctx, const void* hist, bool hist_n
   if (w.bytes + pad > ws_bytes) return LIME_WORKSPACE_TOO_SMALL;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   lime_status s;
-  if ((s = launch_layer_schedules(off, B, w.chunk, w.chunk_start, kHistTile, w.tile_start, w.chunk_user, w.merge_needed, w.groups, st)) != LIME_OK) return s;
+  const bool narrow = encode_small_wanted(c, B, total_tokens);
+  if (!narrow && (s = launch_layer_schedules(off, B, w.chunk, w.chunk_start, kHistTile, w.tile_start, w.chunk_user, w.merge_needed, w.groups, st)) != LIME_OK) return s;
   const int64_t BLd = (int64_t)B * g.ell * g.d;
-  if (layer_on_tensor_cores(c, 0)) {
+  if (narrow) {
+    EncodeSmallArgs a{};
+    a.hist = hist; a.off = off; a.B = B; a.total = total_tokens; a.links = link_ctx ? link_ctx : c->links32; a.links_per_user = link_ctx != nullptr;
+    a.w = &c->w; a.scale = c->attn_scale;
+    a.H = g.H; a.ell = g.ell; a.n_layers = g.n_layers; a.ln = g.ln; a.hist_ln = g.ln && !hist_normalized; a.silu = g.phi == LIME_PHI_SILU;
+    a.eps = c->ln_eps; a.scratch = w.S;
+    const bool direct = !c->w.cand_Wv && c->cand_heads == 1;
+    a.link_states = direct ? link_states : nullptr; a.lp = w.LP;
+    if ((s = launch_encode_small(a, st)) != LIME_OK) return s;
+    if (direct) return LIME_OK;
+  } else if (layer_on_tensor_cores(c, 0)) {
     if ((s = encode_user_tc(c, hist, hist_normalized, off, B, total_tokens, link_ctx, link_states, w, st)) != LIME_OK) return s;
     if (!c->w.cand_Wv && c->cand_heads == 1) return LIME_OK;        // the last layer's kernel wrote the link states
   } else {

@@ -236,6 +236,18 @@ lime_status launch_score_gather_tc(const ScoreArgs& a, int* err, cudaStream_t st
 bool score_rows_preferred(const ScoreArgs& a);
 lime_status launch_score_rows(const ScoreArgs& a, cudaStream_t st);
 
+// the whole encode of a narrow model (bf16, d = d_ff = 32) in one launch, one block per user (k_encode_small.cu)
+struct EncodeSmallArgs {
+  const void* hist; const int32_t* off; int B; int64_t total;
+  const float* links; int links_per_user;      // T^0: [ell x d] fp32, or [B x ell x d]
+  const lime_weights* w;                       // as the caller gave them
+  int H, ell, n_layers, ln, hist_ln, silu; float eps, scale;
+  void* scratch;                               // [total x d] bf16, for histories beyond shared memory
+  void* link_states; float* lp;                // bf16 link states, or (link_states NULL) L^P in fp32
+};
+bool encode_small_supported(int dtype, int d, int d_ff, int H, int ell, int gated_mlp);
+lime_status launch_encode_small(const EncodeSmallArgs& a, cudaStream_t st);
+
 // one-thread kernel whose only wait can never be satisfied (self-test of the bounded waits, tc_host.cu)
 lime_status launch_wait_expiry(int* err, uint64_t limit_ns, int code, cudaStream_t st);
 
