@@ -805,6 +805,7 @@ lime_status lime_score_candidates_head(lime_ctx* ctx, const void* link_states, i
   a.LS = link_states; a.W = cand_w; a.T = cand_emb; a.dtype = g.dtype; a.B = B; a.ell = c->ell_c; a.d = g.d;
   a.cand_off = cand_off; a.C = C; a.total = total_cands; a.cand_ids = cand_ids; a.logits = logits;
   a.corpus_rows = cand_ids ? corpus_rows : 0; a.dev_flag = cand_ids ? dev_flag : nullptr;
+  if (score_mlp3_supported(a, f)) return launch_score_mlp3(a, f, st);
   const bool tc = f.n_hidden == 1 && c->head_W1bT && score_head_tc_supported(a, w0);
   // per user: LSW_b = LS_b W_0[:d]  (the O half of the first layer applied to the link states, so O is never formed)
   lime_status s;

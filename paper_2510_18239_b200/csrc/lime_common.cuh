@@ -274,6 +274,10 @@ struct ScoreHeadArgs {
 bool score_head_tc_supported(const ScoreArgs& a, int n1);
 lime_status launch_score_head_tc(const ScoreArgs& a, const ScoreHeadArgs& h, int* err, cudaStream_t st);
 
+// three hidden layers (w0 <= 512, 128, 64) at d = 32, any candidate form (k_score_mlp3.cu)
+bool score_mlp3_supported(const ScoreArgs& a, const lime_ffn& f);
+lime_status launch_score_mlp3(const ScoreArgs& a, const lime_ffn& f, cudaStream_t st);
+
 // ---- tensor-core XOR layer (bf16, d = d_ff = 128, H * ell = 128) ----------------------------------------------
 // plain_v: WprepT's third segment is W_V^T (link values formed as they stand) instead of the folded gate / up products
 lime_status launch_fold_weights(const void* Wq, const void* Wk, const void* Wv, const void* Wg, const void* Wu, int d,

@@ -163,3 +163,39 @@ def test_narrow_encode_in_one_launch(H, ell, lengths, phi, raw, per_user):
     """d = 32: 16-token tiles, an empty history, one too long for shared memory (its rows stay in global memory)."""
     # SiLU weights are not normalised: stacked layers grow and with them the error of the stored rows
     _encode_against_oracle(synth.BF16, 32, H, ell, 3, lengths, phi, raw, per_user, 6e-2, 4e-2 if phi == "silu" else 1.5e-2)
+
+
+@pytest.mark.parametrize("ell,w0", [(8, 64), (16, 512), (32, 128)])
+@pytest.mark.parametrize("counts,form", [([1], "ids"), ([33, 0, 5, 300], "lists"), ([100] * 5, "ids"), ([17] * 3, "dense")])
+def test_three_layer_interaction_network(ell, w0, counts, form):
+    """d = 32 with hidden widths (w0, 128, 64): 32-slot steps, several users in one step, users without candidates, bad ids."""
+    Bd = _lib()
+    d, dtype, B, V, total = 32, synth.BF16, len(counts), 300, int(sum(counts))
+    r = np.random.default_rng(ell + total)
+    rows = total if form == "dense" else V
+    LS, W, T = (synth.to_storage(x, dtype) for x in (r.normal(size=(B, ell, d)) * 0.5, O.softmax_rows(r.normal(size=(rows, ell)) * 1.5),
+                                                     r.normal(size=(rows, d)) * 0.5))
+    lime = Bd.Lime(d, 4, ell, 1, dtype=Bd.LIME_BF16)
+    layers = synth.ffn_weights(5, "head", (2 * d, w0, 128, 64, 1), dtype)
+    lime.set_head([(Bd.to_device(w, dtype), torch.from_numpy(b).cuda()) for w, b in layers])
+    ids = np.arange(total, dtype=np.int32) if form == "dense" else r.integers(0, V, size=total).astype(np.int32)
+    if form != "dense":
+        ids[total // 2], ids[-1] = V, -1
+    off = O.lengths_to_offsets(np.asarray(counts))
+    flag = torch.full((1,), 2 ** 31 - 1, dtype=torch.int32, device="cuda")
+    got = Hh.to_f64(lime.score_candidates_head(Bd.to_device(LS, dtype), Bd.to_device(W, dtype), Bd.to_device(T, dtype),
+                                               C=0 if form == "lists" else counts[0], total_cands=total, dev_flag=flag,
+                                               cand_off=torch.from_numpy(off.astype(np.int32)).cuda() if form == "lists" else None,
+                                               cand_ids=None if form == "dense" else torch.from_numpy(ids).cuda()))
+    L64 = [(synth.storage_to_f64(w, dtype), b.astype(np.float64)) for w, b in layers]
+    W64, T64, LS64 = (synth.storage_to_f64(x, dtype) for x in (W, T, LS))
+    ok = (ids >= 0) & (ids < rows)
+    want = np.zeros(total)
+    for b in range(B):
+        s = np.arange(off[b], off[b + 1])
+        s = s[ok[s]]
+        if s.size:
+            want[s] = O.score_candidates_head(W64[ids[s]], LS64[b], T64[ids[s]], L64)
+    assert np.abs(got - want).max() <= 2e-2 and np.abs(got - want).max() <= 3e-2 * max(want.std(), 0.1) + 1e-3
+    if form != "dense":
+        assert np.all(got[~ok] == 0.0) and int(flag.item()) == total // 2
