@@ -187,6 +187,25 @@ __global__ void k_transpose_bf16(const __nv_bfloat16* __restrict__ W, int rows, 
   }
 }
 
+struct TransposeMany { const __nv_bfloat16* W[6 * LIME_MAX_LAYERS]; };
+__global__ void k_transpose_square_bf16(const TransposeMany p, int d, __nv_bfloat16* __restrict__ out) {
+  __shared__ __nv_bfloat16 t[32][33];
+  const __nv_bfloat16* W = p.W[blockIdx.z];
+  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+  for (int j = threadIdx.y; j < 32; j += blockDim.y) t[j][threadIdx.x] = __float2bfloat16_rn(w_at(W, r0 + j, c0 + threadIdx.x, d));
+  __syncthreads();
+  for (int j = threadIdx.y; j < 32; j += blockDim.y) out[((int64_t)blockIdx.z * d + c0 + j) * d + r0 + threadIdx.x] = t[threadIdx.x][j];
+}
+lime_status launch_transpose_square_bf16(const void* const* W, int n, int d, void* out, cudaStream_t st) {
+  if (n > 6 * LIME_MAX_LAYERS || d % 32) return LIME_INVALID_ARG;
+  TransposeMany p;
+  for (int i = 0; i < n; ++i) p.W[i] = (const __nv_bfloat16*)W[i];
+  ProfScope _p("k_transpose_square_bf16", st);
+  k_transpose_square_bf16<<<dim3(d / 32, d / 32, n), dim3(32, 8), 0, st>>>(p, d, (__nv_bfloat16*)out);
+  LIME_LAUNCH_CHECK("k_transpose_square_bf16");
+  return LIME_OK;
+}
+
 lime_status launch_transpose_bf16(const void* W, int rows, int cols, void* WT, cudaStream_t st) {
   ProfScope _p("k_transpose_bf16", st);
   dim3 grid((cols + 31) / 32, (rows + 31) / 32), block(32, 8);

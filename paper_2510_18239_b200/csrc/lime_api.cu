@@ -133,6 +133,7 @@ static Workspace carve(const Ctx* c, void* base, int32_t B, int64_t total) {
 
 // True when the whole layer runs on the tensor-core kernels (their set-up data exists for this layer).
 static bool layer_on_tensor_cores(const Ctx* c, int layer) {
+  if (c->side256) return c->side_w && c->WoT[layer] && c->WguT[layer];
   return c->tc_mode != 0 && c->WoT[layer] && c->WprepT[layer] && c->WpostT[layer] && (c->tc_mode == 1 || c->WguT[layer]);
 }
 
@@ -143,6 +144,25 @@ struct LinkOperands {
   const float *cQ, *cK;
   int shared;                 // one set for every user (T^0 = L) or one per user
 };
+
+// The weights half of LinkSide256Args: the GatedMLP of `layer` (-1: none) and the operands of layer `next` (-1: none).
+static LinkSide256Args side256_args(const Ctx* c, int layer, int next, int users) {
+  LinkSide256Args a{};
+  const size_t dd = (size_t)c->cfg.d * c->cfg.d * 2;
+  a.users = users; a.H = c->cfg.H; a.ln = c->cfg.ln; a.eps = c->ln_eps; a.err = c->dev_err;
+  a.scale = c->cfg.phi == LIME_PHI_SILU ? 1.0f : c->attn_scale * 1.4426950408889634f;
+  if (layer >= 0) {
+    a.WvT = static_cast<const char*>(c->side_w) + ((size_t)layer * 6 + 2) * dd;
+    a.WguT = c->WguT[layer]; a.WoT = c->WoT[layer];
+  }
+  if (next >= 0) {
+    const char* at = static_cast<const char*>(c->side_w) + (size_t)next * 6 * dd;
+    a.WqT = at; a.WkT = at + dd; a.WvT_next = at + 2 * dd;
+    a.Wq = c->w.Wq[next] ? c->w.Wq[next] : a.WqT;          // NULL stands for the identity, its own transpose
+    a.Wk = c->w.Wk[next] ? c->w.Wk[next] : a.WkT;
+  }
+  return a;
+}
 
 // LN(links_in) -> bf16 -> PREP GEMM: the operands of `layer` for `rows` link rows, written to the given buffers.
 static lime_status make_link_operands(Ctx* c, int layer, const void* That, int64_t rows, int need_hist, void* Q2, void* K2,
@@ -163,7 +183,7 @@ static lime_status make_link_operands(Ctx* c, int layer, const void* That, int64
 // read (0 when they were stored normalised by the previous layer); `out_ln`: store LayerNorm(S').
 static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const int32_t* off, int32_t B, int64_t total,
                                  const LinkOperands& ops, void* hist_out, int hist_ln, int out_ln, LinkMlpArgs mlp,
-                                 const Workspace& w, cudaStream_t st) {
+                                 const LinkSide256Args* side, const Workspace& w, cudaStream_t st) {
   const lime_config& g = c->cfg;
   lime_status s;
   if (c->tc_mode == 2 && hist_ln && total > 0) {
@@ -185,12 +205,19 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
   const bool pass_stats = hist_ln && hist_out && one_block_update && total > 0;
   la.stats_out = pass_stats ? w.row_stats : nullptr;
   if ((s = c->tc_mode == 2 ? launch_link_attn_d256_tc(la, st) : launch_link_attn_tc(la, st)) != LIME_OK) return s;
+  if (c->side256) {
+    // merge, T^j and what follows from it - the next layer's operands included - in one kernel; `side` says what is wanted
+    LinkSide256Args a = *side;
+    a.Ohat = w.Ohat; a.part_m = w.part_m; a.part_s = w.part_s; a.part_acc = w.part_acc; a.chunk_start = w.chunk_start;
+    if ((s = launch_link_side_d256(a, st)) != LIME_OK) return s;
+  } else {
   if ((s = launch_link_attn_merge_norm(w.chunk_start, w.merge_needed, B, g.ell, g.d, g.H, w.part_m, w.part_s, w.part_acc, w.Ohat, st)) != LIME_OK)
     return s;
   // T^j = GatedMLP(O[T]) with W_V folded into the gate / up weights, and what the next step needs from it
   mlp.Ohat = w.Ohat; mlp.M = (int64_t)B * g.ell; mlp.K = g.H * g.d; mlp.d = g.d; mlp.WpostT = c->WpostT[layer]; mlp.WoT = c->WoT[layer];
   mlp.ln = g.ln; mlp.ln_eps = c->ln_eps; mlp.err = c->dev_err;
   if ((s = launch_link_mlp_tc(mlp, st)) != LIME_OK) return s;
+  }
   if (hist_out && c->tc_mode == 2) {
     HistUpdate256Args hu{};
     hu.hist_in = hist_in; hu.hist_out = hist_out; hu.total = total; hu.K2 = ops.K2; hu.V2t = ops.V2t; hu.WguT = c->WguT[layer];
@@ -218,6 +245,15 @@ static lime_status xor_layer_tc(Ctx* c, int layer, const void* hist_in, const in
                                 const Workspace& w, cudaStream_t st) {
   const lime_config& g = c->cfg;
   lime_status s;
+  if (c->side256) {
+    LinkSide256Args prep = side256_args(c, -1, layer, links_shared ? 1 : B), side = side256_args(c, layer, -1, B);
+    prep.T_in = links_in; prep.t_shared = links_shared; prep.need_hist = hist_out != nullptr;
+    prep.Q2 = w.Q2; prep.K2 = w.K2; prep.V2t = w.V2t;
+    if ((s = launch_link_side_d256(prep, st)) != LIME_OK) return s;
+    side.T_out = links_out;
+    return tc_layer_core(c, layer, hist_in, off, B, total, LinkOperands{w.Q2, w.K2, nullptr, nullptr, w.V2t, nullptr, nullptr, links_shared},
+                         hist_out, g.ln, 0, LinkMlpArgs{}, &side, w, st);
+  }
   const int64_t link_rows = links_shared ? g.ell : (int64_t)B * g.ell;
   if ((s = launch_ln_rows_bf16(links_in, link_rows, g.d, g.ln, c->ln_eps, w.That, st)) != LIME_OK) return s;
   if ((s = make_link_operands(c, layer, w.That, link_rows, hist_out != nullptr, w.Q2, w.K2, w.G2t, w.U2t, w.V2t, w.cQ, w.cK, st)) != LIME_OK)
@@ -225,7 +261,7 @@ static lime_status xor_layer_tc(Ctx* c, int layer, const void* hist_in, const in
   LinkOperands ops{w.Q2, w.K2, w.G2t, w.U2t, w.V2t, w.cQ, w.cK, links_shared};
   LinkMlpArgs mlp{};
   mlp.T_out = links_out;
-  return tc_layer_core(c, layer, hist_in, off, B, total, ops, hist_out, g.ln, 0, mlp, w, st);
+  return tc_layer_core(c, layer, hist_in, off, B, total, ops, hist_out, g.ln, 0, mlp, nullptr, w, st);
 }
 
 // lime_encode_user on the tensor-core path: per layer one link-side GEMM (none on the first layer when the links are
@@ -237,6 +273,29 @@ static lime_status encode_user_tc(Ctx* c, const void* hist, bool hist_normalized
   const lime_config& g = c->cfg;
   lime_status s;
   const int64_t BL = (int64_t)B * g.ell;
+  if (c->side256) {
+    // operands of consecutive layers alternate between two sets: layer j's history update still reads its own while the
+    // link side has written those of layer j + 1
+    const LinkOperands set[2] = {{w.Q2, w.K2, nullptr, nullptr, w.V2t, nullptr, nullptr, 0}, {w.G2t, w.U2t, nullptr, nullptr, w.UTb, nullptr, nullptr, 0}};
+    if (link_ctx) {
+      LinkSide256Args prep = side256_args(c, -1, 0, B);
+      prep.T_in = link_ctx; prep.need_hist = g.n_layers > 1; prep.Q2 = w.Q2; prep.K2 = w.K2; prep.V2t = w.V2t;
+      if ((s = launch_link_side_d256(prep, st)) != LIME_OK) return s;
+    }
+    for (int j = 0; j < g.n_layers; ++j) {
+      const bool last = j == g.n_layers - 1;
+      LinkSide256Args side = side256_args(c, j, last ? -1 : j + 1, B);
+      side.LP = w.LP; side.lp_accumulate = j > 0; side.need_hist = j + 1 < g.n_layers - 1;
+      side.link_states = (last && !c->w.cand_Wv && c->cand_heads == 1) ? link_states : nullptr;
+      const LinkOperands& nx = set[(j + 1) & 1];
+      side.Q2 = const_cast<void*>(nx.Q2); side.K2 = const_cast<void*>(nx.K2); side.V2t = const_cast<void*>(nx.V2t);
+      const LinkOperands ops = (j == 0 && !link_ctx) ? LinkOperands{c->sh_Q2, c->sh_K2, nullptr, nullptr, c->sh_V2t, nullptr, nullptr, 1} : set[j & 1];
+      s = tc_layer_core(c, j, j == 0 ? hist : w.S, off, B, total, ops, last ? nullptr : w.S, (g.ln && j == 0 && !hist_normalized) ? 1 : 0,
+                        (g.ln && !last) ? 1 : 0, LinkMlpArgs{}, &side, w, st);
+      if (s != LIME_OK) return s;
+    }
+    return LIME_OK;
+  }
   for (int j = 0; j < g.n_layers; ++j) {
     const bool last = j == g.n_layers - 1;
     LinkOperands ops;
@@ -252,7 +311,7 @@ static lime_status encode_user_tc(Ctx* c, const void* hist, bool hist_normalized
     mlp.That_next = last ? nullptr : w.That;
     mlp.link_states = (last && !c->w.cand_Wv && c->cand_heads == 1) ? link_states : nullptr;
     s = tc_layer_core(c, j, j == 0 ? hist : w.S, off, B, total, ops, last ? nullptr : w.S, (g.ln && j == 0 && !hist_normalized) ? 1 : 0,
-                      (g.ln && !last) ? 1 : 0, mlp, w, st);
+                      (g.ln && !last) ? 1 : 0, mlp, nullptr, w, st);
     if (s != LIME_OK) return s;
   }
   return LIME_OK;
@@ -436,6 +495,8 @@ lime_status lime_create(const lime_config* cfg, lime_ctx** out) {
   c->have_head = c->have_ctx_mlp = false; c->ctx_dc = 0;
   c->head_W1bT = nullptr; c->head_W1aT = nullptr; c->head_w2 = nullptr; c->ctx_first = nullptr;
   c->tc_mode = tensor_core_mode(g, d_ff);
+  c->side256 = c->tc_mode == 2 && link_side_d256_supported(g.d, d_ff, g.H, g.ell);
+  c->side_w = nullptr;
   for (int j = 0; j < LIME_MAX_LAYERS; ++j) c->WoT[j] = c->WprepT[j] = c->WpostT[j] = c->WguT[j] = nullptr;
   c->sh_That = c->sh_Q2 = c->sh_K2 = c->sh_G2t = c->sh_U2t = c->sh_V2t = nullptr; c->sh_cQ = c->sh_cK = nullptr;
   cudaError_t e = cudaGetDevice(&c->device);
@@ -463,10 +524,14 @@ lime_status lime_destroy(lime_ctx* ctx) {
   cudaFree(c->keff_hl);
   cudaFree(c->links32);
   cudaFree(c->dev_err);
+  if (c->side256) {                                    // these lie inside side_w
+    for (int j = 0; j < LIME_MAX_LAYERS; ++j) c->WoT[j] = c->WguT[j] = nullptr;
+    c->sh_Q2 = c->sh_K2 = c->sh_V2t = nullptr;
+  }
   for (int j = 0; j < LIME_MAX_LAYERS; ++j) { cudaFree(c->WoT[j]); cudaFree(c->WprepT[j]); cudaFree(c->WpostT[j]); cudaFree(c->WguT[j]); }
   cudaFree(c->sh_That); cudaFree(c->sh_Q2); cudaFree(c->sh_K2); cudaFree(c->sh_G2t); cudaFree(c->sh_U2t); cudaFree(c->sh_V2t);
   cudaFree(c->sh_cQ); cudaFree(c->sh_cK);
-  cudaFree(c->head_W1bT); cudaFree(c->head_W1aT); cudaFree(c->head_w2); cudaFree(c->ctx_first);
+  cudaFree(c->head_W1bT); cudaFree(c->head_W1aT); cudaFree(c->head_w2); cudaFree(c->ctx_first); cudaFree(c->side_w);
   delete c;
   return LIME_OK;
 }
@@ -491,9 +556,27 @@ lime_status lime_set_weights(lime_ctx* ctx, const lime_weights* w, void* stream)
   if (precompute_tc_supported(g.dtype, g.d, c->ell_c, g.ell) &&
       (s = launch_keff_split(c->keff, c->ell_c, g.d, c->keff_hl, st)) != LIME_OK)
     return s;
-  // tensor-core path: per layer, W_o as a K-major B operand ([d x d_ff], contraction index contiguous) and the
-  // weight-only products that fold the history-side projections into the link rows
-  if (c->tc_mode != 0) {
+  if (c->side256) {
+    // weights transposed, none folded; the first layer's operands for the shared links T^0 = L follow them in one buffer
+    const size_t dd = (size_t)g.d * g.d * 2, HLd = (size_t)g.H * g.ell * g.d * 2;
+    if (!c->side_w) {
+      LIME_CUDA(cudaMalloc(&c->side_w, (size_t)g.n_layers * 6 * dd + 2 * HLd + (size_t)g.d * g.ell * 2));
+      char* at = static_cast<char*>(c->side_w);
+      for (int j = 0; j < g.n_layers; ++j, at += 6 * dd) { c->WguT[j] = at + 3 * dd; c->WoT[j] = at + 5 * dd; }
+      c->sh_Q2 = at; c->sh_K2 = at + HLd; c->sh_V2t = at + 2 * HLd;
+    }
+    const void* src[6 * LIME_MAX_LAYERS];
+    for (int j = 0; j < g.n_layers; ++j) {
+      const void* m[6] = {w->Wq[j], w->Wk[j], w->Wv[j], w->Wg[j], w->Wu[j], w->Wo[j]};
+      memcpy(src + 6 * j, m, sizeof(m));
+    }
+    if ((s = launch_transpose_square_bf16(src, 6 * g.n_layers, g.d, c->side_w, st)) != LIME_OK) return s;
+    LinkSide256Args prep = side256_args(c, -1, 0, 1);
+    prep.T_in = c->links32; prep.t_shared = 1; prep.need_hist = g.n_layers > 1; prep.Q2 = c->sh_Q2; prep.K2 = c->sh_K2; prep.V2t = c->sh_V2t;
+    if ((s = launch_link_side_d256(prep, st)) != LIME_OK) return s;
+  } else if (c->tc_mode != 0) {
+    // tensor-core path: per layer, W_o as a K-major B operand ([d x d_ff], contraction index contiguous) and the
+    // weight-only products that fold the history-side projections into the link rows
     const bool plain_v = c->tc_mode == 2;
     const size_t prep_rows = 2 * (size_t)g.H * g.d + (plain_v ? (size_t)g.d : 2 * (size_t)g.H * c->d_ff);
     auto need = [](void** p, size_t bytes) -> cudaError_t { return *p ? cudaSuccess : cudaMalloc(p, bytes); };

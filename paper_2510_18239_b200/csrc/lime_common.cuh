@@ -60,6 +60,8 @@ struct Ctx {
   void* WprepT[LIME_MAX_LAYERS]; //   folded PREP operand (k_link_prep.cu), folded link-row GLU operand [2*d_ff x H*d],
   void* WpostT[LIME_MAX_LAYERS]; //   and (tc_mode 2) [W_g | W_u] transposed [2*d_ff x d]
   void* WguT[LIME_MAX_LAYERS];
+  bool side256;                  // d = 256 with 32 links: link side by k_link_side_d256.cu, weights unfolded:
+  void* side_w;                  //   one buffer, per layer W_Q^T | W_K^T | W_V^T | W_g^T | W_u^T | W_o^T, then the sh_ operands
   // link-side operands of the first layer for the shared links T^0 = L (weights only, formed at lime_set_weights)
   void *sh_That, *sh_Q2, *sh_K2, *sh_G2t, *sh_U2t, *sh_V2t;
   float *sh_cQ, *sh_cK;
@@ -285,6 +287,8 @@ lime_status launch_fold_weights(const void* Wq, const void* Wk, const void* Wv, 
 lime_status launch_ln_rows_bf16(const float* T, int64_t rows, int d, int ln, float eps, void* out, cudaStream_t st);
 lime_status launch_link_attn_merge_norm(const int32_t* chunk_start, const int32_t* merge_needed, int B, int ell, int d, int H,
                                         const float* part_m, const float* part_s, const float* part_acc, void* Ohat, cudaStream_t st);
+// n square matrices [d x d] (NULL: identity), transposed one after the other into out
+lime_status launch_transpose_square_bf16(const void* const* W, int n, int d, void* out, cudaStream_t st);
 lime_status launch_transpose_bf16(const void* W, int rows, int cols, void* WT, cudaStream_t st);
 
 // link-row GEMMs on tensor cores (k_gemm_tc.cu); A [M x K] bf16 row-major, Bt [N x K] bf16 (weights, pre-folded)
@@ -350,6 +354,22 @@ lime_status launch_hist_update2_tc(const HistUpdateArgs& a, int H, cudaStream_t 
 // ---- tensor-core XOR layer at d = d_ff = 256 (bf16; ell = 64 with H in {2, 4, 8}, ell = 32 with H in {4, 8}; history rows LayerNorm-ed already) ----
 bool link_attn_d256_tc_supported(int dtype, int d, int H, int ell, int phi);
 lime_status launch_link_attn_d256_tc(const LinkAttnArgs& a, cudaStream_t st);   // a.ln must be 0
+
+// link side of a layer at d = 256, 32 links: merged attention rows -> T and its consumers, and (or) T -> the next layer's operands
+struct LinkSide256Args {
+  int users, H;
+  const void* Ohat; const float *part_m, *part_s, *part_acc; const int32_t* chunk_start;   // Ohat NULL: T is given
+  const float* T_in; int t_shared;
+  const void *WvT, *WguT, *WoT;                             // this layer's, transposed (needed with Ohat)
+  const void *WqT, *WkT, *WvT_next, *Wq, *Wk;               // next layer's, transposed and as stored (WqT NULL: no operands)
+  int need_hist, lp_accumulate, ln;
+  float *T_out, *LP;                                        // nullable
+  void *link_states, *Q2, *K2, *V2t;                        // link_states (nullable): bf16 L^P instead of LP
+  float scale, eps;
+  int* err;
+};
+bool link_side_d256_supported(int d, int d_ff, int H, int ell);
+lime_status launch_link_side_d256(const LinkSide256Args& a, cudaStream_t st);
 
 struct HistUpdate256Args {
   const void* hist_in; void* hist_out; int64_t total;
