@@ -177,12 +177,235 @@ constexpr int NB = NT < 4 ? NT : 4;
   }
 }
 
+// ----------------------------------------------------------------------------- fp32 storage
+// A quad per candidate: lane t holds columns (4 i + t) * 4 .. of its row (64 contiguous bytes a load) and the same columns of the
+// user's link states in registers, which stay there for all candidates of the user a warp works through.
+template <int D, int ELL>
+__global__ void __launch_bounds__(SR_WARPS * 32, 2)
+k_score_rows_f32(const float* __restrict__ LS, const float* __restrict__ W, const float* __restrict__ T, const ScoreRowsParams p) {
+  constexpr int KI = D / 16;
+  pdl_launch_dependents();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  // contiguous groups per warp: neighbouring groups share a user
+  const int64_t w0 = (int64_t)blockIdx.x * SR_WARPS + warp, nw = (int64_t)gridDim.x * SR_WARPS;
+  const int g_begin = (int)(w0 * p.n_groups / nw), g_end = (int)((w0 + 1) * p.n_groups / nw);
+  pdl_wait();
+  float4 ls[ELL][KI];
+  int b = -1, loaded = -1;
+  for (int grp = g_begin; grp < g_end; ++grp) {
+    const int s0 = grp * 8, s1 = min(s0 + 8, p.total), slot = s0 + g;
+    int row = min(slot, p.total - 1);
+    bool in = slot < s1;
+    if (p.ids != nullptr) {
+      const int32_t id = __ldg(p.ids + row);
+      const bool good = id >= 0 && id < p.rows;
+      if (in && !good && t == 0 && p.flag != nullptr) atomicMin(p.flag, row);
+      in = in && good;
+      row = in ? id : 0;
+    }
+    float4 x[KI], w[ELL / 4];
+#pragma unroll
+    for (int i = 0; i < KI; ++i) x[i] = in ? __ldg(reinterpret_cast<const float4*>(T + (int64_t)row * p.ldt) + 4 * i + t) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < ELL / 4; ++i) w[i] = in ? __ldg(reinterpret_cast<const float4*>(W + (int64_t)row * p.ldw) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (p.cand_off == nullptr) b = s0 / p.C;
+    else if (b < 0) b = sr_find_user(p.cand_off, p.B, s0, lane);
+    float out = 0.f;
+    for (;;) {
+      const int u0 = p.cand_off == nullptr ? b * p.C : __ldg(p.cand_off + b), u1 = p.cand_off == nullptr ? u0 + p.C : __ldg(p.cand_off + b + 1);
+      if (u1 > s0) {
+        if (b != loaded) {
+          const float4* src = reinterpret_cast<const float4*>(LS + (int64_t)b * ELL * D) + t;
+#pragma unroll
+          for (int l = 0; l < ELL; ++l)
+#pragma unroll
+            for (int i = 0; i < KI; ++i) ls[l][i] = __ldg(src + l * (D / 4) + 4 * i);
+          loaded = b;
+        }
+        float s = 0.f;
+#pragma unroll
+        for (int l = 0; l < ELL; ++l) {
+          float q = 0.f;
+#pragma unroll
+          for (int i = 0; i < KI; ++i) {
+            q = fmaf(ls[l][i].x, x[i].x, q); q = fmaf(ls[l][i].y, x[i].y, q); q = fmaf(ls[l][i].z, x[i].z, q); q = fmaf(ls[l][i].w, x[i].w, q);
+          }
+          const float4 w4 = w[l / 4];
+          s = fmaf(l % 4 == 0 ? w4.x : l % 4 == 1 ? w4.y : l % 4 == 2 ? w4.z : w4.w, q, s);
+        }
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if (slot >= u0 && slot < u1) out = s;
+      }
+      if (u1 >= s1 || b + 1 >= p.B) break;
+      ++b;
+    }
+    if (t == 0 && slot < s1) p.logits[slot] = out;
+  }
+}
+
+// ----------------------------------------------------------------------------- candidate -> link weights, narrow models
+// out[m, :] = softmax_l <T_m, keff_l>, every warp on its own as above.  bf16: 16 rows a step as A fragments, the keys as a
+// bf16 value and its remainder (keff_hl, [2 ell x d]) in B fragments that stay in registers.
+template <int D, int ELL>
+__global__ void __launch_bounds__(SR_WARPS * 32)
+k_precompute_rows(const __nv_bfloat16* __restrict__ T, int64_t M, const __nv_bfloat16* __restrict__ keff_hl, __nv_bfloat16* __restrict__ out) {
+  constexpr int NT = ELL / 8, NL = ELL / 4, KJ = D / 32;
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  uint4 kf[2][NT][KJ];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int j = 0; j < KJ; ++j)
+        kf[h][n][j] = __ldg(reinterpret_cast<const uint4*>(keff_hl + (int64_t)(h * ELL + (g >> 1) * NL + 2 * n + (g & 1)) * D + j * 32 + t * 8));
+  const int64_t groups = (M + 15) / 16, stride = (int64_t)gridDim.x * SR_WARPS;
+  for (int64_t grp = (int64_t)blockIdx.x * SR_WARPS + (threadIdx.x >> 5); grp < groups; grp += stride) {
+    const int64_t m0 = grp * 16 + g;
+    uint4 a[2][KJ];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < KJ; ++j) a[i][j] = m0 + 8 * i < M ? sr_ld_stream(T + (m0 + 8 * i) * D + j * 32 + t * 8) : make_uint4(0, 0, 0, 0);
+    float acc[NT][4];
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[n][e] = 0.f;
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int j = 0; j < KJ; ++j) {
+          sr_mma(acc[n], a[0][j].x, a[1][j].x, a[0][j].y, a[1][j].y, kf[h][n][j].x, kf[h][n][j].y);
+          sr_mma(acc[n], a[0][j].z, a[1][j].z, a[0][j].w, a[1][j].w, kf[h][n][j].z, kf[h][n][j].w);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {                                 // rows g, g + 8: this thread's links t * NL ..
+      float mx = -INFINITY, sum = 0.f;
+#pragma unroll
+      for (int n = 0; n < NT; ++n) mx = fmaxf(mx, fmaxf(acc[n][2 * i], acc[n][2 * i + 1]));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        acc[n][2 * i] = __expf(acc[n][2 * i] - mx); acc[n][2 * i + 1] = __expf(acc[n][2 * i + 1] - mx);
+        sum += acc[n][2 * i] + acc[n][2 * i + 1];
+      }
+      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+      const float inv = 1.0f / sum;
+      if (m0 + 8 * i < M) {
+        uint32_t o[NT];
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+          const __nv_bfloat162 v = __floats2bfloat162_rn(acc[n][2 * i] * inv, acc[n][2 * i + 1] * inv);
+          o[n] = *reinterpret_cast<const uint32_t*>(&v);
+        }
+        __nv_bfloat16* dst = out + (m0 + 8 * i) * ELL + t * NL;
+        if constexpr (NT == 1) *reinterpret_cast<uint32_t*>(dst) = o[0];
+        else if constexpr (NT == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(o[0], o[1]);
+        else
+#pragma unroll
+          for (int n = 0; n < NT; n += 4) *reinterpret_cast<uint4*>(dst + 2 * n) = make_uint4(o[n], o[n + 1], o[n + 2], o[n + 3]);
+      }
+    }
+  }
+}
+
+// fp32: a quad per row, the keys' columns of a lane in registers
+template <int D, int ELL>
+__global__ void __launch_bounds__(SR_WARPS * 32, 2)
+k_precompute_rows_f32(const float* __restrict__ T, int64_t M, const float* __restrict__ keff, float* __restrict__ out) {
+  constexpr int KI = D / 16, NL = ELL / 4;
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  float4 kf[ELL][KI];
+#pragma unroll
+  for (int l = 0; l < ELL; ++l)
+#pragma unroll
+    for (int i = 0; i < KI; ++i) kf[l][i] = __ldg(reinterpret_cast<const float4*>(keff + l * D) + 4 * i + t);
+  const int64_t groups = (M + 7) / 8, stride = (int64_t)gridDim.x * SR_WARPS;
+  // the next step's rows are requested before this one's products
+  auto load = [&](float4 (&x)[KI], int64_t grp) {
+    const int64_t m = grp * 8 + g;
+#pragma unroll
+    for (int i = 0; i < KI; ++i) x[i] = m < M ? __ldg(reinterpret_cast<const float4*>(T + m * D) + 4 * i + t) : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  float4 x[KI], nx[KI], nx2[KI];
+  int64_t grp = (int64_t)blockIdx.x * SR_WARPS + (threadIdx.x >> 5);
+  load(nx, grp);
+  load(nx2, grp + stride);
+  for (; grp < groups; grp += stride) {
+    const int64_t m = grp * 8 + g;
+#pragma unroll
+    for (int i = 0; i < KI; ++i) { x[i] = nx[i]; nx[i] = nx2[i]; }
+    load(nx2, grp + 2 * stride);
+    float s[ELL], mx = -INFINITY, sum = 0.f;
+#pragma unroll
+    for (int l = 0; l < ELL; ++l) {
+      s[l] = 0.f;
+#pragma unroll
+      for (int i = 0; i < KI; ++i) {
+        s[l] = fmaf(kf[l][i].x, x[i].x, s[l]); s[l] = fmaf(kf[l][i].y, x[i].y, s[l]); s[l] = fmaf(kf[l][i].z, x[i].z, s[l]); s[l] = fmaf(kf[l][i].w, x[i].w, s[l]);
+      }
+      s[l] += __shfl_xor_sync(0xffffffffu, s[l], 1);
+      s[l] += __shfl_xor_sync(0xffffffffu, s[l], 2);
+      mx = fmaxf(mx, s[l]);
+    }
+#pragma unroll
+    for (int l = 0; l < ELL; ++l) { s[l] = __expf(s[l] - mx); sum += s[l]; }
+    const float inv = 1.0f / sum;
+    if (m < M)
+#pragma unroll
+      for (int k = 0; k < NL; k += 2) {                           // lane t writes links t * NL ..
+        float a = s[k], bq = s[k + 1];
+#pragma unroll
+        for (int q = 1; q < 4; ++q) { a = t == q ? s[q * NL + k] : a; bq = t == q ? s[q * NL + k + 1] : bq; }
+        *reinterpret_cast<float2*>(out + m * ELL + t * NL + k) = make_float2(a * inv, bq * inv);
+      }
+  }
+}
+
+bool precompute_rows_supported(int dtype, int d, int rows, int group) {
+  if (rows != group) return false;                                // one softmax per row
+  if (dtype == LIME_F32) return (d == 64 && rows == 8) || (d == 32 && (rows == 8 || rows == 16));
+  return d == 32 && (rows == 8 || rows == 16 || rows == 32);
+}
+
+lime_status launch_precompute_rows(int dtype, const void* cand, int64_t M, int d, int ell, const float* keff, const void* keff_hl, void* out_w,
+                                   cudaStream_t st) {
+  if (M == 0) return LIME_OK;
+  const int64_t blocks = (M / (dtype == LIME_F32 ? 8 : 16) + SR_WARPS) / SR_WARPS, cap = (int64_t)kSMs * (dtype == LIME_F32 ? 3 : 8);
+  const dim3 grid((unsigned)(blocks < cap ? blocks : cap)), block(SR_WARPS * 32);
+  ProfScope _p("k_precompute_rows", st);
+  if (dtype == LIME_F32) {
+    const float* T = (const float*)cand;
+    float* o = (float*)out_w;
+    if (d == 64) k_precompute_rows_f32<64, 8><<<grid, block, 0, st>>>(T, M, keff, o);
+    else if (ell == 8) k_precompute_rows_f32<32, 8><<<grid, block, 0, st>>>(T, M, keff, o);
+    else k_precompute_rows_f32<32, 16><<<grid, block, 0, st>>>(T, M, keff, o);
+  } else {
+    const __nv_bfloat16 *T = (const __nv_bfloat16*)cand, *k = (const __nv_bfloat16*)keff_hl;
+    __nv_bfloat16* o = (__nv_bfloat16*)out_w;
+    if (ell == 8) k_precompute_rows<32, 8><<<grid, block, 0, st>>>(T, M, k, o);
+    else if (ell == 16) k_precompute_rows<32, 16><<<grid, block, 0, st>>>(T, M, k, o);
+    else k_precompute_rows<32, 32><<<grid, block, 0, st>>>(T, M, k, o);
+  }
+  LIME_LAUNCH_CHECK("k_precompute_rows");
+  return LIME_OK;
+}
+
+// ----------------------------------------------------------------------------- dispatch
 static bool score_rows_supported(const ScoreArgs& a) {
-  if (a.dtype != LIME_BF16) return false;
+  if (a.cand_off == nullptr && a.C <= 0) return false;
+  if (a.dtype == LIME_F32) {
+    if (!((a.d == 64 && a.ell == 8) || (a.d == 32 && (a.ell == 8 || a.ell == 16)))) return false;
+    return ((reinterpret_cast<uintptr_t>(a.T) | reinterpret_cast<uintptr_t>(a.W) | reinterpret_cast<uintptr_t>(a.LS)) & 15) == 0 && a.ldt % 4 == 0 && a.ldw % 4 == 0;
+  }
   const bool d_ok = a.d == 32 || a.d == 64 || a.d == 128 || a.d == 256;
   const bool l_ok = a.ell == 8 || a.ell == 16 || a.ell == 32 || a.ell == 64;
   if (!d_ok || !l_ok) return false;
-  if (a.cand_off == nullptr && a.C <= 0) return false;
   const int64_t ldt = a.ldt ? a.ldt : a.d, ldw = a.ldw ? a.ldw : a.ell;
   // 16-byte pieces of T rows; weight pieces of ell / 2 bytes, at most 16
   return (reinterpret_cast<uintptr_t>(a.T) & 15) == 0 && ldt % 8 == 0 && (reinterpret_cast<uintptr_t>(a.W) & 15) == 0 && ldw % 8 == 0 &&
@@ -223,7 +446,26 @@ static lime_status launch_score_rows_d(const ScoreArgs& a, cudaStream_t st) {
   }
 }
 
+template <int D, int ELL>
+static lime_status launch_score_rows_f32_t(const ScoreArgs& a, cudaStream_t st) {
+  ScoreRowsParams p{};
+  p.cand_off = a.cand_off; p.ids = a.cand_ids; p.flag = a.dev_flag; p.logits = a.logits;
+  p.ldt = a.ldt ? (int)a.ldt : D; p.ldw = a.ldw ? (int)a.ldw : ELL;
+  p.rows = (int)(a.cand_ids ? a.corpus_rows : a.total); p.total = (int)a.total; p.B = a.B; p.C = a.C;
+  p.n_groups = (int)((a.total + 7) / 8);
+  const int64_t blocks = (p.n_groups + SR_WARPS - 1) / SR_WARPS, cap = 3 * kSMs;
+  ProfScope _p("k_score_rows", st);
+  launch_pdl(k_score_rows_f32<D, ELL>, dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(SR_WARPS * 32), 0, st, (const float*)a.LS,
+             (const float*)a.W, (const float*)a.T, p);
+  LIME_LAUNCH_CHECK("k_score_rows");
+  return LIME_OK;
+}
+
 lime_status launch_score_rows(const ScoreArgs& a, cudaStream_t st) {
+  if (a.dtype == LIME_F32) {
+    if (a.d == 64) return launch_score_rows_f32_t<64, 8>(a, st);
+    return a.ell == 8 ? launch_score_rows_f32_t<32, 8>(a, st) : launch_score_rows_f32_t<32, 16>(a, st);
+  }
   switch (a.d) {
     case 32: return launch_score_rows_d<32>(a, st);
     case 64: return launch_score_rows_d<64>(a, st);

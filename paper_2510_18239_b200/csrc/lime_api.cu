@@ -553,7 +553,8 @@ lime_status lime_set_weights(lime_ctx* ctx, const lime_weights* w, void* stream)
   if (s != LIME_OK) return s;
   s = launch_keff(g.dtype, w->links, w->cand_Wk, w->cand_Wq, g.ell, g.d, c->cand_heads, c->cand_scale, c->keff, st);
   if (s != LIME_OK) return s;
-  if (precompute_tc_supported(g.dtype, g.d, c->ell_c, g.ell) &&
+  if ((precompute_tc_supported(g.dtype, g.d, c->ell_c, g.ell) ||
+       (g.dtype == LIME_BF16 && precompute_rows_supported(g.dtype, g.d, c->ell_c, g.ell))) &&
       (s = launch_keff_split(c->keff, c->ell_c, g.d, c->keff_hl, st)) != LIME_OK)
     return s;
   if (c->side256) {
@@ -663,6 +664,8 @@ lime_status lime_precompute_candidate_links(lime_ctx* ctx, const void* cand_emb,
   if (precompute_tc_supported(c->cfg.dtype, c->cfg.d, c->ell_c, c->cfg.ell))
     return launch_precompute_tc(cand_emb, M, c->cfg.d, c->ell_c, c->cfg.ell, c->keff_hl, out_w, c->dev_err,
                                 static_cast<cudaStream_t>(stream));
+  if (precompute_rows_supported(c->cfg.dtype, c->cfg.d, c->ell_c, c->cfg.ell))
+    return launch_precompute_rows(c->cfg.dtype, cand_emb, M, c->cfg.d, c->ell_c, c->keff, c->keff_hl, out_w, static_cast<cudaStream_t>(stream));
   return launch_precompute(c->cfg.dtype, cand_emb, M, c->cfg.d, c->ell_c, c->cfg.ell, c->keff, out_w,
                            static_cast<cudaStream_t>(stream));
 }

@@ -234,8 +234,11 @@ lime_status launch_score_tc(const ScoreArgs& a, int* err, cudaStream_t st);
 bool score_gather_tc_supported(const ScoreArgs& a);
 lime_status launch_score_gather_tc(const ScoreArgs& a, int* err, cudaStream_t st);
 
-// warp-level scorer: by id, ragged lists, small widths (bf16, d in {32, 64, 128, 256}, ell in {8, 16, 32, 64}), k_score_rows.cu
+// warp-level scorer: by id, ragged lists, small widths (bf16, d in {32, 64, 128, 256}, ell in {8, 16, 32, 64}; fp32, d in {32, 64}), k_score_rows.cu
 bool score_rows_preferred(const ScoreArgs& a);
+// candidate -> link weights of narrow models, same design (bf16 d = 32; fp32 d = 32, 64)
+bool precompute_rows_supported(int dtype, int d, int rows, int group);
+lime_status launch_precompute_rows(int dtype, const void* cand, int64_t M, int d, int ell, const float* keff, const void* keff_hl, void* out_w, cudaStream_t st);
 lime_status launch_score_rows(const ScoreArgs& a, cudaStream_t st);
 
 // the whole encode of a narrow model (bf16, d = d_ff = 32) in one launch, one block per user (k_encode_small.cu)

@@ -16,14 +16,15 @@ def _lib():
     return binding
 
 
-@pytest.mark.parametrize("d,ell", [(32, 8), (32, 64), (64, 16), (128, 32), (256, 32), (256, 64)])
+@pytest.mark.parametrize("dtype,d,ell", [(synth.BF16, 32, 8), (synth.BF16, 32, 64), (synth.BF16, 64, 16), (synth.BF16, 128, 32), (synth.BF16, 256, 32),
+                                         (synth.BF16, 256, 64), (synth.F32, 64, 8), (synth.F32, 32, 8), (synth.F32, 32, 16)])
 @pytest.mark.parametrize("counts,by_id", [([1], True), ([15, 16, 17], False), ([0, 5, 0, 33, 1, 0], True), ([3] * 70 + [0] * 40 + [400], True)])
-def test_score_lists_by_warp(d, ell, counts, by_id):
+def test_score_lists_by_warp(dtype, d, ell, counts, by_id):
     """The warp-level scorer: lists around its 16-slot step, many users inside one step, users without candidates, ids
     outside the corpus."""
     Bd = _lib()
-    dtype, corpus, B, total = synth.BF16, 500, len(counts), int(sum(counts))
-    lime = Bd.Lime(d, max(1, d // 128), ell, 1, dtype=Bd.LIME_BF16, gated_mlp=False)
+    corpus, B, total = 500, len(counts), int(sum(counts))
+    lime = Bd.Lime(d, max(1, d // 128), ell, 1, dtype=Bd.LIME_F32 if dtype == synth.F32 else Bd.LIME_BF16, gated_mlp=False)
     off = O.lengths_to_offsets(np.asarray(counts))
     rows = corpus if by_id else total
     LS = synth.normal_storage(5, "ls", (B, ell, d), 1.0, dtype)
@@ -46,6 +47,19 @@ def test_score_lists_by_warp(d, ell, counts, by_id):
     assert np.abs(got - want).max() <= 1e-4 * max(1.0, np.abs(want).max())
     if by_id:
         assert np.all(got[~ok] == 0.0) and int(flag.item()) == total // 2
+
+
+@pytest.mark.parametrize("dtype,d,ell", [(synth.BF16, 32, 8), (synth.BF16, 32, 16), (synth.BF16, 32, 32), (synth.F32, 64, 8), (synth.F32, 32, 16)])
+@pytest.mark.parametrize("M", [1, 7, 17, 5000])
+def test_precompute_narrow(dtype, d, ell, M):
+    Bd = _lib()
+    lime = Bd.Lime(d, 1, ell, 1, dtype=Bd.LIME_F32 if dtype == synth.F32 else Bd.LIME_BF16, gated_mlp=False)
+    L, T = synth.normal_storage(1, "l", (ell, d), 1.0, dtype), synth.normal_storage(1, "t", (M, d), 1.0, dtype)
+    lime.set_weights(Bd.to_device(L, dtype), [{}])
+    got = Hh.to_f64(lime.precompute_candidate_links(Bd.to_device(T, dtype)))
+    cfg = O.OracleConfig(d=d, H=1, ell=ell, n_layers=1)
+    want = O.precompute_candidate_links(synth.storage_to_f64(T, dtype), synth.storage_to_f64(L, dtype), cfg)
+    assert np.abs(got - want).max() <= (1e-6 if dtype == synth.F32 else 2.0 ** -8)
 
 
 def _layer_against_oracle(dtype, d, H, ell, lengths, shared, phi, tol_max, tol_mean):
