@@ -60,11 +60,12 @@ static int tensor_core_mode(const lime_config& g, int d_ff) {
     return 2;
   return 0;
 }
-// One block per user serves histories of ordinary length; a few very long ones leave most SMs idle and take the generic
+// One block (or cluster) per user serves histories of ordinary length; a few very long ones leave most SMs idle and take the generic
 // kernels, which split them.
 static bool encode_small_wanted(const Ctx* c, int32_t B, int64_t total) {
   const lime_config& g = c->cfg;
-  return encode_small_supported(g.dtype, g.d, c->d_ff, g.H, g.ell, g.gated_mlp) && total <= 2048ll * B;
+  return (encode_small_supported(g.dtype, g.d, c->d_ff, g.H, g.ell, g.gated_mlp) ||
+          encode_f32_supported(g.dtype, g.d, c->d_ff, g.H, g.ell, g.gated_mlp)) && total <= 2048ll * B;
 }
 constexpr int kHistTile = 128;  // tokens per block of the history<-links attention
 
@@ -718,7 +719,13 @@ static lime_status encode_user_impl(lime_ctx* ctx, const void* hist, bool hist_n
     a.eps = c->ln_eps; a.scratch = w.S;
     const bool direct = !c->w.cand_Wv && c->cand_heads == 1;
     a.link_states = direct ? link_states : nullptr; a.lp = w.LP;
-    if ((s = launch_encode_small(a, st)) != LIME_OK) return s;
+    if (g.dtype == LIME_F32) {
+      if (direct) a.lp = static_cast<float*>(link_states);
+      s = launch_encode_f32(a, c->dev_err, st);
+    } else {
+      s = launch_encode_small(a, st);
+    }
+    if (s != LIME_OK) return s;
     if (direct) return LIME_OK;
   } else if (layer_on_tensor_cores(c, 0)) {
     if ((s = encode_user_tc(c, hist, hist_normalized, off, B, total_tokens, link_ctx, link_states, w, st)) != LIME_OK) return s;

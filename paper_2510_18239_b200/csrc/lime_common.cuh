@@ -252,6 +252,9 @@ struct EncodeSmallArgs {
 };
 bool encode_small_supported(int dtype, int d, int d_ff, int H, int ell, int gated_mlp);
 lime_status launch_encode_small(const EncodeSmallArgs& a, cudaStream_t st);
+// the same for fp32 storage at d = d_ff = 64, a cluster of blocks per user; L^P to a.lp (k_encode_f32.cu)
+bool encode_f32_supported(int dtype, int d, int d_ff, int H, int ell, int gated_mlp);
+lime_status launch_encode_f32(const EncodeSmallArgs& a, int* err, cudaStream_t st);
 
 // one-thread kernel whose only wait can never be satisfied (self-test of the bounded waits, tc_host.cu)
 lime_status launch_wait_expiry(int* err, uint64_t limit_ns, int code, cudaStream_t st);

@@ -213,3 +213,11 @@ def test_three_layer_interaction_network(ell, w0, counts, form):
     assert np.abs(got - want).max() <= 2e-2 and np.abs(got - want).max() <= 3e-2 * max(want.std(), 0.1) + 1e-3
     if form != "dense":
         assert np.all(got[~ok] == 0.0) and int(flag.item()) == total // 2
+
+
+@pytest.mark.parametrize("H,ell", [(2, 8), (4, 8), (2, 16)])
+@pytest.mark.parametrize("lengths", [[1], [0, 15, 100, 257, 3], [1500, 3, 700], [64] * 4, [60] * 300])
+@pytest.mark.parametrize("phi,raw,per_user", [("softmax", False, False), ("silu", False, True), ("softmax", True, True)])
+def test_fp32_encode_in_one_launch(H, ell, lengths, phi, raw, per_user):
+    """fp32 storage at d = 64: one to eight blocks a user, several 256-token rounds a block, histories beyond shared memory."""
+    _encode_against_oracle(synth.F32, 64, H, ell, 3, lengths, phi, raw, per_user, 1e-4, 1e-5)
