@@ -111,6 +111,11 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     return lib
 
 
+def _lib() -> ctypes.CDLL:
+    """The loaded library (every call goes through here: one global read once it is loaded)."""
+    return _lib_handle if _lib_handle is not None else load_library()
+
+
 def _check(status: int, where: str):
     if status != 0:
         detail = load_library().lime_last_cuda_error().decode() if status == 4 else ""
@@ -125,73 +130,81 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return t.data_ptr()
 
 
+# The current stream's handle without building a torch.cuda.Stream around it (0.3 instead of 3 us of a call that has
+# about 10; torch's own generated code takes it this way), or the public route where this torch has no such function.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    if _raw_stream is None or _current_device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_current_device())
 
 
 # ----------------------------------------------------------------------------- 1:1 entry points
 def lime_version() -> str:
-    return load_library().lime_version().decode()
+    return _lib().lime_version().decode()
 
 
 def lime_create(cfg: lime_config) -> int:
     h = ctypes.c_void_p()
-    _check(load_library().lime_create(ctypes.byref(cfg), ctypes.byref(h)), "lime_create")
+    _check(_lib().lime_create(ctypes.byref(cfg), ctypes.byref(h)), "lime_create")
     return h.value
 
 
 def lime_destroy(ctx: int) -> None:
-    _check(load_library().lime_destroy(ctx), "lime_destroy")
+    _check(_lib().lime_destroy(ctx), "lime_destroy")
 
 
 def lime_set_weights(ctx: int, w: lime_weights) -> None:
-    _check(load_library().lime_set_weights(ctx, ctypes.byref(w), _stream()), "lime_set_weights")
+    _check(_lib().lime_set_weights(ctx, ctypes.byref(w), _stream()), "lime_set_weights")
 
 
 def lime_workspace_bytes(ctx: int, B: int, total_tokens: int) -> int:
-    return int(load_library().lime_workspace_bytes(ctx, B, total_tokens))
+    return int(_lib().lime_workspace_bytes(ctx, B, total_tokens))
 
 
 def lime_lengths_to_offsets(ctx: int, lengths: torch.Tensor, off: torch.Tensor) -> None:
-    _check(load_library().lime_lengths_to_offsets(ctx, _ptr(lengths), lengths.numel(), _ptr(off), _stream()),
+    _check(_lib().lime_lengths_to_offsets(ctx, _ptr(lengths), lengths.numel(), _ptr(off), _stream()),
            "lime_lengths_to_offsets")
 
 
 def lime_gather_history(ctx: int, table: torch.Tensor, ids: torch.Tensor, out: torch.Tensor,
                         dev_flag: Optional[torch.Tensor] = None) -> None:
-    _check(load_library().lime_gather_history(ctx, _ptr(table), table.shape[0], _ptr(ids), ids.numel(), _ptr(out),
+    _check(_lib().lime_gather_history(ctx, _ptr(table), table.shape[0], _ptr(ids), ids.numel(), _ptr(out),
                                               _ptr(dev_flag), _stream()), "lime_gather_history")
 
 
 def lime_gather_history_normalized(ctx: int, table: torch.Tensor, ids: torch.Tensor, out: torch.Tensor,
                                    dev_flag: Optional[torch.Tensor] = None) -> None:
-    _check(load_library().lime_gather_history_normalized(ctx, _ptr(table), table.shape[0], _ptr(ids), ids.numel(), _ptr(out),
+    _check(_lib().lime_gather_history_normalized(ctx, _ptr(table), table.shape[0], _ptr(ids), ids.numel(), _ptr(out),
                                                          _ptr(dev_flag), _stream()), "lime_gather_history_normalized")
 
 
 def lime_precompute_candidate_links(ctx: int, cand_emb: torch.Tensor, out_w: torch.Tensor) -> None:
-    _check(load_library().lime_precompute_candidate_links(ctx, _ptr(cand_emb), cand_emb.shape[0], _ptr(out_w), _stream()),
+    _check(_lib().lime_precompute_candidate_links(ctx, _ptr(cand_emb), cand_emb.shape[0], _ptr(out_w), _stream()),
            "lime_precompute_candidate_links")
 
 
 def lime_xor_layer(ctx: int, layer: int, hist_in: torch.Tensor, off: torch.Tensor, B: int, links_in: torch.Tensor,
                    links_shared: bool, hist_out: Optional[torch.Tensor], links_out: torch.Tensor,
                    ws: torch.Tensor) -> None:
-    _check(load_library().lime_xor_layer(ctx, layer, _ptr(hist_in), _ptr(off), B, hist_in.shape[0], _ptr(links_in),
+    _check(_lib().lime_xor_layer(ctx, layer, _ptr(hist_in), _ptr(off), B, hist_in.shape[0], _ptr(links_in),
                                          1 if links_shared else 0, _ptr(hist_out), _ptr(links_out), _ptr(ws),
                                          ws.numel() * ws.element_size(), _stream()), "lime_xor_layer")
 
 
 def lime_encode_user(ctx: int, hist: torch.Tensor, off: torch.Tensor, B: int, link_ctx: Optional[torch.Tensor],
                      link_states: torch.Tensor, ws: torch.Tensor) -> None:
-    _check(load_library().lime_encode_user(ctx, _ptr(hist), _ptr(off), B, hist.shape[0], _ptr(link_ctx),
+    _check(_lib().lime_encode_user(ctx, _ptr(hist), _ptr(off), B, hist.shape[0], _ptr(link_ctx),
                                            _ptr(link_states), _ptr(ws), ws.numel() * ws.element_size(), _stream()),
            "lime_encode_user")
 
 
 def lime_encode_user_normalized(ctx: int, hist_normalized: torch.Tensor, off: torch.Tensor, B: int,
                                 link_ctx: Optional[torch.Tensor], link_states: torch.Tensor, ws: torch.Tensor) -> None:
-    _check(load_library().lime_encode_user_normalized(ctx, _ptr(hist_normalized), _ptr(off), B, hist_normalized.shape[0],
+    _check(_lib().lime_encode_user_normalized(ctx, _ptr(hist_normalized), _ptr(off), B, hist_normalized.shape[0],
                                                       _ptr(link_ctx), _ptr(link_states), _ptr(ws),
                                                       ws.numel() * ws.element_size(), _stream()),
            "lime_encode_user_normalized")
@@ -204,21 +217,21 @@ def lime_score_candidates(ctx: int, link_states: torch.Tensor, B: int, cand_w: t
     """corpus_rows (only with cand_ids): rows of the corpus caches cand_w / cand_emb; by default the row count of cand_emb."""
     if cand_ids is not None and corpus_rows is None:
         corpus_rows = int(cand_emb.shape[0])
-    _check(load_library().lime_score_candidates(ctx, _ptr(link_states), B, _ptr(cand_w), _ptr(cand_emb), _ptr(cand_off),
+    _check(_lib().lime_score_candidates(ctx, _ptr(link_states), B, _ptr(cand_w), _ptr(cand_emb), _ptr(cand_off),
                                                 C, total_cands, _ptr(cand_ids), int(corpus_rows or 0), _ptr(dev_flag),
                                                 _ptr(logits), _stream()),
            "lime_score_candidates")
 
 
 def lime_pack_corpus_cache(ctx: int, cand_emb: torch.Tensor, cand_w: torch.Tensor, packed: torch.Tensor) -> None:
-    _check(load_library().lime_pack_corpus_cache(ctx, _ptr(cand_emb), _ptr(cand_w), cand_emb.shape[0], _ptr(packed), _stream()),
+    _check(_lib().lime_pack_corpus_cache(ctx, _ptr(cand_emb), _ptr(cand_w), cand_emb.shape[0], _ptr(packed), _stream()),
            "lime_pack_corpus_cache")
 
 
 def lime_score_candidates_packed(ctx: int, link_states: torch.Tensor, B: int, packed: torch.Tensor, cand_ids: torch.Tensor,
                                  cand_off: Optional[torch.Tensor], C: int, total_cands: int, logits: torch.Tensor,
                                  dev_flag: Optional[torch.Tensor] = None) -> None:
-    _check(load_library().lime_score_candidates_packed(ctx, _ptr(link_states), B, _ptr(packed), packed.shape[0], _ptr(cand_ids),
+    _check(_lib().lime_score_candidates_packed(ctx, _ptr(link_states), B, _ptr(packed), packed.shape[0], _ptr(cand_ids),
                                                        _ptr(cand_off), C, total_cands, _ptr(dev_flag), _ptr(logits), _stream()),
            "lime_score_candidates_packed")
 
@@ -236,19 +249,19 @@ def make_ffn(layers) -> lime_ffn:
 
 
 def lime_set_context_mlp(ctx: int, d_c: int, mlp: lime_ffn) -> None:
-    _check(load_library().lime_set_context_mlp(ctx, d_c, ctypes.byref(mlp), _stream()), "lime_set_context_mlp")
+    _check(_lib().lime_set_context_mlp(ctx, d_c, ctypes.byref(mlp), _stream()), "lime_set_context_mlp")
 
 
 def lime_contextualize_links(ctx: int, user_ctx: torch.Tensor, B: int, link_ctx: torch.Tensor) -> None:
-    _check(load_library().lime_contextualize_links(ctx, _ptr(user_ctx), B, _ptr(link_ctx), _stream()), "lime_contextualize_links")
+    _check(_lib().lime_contextualize_links(ctx, _ptr(user_ctx), B, _ptr(link_ctx), _stream()), "lime_contextualize_links")
 
 
 def lime_set_head(ctx: int, head: lime_ffn) -> None:
-    _check(load_library().lime_set_head(ctx, ctypes.byref(head), _stream()), "lime_set_head")
+    _check(_lib().lime_set_head(ctx, ctypes.byref(head), _stream()), "lime_set_head")
 
 
 def lime_head_workspace_bytes(ctx: int, B: int) -> int:
-    return int(load_library().lime_head_workspace_bytes(ctx, B))
+    return int(_lib().lime_head_workspace_bytes(ctx, B))
 
 
 def lime_score_candidates_head(ctx: int, link_states: torch.Tensor, B: int, cand_w: torch.Tensor, cand_emb: torch.Tensor,
@@ -257,7 +270,7 @@ def lime_score_candidates_head(ctx: int, link_states: torch.Tensor, B: int, cand
                                dev_flag: Optional[torch.Tensor] = None) -> None:
     if cand_ids is not None and corpus_rows is None:
         corpus_rows = int(cand_emb.shape[0])
-    _check(load_library().lime_score_candidates_head(ctx, _ptr(link_states), B, _ptr(cand_w), _ptr(cand_emb), _ptr(cand_off),
+    _check(_lib().lime_score_candidates_head(ctx, _ptr(link_states), B, _ptr(cand_w), _ptr(cand_emb), _ptr(cand_off),
                                                      C, total_cands, _ptr(cand_ids), int(corpus_rows or 0), _ptr(dev_flag),
                                                      _ptr(logits), _ptr(ws), ws.numel() * ws.element_size(), _stream()),
            "lime_score_candidates_head")
@@ -268,18 +281,18 @@ def lime_precompute_candidate_links_noalloc(dtype: int, d: int, ell: int, cand_s
                                             cand_emb: torch.Tensor, out_w: torch.Tensor) -> None:
     """Context-free, allocation-free precompute for callers that may not allocate device memory; the caller passes
     every buffer, including the output.  Raises LimeError(LIME_EXCEEDS_STATIC_SCRATCH) if ell * d is too large."""
-    st = load_library().lime_precompute_candidate_links_noalloc(dtype, d, ell, cand_scale, _ptr(links), _ptr(cand_Wq),
+    st = _lib().lime_precompute_candidate_links_noalloc(dtype, d, ell, cand_scale, _ptr(links), _ptr(cand_Wq),
                                                                 _ptr(cand_Wk), _ptr(cand_emb), cand_emb.shape[0],
                                                                 _ptr(out_w), _stream())
     if st != 0:
         raise LimeError(st, "lime_precompute_candidate_links_noalloc",
-                        load_library().lime_last_cuda_error().decode() if st in (4, 7) else "")
+                        _lib().lime_last_cuda_error().decode() if st in (4, 7) else "")
 
 
 def lime_device_status(ctx: int) -> int:
     """Synchronises; raises LimeError(LIME_DEVICE_TIMEOUT) if a bounded in-kernel wait gave up, else returns 0."""
     code = ctypes.c_int32(0)
-    st = load_library().lime_device_status(ctx, ctypes.byref(code))
+    st = _lib().lime_device_status(ctx, ctypes.byref(code))
     if st != 0:
         raise LimeError(st, "lime_device_status", f"wait code {code.value}")
     return int(code.value)
@@ -287,11 +300,11 @@ def lime_device_status(ctx: int) -> int:
 
 def lime_selftest_wait_expiry(ctx: int, limit_us: int) -> None:
     """Launches a wait that can never be satisfied, bounded by limit_us; lime_device_status then reports the time-out."""
-    _check(load_library().lime_selftest_wait_expiry(ctx, limit_us, _stream()), "lime_selftest_wait_expiry")
+    _check(_lib().lime_selftest_wait_expiry(ctx, limit_us, _stream()), "lime_selftest_wait_expiry")
 
 
 def lime_profile_start(capacity: int = 4096) -> None:
-    _check(load_library().lime_profile_start(capacity), "lime_profile_start")
+    _check(_lib().lime_profile_start(capacity), "lime_profile_start")
 
 
 def lime_profile_stop(capacity: int = 4096):
@@ -299,7 +312,7 @@ def lime_profile_stop(capacity: int = 4096):
     names = ctypes.create_string_buffer(64 * capacity)
     ms = (ctypes.c_float * capacity)()
     count = ctypes.c_int32(0)
-    _check(load_library().lime_profile_stop(names, len(names), ms, capacity, ctypes.byref(count)), "lime_profile_stop")
+    _check(_lib().lime_profile_stop(names, len(names), ms, capacity, ctypes.byref(count)), "lime_profile_stop")
     nm = names.value.decode().split("\n")[:-1]
     return [(nm[i], float(ms[i])) for i in range(min(len(nm), count.value, capacity))], int(count.value)
 
@@ -323,6 +336,7 @@ class Lime:
     def __init__(self, d: int, H: int, ell: int, n_layers: int, dtype: int = LIME_BF16, d_ff: int = 0,
                  phi: int = LIME_PHI_SOFTMAX, ln: bool = True, gated_mlp: bool = True, attn_scale: float = 0.0,
                  cand_scale: float = 0.0, ln_eps: float = 0.0, cand_heads: int = 0):
+        self.d, self.ell = d, ell
         self.cfg = lime_config(d, H, ell, n_layers, d_ff, dtype, phi, int(ln), int(gated_mlp), attn_scale, cand_scale, ln_eps,
                                cand_heads)
         self.ell_c = ell * (H if cand_heads == H and H > 1 else 1)      # weight columns per candidate, link-state rows
@@ -330,6 +344,8 @@ class Lime:
         self.tdtype = torch_dtype(dtype)
         self._keep = []
         self._ws = None
+        self._ws_for = None             # (B, total_tokens) that _ws is known to serve
+        self._head_ws = None
 
     def close(self):
         if self.ctx:
@@ -362,42 +378,44 @@ class Lime:
         self._keep = keep
 
     def workspace(self, B: int, total_tokens: int) -> torch.Tensor:
-        need = lime_workspace_bytes(self.ctx, B, total_tokens)
-        if self._ws is None or self._ws.numel() < need:
-            self._ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+        if self._ws_for != (B, total_tokens):
+            need = lime_workspace_bytes(self.ctx, B, total_tokens)
+            if self._ws is None or self._ws.numel() < need:
+                self._ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+            self._ws_for = (B, total_tokens)
         return self._ws
 
     def lengths_to_offsets(self, lengths: torch.Tensor) -> torch.Tensor:
-        off = torch.empty(lengths.numel() + 1, dtype=torch.int32, device=lengths.device)
+        off = lengths.new_empty(lengths.numel() + 1)           # int32 on the same device, as the lengths are
         lime_lengths_to_offsets(self.ctx, lengths, off)
         return off
 
     def gather_history(self, table: torch.Tensor, ids: torch.Tensor, flag: Optional[torch.Tensor] = None) -> torch.Tensor:
-        out = torch.empty((ids.numel(), self.cfg.d), dtype=self.tdtype, device=ids.device)
+        out = table.new_empty((ids.numel(), self.d))
         lime_gather_history(self.ctx, table, ids, out, flag)
         return out
 
     def gather_history_normalized(self, table: torch.Tensor, ids: torch.Tensor,
                                   flag: Optional[torch.Tensor] = None) -> torch.Tensor:
-        out = torch.empty((ids.numel(), self.cfg.d), dtype=self.tdtype, device=ids.device)
+        out = table.new_empty((ids.numel(), self.d))
         lime_gather_history_normalized(self.ctx, table, ids, out, flag)
         return out
 
     def encode_user_normalized(self, hist_normalized: torch.Tensor, off: torch.Tensor,
                                link_ctx: Optional[torch.Tensor] = None) -> torch.Tensor:
         B = off.numel() - 1
-        ls = torch.empty((B, self.ell_c, self.cfg.d), dtype=self.tdtype, device=hist_normalized.device)
+        ls = hist_normalized.new_empty((B, self.ell_c, self.d))
         lime_encode_user_normalized(self.ctx, hist_normalized, off, B, link_ctx, ls, self.workspace(B, hist_normalized.shape[0]))
         return ls
 
     def precompute_candidate_links(self, cand_emb: torch.Tensor) -> torch.Tensor:
-        out = torch.empty((cand_emb.shape[0], self.ell_c), dtype=self.tdtype, device=cand_emb.device)
+        out = cand_emb.new_empty((cand_emb.shape[0], self.ell_c))
         lime_precompute_candidate_links(self.ctx, cand_emb, out)
         return out
 
     def encode_user(self, hist: torch.Tensor, off: torch.Tensor, link_ctx: Optional[torch.Tensor] = None) -> torch.Tensor:
         B = off.numel() - 1
-        ls = torch.empty((B, self.ell_c, self.cfg.d), dtype=self.tdtype, device=hist.device)
+        ls = hist.new_empty((B, self.ell_c, self.d))
         lime_encode_user(self.ctx, hist, off, B, link_ctx, ls, self.workspace(B, hist.shape[0]))
         return ls
 
@@ -430,7 +448,7 @@ class Lime:
 
     def contextualize_links(self, user_ctx: torch.Tensor) -> torch.Tensor:
         B = user_ctx.shape[0]
-        out = torch.empty((B, self.cfg.ell, self.cfg.d), dtype=torch.float32, device=user_ctx.device)
+        out = torch.empty((B, self.ell, self.d), dtype=torch.float32, device=user_ctx.device)
         lime_contextualize_links(self.ctx, user_ctx, B, out)
         return out
 
@@ -446,7 +464,7 @@ class Lime:
         total = total_cands if total_cands is not None else (cand_ids.numel() if cand_ids is not None else cand_emb.shape[0])
         logits = torch.empty(total, dtype=torch.float32, device=link_states.device)
         need = lime_head_workspace_bytes(self.ctx, B)
-        if getattr(self, "_head_ws", None) is None or self._head_ws.numel() < need:
+        if self._head_ws is None or self._head_ws.numel() < need:
             self._head_ws = torch.empty(need, dtype=torch.uint8, device=link_states.device)
         lime_score_candidates_head(self.ctx, link_states, B, cand_w, cand_emb, cand_off, C, total, cand_ids, logits,
                                    self._head_ws, corpus_rows, dev_flag)
