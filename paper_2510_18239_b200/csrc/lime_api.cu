@@ -184,7 +184,7 @@ static lime_status make_link_operands(Ctx* c, int layer, const void* That, int64
 // read (0 when they were stored normalised by the previous layer); `out_ln`: store LayerNorm(S').
 static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const int32_t* off, int32_t B, int64_t total,
                                  const LinkOperands& ops, void* hist_out, int hist_ln, int out_ln, LinkMlpArgs mlp,
-                                 const LinkSide256Args* side, const Workspace& w, cudaStream_t st) {
+                                 const LinkSide256Args* side, const LinkSide128Args* side1, const Workspace& w, cudaStream_t st) {
   const lime_config& g = c->cfg;
   lime_status s;
   if (c->tc_mode == 2 && hist_ln && total > 0) {
@@ -211,7 +211,7 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
     LinkSide256Args a = *side;
     a.Ohat = w.Ohat; a.part_m = w.part_m; a.part_s = w.part_s; a.part_acc = w.part_acc; a.chunk_start = w.chunk_start;
     if ((s = launch_link_side_d256(a, st)) != LIME_OK) return s;
-  } else {
+  } else if (side1 == nullptr) {
   if ((s = launch_link_attn_merge_norm(w.chunk_start, w.merge_needed, B, g.ell, g.d, g.H, w.part_m, w.part_s, w.part_acc, w.Ohat, st)) != LIME_OK)
     return s;
   // T^j = GatedMLP(O[T]) with W_V folded into the gate / up weights, and what the next step needs from it
@@ -237,6 +237,13 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
     else s = launch_hist_update2_tc(hu, g.H, st);
     if (s != LIME_OK) return s;
   }
+  if (side1 != nullptr) {
+    // few link rows: merge, T^j and the next layer's operands in one kernel, behind the history update that reads this layer's
+    LinkSide128Args a = *side1;
+    a.users = B; a.ell = g.ell; a.Ohat = w.Ohat; a.part_m = w.part_m; a.part_s = w.part_s; a.part_acc = w.part_acc;
+    a.chunk_start = w.chunk_start; a.WpostT = c->WpostT[layer]; a.WoT = c->WoT[layer]; a.ln = g.ln; a.eps = c->ln_eps; a.err = c->dev_err;
+    if ((s = launch_link_side_d128(a, st)) != LIME_OK) return s;
+  }
   return LIME_OK;
 }
 
@@ -253,7 +260,7 @@ static lime_status xor_layer_tc(Ctx* c, int layer, const void* hist_in, const in
     if ((s = launch_link_side_d256(prep, st)) != LIME_OK) return s;
     side.T_out = links_out;
     return tc_layer_core(c, layer, hist_in, off, B, total, LinkOperands{w.Q2, w.K2, nullptr, nullptr, w.V2t, nullptr, nullptr, links_shared},
-                         hist_out, g.ln, 0, LinkMlpArgs{}, &side, w, st);
+                         hist_out, g.ln, 0, LinkMlpArgs{}, &side, nullptr, w, st);
   }
   const int64_t link_rows = links_shared ? g.ell : (int64_t)B * g.ell;
   if ((s = launch_ln_rows_bf16(links_in, link_rows, g.d, g.ln, c->ln_eps, w.That, st)) != LIME_OK) return s;
@@ -262,7 +269,7 @@ static lime_status xor_layer_tc(Ctx* c, int layer, const void* hist_in, const in
   LinkOperands ops{w.Q2, w.K2, w.G2t, w.U2t, w.V2t, w.cQ, w.cK, links_shared};
   LinkMlpArgs mlp{};
   mlp.T_out = links_out;
-  return tc_layer_core(c, layer, hist_in, off, B, total, ops, hist_out, g.ln, 0, mlp, nullptr, w, st);
+  return tc_layer_core(c, layer, hist_in, off, B, total, ops, hist_out, g.ln, 0, mlp, nullptr, nullptr, w, st);
 }
 
 // lime_encode_user on the tensor-core path: per layer one link-side GEMM (none on the first layer when the links are
@@ -292,11 +299,12 @@ static lime_status encode_user_tc(Ctx* c, const void* hist, bool hist_normalized
       side.Q2 = const_cast<void*>(nx.Q2); side.K2 = const_cast<void*>(nx.K2); side.V2t = const_cast<void*>(nx.V2t);
       const LinkOperands ops = (j == 0 && !link_ctx) ? LinkOperands{c->sh_Q2, c->sh_K2, nullptr, nullptr, c->sh_V2t, nullptr, nullptr, 1} : set[j & 1];
       s = tc_layer_core(c, j, j == 0 ? hist : w.S, off, B, total, ops, last ? nullptr : w.S, (g.ln && j == 0 && !hist_normalized) ? 1 : 0,
-                        (g.ln && !last) ? 1 : 0, LinkMlpArgs{}, &side, w, st);
+                        (g.ln && !last) ? 1 : 0, LinkMlpArgs{}, &side, nullptr, w, st);
       if (s != LIME_OK) return s;
     }
     return LIME_OK;
   }
+  const bool few_rows = c->tc_mode == 1 && link_side_d128_wanted(g.d, c->d_ff, g.H, g.ell, B);
   for (int j = 0; j < g.n_layers; ++j) {
     const bool last = j == g.n_layers - 1;
     LinkOperands ops;
@@ -304,15 +312,24 @@ static lime_status encode_user_tc(Ctx* c, const void* hist, bool hist_normalized
       ops = LinkOperands{c->sh_Q2, c->sh_K2, c->sh_G2t, c->sh_U2t, c->sh_V2t, c->sh_cQ, c->sh_cK, 1};
     } else {
       if (j == 0 && (s = launch_ln_rows_bf16(link_ctx, BL, g.d, g.ln, c->ln_eps, w.That, st)) != LIME_OK) return s;
-      if ((s = make_link_operands(c, j, w.That, BL, !last, w.Q2, w.K2, w.G2t, w.U2t, w.V2t, w.cQ, w.cK, st)) != LIME_OK) return s;
+      if ((j == 0 || !few_rows) &&
+          (s = make_link_operands(c, j, w.That, BL, !last, w.Q2, w.K2, w.G2t, w.U2t, w.V2t, w.cQ, w.cK, st)) != LIME_OK)
+        return s;
       ops = LinkOperands{w.Q2, w.K2, w.G2t, w.U2t, w.V2t, w.cQ, w.cK, 0};
+    }
+    LinkSide128Args side1{};
+    if (few_rows) {
+      side1.LP = w.LP; side1.lp_accumulate = j > 0; side1.need_hist = j + 1 < g.n_layers - 1;
+      side1.WprepT = last ? nullptr : c->WprepT[j + 1];
+      side1.link_states = (last && !c->w.cand_Wv && c->cand_heads == 1) ? link_states : nullptr;
+      side1.Q2 = w.Q2; side1.K2 = w.K2; side1.G2t = w.G2t; side1.U2t = w.U2t;
     }
     LinkMlpArgs mlp{};
     mlp.LP = w.LP; mlp.lp_accumulate = j > 0;                                   // L^P = sum_j T^j  (Eq. 8)
     mlp.That_next = last ? nullptr : w.That;
     mlp.link_states = (last && !c->w.cand_Wv && c->cand_heads == 1) ? link_states : nullptr;
     s = tc_layer_core(c, j, j == 0 ? hist : w.S, off, B, total, ops, last ? nullptr : w.S, (g.ln && j == 0 && !hist_normalized) ? 1 : 0,
-                      (g.ln && !last) ? 1 : 0, mlp, nullptr, w, st);
+                      (g.ln && !last) ? 1 : 0, mlp, nullptr, few_rows ? &side1 : nullptr, w, st);
     if (s != LIME_OK) return s;
   }
   return LIME_OK;

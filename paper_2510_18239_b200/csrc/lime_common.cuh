@@ -377,6 +377,20 @@ struct LinkSide256Args {
 bool link_side_d256_supported(int d, int d_ff, int H, int ell);
 lime_status launch_link_side_d256(const LinkSide256Args& a, cudaStream_t st);
 
+// the same for d = 128 with four heads and few link rows: merge, GatedMLP and the next layer's operands (k_link_side_d128.cu)
+struct LinkSide128Args {
+  int users, ell;
+  const void* Ohat; const float *part_m, *part_s, *part_acc; const int32_t* chunk_start;
+  const void *WpostT, *WoT, *WprepT;                        // this layer's GatedMLP; next layer's operands (NULL: none wanted)
+  int need_hist, lp_accumulate, ln;
+  float *T_out, *LP;                                        // nullable
+  void *link_states, *Q2, *K2, *G2t, *U2t;                  // link_states (nullable): bf16 L^P instead of LP
+  float eps;
+  int* err;
+};
+bool link_side_d128_wanted(int d, int d_ff, int H, int ell, int64_t users);
+lime_status launch_link_side_d128(const LinkSide128Args& a, cudaStream_t st);
+
 struct HistUpdate256Args {
   const void* hist_in; void* hist_out; int64_t total;
   const void* K2;                       // folded link keys [users x H*ell x d] bf16

@@ -221,3 +221,14 @@ def test_three_layer_interaction_network(ell, w0, counts, form):
 def test_fp32_encode_in_one_launch(H, ell, lengths, phi, raw, per_user):
     """fp32 storage at d = 64: one to eight blocks a user, several 256-token rounds a block, histories beyond shared memory."""
     _encode_against_oracle(synth.F32, 64, H, ell, 3, lengths, phi, raw, per_user, 1e-4, 1e-5)
+
+
+@pytest.mark.parametrize("ell,B", [(32, 1), (32, 33), (32, 64), (64, 1), (64, 17), (64, 32)])
+@pytest.mark.parametrize("longest,per_user", [(40, False), (1300, True)])
+def test_link_side_of_few_rows(ell, B, longest, per_user):
+    """d = 128, four heads: 32 and 64 link rows a cluster, a last cluster that is not full, users without history or with
+    several chunks."""
+    r = np.random.default_rng(B)
+    lengths = [int(x) for x in r.integers(0, 40, size=B)]
+    lengths[B // 2] = longest
+    _encode_against_oracle(synth.BF16, 128, 4, ell, 3, lengths, "softmax", False, per_user, 6e-2, 2.5e-2)
