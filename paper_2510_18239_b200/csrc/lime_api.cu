@@ -2,9 +2,11 @@
 // method lives here; every step runs in the kernels of this directory.
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include "lime_common.cuh"
+#include "tc_common.cuh"
 
 namespace lime {
 
@@ -36,6 +38,40 @@ ProfScope::~ProfScope() {
 
 static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 static inline size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
+// Memory of weight copies comes from a pool per device: a cudaMalloc of 2 MB or more maps fresh pages every time (0.34 ms).
+// The pool keeps at most 64 MB that no context uses, and gives all of it back when the device's last context with such
+// copies goes.
+struct WeightPool {
+  std::mutex lock;
+  cudaMemPool_t pool = nullptr;
+  int users = 0;
+};
+static WeightPool g_weight_pool[kMaxDeviceOrdinals];
+static cudaError_t weight_alloc(int device, void** p, size_t bytes, cudaStream_t st) {
+  if (device < 0 || device >= kMaxDeviceOrdinals) return cudaErrorInvalidDevice;
+  WeightPool& w = g_weight_pool[device];
+  std::lock_guard<std::mutex> hold(w.lock);
+  if (w.pool == nullptr) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    cudaError_t e = cudaMemPoolCreate(&w.pool, &props);
+    uint64_t keep = 64ull << 20;
+    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(w.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e != cudaSuccess) return e;
+  }
+  const cudaError_t e = cudaMallocFromPoolAsync(p, bytes, w.pool, st);
+  if (e == cudaSuccess) ++w.users;
+  return e;
+}
+static void weight_free(int device, void* p) {
+  if (p == nullptr) return;
+  cudaFree(p);                                          // waits for the device, as every lime_destroy does
+  WeightPool& w = g_weight_pool[device];
+  std::lock_guard<std::mutex> hold(w.lock);
+  if (--w.users == 0) cudaMemPoolTrimTo(w.pool, 0);
+}
 static inline int elem_size(int dtype) { return dtype == LIME_F32 ? 4 : 2; }
 
 // Tokens per work item of the link<-history attention: a power of two in [lo, 2048] giving about three work items per
@@ -549,7 +585,7 @@ lime_status lime_destroy(lime_ctx* ctx) {
   for (int j = 0; j < LIME_MAX_LAYERS; ++j) { cudaFree(c->WoT[j]); cudaFree(c->WprepT[j]); cudaFree(c->WpostT[j]); cudaFree(c->WguT[j]); }
   cudaFree(c->sh_That); cudaFree(c->sh_Q2); cudaFree(c->sh_K2); cudaFree(c->sh_G2t); cudaFree(c->sh_U2t); cudaFree(c->sh_V2t);
   cudaFree(c->sh_cQ); cudaFree(c->sh_cK);
-  cudaFree(c->head_W1bT); cudaFree(c->head_W1aT); cudaFree(c->head_w2); cudaFree(c->ctx_first); cudaFree(c->side_w);
+  cudaFree(c->head_W1bT); cudaFree(c->head_W1aT); cudaFree(c->head_w2); cudaFree(c->ctx_first); weight_free(c->device, c->side_w);
   delete c;
   return LIME_OK;
 }
@@ -579,9 +615,7 @@ lime_status lime_set_weights(lime_ctx* ctx, const lime_weights* w, void* stream)
     // weights transposed, none folded; the first layer's operands for the shared links T^0 = L follow them in one buffer
     const size_t dd = (size_t)g.d * g.d * 2, HLd = (size_t)g.H * g.ell * g.d * 2;
     if (!c->side_w) {
-      // from the device's stream-ordered pool: a cudaMalloc of this size maps fresh 2 MB pages every time (0.34 ms), the pool keeps
-      // its mapping while any context is alive
-      LIME_CUDA(cudaMallocAsync(&c->side_w, (size_t)g.n_layers * 6 * dd + 2 * HLd + (size_t)g.d * g.ell * 2, st));
+      LIME_CUDA(weight_alloc(c->device, &c->side_w, (size_t)g.n_layers * 6 * dd + 2 * HLd + (size_t)g.d * g.ell * 2, st));
       char* at = static_cast<char*>(c->side_w);
       for (int j = 0; j < g.n_layers; ++j, at += 6 * dd) { c->WguT[j] = at + 3 * dd; c->WoT[j] = at + 5 * dd; }
       c->sh_Q2 = at; c->sh_K2 = at + HLd; c->sh_V2t = at + 2 * HLd;
