@@ -889,6 +889,8 @@ lime_status lime_contextualize_links(lime_ctx* ctx, const void* user_ctx, int32_
   const lime_ffn& f = c->ctx_mlp;
   const int w0 = f.n_hidden > 0 ? f.widths[0] : g.d;
   const char* W0c = static_cast<const char*>(f.W[0]) + (size_t)g.d * w0 * elem_size(g.dtype);     // rows d.. act on E^C
+  if (link_ctx_mma_supported(g.dtype, c->ctx_dc, w0, g.ell, g.d, ffn_tail(f, g.d)))
+    return launch_link_ctx_mma(c->ctx_first, user_ctx, c->ctx_dc, W0c, w0, B, g.ell, g.d, ffn_tail(f, g.d), link_ctx, static_cast<cudaStream_t>(stream));
   return launch_link_ctx_mlp(g.dtype, c->ctx_first, user_ctx, c->ctx_dc, W0c, w0, B, g.ell, ffn_tail(f, g.d), link_ctx,
                              static_cast<cudaStream_t>(stream));
 }

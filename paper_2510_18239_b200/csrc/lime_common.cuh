@@ -272,6 +272,10 @@ lime_status launch_rows_times_w(const void* X, int x_dtype, int64_t M, int K, co
                                 const float* bias, float* Y, void* Yt, int group, const char* name, cudaStream_t st);
 lime_status launch_link_ctx_mlp(int dtype, const float* first, const void* user_ctx, int d_c, const void* W0c, int w0, int B,
                                 int ell, const FfnArgs& f, float* out, cudaStream_t st);
+// the same with one hidden layer on tensor cores (k_link_ctx_mma.cu)
+bool link_ctx_mma_supported(int dtype, int d_c, int w0, int ell, int d, const FfnArgs& f);
+lime_status launch_link_ctx_mma(const float* first, const void* user_ctx, int d_c, const void* W0c, int w0, int B, int ell, int d,
+                                const FfnArgs& f, float* out, cudaStream_t st);
 // generic scorer through the interaction network; LSW fp32 [B x ell x w0], W0t = rows d.. of the first layer [d x w0]
 lime_status launch_score_head_simt(const ScoreArgs& a, const float* LSW, const void* W0t, const float* b0, int w0,
                                    const FfnArgs& f, cudaStream_t st);

@@ -232,3 +232,21 @@ def test_link_side_of_few_rows(ell, B, longest, per_user):
     lengths = [int(x) for x in r.integers(0, 40, size=B)]
     lengths[B // 2] = longest
     _encode_against_oracle(synth.BF16, 128, 4, ell, 3, lengths, "softmax", False, per_user, 6e-2, 2.5e-2)
+
+
+@pytest.mark.parametrize("d,ell,w0,d_c,B", [(128, 32, 128, 32, 3), (128, 16, 64, 1, 1), (256, 64, 256, 70, 2), (64, 48, 192, 8, 5)])
+def test_link_contextualisation_with_one_hidden_layer(d, ell, w0, d_c, B):
+    Bd = _lib()
+    dtype = synth.BF16
+    lime = Bd.Lime(d, 4, ell, 1, dtype=Bd.LIME_BF16)
+    links = synth.normal_storage(1, "l", (ell, d), 1.0, dtype)
+    w = {k: Bd.to_device(synth.normal_storage(2, k, (d, d), d ** -0.5, dtype), dtype) for k in ("Wq", "Wk", "Wv", "Wg", "Wu", "Wo")}
+    links_d = Bd.to_device(links, dtype)
+    lime.set_weights(links_d, [w])
+    layers = synth.ffn_weights(7, "ctx", (d + d_c, w0, d), dtype)
+    lime.set_context_mlp(d_c, [(Bd.to_device(a, dtype), torch.from_numpy(b).cuda()) for a, b in layers])
+    ec = synth.normal_storage(8, "ec", (B, d_c), 1.0, dtype)
+    got = Hh.to_f64(lime.contextualize_links(Bd.to_device(ec, dtype)))
+    L64 = [(synth.storage_to_f64(a, dtype), b.astype(np.float64)) for a, b in layers]
+    want = np.stack([O.contextualize_links(synth.storage_to_f64(links, dtype), synth.storage_to_f64(ec, dtype)[b], L64) for b in range(B)])
+    assert np.abs(got - want).max() <= 2e-5 * max(1.0, np.abs(want).max())
