@@ -14,7 +14,7 @@
 // The H * ell stacked (head, link) rows are processed in blocks of 128 = the TMEM lanes (one block per work item; a
 // second block of the same tokens finds them in L2).  Online softmax whose reference maximum is only raised
 // when the true maximum exceeds it by more than 8 (then the accumulator row is rescaled in TMEM), so most tiles need
-// no correction pass.  With LN = false the rows of X are LayerNorm-ed already and the corrections vanish.
+// no correction pass.  Rows that are LayerNorm-ed already need no corrections: k_link_attn_tmem_tc.cu.
 // With `silu` set the activation is SiLU(s) / N(U) (Algorithms 1-2): one pass per tile, no maximum, no row sums; the
 // divisor is the number of keys, and per-chunk partials are summed with equal weights.
 // Shared memory: three token stages, the folded queries of the current user, two P' buffers (the second MMA of a
@@ -101,15 +101,13 @@ __device__ __forceinline__ bool la_group_sync(uint64_t* bar, uint32_t& uses, int
 }
 
 // Pass 1 over this thread's LA_COLS scores: LayerNorm correction (LN) and the maximum over the valid columns.
-template <bool LN, bool MASK>
+template <bool MASK>
 __device__ __forceinline__ float la_pass1(float (&v)[LA_COLS], const float2* __restrict__ st, float cq, int col0, int nvalid) {
   float mx = -INFINITY;
 #pragma unroll
   for (int j = 0; j < LA_COLS; ++j) {
-    if (LN) {
-      const float2 c2 = st[col0 + j];
-      v[j] = (v[j] - cq * c2.y) * c2.x;
-    }
+    const float2 c2 = st[col0 + j];
+    v[j] = (v[j] - cq * c2.y) * c2.x;
     if (!MASK || col0 + j < nvalid) mx = fmaxf(mx, v[j]);
   }
   return mx;
@@ -118,7 +116,7 @@ __device__ __forceinline__ float la_pass1(float (&v)[LA_COLS], const float2* __r
 // Pass 2: p = 2^(s - m_ref) (softmax) or SiLU(s) (SILU: no reference maximum, no row sum), P' = p * rstd as bf16 into
 // the A-operand buffer (K-major over the tile's tokens, 128-byte swizzle); returns the sums of p and of P' * mu
 // through l_sum / mean_corr.
-template <bool LN, bool MASK, bool SILU>
+template <bool MASK, bool SILU>
 __device__ __forceinline__ void la_pass2(const float (&v)[LA_COLS], const float2* __restrict__ st, float m_ref, int col0, int nvalid,
                                          uint8_t* prow_base, uint32_t r, uint32_t chunk0, float& l_sum, float& mean_corr) {
   float ls0 = 0.f, ls1 = 0.f, mc0 = 0.f, mc1 = 0.f;
@@ -135,16 +133,12 @@ __device__ __forceinline__ void la_pass2(const float (&v)[LA_COLS], const float2
       }
       ls0 += e0;
       ls1 += e1;
-      if (LN) {
-        const float2 a = st[col0 + j], b = st[col0 + j + 1];
-        // what the MMA will see is the bf16-rounded P'; use the same rounded values for the mean term
-        const uint32_t pk = la_pack(e0 * a.x, e1 * b.x);
-        mc0 = fmaf(__uint_as_float(pk << 16), a.y, mc0);
-        mc1 = fmaf(__uint_as_float(pk & 0xffff0000u), b.y, mc1);
-        packed[j2] = pk;
-      } else {
-        packed[j2] = la_pack(e0, e1);
-      }
+      const float2 a = st[col0 + j], b = st[col0 + j + 1];
+      // what the MMA will see is the bf16-rounded P'; use the same rounded values for the mean term
+      const uint32_t pk = la_pack(e0 * a.x, e1 * b.x);
+      mc0 = fmaf(__uint_as_float(pk << 16), a.y, mc0);
+      mc1 = fmaf(__uint_as_float(pk & 0xffff0000u), b.y, mc1);
+      packed[j2] = pk;
     }
     *reinterpret_cast<uint4*>(prow_base + la_chunk_addr(r, chunk0 + (uint32_t)c8)) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
   }
@@ -171,7 +165,6 @@ struct ItemWalk {
   __device__ __forceinline__ void advance() { ci += stride; b0 = b1; b1 = b2; }
 };
 
-template <bool LN>
 __global__ void __launch_bounds__(LA_THREADS, 1)
 k_link_attn_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmQ2, const LinkAttnParams p) {
   using namespace tc;
@@ -367,53 +360,51 @@ k_link_attn_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
       int tok0, tok1;
       item_range(w.ci, b, tok0, tok1);
       const int n_tiles = (tok1 - tok0 + LA_TILE - 1) / LA_TILE;
-      const float cq = LN ? p.cQ[(int64_t)(p.shared ? 0 : b) * p.HL + rb * 128 + r] : 0.f;
+      const float cq = p.cQ[(int64_t)(p.shared ? 0 : b) * p.HL + rb * 128 + r];
       float m_ref = -INFINITY, l_sum = 0.f, mean_corr = 0.f;
       for (int t = 0; t < n_tiles && ok; ++t, ++g) {
         const int s = g % LA_XSTAGES, pb = g & 1;
         const int nvalid = min(LA_TILE, tok1 - tok0 - t * LA_TILE);
         const float2* st = stats + s * 128;
-        if (LN) {
-          // LayerNorm statistics of the tile's tokens: four lanes per token, 32 features each, held in registers
-          if (!mbar_wait(&x_full[s], (uint32_t)(g / LA_XSTAGES) & 1u, p.err, 61)) { ok = false; break; }
-          const int tok = 8 * sw + (lane >> 2), p4 = lane & 3;
-          const uint8_t* xs = smem + LA_OFF_X + s * LA_X_STAGE + (p4 >> 1) * LA_SUB + tok * 128;
-          uint4 u[4];
+        // LayerNorm statistics of the tile's tokens: four lanes per token, 32 features each, held in registers
+        if (!mbar_wait(&x_full[s], (uint32_t)(g / LA_XSTAGES) & 1u, p.err, 61)) { ok = false; break; }
+        const int tok = 8 * sw + (lane >> 2), p4 = lane & 3;
+        const uint8_t* xs = smem + LA_OFF_X + s * LA_X_STAGE + (p4 >> 1) * LA_SUB + tok * 128;
+        uint4 u[4];
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const int ch = (p4 & 1) * 4 + ((c + (p4 >> 1)) & 3);             // this lane's 4 chunks, rotated start
-            u[c] = *reinterpret_cast<const uint4*>(xs + ((ch ^ (tok & 7)) << 4));
-          }
-          float sum = 0.f;
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const uint32_t w[4] = {u[c].x, u[c].y, u[c].z, u[c].w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) sum += __uint_as_float(w[j] << 16) + __uint_as_float(w[j] & 0xffff0000u);
-          }
-          sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-          sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-          const float mu = sum * (1.0f / LA_D);
-          float var = 0.f;
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const uint32_t w[4] = {u[c].x, u[c].y, u[c].z, u[c].w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const float a = __uint_as_float(w[j] << 16) - mu, bb = __uint_as_float(w[j] & 0xffff0000u) - mu;
-              var = fmaf(a, a, var);
-              var = fmaf(bb, bb, var);
-            }
-          }
-          var += __shfl_xor_sync(0xffffffffu, var, 1);
-          var += __shfl_xor_sync(0xffffffffu, var, 2);
-          if (p4 == 0) {
-            const float2 rm = make_float2(rsqrtf(var * (1.0f / LA_D) + p.ln_eps), mu);
-            stats[s * 128 + tok] = rm;
-            if (p.stats_out != nullptr && rb == 0 && tok < nvalid) p.stats_out[tok0 + t * LA_TILE + tok] = rm;
-          }
-          if (!la_group_sync(stats_bar, stats_uses, lane, p.err, 62)) { ok = false; break; }
+        for (int c = 0; c < 4; ++c) {
+          const int ch = (p4 & 1) * 4 + ((c + (p4 >> 1)) & 3);             // this lane's 4 chunks, rotated start
+          u[c] = *reinterpret_cast<const uint4*>(xs + ((ch ^ (tok & 7)) << 4));
         }
+        float sum = 0.f;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const uint32_t w[4] = {u[c].x, u[c].y, u[c].z, u[c].w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) sum += __uint_as_float(w[j] << 16) + __uint_as_float(w[j] & 0xffff0000u);
+        }
+        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+        const float mu = sum * (1.0f / LA_D);
+        float var = 0.f;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const uint32_t w[4] = {u[c].x, u[c].y, u[c].z, u[c].w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float a = __uint_as_float(w[j] << 16) - mu, bb = __uint_as_float(w[j] & 0xffff0000u) - mu;
+            var = fmaf(a, a, var);
+            var = fmaf(bb, bb, var);
+          }
+        }
+        var += __shfl_xor_sync(0xffffffffu, var, 1);
+        var += __shfl_xor_sync(0xffffffffu, var, 2);
+        if (p4 == 0) {
+          const float2 rm = make_float2(rsqrtf(var * (1.0f / LA_D) + p.ln_eps), mu);
+          stats[s * 128 + tok] = rm;
+          if (p.stats_out != nullptr && rb == 0 && tok < nvalid) p.stats_out[tok0 + t * LA_TILE + tok] = rm;
+        }
+        if (!la_group_sync(stats_bar, stats_uses, lane, p.err, 62)) { ok = false; break; }
         if (!mbar_wait(&s_full[pb], (uint32_t)(g >> 1) & 1u, p.err, 63)) { ok = false; break; }
         tc_fence_after();
 
@@ -421,14 +412,14 @@ k_link_attn_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
         float v[LA_COLS];
         tmem_ld_32x32(lane_addr + COL_S + pb * 128 + col0, v);
         tmem_wait_ld();
-        float mx = nvalid == LA_TILE ? la_pass1<LN, false>(v, st, cq, col0, nvalid) : la_pass1<LN, true>(v, st, cq, col0, nvalid);
+        float mx = nvalid == LA_TILE ? la_pass1<false>(v, st, cq, col0, nvalid) : la_pass1<true>(v, st, cq, col0, nvalid);
         if (p.silu) {
           // SiLU(s) / N(U) needs neither a reference maximum nor row sums: one pass, no exchange between the row's threads
           if (g >= LA_PBUFS && !mbar_wait(&p_free[g % LA_PBUFS], (uint32_t)((g - LA_PBUFS) / LA_PBUFS) & 1u, p.err, 65)) { ok = false; break; }
           uint8_t* pbuf = smem + LA_OFF_P + (g % LA_PBUFS) * LA_P_BUF + (col0 >> 6) * LA_SUB;
           const uint32_t chunk0 = (uint32_t)(col0 & 63) >> 3;
-          if (nvalid == LA_TILE) la_pass2<LN, false, true>(v, st, 0.f, col0, nvalid, pbuf, r, chunk0, l_sum, mean_corr);
-          else la_pass2<LN, true, true>(v, st, 0.f, col0, nvalid, pbuf, r, chunk0, l_sum, mean_corr);
+          if (nvalid == LA_TILE) la_pass2<false, true>(v, st, 0.f, col0, nvalid, pbuf, r, chunk0, l_sum, mean_corr);
+          else la_pass2<true, true>(v, st, 0.f, col0, nvalid, pbuf, r, chunk0, l_sum, mean_corr);
           tc_fence_before();
           fence_proxy_async_smem();
           __syncwarp();
@@ -465,8 +456,8 @@ k_link_attn_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
         // pass 2: P' -> smem; K index = token column, so columns col0.. live in K-block col0 / 64, chunk (col0 % 64) / 8..
         uint8_t* pbuf = smem + LA_OFF_P + (g % LA_PBUFS) * LA_P_BUF + (col0 >> 6) * LA_SUB;
         const uint32_t chunk0 = (uint32_t)(col0 & 63) >> 3;
-        if (nvalid == LA_TILE) la_pass2<LN, false, false>(v, st, m_ref, col0, nvalid, pbuf, r, chunk0, l_sum, mean_corr);
-        else la_pass2<LN, true, false>(v, st, m_ref, col0, nvalid, pbuf, r, chunk0, l_sum, mean_corr);
+        if (nvalid == LA_TILE) la_pass2<false, false>(v, st, m_ref, col0, nvalid, pbuf, r, chunk0, l_sum, mean_corr);
+        else la_pass2<true, false>(v, st, m_ref, col0, nvalid, pbuf, r, chunk0, l_sum, mean_corr);
         tc_fence_before();
         fence_proxy_async_smem();
         __syncwarp();
@@ -563,6 +554,7 @@ bool link_attn_tc_supported(int dtype, int d, int H, int ell, int phi) {
 
 lime_status launch_link_attn_tc(const LinkAttnArgs& a, cudaStream_t st) {
   if (a.n_chunk_upper <= 0 || a.total == 0) return LIME_OK;   // no history: the merge step writes zeros
+  if (!a.ln) return launch_link_attn_d128_tmem(a, st);
   CUtensorMap tmX, tmQ2;
   const uint64_t users = a.shared ? 1 : (uint64_t)a.B;
   if (!make_tmap_bf16_sw128(&tmX, a.hist, (uint64_t)a.total, LA_D, LA_D, LA_TILE) ||
@@ -571,16 +563,14 @@ lime_status launch_link_attn_tc(const LinkAttnArgs& a, cudaStream_t st) {
   LinkAttnParams p;
   p.cQ = a.cQ; p.off = a.off; p.chunk_start = a.chunk_start; p.chunk_user = a.chunk_user; p.silu = a.silu; p.B = a.B; p.chunk = a.chunk; p.shared = a.shared;
   p.ell = a.ell; p.H = a.H; p.HL = a.H * a.ell; p.RB = p.HL / 128; p.ln_eps = a.ln_eps; p.part_m = a.part_m; p.part_s = a.part_s; p.part_acc = a.part_acc;
-  p.Ohat = (__nv_bfloat16*)a.Ohat; p.stats_out = a.ln ? a.stats_out : nullptr; p.err = a.err;
+  p.Ohat = (__nv_bfloat16*)a.Ohat; p.stats_out = a.stats_out; p.err = a.err;
   int grid = a.n_chunk_upper * p.RB < kSMs ? a.n_chunk_upper * p.RB : kSMs;
   grid -= grid % p.RB;                              // a CTA's work items then all share its row block
-  static bool smem_ln[kMaxDeviceOrdinals] = {}, smem_plain[kMaxDeviceOrdinals] = {};
-  lime_status es = a.ln ? ensure_dynamic_smem((const void*)k_link_attn_tc<true>, (int)LA_SMEM, smem_ln)
-                        : ensure_dynamic_smem((const void*)k_link_attn_tc<false>, (int)LA_SMEM, smem_plain);
+  static bool smem_set[kMaxDeviceOrdinals] = {};
+  const lime_status es = ensure_dynamic_smem((const void*)k_link_attn_tc, (int)LA_SMEM, smem_set);
   if (es != LIME_OK) return es;
   ProfScope _p("k_link_attn_tc", st);
-  if (a.ln) launch_pdl(k_link_attn_tc<true>, dim3(grid), dim3(LA_THREADS), LA_SMEM, st, tmX, tmQ2, p);
-  else launch_pdl(k_link_attn_tc<false>, dim3(grid), dim3(LA_THREADS), LA_SMEM, st, tmX, tmQ2, p);
+  launch_pdl(k_link_attn_tc, dim3(grid), dim3(LA_THREADS), LA_SMEM, st, tmX, tmQ2, p);
   LIME_LAUNCH_CHECK("k_link_attn_tc");
   return LIME_OK;
 }

@@ -344,6 +344,7 @@ struct LinkAttnArgs {
 bool link_attn_tc_supported(int dtype, int d, int H, int ell, int phi);
 int link_attn_d256_groups(int n_chunk_upper, int H, int ell);   // groups of CTAs (one CTA per 128-row block) of that kernel
 lime_status launch_link_attn_tc(const LinkAttnArgs& a, cudaStream_t st);
+lime_status launch_link_attn_d128_tmem(const LinkAttnArgs& a, cudaStream_t st);   // the same for rows LayerNorm-ed already (a.ln must be 0)
 
 struct HistUpdateArgs {
   const void* hist_in; void* hist_out; int64_t total;

@@ -250,3 +250,11 @@ def test_link_contextualisation_with_one_hidden_layer(d, ell, w0, d_c, B):
     L64 = [(synth.storage_to_f64(a, dtype), b.astype(np.float64)) for a, b in layers]
     want = np.stack([O.contextualize_links(synth.storage_to_f64(links, dtype), synth.storage_to_f64(ec, dtype)[b], L64) for b in range(B)])
     assert np.abs(got - want).max() <= 2e-5 * max(1.0, np.abs(want).max())
+
+
+@pytest.mark.parametrize("d,H,ell", [(128, 4, 32), (128, 4, 64), (256, 4, 32), (256, 8, 64)])
+@pytest.mark.parametrize("lengths", [[1], [95, 96, 97, 0, 127, 128, 129, 191, 193, 257, 289], [4500, 3, 700], [130] * 160])
+@pytest.mark.parametrize("phi,per_user", [("softmax", True), ("silu", False)])
+def test_attention_over_token_tiles(d, H, ell, lengths, phi, per_user):
+    """Histories around the 96- and 128-token tiles, one of several chunks, more users than CTAs."""
+    _encode_against_oracle(synth.BF16, d, H, ell, 2, lengths, phi, False, per_user, 6e-2, 4e-2 if phi == "silu" else 2.5e-2)
