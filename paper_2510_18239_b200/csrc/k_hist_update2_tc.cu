@@ -513,6 +513,7 @@ static lime_status launch_hu2(const HistUpdateArgs& a, int HL, cudaStream_t st) 
 
 lime_status launch_hist_update2_tc(const HistUpdateArgs& a, int H, cudaStream_t st) {
   if (a.total == 0) return LIME_OK;
+  if (!a.ln && hist_update_tmem_supported(H * a.ell, a.ell)) return launch_hist_update_tmem(a, H * a.ell, st);
   switch (a.ell) {
     case 32: return launch_hu2<32>(a, H * a.ell, st);
     case 64: return launch_hu2<64>(a, H * a.ell, st);

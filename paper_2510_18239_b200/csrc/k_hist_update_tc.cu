@@ -22,7 +22,8 @@
 // [gate | up].  Shared memory: one token stage (32 KB), K2, [G2 | U2], W_o (128 KB), one P/U buffer (32 KB).
 //
 // With `out_ln` the rows are written already LayerNorm-ed (the next layer applies LayerNorm to every row it reads and
-// nothing else reads them, Eq. 8), so that the next layer's kernels run with LN = false.
+// nothing else reads them, Eq. 8), so that the next layer's kernels are those for
+// rows LayerNorm-ed already (k_hist_update_tmem_tc.cu).
 //
 // Built for d = d_ff = 128, H * ell = 128 and ell in {16, 32}.
 #include "lime_common.cuh"
@@ -52,7 +53,7 @@ static_assert(HU_SMEM <= 232448, "shared memory budget of one CTA");
 struct HistUpdateParams {
   __nv_bfloat16* out;            // [total x d]
   const float* cK;               // [users x HL] row sums of K2
-  const float2* stats_in;        // nullable (LN): {rstd, mean} of every history row, computed by the attention kernel
+  const float2* stats_in;        // nullable: {rstd, mean} of every history row, computed by the attention kernel
   const int32_t* off;            // [B+1]
   const int32_t* tile_start;     // [B+1] prefix of per-user tile counts (tile = 128 tokens)
   int B, ell, shared, out_ln;
@@ -117,7 +118,7 @@ __device__ __forceinline__ bool hu_group_sync(uint64_t* bar, uint32_t& uses, int
   return ok;
 }
 
-template <int ELL, bool LN>
+template <int ELL>
 __global__ void __launch_bounds__(HU_THREADS, 1)
 k_hist_update_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmK2,
                  const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmU,
@@ -321,53 +322,49 @@ k_hist_update_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
       st_ahead = row < tr_next.row_hi ? __ldg(p.stats_in + row) : make_float2(1.f, 0.f);
     };
     auto take_stats = [&](int g) -> bool {
-      if (LN && p.stats_in != nullptr) {
+      if (p.stats_in != nullptr) {
         rstd_r = st_ahead.x; mu_r = st_ahead.y;
         if (lane == 0) mbar_arrive(x_empty);
         return true;
       }
-      if (LN) {
-        if (!mbar_wait(x_full, (uint32_t)g & 1u, p.err, 31)) return false;
-        const int tok = 8 * rw + (lane >> 2), p4 = lane & 3;
-        const uint8_t* xs = smem + HU_OFF_X + (p4 >> 1) * HU_SUB + tok * 128;
-        uint4 u[4];
+      if (!mbar_wait(x_full, (uint32_t)g & 1u, p.err, 31)) return false;
+      const int tok = 8 * rw + (lane >> 2), p4 = lane & 3;
+      const uint8_t* xs = smem + HU_OFF_X + (p4 >> 1) * HU_SUB + tok * 128;
+      uint4 u[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int ch = (p4 & 1) * 4 + ((c + (p4 >> 1)) & 3);
-          u[c] = *reinterpret_cast<const uint4*>(xs + ((ch ^ (tok & 7)) << 4));
-        }
-        float sum = 0.f;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const uint32_t w[4] = {u[c].x, u[c].y, u[c].z, u[c].w};
-#pragma unroll
-          for (int j = 0; j < 4; ++j) sum += __uint_as_float(w[j] << 16) + __uint_as_float(w[j] & 0xffff0000u);
-        }
-        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-        const float mu = sum * (1.0f / HU_D);
-        float var = 0.f;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const uint32_t w[4] = {u[c].x, u[c].y, u[c].z, u[c].w};
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float a = __uint_as_float(w[j] << 16) - mu, bb = __uint_as_float(w[j] & 0xffff0000u) - mu;
-            var = fmaf(a, a, var);
-            var = fmaf(bb, bb, var);
-          }
-        }
-        var += __shfl_xor_sync(0xffffffffu, var, 1);
-        var += __shfl_xor_sync(0xffffffffu, var, 2);
-        if (p4 == 0) stats[(g & 1) * 128 + tok] = make_float2(rsqrtf(var * (1.0f / HU_D) + p.ln_eps), mu);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(x_empty);                 // this warp is done with the staged tile
-        if (!hu_group_sync(stats_bar, stats_uses, lane, p.err, 35)) return false;
-        const float2 st = stats[(g & 1) * 128 + r];
-        rstd_r = st.x; mu_r = st.y;
-      } else {
-        if (lane == 0) mbar_arrive(x_empty);
+      for (int c = 0; c < 4; ++c) {
+        const int ch = (p4 & 1) * 4 + ((c + (p4 >> 1)) & 3);
+        u[c] = *reinterpret_cast<const uint4*>(xs + ((ch ^ (tok & 7)) << 4));
       }
+      float sum = 0.f;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const uint32_t w[4] = {u[c].x, u[c].y, u[c].z, u[c].w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) sum += __uint_as_float(w[j] << 16) + __uint_as_float(w[j] & 0xffff0000u);
+      }
+      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+      const float mu = sum * (1.0f / HU_D);
+      float var = 0.f;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const uint32_t w[4] = {u[c].x, u[c].y, u[c].z, u[c].w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float a = __uint_as_float(w[j] << 16) - mu, bb = __uint_as_float(w[j] & 0xffff0000u) - mu;
+          var = fmaf(a, a, var);
+          var = fmaf(bb, bb, var);
+        }
+      }
+      var += __shfl_xor_sync(0xffffffffu, var, 1);
+      var += __shfl_xor_sync(0xffffffffu, var, 2);
+      if (p4 == 0) stats[(g & 1) * 128 + tok] = make_float2(rsqrtf(var * (1.0f / HU_D) + p.ln_eps), mu);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(x_empty);                 // this warp is done with the staged tile
+      if (!hu_group_sync(stats_bar, stats_uses, lane, p.err, 35)) return false;
+      const float2 st = stats[(g & 1) * 128 + r];
+      rstd_r = st.x; mu_r = st.y;
       return true;
     };
 
@@ -378,7 +375,7 @@ k_hist_update_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
       const int b = tr_next.tu.b;
       if (!mbar_wait(s2_full, (uint32_t)g & 1u, p.err, 32)) return false;
       tc_fence_after();
-      if (LN && b != ck_user && (ck_user < 0 || !p.shared)) {
+      if (b != ck_user && (ck_user < 0 || !p.shared)) {
         // scores(g) exist, so every warp has finished the softmax of tile g-1 (its P was needed first): nobody still
         // reads the previous user's sums.  Every warp of a part writes the same values.
         float* ckw = reinterpret_cast<float*>(smem + HU_OFF_CK) + col0;
@@ -394,7 +391,7 @@ k_hist_update_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
 #pragma unroll
         for (int j = 0; j < ELL; ++j) {
           const int c = h * ELL + j;
-          if (LN) v[c] = (v[c] - mu_r * ck_s[c]) * rstd_r;
+          v[c] = (v[c] - mu_r * ck_s[c]) * rstd_r;
           mx = fmaxf(mx, v[c]);
         }
         float inv;
@@ -525,10 +522,10 @@ k_hist_update_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
       return true;
     };
 
-    if (LN && p.stats_in != nullptr) fetch_stats(0);
+    if (p.stats_in != nullptr) fetch_stats(0);
     ok = take_stats(0) && softmax(0);
     for (int g = 0; g < n && ok; ++g) {
-      if (LN && p.stats_in != nullptr && g + 1 < n) fetch_stats(g + 1);
+      if (p.stats_in != nullptr && g + 1 < n) fetch_stats(g + 1);
       if (!silu_mul(g)) { ok = false; break; }                                   // [gate|up](g) ran under store(g-1)
       // statistics of the next tile while S'(g) is formed, so that its stage can be refilled a whole tile early
       if (g + 1 < n && !take_stats(g + 1)) { ok = false; break; }
@@ -564,23 +561,22 @@ static lime_status launch_hu(const HistUpdateArgs& a, cudaStream_t st) {
       !make_tmap_bf16_sw128(&tmWo, a.WoT, HU_D, HU_F, HU_F, 128))
     return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
   HistUpdateParams p;
-  p.out = (__nv_bfloat16*)a.hist_out; p.cK = a.cK; p.stats_in = a.ln ? a.stats_in : nullptr; p.off = a.off; p.tile_start = a.tile_start; p.B = a.B; p.silu = a.silu; p.ell = ELL;
+  p.out = (__nv_bfloat16*)a.hist_out; p.cK = a.cK; p.stats_in = a.stats_in; p.off = a.off; p.tile_start = a.tile_start; p.B = a.B; p.silu = a.silu; p.ell = ELL;
   p.shared = a.shared; p.out_ln = a.out_ln; p.ln_eps = a.ln_eps; p.err = a.err;
   int grid = a.n_tile_upper < kSMs ? a.n_tile_upper : kSMs;
   if (grid < 1) return LIME_OK;
-  static bool smem_ln[kMaxDeviceOrdinals] = {}, smem_plain[kMaxDeviceOrdinals] = {};
-  lime_status es = a.ln ? ensure_dynamic_smem((const void*)k_hist_update_tc<ELL, true>, (int)HU_SMEM, smem_ln)
-                        : ensure_dynamic_smem((const void*)k_hist_update_tc<ELL, false>, (int)HU_SMEM, smem_plain);
+  static bool smem_set[kMaxDeviceOrdinals] = {};
+  const lime_status es = ensure_dynamic_smem((const void*)k_hist_update_tc<ELL>, (int)HU_SMEM, smem_set);
   if (es != LIME_OK) return es;
   ProfScope _p("k_hist_update_tc", st);
-  if (a.ln) launch_pdl(k_hist_update_tc<ELL, true>, dim3(grid), dim3(HU_THREADS), HU_SMEM, st, tmX, tmK2, tmG, tmU, tmWo, p);
-  else launch_pdl(k_hist_update_tc<ELL, false>, dim3(grid), dim3(HU_THREADS), HU_SMEM, st, tmX, tmK2, tmG, tmU, tmWo, p);
+  launch_pdl(k_hist_update_tc<ELL>, dim3(grid), dim3(HU_THREADS), HU_SMEM, st, tmX, tmK2, tmG, tmU, tmWo, p);
   LIME_LAUNCH_CHECK("k_hist_update_tc");
   return LIME_OK;
 }
 
 lime_status launch_hist_update_tc(const HistUpdateArgs& a, cudaStream_t st) {
   if (a.total == 0) return LIME_OK;
+  if (!a.ln) return launch_hist_update_tmem(a, 128, st);
   switch (a.ell) {
     case 16: return launch_hu<16>(a, st);
     case 32: return launch_hu<32>(a, st);

@@ -101,22 +101,27 @@ __device__ __forceinline__ float lt_ex2(float x) {
 template <bool SILU, int COLS>
 __device__ __forceinline__ float lt_probabilities(const float (&v)[COLS], float m_ref, uint32_t taddr) {
   constexpr int STEP = COLS % 32 == 0 ? 32 : 16;
-  float ls[4] = {0.f, 0.f, 0.f, 0.f};
+  float2 s0 = make_float2(0.f, 0.f), s1 = s0;
 #pragma unroll
   for (int c = 0; c < COLS; c += STEP) {
     float packed[STEP / 2];
 #pragma unroll
     for (int j = 0; j < STEP / 2; ++j) {
-      const float e0 = SILU ? lt_silu(v[c + 2 * j]) : lt_ex2(v[c + 2 * j] - m_ref);
-      const float e1 = SILU ? lt_silu(v[c + 2 * j + 1]) : lt_ex2(v[c + 2 * j + 1] - m_ref);
-      ls[(2 * j) & 3] += e0;
-      ls[(2 * j + 1) & 3] += e1;
-      packed[j] = __uint_as_float(lt_pack(e0, e1));
+      float2 e = make_float2(v[c + 2 * j], v[c + 2 * j + 1]);
+      if (SILU) {
+        e = make_float2(lt_silu(e.x), lt_silu(e.y));
+      } else {
+        e = __fadd2_rn(e, make_float2(-m_ref, -m_ref));
+        e = make_float2(lt_ex2(e.x), lt_ex2(e.y));
+        if (j & 1) s1 = __fadd2_rn(s1, e); else s0 = __fadd2_rn(s0, e);
+      }
+      packed[j] = __uint_as_float(lt_pack(e.x, e.y));
     }
     if constexpr (STEP == 32) tc::tmem_st_32x16(taddr + (uint32_t)(c >> 1), packed);
     else tc::tmem_st_32x8(taddr + (uint32_t)(c >> 1), packed);
   }
-  return (ls[0] + ls[1]) + (ls[2] + ls[3]);
+  s0 = __fadd2_rn(s0, s1);
+  return s0.x + s0.y;
 }
 
 // Walk over the (user, chunk) items of a CTA's group.  The index arrays stay in global memory; the items and users of the

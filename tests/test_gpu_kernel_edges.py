@@ -252,7 +252,7 @@ def test_link_contextualisation_with_one_hidden_layer(d, ell, w0, d_c, B):
     assert np.abs(got - want).max() <= 2e-5 * max(1.0, np.abs(want).max())
 
 
-@pytest.mark.parametrize("d,H,ell", [(128, 4, 32), (128, 4, 64), (256, 4, 32), (256, 8, 64)])
+@pytest.mark.parametrize("d,H,ell", [(128, 4, 32), (128, 8, 16), (128, 4, 64), (128, 8, 32), (256, 4, 32), (256, 8, 64)])
 @pytest.mark.parametrize("lengths", [[1], [95, 96, 97, 0, 127, 128, 129, 191, 193, 257, 289], [4500, 3, 700], [130] * 160])
 @pytest.mark.parametrize("phi,per_user", [("softmax", True), ("silu", False)])
 def test_attention_over_token_tiles(d, H, ell, lengths, phi, per_user):
