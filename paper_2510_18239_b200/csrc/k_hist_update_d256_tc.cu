@@ -9,8 +9,8 @@
 // the GatedMLP weights follow unfolded - at this width folding W_V W_g into the link side (as the d = 128 kernels do)
 // would cost twice the tensor work and twice the operand traffic:
 //   scores [128 x H*ell] = X . K2^T, 256 stacked (head, link) rows per contraction
-//   per group c of 128 stacked rows (two heads of 64 links, four of 32): per-head softmax over the links, unnormalised (or
-//                             SiLU(s) / ell) -> P_c (bf16);  O[:, head] = P_head [128 x ell] . V_head [ell x d_h]
+//   per-head softmax over the links, unnormalised (or SiLU(s) / ell) -> P (bf16)
+//   O[:, head] = P_head [128 x ell] . V_head [ell x d_h]
 //   O * 1 / (row sum of the head) -> bf16
 //   per half hf of the hidden columns:   [gate | up] = O . [W_g | W_u][:, hf]  ->  U = SiLU(gate) * up (bf16)
 //                                        S' (+)= U . W_o[hf rows, :]
@@ -18,18 +18,21 @@
 // Every contraction but the value mix is issued 256 columns wide: at 128 columns an MMA re-reads its A operand from
 // shared memory twice as often per flop, and shared-memory bandwidth (operands in, TMA writes, the row warps) is what
 // the tensor pipe waits for here.
-// TMEM (512 columns) as two regions that swap roles every tile.  R0: scores of heads 0-3, overwritten head by head by
-// O as its scores are consumed, later S'.  R1: scores of heads 4-7, later [gate | up] of one half.  The next tile's
-// R0 is this tile's R1, which is free before S' is even complete.
-// Shared memory: X tile 64 KB (dead once the scores are formed: then the two P buffers, then O); V[T]^T of the user, later
-// U, later the patches S' leaves through, 32 KB; a ring of three 32 KB operand slabs ([256 rows x 64 of the contraction
-// index]) through which K2, [W_g | W_u] and W_o stream from L2 in the order the MMA issuer consumes them.  (Seven
-// 16 KB slabs of 32 of the contraction index, 64-byte swizzle - half again as many bytes in flight - were measured:
-// 8.3 against 7.4 ms per production_ragged step; what limits the stream is not its depth but the 64-byte pieces.)
-// Warp 0 TMA producer, warp 1 MMA issuer, warps 2-17 token rows.  For the softmax the row warps form two groups that
-// take alternate groups of 128 stacked rows, one thread per token and 64 of them (one head of 64 links, or two of 32, whose
-// maxima and sums are the two halves' own): no exchange between threads, and one group's exponentials overlap the other
-// group's value mix.  Elsewhere four threads share a token, a quarter of the columns each.
+// TMEM (512 columns) as two regions.  A: scores of the first 256 stacked rows, then P of all of them (a thread's bf16 pairs
+// over its own scores: the first group's in the first half of its columns, the second's in the other), then [gate | up] of one
+// half, then U over the gates.  B: scores of the other 256 stacked rows, then O, then S'.  P and U are A operands there: no
+// shared memory, no proxy fence.  A takes the next tile's first scores right behind this tile's last contraction.
+// Shared memory: X tile 64 KB (dead once the scores are formed, then O as bf16) and a ring of four 32 KB operand slabs
+// ([256 rows x 64 of the contraction index]) through which K2, V[T]^T, [W_g | W_u] and W_o stream from L2 in the order the MMA
+// issuer consumes them.  (16 KB slabs of 32 of the contraction index, 64-byte swizzle - half again as many in flight - were
+// measured and lose: what limits the stream is not its depth but the 64-byte pieces.)
+// Warp 0 TMA producer, warp 1 MMA issuer, warps 2-17 token rows: for the softmax one thread per token and 64 stacked rows of
+// each region (one head of 64 links, or two of 32, whose maxima and sums are the two halves' own: no exchange between
+// threads); elsewhere four threads share a token, a quarter of the columns each.
+// Measured (1024 users of 1024..4096 tokens, 64 links x 8 heads): 27500 cycles a tile against 32000 with P and U in shared memory
+// (over the token tile, so that the softmax had to wait for every score), 11300 of them tensor time; 2.65 -> 2.41 ms a launch at
+// the 1 kW power cap, where the batch runs.  What is left: the chain of one tile (TMEM has no room for a second), of which the
+// slabs' arrival (640 KB a tile from L2) takes 6300 and the rows' way out 6500.
 #include "lime_common.cuh"
 #include "tc_common.cuh"
 
@@ -37,14 +40,15 @@ namespace lime {
 
 constexpr int HC_D = 256, HC_F = 256, HC_TILE = 128;
 constexpr int HC_PARTS = 4, HC_ROW_WARPS = 4 * HC_PARTS, HC_THREADS = 64 + 32 * HC_ROW_WARPS;
-constexpr int HC_RING = 3;
+constexpr int HC_RING = 4;
 constexpr uint32_t HC_SUB = 128 * 128;                          // bytes of one [128 rows x 64 bf16] swizzled sub-tile
 constexpr uint32_t HC_SLAB = 2 * HC_SUB;                        // one ring slot: [256 rows x 64 bf16]
-constexpr uint32_t HC_OFF_XO = 0;                               // token tile, then P of two groups, then O: 4 K-blocks
-constexpr uint32_t HC_OFF_PU = HC_OFF_XO + 4 * HC_SUB;          // V[T]^T [256 features x 64 links], later U: 2 K-blocks
-constexpr uint32_t HC_OFF_RING = HC_OFF_PU + 2 * HC_SUB;
-constexpr uint32_t HC_OFF_EXCH = HC_OFF_RING + HC_RING * HC_SLAB;     // [2 parities][PARTS][128] float2
-constexpr uint32_t HC_OFF_INV = HC_OFF_EXCH + 2 * HC_PARTS * 128 * 8; // [8 heads][128 rows] 1 / softmax row sum
+constexpr uint32_t HC_OFF_XO = 0;                               // token tile, then O: 4 K-blocks
+constexpr uint32_t HC_OFF_RING = HC_OFF_XO + 4 * HC_SUB;
+constexpr uint32_t HC_PATCH = 8 * 128;                          // a row warp's own: 8 of its 32 rows on their way out
+constexpr uint32_t HC_OFF_PATCH = HC_OFF_RING + HC_RING * HC_SLAB;
+constexpr uint32_t HC_OFF_EXCH = HC_OFF_PATCH + HC_ROW_WARPS * HC_PATCH;   // [PARTS][128] float2
+constexpr uint32_t HC_OFF_INV = HC_OFF_EXCH + HC_PARTS * 128 * 8;     // [8 heads][128 rows] 1 / softmax row sum
 constexpr uint32_t HC_OFF_BAR = HC_OFF_INV + 8 * 128 * 4;
 constexpr int HC_IDX_CAP = 1025;                                // users + 1 whose offsets are staged in shared memory
 constexpr uint32_t HC_OFF_IDX = HC_OFF_BAR + 512;
@@ -55,7 +59,7 @@ struct HistUpdate256Params {
   __nv_bfloat16* out;            // [total x d]
   const int32_t* off;            // [B+1]
   const int32_t* tile_start;     // [B+1] prefix of per-user tile counts (tile = 128 tokens)
-  int B, H, HL, NG, shared, out_ln;   // NG = HL / 128 groups of 128 stacked rows
+  int B, H, HL, shared, out_ln;
   int silu;                      // 1: P = SiLU(scores) / ell (Algorithm 2) instead of the per-head softmax
   float ln_eps;
   int* err;
@@ -110,41 +114,36 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   }
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + HC_OFF_BAR);
   uint64_t* full = bars;              // [HC_RING] operand slab landed
-  uint64_t* empty = bars + 3;         // [HC_RING] the MMAs that read the slab have run
-  uint64_t* x_full = bars + 6;        // per tile
-  uint64_t* x_free = bars + 7;        // per tile: the last contraction that reads the X / P / O buffer has run
-  uint64_t* v_full = bars + 8;        // per tile: V[T]^T of the tile's user landed
-  uint64_t* pu_free = bars + 9;       // per tile: every row warp is done with its patch of the V / U buffer (16 warps)
-  uint64_t* s_full = bars + 10;       // [2] per tile: scores of heads 0-3 / 4-7 in TMEM
-  uint64_t* p_ready = bars + 12;      // [2] per group, by row-warp group: P_c in smem (8 warps)
-  uint64_t* pv_done = bars + 14;      // [2] per group: value mix done (that P buffer free)
-  uint64_t* o_full = bars + 16;       // per tile: O complete in TMEM
-  uint64_t* o_ready = bars + 17;      // per tile: O as bf16 in smem (16 warps)
-  uint64_t* gu_full = bars + 18;      // per (tile, half): [gate | up] complete
-  uint64_t* u_ready = bars + 19;      // per (tile, half): U in smem, [gate | up] read (16 warps)
-  uint64_t* sp_full = bars + 20;      // per tile: S' complete
-  uint64_t* sp_read = bars + 21;      // per tile: S' read out of TMEM (16 warps)
-  uint64_t* row_bar = bars + 22;      // [4] rendezvous of the four warps sharing a TMEM lane quarter
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 26);
-  static_assert(HC_RING == 3, "barrier table above");
+  uint64_t* empty = bars + 4;         // [HC_RING] the MMAs that read the slab have run
+  uint64_t* x_full = bars + 8;        // per tile
+  uint64_t* x_free = bars + 9;        // per tile: the last contraction that reads the X / O buffer has run
+  uint64_t* s_full = bars + 10;       // [2] per tile: scores in region A / B
+  uint64_t* p_ready = bars + 12;      // per tile: P in TMEM, scores consumed (16 warps)
+  uint64_t* o_full = bars + 13;       // per tile: O complete in TMEM
+  uint64_t* o_ready = bars + 14;      // per tile: O as bf16 in smem (16 warps)
+  uint64_t* gu_full = bars + 15;      // per (tile, half): [gate | up] complete
+  uint64_t* u_ready = bars + 16;      // per (tile, half): U in TMEM, [gate | up] read (16 warps)
+  uint64_t* sp_full = bars + 17;      // per tile: S' complete
+  uint64_t* sp_read = bars + 18;      // per tile: S' read out of TMEM (16 warps)
+  uint64_t* row_bar = bars + 19;      // [4] rendezvous of the four warps sharing a TMEM lane quarter
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 23);
+  static_assert(HC_RING == 4, "barrier table above");
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_tiles_all = p.tile_start[p.B];
   const int t_begin = (int)(((int64_t)blockIdx.x * n_tiles_all) / gridDim.x);
   const int t_end = (int)(((int64_t)(blockIdx.x + 1) * n_tiles_all) / gridDim.x);
   const int n = t_end - t_begin;
-  constexpr int HPG = 128 / ELL;                             // heads per group of 128 stacked rows
   constexpr uint32_t V_ROW = ELL * 2;                        // bytes of a V[T]^T row (its swizzle span)
   constexpr uint32_t V_BYTES = HC_D * V_ROW;
-  const int NG = p.NG;                                       // groups of 128 stacked rows
   const int d_h = HC_D / p.H;
   const int n_sg = (p.HL + 255) / 256;                       // score contractions per tile (four heads each)
   const int sc_boxes = p.HL >= 256 ? 2 : 1;                  // 128-row boxes of K2 per score slab
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < HC_RING; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
-    mbar_init(x_full, 1); mbar_init(x_free, 1); mbar_init(v_full, 1); mbar_init(pu_free, HC_ROW_WARPS);
-    for (int i = 0; i < 2; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_ready[i], HC_ROW_WARPS / 2); mbar_init(&pv_done[i], 1); }
+    mbar_init(x_full, 1); mbar_init(x_free, 1);
+    mbar_init(&s_full[0], 1); mbar_init(&s_full[1], 1); mbar_init(p_ready, HC_ROW_WARPS);
     mbar_init(o_full, 1); mbar_init(o_ready, HC_ROW_WARPS); mbar_init(gu_full, 1); mbar_init(u_ready, HC_ROW_WARPS);
     mbar_init(sp_full, 1); mbar_init(sp_read, HC_ROW_WARPS);
     for (int i = 0; i < 4; ++i) mbar_init(&row_bar[i], HC_PARTS);
@@ -171,7 +170,6 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
       const uint64_t pol_stream = policy_evict_first(), pol_keep = policy_evict_last();
       bool ok = true;
       int g = 0, sl = 0;
-      bool v_sent = false;
       // one ring slab: one or two boxes of 128 rows at contraction offset x
       auto slab = [&](const CUtensorMap* m, int x, int y0, int y1, int boxes) -> bool {
         const int s = sl % HC_RING;
@@ -195,7 +193,7 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         // only needs a free ring slot, so it travels while the previous tile is still being finished.
         ok = k2_slab(0, 0);
         if (!ok) break;
-        // the X / P / O buffer is free once the previous tile's last contraction over O has run
+        // the X / O buffer is free once the previous tile's last contraction over O has run
         if (g > 0 && !mbar_wait(x_free, (uint32_t)(g - 1) & 1u, p.err, 12)) { ok = false; break; }
         const int row0 = off[b] + (t - tu.lo) * HC_TILE;
         mbar_arrive_expect_tx(x_full, 4 * HC_SUB);
@@ -204,11 +202,14 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         for (int sg = 1; sg < n_sg && ok; ++sg)
           for (int kb = 0; kb < 4 && ok; ++kb) ok = k2_slab(sg, kb);
         if (!ok) break;
-        // the user's link values go where U of the previous tile was and where its rows left through
-        if (g > 0 && !mbar_wait(pu_free, (uint32_t)(g - 1) & 1u, p.err, 13)) { ok = false; break; }
-        mbar_arrive_expect_tx(v_full, V_BYTES);
-        tma_load_2d_hint(smem + HC_OFF_PU, &tmV, 0, urow * HC_D, v_full, pol_keep);
-        v_sent = true;
+        // the user's link values, a slab of their own layout ([256 features x ell links])
+        {
+          const int s = sl % HC_RING;
+          if (!mbar_wait(&empty[s], ((uint32_t)(sl / HC_RING) & 1u) ^ 1u, p.err, 13)) { ok = false; break; }
+          mbar_arrive_expect_tx(&full[s], V_BYTES);
+          tma_load_2d_hint(smem + HC_OFF_RING + s * HC_SLAB, &tmV, 0, urow * HC_D, &full[s], pol_keep);
+          ++sl;
+        }
         // then per half of the hidden columns the gate and up columns of W_g / W_u (contraction over d) and that half's
         // rows of W_o (all output columns)
         for (int hf = 0; hf < 2 && ok; ++hf) {
@@ -222,87 +223,94 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         // giving up: let the copies already issued land (bounded) before this CTA's shared memory goes away
         const int gl = g < n ? g : n - 1;
         if (g > 0 || sl > 0) mbar_wait_quiet(x_full, (uint32_t)gl & 1u);
-        if (v_sent) mbar_wait_quiet(v_full, (uint32_t)gl & 1u);
         for (int j = 0; j < sl && j < HC_RING; ++j) mbar_wait_quiet(&full[(sl - 1 - j) % HC_RING], (uint32_t)((sl - 1 - j) / HC_RING) & 1u);
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0 && n > 0) {
+    // The whole warp runs this code and one elected lane issues (warp-uniform descriptors, see k_link_attn_tmem_tc.cu).
+    if (n > 0) {
       constexpr uint32_t idesc_256 = make_idesc_bf16(128, 256);
       const uint32_t idesc_sc = p.HL >= 256 ? idesc_256 : make_idesc_bf16(128, 128);
       const uint32_t idesc_v = make_idesc_bf16(128, d_h);
       const uint32_t sbase = smem_u32(smem);
-      const uint32_t xo = sbase + HC_OFF_XO, pu = sbase + HC_OFF_PU;
-      bool ok = true;
-      int sl = 0;
-      uint32_t p_uses[2] = {0u, 0u};
-      // one operand slab (64 of the contraction index): D[128 x N] (+)= A_kblock . slab^T
-      auto slab_mma = [&](uint32_t d_col, uint32_t a_kblock, uint32_t idesc, bool first) -> bool {
-        const int s = sl % HC_RING;
-        if (!mbar_wait(&full[s], (uint32_t)(sl / HC_RING) & 1u, p.err, 22)) return false;
+      const uint32_t A = __shfl_sync(0xffffffffu, tmem_base, 0), B = A + 256u;
+      const uint64_t dxo = make_sdesc_k_sw128(sbase + HC_OFF_XO), dring = make_sdesc_k_sw128(sbase + HC_OFF_RING);
+      auto wait = [&](uint64_t* bar, uint32_t parity, int where) -> bool {
+        const bool got = __all_sync(0xffffffffu, mbar_wait(bar, parity, p.err, where));
         tc_fence_after();
+        return got;
+      };
+      bool ok = true;
+      uint32_t slot = 0, slot_ph = 0;
+      auto next_slot = [&]() { if (++slot == HC_RING) { slot = 0; slot_ph ^= 1u; } };
+      // one operand slab (64 of the contraction index): D[128 x N] (+)= X / O K-block . slab^T, then up to two commits
+      auto slab_ss = [&](uint32_t d, int kb, uint32_t idesc, bool first, uint64_t* done, uint64_t* done2) -> bool {
+        if (!wait(&full[slot], slot_ph, 22)) return false;
+        if (elect_one()) {
+          const uint64_t da = dxo + (uint64_t)((uint32_t)kb * HC_SUB >> 4), db = dring + (uint64_t)(slot * HC_SLAB >> 4);
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          mma_bf16_ss(tmem_base + d_col, make_sdesc_k_sw128(a_kblock + k * 32), make_sdesc_k_sw128(sbase + HC_OFF_RING + s * HC_SLAB + k * 32),
-                      idesc, (first && k == 0) ? 0u : 1u);
-        mma_commit(&empty[s]);
-        ++sl;
+          for (int k = 0; k < 4; ++k) mma_bf16_ss(d, da + ((k * 32) >> 4), db + ((k * 32) >> 4), idesc, (first && k == 0) ? 0u : 1u);
+          mma_commit(&empty[slot]);
+          if (done != nullptr) mma_commit(done);
+          if (done2 != nullptr) mma_commit(done2);
+        }
+        __syncwarp();
+        next_slot();
+        return true;
+      };
+      // the same with U in TMEM: 64 hidden columns are two threads' 16 columns each, 32 apart
+      auto slab_u = [&](int kb, bool first, uint64_t* done) -> bool {
+        if (!wait(&full[slot], slot_ph, 22)) return false;
+        if (elect_one()) {
+          const uint64_t db = dring + (uint64_t)(slot * HC_SLAB >> 4);
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            mma_bf16_ts(B, A + (uint32_t)((kb * 2 + (k >> 1)) * 32 + (k & 1) * 8), db + ((k * 32) >> 4), idesc_256, (first && k == 0) ? 0u : 1u);
+          mma_commit(&empty[slot]);
+          if (done != nullptr) mma_commit(done);
+        }
+        __syncwarp();
+        next_slot();
         return true;
       };
       for (int g = 0; g < n && ok; ++g) {
-        const uint32_t R0 = (uint32_t)(g & 1) * 256u, R1 = 256u - R0;
-        if (!mbar_wait(x_full, (uint32_t)g & 1u, p.err, 23)) break;
-        // 1. scores.  R0 was [gate | up] of the previous tile (u_ready waited); R1 was its S'.
-        for (int kb = 0; kb < 4 && ok; ++kb) ok = slab_mma(R0, xo + kb * HC_SUB, idesc_sc, kb == 0);
+        if (!wait(x_full, (uint32_t)g & 1u, 23)) break;
+        // 1. scores.  A held U of the previous tile (handed to the pipe, which keeps the order); B its S'
+        for (int kb = 0; kb < 4 && ok; ++kb) ok = slab_ss(A, kb, idesc_sc, kb == 0, kb == 3 ? &s_full[0] : nullptr, nullptr);
         if (!ok) break;
-        mma_commit(&s_full[0]);
-        if (g > 0 && !mbar_wait(sp_read, (uint32_t)(g - 1) & 1u, p.err, 26)) break;
-        tc_fence_after();
-        if (n_sg == 2) {
-          for (int kb = 0; kb < 4 && ok; ++kb) ok = slab_mma(R1, xo + kb * HC_SUB, idesc_256, kb == 0);
-          if (!ok) break;
-          mma_commit(&s_full[1]);
-        }
-        if (!mbar_wait(v_full, (uint32_t)g & 1u, p.err, 28)) break;
-        // 2. value mix, head by head: O[:, head] = P_head . V_head  (contraction over the 64 links of the head).  The O
-        //    columns of group c lie inside score columns that groups <= c / 2 held, all consumed once P_c exists and the
-        //    groups are taken in order.
-        for (int c = 0; c < NG && ok; ++c) {
-          const int rg = c & 1;
-          if (!mbar_wait(&p_ready[rg], p_uses[rg] & 1u, p.err, 24)) { ok = false; break; }
-          ++p_uses[rg];
-          tc_fence_after();
-          for (int hl = 0; hl < HPG; ++hl) {
-            const int h = c * HPG + hl;
-            const uint32_t a0 = xo + (uint32_t)(rg * 2) * HC_SUB + (uint32_t)(hl * ELL / 64) * HC_SUB + (uint32_t)(hl * ELL % 64) * 2;
+        if (g > 0 && !wait(sp_read, (uint32_t)(g - 1) & 1u, 26)) break;
+        if (n_sg == 2)
+          for (int kb = 0; kb < 4 && ok; ++kb) ok = slab_ss(B, kb, idesc_256, kb == 0, kb == 3 ? &s_full[1] : nullptr, nullptr);
+        if (!ok) break;
+        // 2. value mix, head by head: O[:, head] = P_head . V_head (contraction over the links of the head), over the scores of
+        //    B, once they are all consumed
+        if (!wait(&full[slot], slot_ph, 28) || !wait(p_ready, (uint32_t)g & 1u, 24)) break;
+        if (elect_one()) {
+          const uint64_t dv = make_sdesc_k_sw(sbase + HC_OFF_RING + slot * HC_SLAB, V_ROW);
+          for (int h = 0; h < p.H; ++h) {
+            const int row = h * ELL, c = row >> 7;          // stacked row, group of 128: P of 64 rows is 32 columns
+            const uint32_t pa = A + (uint32_t)((c & 1) * 128 + ((row >> 6) & 1) * 64 + (c >> 1) * 32 + ((row & 63) >> 1));
+#pragma unroll
             for (int kk = 0; kk < ELL / 16; ++kk)
-              mma_bf16_ss(tmem_base + R0 + (uint32_t)(h * d_h), make_sdesc_k_sw128(a0 + kk * 32),
-                          make_sdesc_k_sw(pu + (uint32_t)(h * d_h) * V_ROW + kk * 32, V_ROW), idesc_v, kk != 0);
+              mma_bf16_ts(B + (uint32_t)(h * d_h), pa + kk * 8, dv + ((uint32_t)(h * d_h) * V_ROW >> 4) + ((kk * 32) >> 4), idesc_v, kk != 0);
           }
-          mma_commit(&pv_done[rg]);
-          if (c == NG - 1) mma_commit(o_full);
+          mma_commit(&empty[slot]);
+          mma_commit(o_full);
         }
-        if (!ok) break;
-        // 3. GatedMLP on O (bf16 in the X / P / O buffer), the hidden columns in two halves
-        if (!mbar_wait(o_ready, (uint32_t)g & 1u, p.err, 25)) break;
-        tc_fence_after();
+        __syncwarp();
+        next_slot();
+        // 3. GatedMLP on O (bf16 in the X / O buffer), the hidden columns in two halves
+        if (!wait(o_ready, (uint32_t)g & 1u, 25)) break;
         for (int hf = 0; hf < 2 && ok; ++hf) {
-          if (hf == 1) {
-            // S' = U(0) . W_o[0..127, :] first: it frees the U buffer for the second half
-            for (int kb = 0; kb < 2 && ok; ++kb) ok = slab_mma(R0, pu + kb * HC_SUB, idesc_256, kb == 0);
-          }
-          for (int kb = 0; kb < 4 && ok; ++kb) ok = slab_mma(R1, xo + kb * HC_SUB, idesc_256, kb == 0);
-          if (!ok) break;
-          mma_commit(gu_full);
-          if (hf == 1) mma_commit(x_free);
-          if (!mbar_wait(u_ready, (uint32_t)(2 * g + hf) & 1u, p.err, 27)) { ok = false; break; }
-          tc_fence_after();
+          // S' = U(0) . W_o[0..127, :] before the second half's [gate | up] is formed over it
+          if (hf == 1)
+            for (int kb = 0; kb < 2 && ok; ++kb) ok = slab_u(kb, kb == 0, nullptr);
+          for (int kb = 0; kb < 4 && ok; ++kb)
+            ok = slab_ss(A, kb, idesc_256, kb == 0, kb == 3 ? gu_full : nullptr, kb == 3 && hf == 1 ? x_free : nullptr);
+          if (ok) ok = wait(u_ready, (uint32_t)hf, 27);            // two phases a tile
         }
-        if (!ok) break;
-        for (int kb = 0; kb < 2 && ok; ++kb) ok = slab_mma(R0, pu + kb * HC_SUB, idesc_256, false);
-        if (!ok) break;
-        mma_commit(sp_full);
+        for (int kb = 0; kb < 2 && ok; ++kb) ok = slab_u(kb, false, kb == 1 ? sp_full : nullptr);
       }
     }
   } else if (n > 0) {
@@ -310,92 +318,82 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     const int rw = warp - 2;                                 // 0..15
     const int q4 = warp & 3;                                 // TMEM lane quarter of this warp
     const int part = rw >> 2;                                // which quarter of the columns of every step
-    const int rg = part >> 1, hh = part & 1;                 // softmax: row-warp group, half (64 columns) of a group of 128 stacked rows
     const uint32_t r = (uint32_t)(q4 * 32 + lane);           // token row of the tile == TMEM lane
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q4 * 32) << 16);
-    float2* exch = reinterpret_cast<float2*>(smem + HC_OFF_EXCH);         // [2][PARTS][128]
+    constexpr uint32_t RA = 0, RB = 256;                     // the two regions
+    float2* exch = reinterpret_cast<float2*>(smem + HC_OFF_EXCH);         // [PARTS][128]
     float* inv_sum = reinterpret_cast<float*>(smem + HC_OFF_INV);         // [8][128]
-    uint8_t* p_head = smem + HC_OFF_XO + (uint32_t)(rg * 2 + hh) * HC_SUB;   // P of this thread's 64 columns: one K-block
-    uint8_t* pu_part = smem + HC_OFF_PU + (part >> 1) * HC_SUB;           // U: K-block part / 2, chunks (part % 2) * 4 ..
-    const uint32_t pu_chunk0 = (uint32_t)(part & 1) * 4;
-    uint32_t row_uses = 0, my_p = 0;
+    uint8_t* patch = smem + HC_OFF_PATCH + rw * HC_PATCH;
+    uint32_t row_uses = 0;
     bool ok = true;
     HcTileUser tu;
     for (int g = 0; g < n && ok; ++g) {
       const int t = t_begin + g;
       const int b = tu.of(tile_start, p.B, t);
       const int row0 = off[b] + (t - tu.lo) * HC_TILE;
-      const uint32_t R0 = (uint32_t)(g & 1) * 256u, R1 = 256u - R0;
-      // ---- this row-warp group's groups: softmax over the links of this thread's head (or two heads of 32), P_c -> smem
-      for (int c = rg; c < NG && ok; c += 2, ++my_p) {
-        const int sg = c >> 1;
+      // ---- softmax over the links of this thread's heads: 64 stacked rows of either region, P over its own scores in A
+      for (int sg = 0; sg < n_sg && ok; ++sg) {
         if (!mbar_wait(&s_full[sg], (uint32_t)g & 1u, p.err, 32)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t col = lane_addr + (sg ? R1 : R0) + (uint32_t)(c & 1) * 128u + (uint32_t)hh * 64u;
-        float v[32];
-        float mx[64 / ELL] = {}, sum[64 / ELL] = {};       // by head; with ELL = 32 the two halves are heads of their own
-        if (!p.silu) {
-          tmem_ld_32x32(col, v);
-          tmem_wait_ld();
-          mx[0] = v[0];
+        const int first = sg * 256 + part * 64;              // first stacked row
+        if (first >= p.HL) break;
+        float v[64];
+        tmem_ld_32x32(lane_addr + (sg ? RB : RA) + part * 64, *reinterpret_cast<float(*)[32]>(&v[0]));
+        tmem_ld_32x32(lane_addr + (sg ? RB : RA) + part * 64 + 32, *reinterpret_cast<float(*)[32]>(&v[32]));
+        tmem_wait_ld();
 #pragma unroll
-          for (int j = 1; j < 32; ++j) mx[0] = fmaxf(mx[0], v[j]);
-          tmem_ld_32x32(col + 32, v);
-          tmem_wait_ld();
-          float& m1 = mx[64 / ELL - 1];
-          if (ELL == 32) m1 = v[0];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) m1 = fmaxf(m1, v[j]);
-        }
-        // the P buffers lie over the token tile: every score contraction of the tile must have read it, and the value mix
-        // that read this buffer last must have run
-        if (!mbar_wait(&s_full[n_sg - 1], (uint32_t)g & 1u, p.err, 35)) { ok = false; break; }
-        if (my_p > 0 && !mbar_wait(&pv_done[rg], (my_p - 1) & 1u, p.err, 36)) { ok = false; break; }
-#pragma unroll
-        for (int hv = 0; hv < 2; ++hv) {
-          tmem_ld_32x32(col + hv * 32, v);
-          tmem_wait_ld();
+        for (int h = 0; h < 64 / ELL; ++h) {                 // with ELL = 32 the two halves are heads of their own
+          float2* w = reinterpret_cast<float2*>(&v[h * ELL]);
+          float inv = 1.0f;
           if (p.silu) {
             // SiLU(s) / ell: every history query attends to the ell links of the head (Algorithm 1)
 #pragma unroll
-            for (int j = 0; j < 32; ++j) { const float hx = 0.5f * v[j]; v[j] = fmaf(hx, hc_tanh(hx), hx) * (1.0f / ELL); }
-          } else {
-            float s0 = 0.f, s1 = 0.f;
-            const float m = mx[hv * (64 / ELL - 1)];
-#pragma unroll
-            for (int j = 0; j < 32; j += 2) {
-              v[j] = hc_ex2(v[j] - m);
-              v[j + 1] = hc_ex2(v[j + 1] - m);
-              s0 += v[j];
-              s1 += v[j + 1];
+            for (int j = 0; j < ELL / 2; ++j) {
+              const float2 hx = __fmul2_rn(w[j], make_float2(0.5f, 0.5f));
+              w[j] = __fmul2_rn(__ffma2_rn(hx, make_float2(hc_tanh(hx.x), hc_tanh(hx.y)), hx), make_float2(1.0f / ELL, 1.0f / ELL));
             }
-            sum[hv * (64 / ELL - 1)] += s0 + s1;
-          }
+          } else {
+            float m0 = w[0].x, m1 = w[0].y, m2 = w[1].x, m3 = w[1].y;
 #pragma unroll
-          for (int c8 = 0; c8 < 4; ++c8) {
-            uint4 o;
-            o.x = hc_pack(v[c8 * 8 + 0], v[c8 * 8 + 1]); o.y = hc_pack(v[c8 * 8 + 2], v[c8 * 8 + 3]);
-            o.z = hc_pack(v[c8 * 8 + 4], v[c8 * 8 + 5]); o.w = hc_pack(v[c8 * 8 + 6], v[c8 * 8 + 7]);
-            *reinterpret_cast<uint4*>(p_head + hc_chunk(r, (uint32_t)(hv * 4 + c8))) = o;
+            for (int j = 2; j < ELL / 2; j += 2) {
+              m0 = fmaxf(m0, w[j].x); m1 = fmaxf(m1, w[j].y); m2 = fmaxf(m2, w[j + 1].x); m3 = fmaxf(m3, w[j + 1].y);
+            }
+            const float mx = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
+            float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+#pragma unroll
+            for (int j = 0; j < ELL / 2; j += 2) {
+              const float2 a0 = __fadd2_rn(w[j], make_float2(-mx, -mx)), a1 = __fadd2_rn(w[j + 1], make_float2(-mx, -mx));
+              w[j] = make_float2(hc_ex2(a0.x), hc_ex2(a0.y));
+              w[j + 1] = make_float2(hc_ex2(a1.x), hc_ex2(a1.y));
+              s0 = __fadd2_rn(s0, w[j]);
+              s1 = __fadd2_rn(s1, w[j + 1]);
+            }
+            s0 = __fadd2_rn(s0, s1);
+            inv = __fdividef(1.0f, s0.x + s0.y);
           }
+          // the exponentials go to the value mix unnormalised; O is divided by the row sum of its head afterwards
+          inv_sum[(first / ELL + h) * 128 + (int)r] = inv;
         }
-        // the exponentials go to the value mix unnormalised; O is divided by the row sum of its head afterwards
 #pragma unroll
-        for (int i = 0; i < 64 / ELL; ++i)
-          inv_sum[(c * HPG + hh * (64 / ELL) + i) * 128 + (int)r] = p.silu ? 1.0f : __fdividef(1.0f, sum[i]);
-        tc_fence_before();
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&p_ready[rg]);
+        for (int c = 0; c < 64; c += 32) {
+          float pk[16];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) pk[j] = __uint_as_float(hc_pack(v[c + 2 * j], v[c + 2 * j + 1]));
+          tmem_st_32x16(lane_addr + RA + (uint32_t)(part * 64 + sg * 32 + (c >> 1)), pk);
+        }
       }
       if (!ok) break;
+      tmem_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(p_ready);
       // ---- O: this thread's 64 columns / row sum of their heads -> bf16 -> K-block `part` of the X / P / O buffer
       if (!mbar_wait(o_full, (uint32_t)g & 1u, p.err, 33)) { ok = false; break; }
       tc_fence_after();
 #pragma unroll
       for (int c = 0; c < 64; c += 32) {
         float a[32];
-        tmem_ld_32x32(lane_addr + R0 + part * 64 + c, a);
+        tmem_ld_32x32(lane_addr + RB + part * 64 + c, a);
         const float sc = inv_sum[((part * 64 + c) / d_h) * 128 + (int)r];
         tmem_wait_ld();
 #pragma unroll
@@ -410,28 +408,23 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(o_ready);
-      // ---- per half of the hidden columns: U = SiLU(gate) * up for this thread's 32 columns -> smem
+      // ---- per half of the hidden columns: U = SiLU(gate) * up for this thread's 32 columns, over its own gates
       for (int hf = 0; hf < 2 && ok; ++hf) {
-        if (!mbar_wait(gu_full, (uint32_t)(2 * g + hf) & 1u, p.err, 34)) { ok = false; break; }
+        if (!mbar_wait(gu_full, (uint32_t)hf, p.err, 34)) { ok = false; break; }          // two phases a tile
         tc_fence_after();
-        float gt[32], up[32];
-        tmem_ld_32x32(lane_addr + R1 + part * 32, gt);
-        tmem_ld_32x32(lane_addr + R1 + 128 + part * 32, up);
+        float gt[32], up[32], pk[16];
+        tmem_ld_32x32(lane_addr + RA + part * 32, gt);
+        tmem_ld_32x32(lane_addr + RA + 128 + part * 32, up);
         tmem_wait_ld();
 #pragma unroll
-        for (int c8 = 0; c8 < 4; ++c8) {
-          float y[8];
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float hx = 0.5f * gt[c8 * 8 + j];
-            y[j] = fmaf(hx, hc_tanh(hx), hx) * up[c8 * 8 + j];
-          }
-          uint4 o;
-          o.x = hc_pack(y[0], y[1]); o.y = hc_pack(y[2], y[3]); o.z = hc_pack(y[4], y[5]); o.w = hc_pack(y[6], y[7]);
-          *reinterpret_cast<uint4*>(pu_part + hc_chunk(r, pu_chunk0 + (uint32_t)c8)) = o;
+        for (int j = 0; j < 16; ++j) {
+          const float2 hx = __fmul2_rn(make_float2(gt[2 * j], gt[2 * j + 1]), make_float2(0.5f, 0.5f));
+          const float2 y = __fmul2_rn(__ffma2_rn(hx, make_float2(hc_tanh(hx.x), hc_tanh(hx.y)), hx), make_float2(up[2 * j], up[2 * j + 1]));
+          pk[j] = __uint_as_float(hc_pack(y.x, y.y));
         }
+        tmem_st_32x16(lane_addr + RA + part * 32, pk);
+        tmem_wait_st();
         tc_fence_before();
-        fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(u_ready);
       }
@@ -439,74 +432,69 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
       // ---- S': this thread's 64 columns of its row -> (LayerNorm) -> bf16 -> global, straight from registers
       if (!mbar_wait(sp_full, (uint32_t)g & 1u, p.err, 37)) { ok = false; break; }
       tc_fence_after();
-      float a0[32], a1[32];
-      tmem_ld_32x32(lane_addr + R0 + part * 64, a0);
-      tmem_ld_32x32(lane_addr + R0 + part * 64 + 32, a1);
+      float v[64];
+      tmem_ld_32x32(lane_addr + RB + part * 64, *reinterpret_cast<float(*)[32]>(&v[0]));
+      tmem_ld_32x32(lane_addr + RB + part * 64 + 32, *reinterpret_cast<float(*)[32]>(&v[32]));
       tmem_wait_ld();
-      // S' is in registers: the columns may take the next tile's value mix while this tile is normalised and stored
+      // S' is in registers: the columns may take the next tile's scores while this tile is normalised and stored
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(sp_read);
-      float mu = 0.f, rstd = 1.f;
       if (p.out_ln) {
-        // each quarter sends the mean of its 64 columns and their squared deviations from it; the four combine exactly
-        float s = 0.f;
+        // each quarter sends the mean of its 64 columns and their squared deviations from it; the four combine exactly.
+        // (The slots are rewritten a tile later, when every warp has moved on.)
+        float2* w = reinterpret_cast<float2*>(v);
+        float2 s0 = w[0], s1 = w[1];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) s += a0[j] + a1[j];
-        const float m_q = s * (1.0f / 64);
-        float m2 = 0.f;
+        for (int j = 2; j < 32; j += 2) { s0 = __fadd2_rn(s0, w[j]); s1 = __fadd2_rn(s1, w[j + 1]); }
+        s0 = __fadd2_rn(s0, s1);
+        const float m_q = (s0.x + s0.y) * (1.0f / 64);
+        float2 q0 = make_float2(0.f, 0.f), q1 = q0;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const float d0 = a0[j] - m_q, d1 = a1[j] - m_q;
-          m2 = fmaf(d0, d0, m2);
-          m2 = fmaf(d1, d1, m2);
+        for (int j = 0; j < 32; j += 2) {
+          const float2 d0 = __fadd2_rn(w[j], make_float2(-m_q, -m_q)), d1 = __fadd2_rn(w[j + 1], make_float2(-m_q, -m_q));
+          q0 = __ffma2_rn(d0, d0, q0);
+          q1 = __ffma2_rn(d1, d1, q1);
         }
-        float2* ex = exch + (row_uses & 1u) * (HC_PARTS * 128);
-        ex[part * 128 + r] = make_float2(m_q, m2);
+        q0 = __fadd2_rn(q0, q1);
+        exch[part * 128 + r] = make_float2(m_q, q0.x + q0.y);
         if (!hc_group_sync(&row_bar[q4], row_uses, lane, p.err, 38)) { ok = false; break; }
         float2 e[HC_PARTS];
 #pragma unroll
-        for (int i = 0; i < HC_PARTS; ++i) e[i] = ex[i * 128 + r];
-        mu = 0.25f * (e[0].x + e[1].x + e[2].x + e[3].x);
+        for (int i = 0; i < HC_PARTS; ++i) e[i] = exch[i * 128 + r];
+        const float mu = 0.25f * (e[0].x + e[1].x + e[2].x + e[3].x);
         float tot = 0.f;
 #pragma unroll
         for (int i = 0; i < HC_PARTS; ++i) { const float dm = e[i].x - mu; tot += e[i].y + 64.0f * dm * dm; }
-        rstd = rsqrtf(tot * (1.0f / HC_D) + p.ln_eps);
+        const float rstd = rsqrtf(tot * (1.0f / HC_D) + p.ln_eps);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) w[j] = __fmul2_rn(__fadd2_rn(w[j], make_float2(-mu, -mu)), make_float2(rstd, rstd));
       }
-      // Out through a 2 KB patch of the V / U buffer that belongs to this warp alone (S' has consumed U): the warp stages
-      // 32 columns of its 32 rows (row R at R * 64 bytes, 16-byte chunk c at position c ^ ((R >> 1) & 3): conflict-free
-      // both ways), then writes them with four lanes per row, 64 contiguous bytes each.  Only the warp itself has to
-      // rendezvous.
-      {
-        uint8_t* patch = smem + HC_OFF_PU + (part >> 1) * HC_SUB + q4 * 4096 + (part & 1) * 2048;
-        const int row_end = off[b + 1];
-        const uint32_t rr = (uint32_t)lane >> 2, rc = (uint32_t)lane & 3u;
+      // Out through the warp's own patch, eight rows of its 64 columns at a time (128 bytes a row, 16-byte chunk c at position
+      // c ^ row: no bank conflicts), so that a store writes whole 128-byte lines.  (32-byte stores straight from the thread's
+      // row, one line per lane, were measured: as fast here, 2 us slower in the d = 128 kernel.)
+      const uint32_t x7 = (uint32_t)(lane & 7);
+      const int rsub = lane >> 3, row_end = off[b + 1];
+      __nv_bfloat16* dst = p.out + part * 64 + (lane & 7) * 8;
+      uint4 o[8];
 #pragma unroll
-        for (int hcol = 0; hcol < 2; ++hcol) {
-          const float* a = hcol ? a1 : a0;
+      for (int c = 0; c < 8; ++c)
+        o[c] = make_uint4(hc_pack(v[c * 8], v[c * 8 + 1]), hc_pack(v[c * 8 + 2], v[c * 8 + 3]), hc_pack(v[c * 8 + 4], v[c * 8 + 5]),
+                          hc_pack(v[c * 8 + 6], v[c * 8 + 7]));
 #pragma unroll
-          for (int c8 = 0; c8 < 4; ++c8) {
-            uint4 o;
-            o.x = hc_pack((a[c8 * 8 + 0] - mu) * rstd, (a[c8 * 8 + 1] - mu) * rstd);
-            o.y = hc_pack((a[c8 * 8 + 2] - mu) * rstd, (a[c8 * 8 + 3] - mu) * rstd);
-            o.z = hc_pack((a[c8 * 8 + 4] - mu) * rstd, (a[c8 * 8 + 5] - mu) * rstd);
-            o.w = hc_pack((a[c8 * 8 + 6] - mu) * rstd, (a[c8 * 8 + 7] - mu) * rstd);
-            *reinterpret_cast<uint4*>(patch + lane * 64 + (((uint32_t)c8 ^ (((uint32_t)lane >> 1) & 3u)) << 4)) = o;
-          }
-          __syncwarp();
+      for (int m = 0; m < 4; ++m) {
+        if (rsub == m) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const uint32_t R = (uint32_t)i * 8 + rr;
-            const uint4 o = *reinterpret_cast<const uint4*>(patch + R * 64 + ((rc ^ ((R >> 1) & 3u)) << 4));
-            const int grow = row0 + q4 * 32 + (int)R;
-            if (grow < row_end)
-              *reinterpret_cast<uint4*>(p.out + (int64_t)grow * HC_D + part * 64 + hcol * 32 + rc * 8) = o;
-          }
-          __syncwarp();
+          for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(patch + hc_chunk(x7, (uint32_t)c)) = o[c];
         }
+        __syncwarp();
+        const uint4 o0 = *reinterpret_cast<const uint4*>(patch + hc_chunk((uint32_t)rsub, x7));
+        const uint4 o1 = *reinterpret_cast<const uint4*>(patch + hc_chunk((uint32_t)rsub + 4, x7));
+        __syncwarp();
+        const int row = row0 + q4 * 32 + m * 8 + rsub;
+        if (row < row_end) *reinterpret_cast<uint4*>(dst + (int64_t)row * HC_D) = o0;
+        if (row + 4 < row_end) *reinterpret_cast<uint4*>(dst + (int64_t)(row + 4) * HC_D) = o1;
       }
-      // the V / U buffer may take the next tile's link values
-      if (lane == 0) mbar_arrive(pu_free);
     }
   }
 
@@ -537,7 +525,7 @@ static lime_status launch_hist_update_d256_t(const HistUpdate256Args& a, cudaStr
     return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
   HistUpdate256Params p;
   p.out = (__nv_bfloat16*)a.hist_out; p.off = a.off; p.tile_start = a.tile_start; p.B = a.B; p.H = a.H; p.HL = HL;
-  p.NG = HL / 128; p.shared = a.shared; p.silu = a.silu; p.out_ln = a.out_ln; p.ln_eps = a.ln_eps; p.err = a.err;
+  p.shared = a.shared; p.silu = a.silu; p.out_ln = a.out_ln; p.ln_eps = a.ln_eps; p.err = a.err;
   int grid = a.n_tile_upper < kSMs ? a.n_tile_upper : kSMs;
   if (grid < 1) return LIME_OK;
   static bool smem_set[kMaxDeviceOrdinals] = {};
