@@ -289,7 +289,9 @@ static lime_status launch_score_gather_t(const ScoreArgs& a, int* err, cudaStrea
   p.n_tiles = p.tiles_per_user * a.B;
   p.stages = S; p.err = err;
   const int grid = p.n_tiles < kSMs ? p.n_tiles : kSMs;
-  LIME_CUDA(cudaFuncSetAttribute(k_score_gather_tc<ELL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  static bool smem_set[kMaxDeviceOrdinals] = {};
+  const lime_status es = ensure_dynamic_smem((const void*)k_score_gather_tc<ELL>, 227 * 1024, smem_set);      // `smem` differs by d
+  if (es != LIME_OK) return es;
   ProfScope _p("k_score_gather_tc", st);
   launch_pdl(k_score_gather_tc<ELL>, dim3(grid), dim3(SG_THREADS), smem, st, tmLS, tmT, tmW, p);
   LIME_LAUNCH_CHECK("k_score_gather_tc");

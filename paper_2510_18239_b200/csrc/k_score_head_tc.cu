@@ -84,16 +84,20 @@ k_score_head_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__
     fence_barrier_init();
     prefetch_tmap(&tmT); prefetch_tmap(&tmW); prefetch_tmap(&tmLSW); prefetch_tmap(&tmW1b);
   }
-  for (int i = threadIdx.x; i < n1; i += SH_THREADS) {
-    consts[i] = p.b1 ? p.b1[i] : 0.f;
-    consts[256 + i] = p.w2[i];
-  }
-  if (threadIdx.x == 0) consts[512] = p.b2 ? p.b2[0] : 0.f;
   if (warp == 1) { tmem_alloc(tmem_slot, tmem_cols); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // set-up done: the next kernel's CTAs may become resident; nothing an earlier kernel wrote is read before the wait
+  pdl_launch_dependents();
+  pdl_wait();
+  for (int i = threadIdx.x; i < n1; i += SH_THREADS) {
+    consts[i] = p.b1 ? p.b1[i] : 0.f;
+    consts[256 + i] = p.w2[i];
+  }
+  if (threadIdx.x == 0) consts[512] = p.b2 ? p.b2[0] : 0.f;
+  __syncthreads();
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -304,9 +308,11 @@ static lime_status launch_score_head_tc_t(const ScoreArgs& a, const ScoreHeadArg
   p.n_tiles = p.tiles_per_user * a.B;
   p.stages = S; p.lsw_bufs = lb; p.err = err;
   const int grid = p.n_tiles < kSMs ? p.n_tiles : kSMs;
-  LIME_CUDA(cudaFuncSetAttribute(k_score_head_tc<ELL, GATHER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  static bool smem_set[kMaxDeviceOrdinals] = {};
+  const lime_status es = ensure_dynamic_smem((const void*)k_score_head_tc<ELL, GATHER>, 227 * 1024, smem_set);      // `smem` differs by d
+  if (es != LIME_OK) return es;
   ProfScope _p("k_score_head_tc", st);
-  k_score_head_tc<ELL, GATHER><<<grid, SH_THREADS, smem, st>>>(tmT, tmW, tmLSW, tmW1b, p);
+  launch_pdl(k_score_head_tc<ELL, GATHER>, dim3(grid), dim3(SH_THREADS), smem, st, tmT, tmW, tmLSW, tmW1b, p);
   LIME_LAUNCH_CHECK("k_score_head_tc");
   return LIME_OK;
 }

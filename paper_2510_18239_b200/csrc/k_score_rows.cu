@@ -19,6 +19,7 @@
 namespace lime {
 
 constexpr int SR_WARPS = 4;
+constexpr int SR_AHEAD = 4;      // groups of slots a warp asks L2 for before it may read the link states
 // blocks an SM can hold: what a thread keeps of its rows (d / 16 words each of two), weights and accumulators sets the
 // registers it needs, and the rest goes into warps
 constexpr int sr_blocks(int d, int ell) { return d * ell >= 8192 ? (d == 256 && ell == 64 ? 2 : 3) : 4; }
@@ -75,6 +76,19 @@ k_score_rows(const ScoreRowsParams p) {
   const int g = lane >> 2, t = lane & 3;
   const int g_begin = (int)(((int64_t)blockIdx.x * p.n_groups) / gridDim.x);
   const int g_end = (int)(((int64_t)(blockIdx.x + 1) * p.n_groups) / gridDim.x);
+  // What the block waits for is the link states (and the list offsets): its first rows move into L2 meanwhile, two lanes per
+  // slot taking every other line of the row (memory is idle while the last link-side kernel runs on a few SMs, and all blocks of
+  // this kernel fit beside it: 100 lists of 20..1500 ids, the batch 142 -> 134 us.  The tcgen05 scorers do not gain: their CTAs
+  // take a whole SM, so those that wait for one of the busy SMs start late whatever the others have prefetched)
+  for (int grp = g_begin + warp; grp < min(g_end, g_begin + SR_AHEAD * SR_WARPS); grp += SR_WARPS) {
+    const int slot = grp * (16 * MT) + (lane & 15);
+    const int id = slot < p.total ? (p.ids != nullptr ? __ldcg(p.ids + slot) : slot) : -1;
+    if (id >= 0 && id < p.rows) {
+      const char* row = reinterpret_cast<const char*>(p.T + (int64_t)id * p.ldt);
+      for (int o = (lane >> 4) * 128; o < D * 2; o += 256) prefetch_l2(row + o);
+      if (lane < 16) prefetch_l2_row(p.W + (int64_t)id * p.ldw, ELL * 2);
+    }
+  }
   pdl_wait();
   int b = -1;
   for (int grp = g_begin + warp; grp < g_end; grp += SR_WARPS) {

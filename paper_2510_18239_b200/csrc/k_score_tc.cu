@@ -238,7 +238,9 @@ static lime_status launch_score_tc_t(const ScoreArgs& a, int* err, cudaStream_t 
   p.n_tiles = p.tiles_per_user * a.B;
   p.stages = S; p.err = err;
   int grid = p.n_tiles < kSMs ? p.n_tiles : kSMs;
-  LIME_CUDA(cudaFuncSetAttribute(k_score_tc<ELL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  static bool smem_set[kMaxDeviceOrdinals] = {};
+  const lime_status es = ensure_dynamic_smem((const void*)k_score_tc<ELL>, 227 * 1024, smem_set);      // `smem` differs by d
+  if (es != LIME_OK) return es;
   ProfScope _p("k_score_tc", st);
   launch_pdl(k_score_tc<ELL>, dim3(grid), dim3(SCT_THREADS), smem, st, tmT, tmLS, tmW, p);
   LIME_LAUNCH_CHECK("k_score_tc");

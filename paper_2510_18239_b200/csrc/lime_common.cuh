@@ -96,13 +96,22 @@ lime_status cuda_fail(cudaError_t e, const char* where);
 // kernel's CTAs may become resident while its predecessor still runs (as soon as every CTA of the predecessor has
 // executed pdl_launch_dependents() or exited), set up their barriers and tensor memory, and then block in pdl_wait()
 // until the predecessor has completed and its writes are visible.  Rules kept by every kernel launched this way:
-//  - nothing produced by an earlier kernel is read, and no global memory is written, before pdl_wait();
+//  - nothing produced by an earlier kernel is read, and no global memory is written, before pdl_wait().  The warp-level scorer
+//    (k_score_rows.cu) does ask L2 for candidate rows before it: prefetches hold no value, and ids read that early only choose
+//    what to prefetch, past L1, and are read again afterwards;
 //  - a kernel that allocates tensor memory calls pdl_launch_dependents() only after its allocation, so a dependent CTA
 //    that shares the SM can never hold the columns a CTA of the running kernel still waits for.
 // A kernel launched the ordinary way after such a kernel still waits for its completion, as always.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// the 128-byte line at `p` into L2
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+// a row of `bytes`
+__device__ __forceinline__ void prefetch_l2_row(const void* p, int bytes) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+  for (uintptr_t l = a & ~(uintptr_t)127; l < a + bytes; l += 128) prefetch_l2(reinterpret_cast<const void*>(l < a ? a : l));
+}
 #endif
 bool pdl_enabled();      // environment LIME_PDL=0 turns the attribute off (every launch then serialises fully)
 template <typename... KArgs, typename... Args>
