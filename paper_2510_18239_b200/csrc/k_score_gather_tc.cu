@@ -127,7 +127,7 @@ k_score_gather_tc(const __grid_constant__ CUtensorMap tmLS, const __grid_constan
 #pragma unroll
       for (int i = 0; i < 4; ++i) { id_now[i] = id_next[i]; id_next[i] = id_after[i]; }
       read_ids(t + 2, id_after);
-      if (!mbar_wait(&empty[s], ((uint32_t)(it / S) & 1u) ^ 1u, p.err, 101)) { ok = false; break; }
+      if (!mbar_wait_spin(&empty[s], ((uint32_t)(it / S) & 1u) ^ 1u, p.err, 101)) { ok = false; break; }
       const int b = t / p.tiles_per_user;
       uint8_t* st = smem + (size_t)s * stage_bytes;
       // every thread announces its own bytes before it issues its copies, so the phase cannot complete early
@@ -170,8 +170,8 @@ k_score_gather_tc(const __grid_constant__ CUtensorMap tmLS, const __grid_constan
         const uint32_t ph = (uint32_t)(it / S) & 1u;
         const int buf = it & 1;
         const uint32_t bph = (uint32_t)(it >> 1) & 1u;
-        if (!mbar_wait(&tmem_empty[buf], bph ^ 1u, p.err, 102)) break;
-        if (!mbar_wait(&full[s], ph, p.err, 103)) break;
+        if (!mbar_wait_spin(&tmem_empty[buf], bph ^ 1u, p.err, 102)) break;
+        if (!mbar_wait_spin(&full[s], ph, p.err, 103)) break;
         tc_fence_after();
         const uint32_t a0 = smem_u32(smem + (size_t)s * stage_bytes);
         const uint32_t b0 = a0 + t_bytes;
@@ -202,7 +202,7 @@ k_score_gather_tc(const __grid_constant__ CUtensorMap tmLS, const __grid_constan
       const int64_t grow = (int64_t)b * p.C + c0 + r;
       const int s = it % S;
       const int32_t my_id = valid ? __ldg(p.ids + grow) : 0;        // in L2 since the producers read it; used at the very end
-      if (!mbar_wait(&full[s], (uint32_t)(it / S) & 1u, p.err, 105)) break;
+      if (!mbar_wait_spin(&full[s], (uint32_t)(it / S) & 1u, p.err, 105)) break;
       uint4 w[ELL / 8];
       {
         const uint4* wp = reinterpret_cast<const uint4*>(smem + (size_t)s * stage_bytes + t_bytes + ls_bytes) + r * (ELL / 8);
@@ -211,7 +211,7 @@ k_score_gather_tc(const __grid_constant__ CUtensorMap tmLS, const __grid_constan
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[s]);       // this warp has taken its rows out of the stage
-      if (!mbar_wait(&tmem_full[buf], bph, p.err, 104)) break;
+      if (!mbar_wait_spin(&tmem_full[buf], bph, p.err, 104)) break;
       tc_fence_after();
       constexpr int CH = ELL >= 32 ? 32 : 16;
       float acc4[4] = {0.f, 0.f, 0.f, 0.f};

@@ -131,7 +131,7 @@ k_score_head_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__
         }
         if (b != prev_user) {
           const int lb = un % LB;
-          if (!all(mbar_wait(&lsw_empty[lb], ((uint32_t)(un / LB) & 1u) ^ 1u, p.err, 101))) { ok = false; break; }
+          if (!all(mbar_wait_spin(&lsw_empty[lb], ((uint32_t)(un / LB) & 1u) ^ 1u, p.err, 101))) { ok = false; break; }
           if (lane == 0) {
             mbar_arrive_expect_tx(&lsw_full[lb], (uint32_t)n1 * ELL * 2);
             for (int kb = 0; kb < WKB; ++kb)
@@ -141,7 +141,7 @@ k_score_head_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__
           prev_user = b;
         }
         const int s = it % S;
-        if (!all(mbar_wait(&empty[s], ((uint32_t)(it / S) & 1u) ^ 1u, p.err, 102))) { ok = false; break; }
+        if (!all(mbar_wait_spin(&empty[s], ((uint32_t)(it / S) & 1u) ^ 1u, p.err, 102))) { ok = false; break; }
         uint8_t* st = smem + (size_t)s * stage_bytes;
         if (lane == 0) mbar_arrive_expect_tx(&full[s], stage_bytes);
         if constexpr (GATHER) {
@@ -177,14 +177,14 @@ k_score_head_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__
         const int b = t / p.tiles_per_user;
         if (b != prev_user) {
           const int lb = un % LB;
-          if (!mbar_wait(&lsw_full[lb], (uint32_t)(un / LB) & 1u, p.err, 104)) break;
+          if (!mbar_wait_spin(&lsw_full[lb], (uint32_t)(un / LB) & 1u, p.err, 104)) break;
           lsw_addr = smem_u32(lsw_base + (size_t)lb * lsw_bytes);
           ++un;
           prev_user = b;
         }
         const int s = it % S, buf = it & 1;
-        if (!mbar_wait(&tmem_empty[buf], ((uint32_t)(it >> 1) & 1u) ^ 1u, p.err, 105)) break;
-        if (!mbar_wait(&full[s], (uint32_t)(it / S) & 1u, p.err, 106)) break;
+        if (!mbar_wait_spin(&tmem_empty[buf], ((uint32_t)(it >> 1) & 1u) ^ 1u, p.err, 105)) break;
+        if (!mbar_wait_spin(&full[s], (uint32_t)(it / S) & 1u, p.err, 106)) break;
         tc_fence_after();
         const uint32_t a0 = smem_u32(smem + (size_t)s * stage_bytes);
         const uint32_t d_tmem = tmem_base + (uint32_t)buf * acc_cols;
@@ -222,7 +222,7 @@ k_score_head_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__
       const int buf = it & 1;
       const int b = t / p.tiles_per_user;
       const int c0 = (t % p.tiles_per_user) * SH_TILE;
-      if (!mbar_wait(&tmem_full[buf], (uint32_t)(it >> 1) & 1u, p.err, 107)) break;
+      if (!mbar_wait_spin(&tmem_full[buf], (uint32_t)(it >> 1) & 1u, p.err, 107)) break;
       tc_fence_after();
       float acc4[4] = {0.f, 0.f, 0.f, 0.f};
       const uint32_t ta = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)buf * acc_cols;

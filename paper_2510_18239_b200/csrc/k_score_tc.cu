@@ -90,7 +90,7 @@ k_score_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUte
       for (int t = t_begin; t < t_end; ++t, ++it) {
         const int s = it % S;
         const uint32_t ph = (uint32_t)(it / S) & 1u;
-        if (!mbar_wait(&empty[s], ph ^ 1u, p.err, 1)) { ok = false; break; }
+        if (!mbar_wait_spin(&empty[s], ph ^ 1u, p.err, 1)) { ok = false; break; }
         const int b = t / p.tiles_per_user;
         const int row0 = b * p.C + (t % p.tiles_per_user) * SCT_TILE;
         bool load_ls = false;
@@ -124,8 +124,8 @@ k_score_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUte
         const uint32_t ph = (uint32_t)(it / S) & 1u;
         const int buf = it & 1;
         const uint32_t bph = (uint32_t)(it >> 1) & 1u;
-        if (!mbar_wait(&tmem_empty[buf], bph ^ 1u, p.err, 2)) break;
-        if (!mbar_wait(&full[s], ph, p.err, 3)) break;
+        if (!mbar_wait_spin(&tmem_empty[buf], bph ^ 1u, p.err, 2)) break;
+        if (!mbar_wait_spin(&full[s], ph, p.err, 3)) break;
         tc_fence_after();
         const uint32_t a0 = smem_u32(smem + (size_t)s * stage_bytes);
         const uint32_t b0 = a0 + t_bytes;
@@ -155,7 +155,7 @@ k_score_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUte
       const bool valid = c0 + r < p.C;
       const int64_t grow = (int64_t)b * p.C + c0 + r;
       const int s = it % S;
-      if (!mbar_wait(&full[s], (uint32_t)(it / S) & 1u, p.err, 5)) break;
+      if (!mbar_wait_spin(&full[s], (uint32_t)(it / S) & 1u, p.err, 5)) break;
       uint4 w[ELL / 8];
       {
         const uint4* wp = reinterpret_cast<const uint4*>(smem + (size_t)s * stage_bytes + t_bytes + ls_bytes) + r * (ELL / 8);
@@ -164,7 +164,7 @@ k_score_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUte
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[s]);       // this warp has taken its rows out of the stage
-      if (!mbar_wait(&tmem_full[buf], bph, p.err, 4)) break;
+      if (!mbar_wait_spin(&tmem_full[buf], bph, p.err, 4)) break;
       tc_fence_after();
       // dot of the weight row with the accumulator row, CH columns per TMEM load, four independent partial sums
       constexpr int CH = ELL >= 32 ? 32 : 16;

@@ -63,16 +63,33 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
 // in *err (if not already set) and returns false; callers then leave their loops, so the CTA always reaches its
 // final barrier, frees its TMEM and exits.
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s
-// (The clock is first read after 1024 polls: read on the way into a wait, it delays the end of a short one.  Letting the
-// hardware suspend the thread with a time hint was measured and wakes later than polling does.)
+// The clock is read on the way into the polling loop, which also keeps a warp that has just found its phase incomplete from
+// taking issue slots for a few hundred cycles.  (Letting the hardware suspend the thread with a time hint was measured and
+// wakes later.)
 __device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, int* err, int where, uint64_t limit_ns) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const uint64_t t0 = global_timer_ns();
+  uint32_t spins = 0;
+  while (!mbar_try_wait(bar, parity)) {
+    if ((++spins & 0x3ff) == 0) {
+      if (global_timer_ns() - t0 > limit_ns || *(volatile int*)err != 0) {
+        atomicCAS(err, 0, where);
+        return false;
+      }
+    }
+  }
+  return true;
+}
+// The same for kernels whose waits are short and whose warps are few (the scorers; the dense one streams at the memory rate:
+// 111 -> 105 us): polls at once, and first reads the clock after 1024 polls.
+__device__ __forceinline__ bool mbar_wait_spin(uint64_t* bar, uint32_t parity, int* err, int where) {
   uint64_t t0 = 0;
   uint32_t spins = 0;
   while (!mbar_try_wait(bar, parity)) {
     if ((++spins & 0x3ff) == 0) {
       const uint64_t now = global_timer_ns();
       if (t0 == 0) t0 = now;
-      if (now - t0 > limit_ns || *(volatile int*)err != 0) {
+      if (now - t0 > kWaitLimitNs || *(volatile int*)err != 0) {
         atomicCAS(err, 0, where);
         return false;
       }
