@@ -74,7 +74,7 @@ static void weight_free(int device, void* p) {
 }
 static inline int elem_size(int dtype) { return dtype == LIME_F32 ? 4 : 2; }
 
-// Tokens per work item of the link<-history attention: a power of two in [lo, 2048] giving about three work items per
+// Tokens per work item of the link<-history attention: a power of two in [lo, hi] giving about three work items per
 // SM (`row_blocks` items per chunk).  Every chunk of a multi-chunk history costs a set of fp32 partials and a pipeline
 // refill, so long histories take long chunks.
 static int pick_chunk(int64_t total_tokens, int row_blocks, int lo, int hi = 2048) {
@@ -140,8 +140,11 @@ static Workspace carve(const Ctx* c, void* base, int32_t B, int64_t total) {
   const bool tc_link = c->tc_mode != 0;
   // tensor-core path: at least 4 token tiles per work item, one item per 128-row block of H * ell (at d = 256 a set of
   // partials is 4 x larger and the batches served have many users, so chunks may be longer still)
-  w.chunk = c->tc_mode == 2 ? pick_chunk(total, (g.H * g.ell + 127) / 128, 512, 4096)
-                            : (tc_link ? pick_chunk(total, (g.H * g.ell + 127) / 128, 512) : pick_chunk(total, 1, 64));
+  // At least 2048 tokens once the users alone make 64 work items: splitting histories of some hundred tokens then evens out less
+  // than the merge of the partials costs (100 users of 250..1000 tokens, two layers: 105 -> 87 us with 32 links, 142 -> 113 us
+  // with 64).  With fewer users the split is what occupies the SMs (16 users of 375..1500 tokens: 57 us, 64 us unsplit).
+  const int row_blocks = (g.H * g.ell + 127) / 128, lo = (int64_t)B * row_blocks >= 64 ? 2048 : 512;
+  w.chunk = c->tc_mode == 2 ? pick_chunk(total, row_blocks, lo, 4096) : (tc_link ? pick_chunk(total, row_blocks, lo) : pick_chunk(total, 1, 64));
   w.n_chunk_upper = (int)((total + w.chunk - 1) / w.chunk + B);
   w.n_tile_upper = (int)((total + kHistTile - 1) / kHistTile + B);
   w.chunk_user = (int32_t*)take((size_t)w.n_chunk_upper * 4);
