@@ -15,6 +15,7 @@ namespace lime {
 
 constexpr int GM_THREADS = 64 + 256, GM_MAX_STAGES = 6;   // producer, MMA issuer, eight epilogue warps
 constexpr uint32_t GM_SUB = 128 * 128;    // [128 rows x 64 bf16]
+constexpr uint32_t GM_PATCH = 8 * 128;    // 8 rows x 64 bf16
 
 enum { GM_EPI_PREP = 0, GM_EPI_ROWS_T = 1 };
 
@@ -48,7 +49,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   constexpr uint32_t B_SUB = (uint32_t)NT * 128;
   constexpr uint32_t STAGE = GM_SUB + B_SUB;
   const int S = p.stages;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)S * STAGE);
+  uint8_t* patches = smem + (size_t)S * STAGE;              // PREP: 1 KB per epilogue warp, rows on their way out
+  uint64_t* bars = reinterpret_cast<uint64_t*>(patches + (EPI == GM_EPI_PREP ? 8 * GM_PATCH : 0));
   uint64_t* full = bars;
   uint64_t* empty = bars + GM_MAX_STAGES;
   uint64_t* acc_full = bars + 2 * GM_MAX_STAGES;          // [2] accumulator of a tile complete
@@ -96,26 +98,29 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         for (int j = 0; j < it && j < S; ++j) mbar_wait_quiet(&full[(it - 1 - j) % S], (uint32_t)((it - 1 - j) / S) & 1u);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc_bf16(128, NT);
-      const uint32_t sbase = smem_u32(smem);
-      bool ok = true;
-      int it = 0, n = 0;
-      for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++n) {
-        const int buf = n & 1;
-        if (!mbar_wait(&acc_empty[buf], ((uint32_t)(n >> 1) & 1u) ^ 1u, p.err, 74)) { ok = false; break; }
+    // the whole warp runs this code and one elected lane issues (warp-uniform descriptors, see k_link_attn_tmem_tc.cu)
+    constexpr uint32_t idesc = make_idesc_bf16(128, NT);
+    const uint64_t da0 = make_sdesc_k_sw128(smem_u32(smem)), db0 = make_sdesc_k_sw128(smem_u32(smem) + GM_SUB);
+    const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
+    bool ok = true;
+    int s = 0, n = 0;
+    uint32_t ph = 0;
+    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++n) {
+      const int buf = n & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(&acc_empty[buf], ((uint32_t)(n >> 1) & 1u) ^ 1u, p.err, 74))) break;
+      for (int kb = 0; kb < KB; ++kb) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&full[s], ph, p.err, 72))) { ok = false; break; }
         tc_fence_after();
-        for (int kb = 0; kb < KB && ok; ++kb, ++it) {
-          const int s = it % S;
-          if (!mbar_wait(&full[s], (uint32_t)(it / S) & 1u, p.err, 72)) { ok = false; break; }
-          tc_fence_after();
+        if (elect_one()) {
+          const uint64_t o = (uint64_t)((uint32_t)s * STAGE >> 4);
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            mma_bf16_ss(tmem_base + (uint32_t)buf * NT, make_sdesc_k_sw128(sbase + s * STAGE + k * 32),
-                        make_sdesc_k_sw128(sbase + s * STAGE + GM_SUB + k * 32), idesc, (kb | k) != 0);
+            mma_bf16_ss(tmem_u + (uint32_t)buf * NT, da0 + o + ((k * 32) >> 4), db0 + o + ((k * 32) >> 4), idesc, (kb | k) != 0);
           mma_commit(&empty[s]);
+          if (kb == KB - 1) mma_commit(&acc_full[buf]);
         }
-        if (ok) mma_commit(&acc_full[buf]);
+        __syncwarp();
+        if (++s == S) { s = 0; ph ^= 1u; }
       }
     }
   } else {
@@ -140,24 +145,42 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         const int HL = p.H * p.ell;
         if (n0 < qk_cols) {
           const int seg = n0 / (p.H * p.d), h = (n0 / p.d) % p.H, i0 = n0 % p.d;
-          __nv_bfloat16* dst = (seg == 0 ? p.Q2 : p.K2) + ((u * HL) + h * p.ell + l) * p.d + i0;
           float* cs = seg == 0 ? p.cQ : p.cK;
+          static_assert(EPI != GM_EPI_PREP || NT == 128, "64 columns a thread");
+          float v[64];
+          tmem_ld_32x32(lane_addr + cb, *reinterpret_cast<float(*)[32]>(&v[0]));
+          tmem_ld_32x32(lane_addr + cb + 32, *reinterpret_cast<float(*)[32]>(&v[32]));
+          tmem_wait_ld();
           float rs = 0.f;
+          if (cs != nullptr && half == 0) {
 #pragma unroll
-          for (int c = cb; c < ce; c += 16) {
-            float v[16];
-            tmem_ld_32x16(lane_addr + c, v);
-            tmem_wait_ld();
-            uint4 o0, o1;
-            o0.x = gm_pack(v[0], v[1]); o0.y = gm_pack(v[2], v[3]); o0.z = gm_pack(v[4], v[5]); o0.w = gm_pack(v[6], v[7]);
-            o1.x = gm_pack(v[8], v[9]); o1.y = gm_pack(v[10], v[11]); o1.z = gm_pack(v[12], v[13]); o1.w = gm_pack(v[14], v[15]);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) rs += __bfloat162float(__float2bfloat16_rn(v[j]));   // sum of what is stored
-            if (valid) {
-              *reinterpret_cast<uint4*>(dst + c) = o0;
-              *reinterpret_cast<uint4*>(dst + c + 8) = o1;
-            }
+            for (int j = 0; j < 64; ++j) rs += __bfloat162float(__float2bfloat16_rn(v[j]));   // sum of what is stored
           }
+          // Out through the warp's own patch, eight rows of its 64 columns at a time (16-byte chunk c at position c ^ row), so
+          // that a store writes whole 128-byte lines: a 16-byte piece per lane made the stores the bound of the kernel.
+          uint4 o[8];
+#pragma unroll
+          for (int c = 0; c < 8; ++c)
+            o[c] = make_uint4(gm_pack(v[c * 8], v[c * 8 + 1]), gm_pack(v[c * 8 + 2], v[c * 8 + 3]), gm_pack(v[c * 8 + 4], v[c * 8 + 5]),
+                              gm_pack(v[c * 8 + 6], v[c * 8 + 7]));
+          uint8_t* patch = patches + (warp - 2) * GM_PATCH;
+          const int out_row = valid ? (int)(u * HL + h * p.ell + l) : -1;
+          __nv_bfloat16* dst = (seg == 0 ? p.Q2 : p.K2) + i0 + cb + (lane & 7) * 8;
+          const int x7 = lane & 7, rsub = lane >> 3;
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            if (rsub == m) {
+#pragma unroll
+              for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(patch + x7 * 128 + ((c ^ x7) << 4)) = o[c];
+            }
+            __syncwarp();
+            const uint4 o0 = *reinterpret_cast<const uint4*>(patch + rsub * 128 + ((x7 ^ rsub) << 4));
+            const uint4 o1 = *reinterpret_cast<const uint4*>(patch + (rsub + 4) * 128 + ((x7 ^ (rsub + 4)) << 4));
+            const int r0 = __shfl_sync(0xffffffffu, out_row, m * 8 + rsub), r1 = __shfl_sync(0xffffffffu, out_row, m * 8 + rsub + 4);
+            if (r0 >= 0) *reinterpret_cast<uint4*>(dst + (int64_t)r0 * p.d) = o0;
+            if (r1 >= 0) *reinterpret_cast<uint4*>(dst + (int64_t)r1 * p.d) = o1;
+          }
+          __syncwarp();
           if (cs != nullptr && half == 0) {
             // the row sum spans the whole tile: this warp also reads the other half's columns for it
 #pragma unroll
@@ -238,8 +261,11 @@ static lime_status launch_gemm(const void* A, int64_t M, int K, const void* Bt, 
   if (m_tiles * n_tiles > 0x7fffffffLL) return LIME_UNSUPPORTED_SHAPE;
   p.M = M; p.kblocks = K / 64; p.m_tiles = (int)m_tiles; p.n_tiles = n_tiles;
   p.stages = GM_MAX_STAGES;
-  const size_t smem = p.stages * stage + 256 + 1024;
-  LIME_CUDA(cudaFuncSetAttribute(k_gemm_tc<EPI, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  constexpr size_t smem = GM_MAX_STAGES * stage + (EPI == GM_EPI_PREP ? 8 * GM_PATCH : 0) + 256 + 1024;
+  static_assert(smem <= 232448, "shared memory budget of one CTA");
+  static bool smem_set[kMaxDeviceOrdinals] = {};
+  const lime_status es = ensure_dynamic_smem((const void*)k_gemm_tc<EPI, NT>, (int)smem, smem_set);
+  if (es != LIME_OK) return es;
   ProfScope _p(name, st);
   const int64_t tiles = m_tiles * n_tiles;
   const unsigned grid = (unsigned)(tiles < kSMs ? tiles : kSMs);

@@ -346,13 +346,14 @@ static lime_status encode_user_tc(Ctx* c, const void* hist, bool hist_normalized
   const bool few_rows = c->tc_mode == 1 && link_side_d128_wanted(g.d, c->d_ff, g.H, g.ell, B);
   for (int j = 0; j < g.n_layers; ++j) {
     const bool last = j == g.n_layers - 1;
+    const bool raw = g.ln && j == 0 && !hist_normalized;      // rows that still need their LayerNorm want the operands' row sums
     LinkOperands ops;
     if (j == 0 && !link_ctx) {
       ops = LinkOperands{c->sh_Q2, c->sh_K2, c->sh_G2t, c->sh_U2t, c->sh_V2t, c->sh_cQ, c->sh_cK, 1};
     } else {
       if (j == 0 && (s = launch_ln_rows_bf16(link_ctx, BL, g.d, g.ln, c->ln_eps, w.That, st)) != LIME_OK) return s;
       if ((j == 0 || !few_rows) &&
-          (s = make_link_operands(c, j, w.That, BL, !last, w.Q2, w.K2, w.G2t, w.U2t, w.V2t, w.cQ, w.cK, st)) != LIME_OK)
+          (s = make_link_operands(c, j, w.That, BL, !last, w.Q2, w.K2, w.G2t, w.U2t, w.V2t, raw ? w.cQ : nullptr, raw ? w.cK : nullptr, st)) != LIME_OK)
         return s;
       ops = LinkOperands{w.Q2, w.K2, w.G2t, w.U2t, w.V2t, w.cQ, w.cK, 0};
     }
@@ -367,7 +368,7 @@ static lime_status encode_user_tc(Ctx* c, const void* hist, bool hist_normalized
     mlp.LP = w.LP; mlp.lp_accumulate = j > 0;                                   // L^P = sum_j T^j  (Eq. 8)
     mlp.That_next = last ? nullptr : w.That;
     mlp.link_states = (last && !c->w.cand_Wv && c->cand_heads == 1) ? link_states : nullptr;
-    s = tc_layer_core(c, j, j == 0 ? hist : w.S, off, B, total, ops, last ? nullptr : w.S, (g.ln && j == 0 && !hist_normalized) ? 1 : 0,
+    s = tc_layer_core(c, j, j == 0 ? hist : w.S, off, B, total, ops, last ? nullptr : w.S, raw ? 1 : 0,
                       (g.ln && !last) ? 1 : 0, mlp, nullptr, few_rows ? &side1 : nullptr, w, st);
     if (s != LIME_OK) return s;
   }
