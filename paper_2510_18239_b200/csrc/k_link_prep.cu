@@ -72,6 +72,8 @@ lime_status launch_fold_weights(const void* Wq, const void* Wk, const void* Wv, 
 // out[r, :] = bf16( LN(T[r, :]) )  (or bf16(T) when ln == 0); one warp per row
 __global__ void __launch_bounds__(256)
 k_ln_rows_bf16(const float* __restrict__ T, int64_t rows, int d, int ln, float eps, __nv_bfloat16* __restrict__ out) {
+  pdl_launch_dependents();     // simple kernel: the next one may set itself up beside it
+  pdl_wait();                  // nothing is read or written before the previous kernel is complete
   const int lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (r >= rows) return;
@@ -91,7 +93,7 @@ k_ln_rows_bf16(const float* __restrict__ T, int64_t rows, int d, int ln, float e
 lime_status launch_ln_rows_bf16(const float* T, int64_t rows, int d, int ln, float eps, void* out, cudaStream_t st) {
   if (rows == 0) return LIME_OK;
   ProfScope _p("k_ln_rows_bf16", st);
-  k_ln_rows_bf16<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(T, rows, d, ln, eps, (__nv_bfloat16*)out);
+  launch_pdl(k_ln_rows_bf16, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, T, rows, d, ln, eps, (__nv_bfloat16*)out);
   LIME_LAUNCH_CHECK("k_ln_rows_bf16");
   return LIME_OK;
 }

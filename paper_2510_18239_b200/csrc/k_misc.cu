@@ -183,6 +183,8 @@ template <int LANES>
 __global__ void __launch_bounds__(256)
 k_gather(const uint4* __restrict__ table, int64_t V, int row_vec, const int32_t* __restrict__ ids, int64_t total,
          uint4* __restrict__ out, int32_t* __restrict__ dev_flag) {
+  pdl_launch_dependents();     // simple kernel: the next one may set itself up beside it
+  pdl_wait();                  // nothing is read or written before the previous kernel is complete
   const int rows_per_block = blockDim.x / LANES;
   const int sub = threadIdx.x % LANES;
   const int64_t stride = (int64_t)gridDim.x * rows_per_block;
@@ -367,10 +369,10 @@ lime_status launch_gather(int dtype, const void* table, int64_t V, int d, const 
   const uint4* tb = (const uint4*)table;
   uint4* o = (uint4*)out;
   switch (lanes) {
-    case 32: k_gather<32><<<(int)blocks, threads, 0, st>>>(tb, V, row_vec, ids, total, o, dev_flag); break;
-    case 16: k_gather<16><<<(int)blocks, threads, 0, st>>>(tb, V, row_vec, ids, total, o, dev_flag); break;
-    case 8:  k_gather<8><<<(int)blocks, threads, 0, st>>>(tb, V, row_vec, ids, total, o, dev_flag); break;
-    default: k_gather<4><<<(int)blocks, threads, 0, st>>>(tb, V, row_vec, ids, total, o, dev_flag); break;
+    case 32: launch_pdl(k_gather<32>, dim3((unsigned)blocks), dim3(threads), 0, st, tb, V, row_vec, ids, total, o, dev_flag); break;
+    case 16: launch_pdl(k_gather<16>, dim3((unsigned)blocks), dim3(threads), 0, st, tb, V, row_vec, ids, total, o, dev_flag); break;
+    case 8:  launch_pdl(k_gather<8>, dim3((unsigned)blocks), dim3(threads), 0, st, tb, V, row_vec, ids, total, o, dev_flag); break;
+    default: launch_pdl(k_gather<4>, dim3((unsigned)blocks), dim3(threads), 0, st, tb, V, row_vec, ids, total, o, dev_flag); break;
   }
   LIME_LAUNCH_CHECK("k_gather");
   return LIME_OK;
