@@ -265,19 +265,19 @@ def launch_mode(args):
 # kernel and workload, with the hash of the kernel's source at capture time: once the source changes the figure
 # is stale and the bench reports null.
 NCU_TRAFFIC = {
-    # dense scorer: 169.9 MB read + 4.0-4.5 MB written per launch
-    ("k_score_tc", "bf16_baseline", 256, 2048): {"bytes": 174.2e6, "source": "k_score_tc.cu", "sha": "823248ada31d3d04"},
-    # XOR-layer kernels: 33.7 MB (layer 1) and 42.2 MB (layer 2) read + written; average per launch
-    ("k_link_attn_tc", "bf16_baseline", 256, 2048): {"bytes": 37.9e6, "source": "k_link_attn_tc.cu", "sha": "81680b45282491ef"},
-    ("k_hist_update_tc", "bf16_baseline", 256, 2048): {"bytes": 34.6e6, "source": "k_hist_update_tc.cu", "sha": "a47ccfb7ddd4247f"},
+    # dense scorer: 169.9 MB read + 3.5 MB written
+    ("k_score_tc", "bf16_baseline", 256, 2048): {"bytes": 173.5e6, "source": "k_score_tc.cu", "sha": "af919608f4657e09"},
+    # XOR-layer kernels: average per launch
+    ("k_link_attn_tc", "bf16_baseline", 256, 2048): {"bytes": 37.8e6, "source": "k_link_attn_tmem_tc.cu", "sha": "74a161f19f4064a1"},
+    ("k_hist_update_tc", "bf16_baseline", 256, 2048): {"bytes": 33.8e6, "source": "k_hist_update_tmem_tc.cu", "sha": "6d27de4cb38a127f"},
     # scorer by id over packed corpus records: 174.5 MB read + 4.1 MB written per launch
     ("k_score_gather_tc", "bf16_baseline", 256, 2048): {"bytes": 178.6e6, "source": "k_score_gather_tc.cu", "sha": "580e539a2d79f57c"},
     # scorer through the interaction network (--head 96): 169.4 MB read + 4.4 MB written per launch
     ("k_score_head_tc", "bf16_baseline", 256, 2048): {"bytes": 173.8e6, "source": "k_score_head_tc.cu", "sha": "614556b96c1342b2"},
-    # d = 256 kernels: captured on 128 users of the same model and length mix (327,693 tokens) and scaled by the tokens of
+    # d = 256 kernels: captured on 128 users of the same model and length mix (327,680 tokens) and scaled by the tokens of
     # a launch (persistent kernels, identical tiles: traffic grows in proportion): bytes per token, average of the layers
-    ("k_link_attn_d256_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 560.0, "source": "k_link_attn_t64_tc.cu", "sha": "b26d676843314aed"},
-    ("k_hist_update_d256_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 893.0, "source": "k_hist_update_d256_tc.cu", "sha": "b84060b13975253c"},
+    ("k_link_attn_d256_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 578.7, "source": "k_link_attn_tmem_tc.cu", "sha": "74a161f19f4064a1"},
+    ("k_hist_update_d256_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 846.5, "source": "k_hist_update_d256_tc.cu", "sha": "b0e365c3aee6d1d3"},
 }
 
 
