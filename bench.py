@@ -269,7 +269,7 @@ NCU_TRAFFIC = {
     ("k_score_tc", "bf16_baseline", 256, 2048): {"bytes": 173.5e6, "source": "k_score_tc.cu", "sha": "af919608f4657e09"},
     # XOR-layer kernels: average per launch
     ("k_link_attn_tc", "bf16_baseline", 256, 2048): {"bytes": 37.8e6, "source": "k_link_attn_tmem_tc.cu", "sha": "74a161f19f4064a1"},
-    ("k_hist_update_tc", "bf16_baseline", 256, 2048): {"bytes": 33.8e6, "source": "k_hist_update_tmem_tc.cu", "sha": "6d27de4cb38a127f"},
+    ("k_hist_update_tc", "bf16_baseline", 256, 2048): {"bytes": 33.8e6, "source": "k_hist_update_tmem_tc.cu", "sha": "bbde8b584842ab94"},
     # scorer by id over packed corpus records: 174.5 MB read + 4.1 MB written per launch
     ("k_score_gather_tc", "bf16_baseline", 256, 2048): {"bytes": 178.6e6, "source": "k_score_gather_tc.cu", "sha": "580e539a2d79f57c"},
     # scorer through the interaction network (--head 96): 169.4 MB read + 4.4 MB written per launch

@@ -1,9 +1,9 @@
 // History update of one XOR layer on tcgen05 for more stacked (head, link) rows than one SM can keep resident
-// (H * ell = 256 .. 512 at d = d_ff = 128, e.g. 4 heads x 64 links):
+// (H * ell = 384 or 512 at d = d_ff = 128, e.g. 8 heads x 64 links):
 //
 //   S'[t,:] = GatedMLP( O[S]_t ),   O[S]_t = concat_h softmax_l( Q[S]_{t,h} K[T]_{l,h}^T * scale ) V[T]_{l,h}     (Eq. 7, Eq. 5)
 //
-// Same chain of contractions per 128-token tile as k_hist_update_tc.cu (scores -> per-head softmax -> [gate | up] ->
+// Same chain of contractions per 128-token tile as k_hist_update_tmem_tc.cu (scores -> per-head softmax -> [gate | up] ->
 // SiLU(gate) * up -> W_o), but the folded link-side operands K2 [HL x d] and [G2 | U2] [2f x HL] (k_link_prep.cu) no
 // longer fit in shared memory next to the token tile.  The (head, link) rows are therefore walked in groups of 128:
 //   for each group c:  scores_c = X . K2_c^T  ->  softmax per head  ->  [gate | up] += P_c . [G2 | U2]_c
@@ -13,7 +13,7 @@
 //
 // Warp 0 TMA producer, warp 1 MMA issuer, warps 2-9 token rows: two threads per token (TMEM lane), 64 columns each -
 // whole heads of the softmax (ell in {32, 64}).  TMEM: 128 columns of scores, 256 [gate | up], 128 S'.
-// With `out_ln` the rows are written LayerNorm-ed for the next layer (see k_hist_update_tc.cu).
+// With `out_ln` the rows are written LayerNorm-ed for the next layer (see k_hist_update_tmem_tc.cu).
 #include "lime_common.cuh"
 #include "tc_common.cuh"
 
@@ -481,7 +481,7 @@ k_hist_update2_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant
 
 bool hist_update2_tc_supported(int dtype, int d, int f, int H, int ell, int phi, int gated_mlp) {
   const int HL = H * ell;
-  return dtype == LIME_BF16 && d == H2_D && f == H2_F && HL % 128 == 0 && HL >= 256 && HL <= 512 && (ell == 32 || ell == 64) &&
+  return dtype == LIME_BF16 && d == H2_D && f == H2_F && HL % 128 == 0 && HL >= 384 && HL <= 512 && (ell == 32 || ell == 64) &&
          (phi == LIME_PHI_SOFTMAX || phi == LIME_PHI_SILU) && gated_mlp != 0;
 }
 
@@ -513,7 +513,6 @@ static lime_status launch_hu2(const HistUpdateArgs& a, int HL, cudaStream_t st) 
 
 lime_status launch_hist_update2_tc(const HistUpdateArgs& a, int H, cudaStream_t st) {
   if (a.total == 0) return LIME_OK;
-  if (!a.ln && hist_update_tmem_supported(H * a.ell, a.ell)) return launch_hist_update_tmem(a, H * a.ell, st);
   switch (a.ell) {
     case 32: return launch_hu2<32>(a, H * a.ell, st);
     case 64: return launch_hu2<64>(a, H * a.ell, st);

@@ -1,12 +1,15 @@
-// History update of one XOR layer on tcgen05, two token tiles in flight per SM (bf16 storage, rows LayerNorm-ed already,
-// d = d_ff = 128, H * ell = 128 or 256):
+// History update of one XOR layer on tcgen05, two token tiles in flight per SM (bf16 storage, d = d_ff = 128, H * ell = 128 or
+// 256):
 //
 //   S'[t,:] = GatedMLP( O[S]_t ),   O[S]_t = concat_h phi( Q[S]_{t,h} K[T]_{l,h}^T * scale ) V[T]_{l,h}          (Eq. 7, Eq. 5)
 //
-// Same folded operands and the same rounding places as k_hist_update_tc.cu and k_hist_update2_tc.cu (which serve rows that
-// still need their LayerNorm, and more stacked rows):
+// With W_K and scale * log2(e) folded into the link keys (K2) and W_V with the GatedMLP's first weights into [G2 | U2]
+// (k_link_prep.cu).  Rows that still need their LayerNorm (LN, the first layer of a raw lookup) get it afterwards, exact for
+// the bf16 operands, from the statistics the attention kernel leaves.  More stacked rows: k_hist_update2_tc.cu.
 //   scores [128 x HL]      = X . K2^T;   per-head softmax over the links (or SiLU(s) / ell) -> P (bf16)
 //   [gate | up] [128 x 2f] = P . [G2 | U2];   U = SiLU(gate) * up (bf16);   S' = U . W_o -> (LayerNorm) -> bf16 -> global
+// With `out_ln` the rows are written LayerNorm-ed: the next layer normalises every row it reads and nothing else reads them
+// (Eq. 8).
 //
 // What bounds it: the chain of four contractions and three passes of the row warps between them, which takes several times
 // the tensor time of a tile.  So two tiles are in the chain at once, half a period apart, each with its own issuing warp,
@@ -39,7 +42,8 @@ constexpr uint32_t HT_OFF_RING = HT_OFF_X + 2 * HT_SUB;       // slabs [64 gate 
 constexpr uint32_t HT_PATCH = 32 * 32;                        // a row warp's own: 8 of its 32 rows on their way out
 constexpr uint32_t HT_OFF_PATCH = HT_OFF_RING + HT_RING * HT_SUB;
 constexpr uint32_t HT_OFF_EXCH = HT_OFF_PATCH + 2 * HT_GROUP_WARPS * HT_PATCH;      // [2 groups][PARTS][128] float2 {mean, M2}
-constexpr uint32_t HT_OFF_BAR = HT_OFF_EXCH + 2 * HT_PARTS * 128 * 8;
+constexpr uint32_t HT_OFF_CK = HT_OFF_EXCH + 2 * HT_PARTS * 128 * 8;  // [2 groups][256] (LN) row sums of their user's K2
+constexpr uint32_t HT_OFF_BAR = HT_OFF_CK + 2 * 256 * 4;
 constexpr int HT_IDX_CAP = 1025;                              // users + 1 whose offsets are staged in shared memory (the
 constexpr uint32_t HT_OFF_IDX = HT_OFF_BAR + 512;             // search for a tile's user is a chain of dependent reads)
 constexpr uint32_t HT_SMEM = HT_OFF_IDX + 2 * HT_IDX_CAP * 4 + 8;
@@ -49,6 +53,8 @@ static_assert(128 * HT_REGS_CONTROL + (HT_THREADS - 128) * HT_REGS_ROWS <= HT_TH
 
 struct HistUpdateTmemParams {
   __nv_bfloat16* out;            // [total x d]
+  const float* cK;               // [users x HL] (LN) row sums of K2
+  const float2* stats_in;        // (LN) {rstd, mean} of every row read, left by the attention kernel of the layer
   const int32_t* off;            // [B+1]
   const int32_t* tile_start;     // [B+1] prefix of per-user tile counts (tile = 128 tokens)
   int B, shared, out_ln;
@@ -95,7 +101,7 @@ struct HtTileUser {
   }
 };
 
-template <int NG, int ELL>
+template <int NG, int ELL, bool LN>
 __global__ void __launch_bounds__(HT_THREADS, 1)
 k_hist_update_tmem_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmK2,
                       const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmU,
@@ -316,6 +322,8 @@ k_hist_update_tmem_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     const uint32_t L = base + (uint32_t)part * 64u, R = base + 128u;      // this thread's columns of L; R as a whole
     float2* exch = reinterpret_cast<float2*>(smem + HT_OFF_EXCH) + grp * HT_PARTS * 128;
     uint8_t* patch = smem + HT_OFF_PATCH + (warp - 4) * HT_PATCH;
+    float* ck_s = reinterpret_cast<float*>(smem + HT_OFF_CK) + grp * 256;
+    int ck_user = -1;
     uint32_t i_ph = 0, gu_ph = 0;
     bool ok = true;
     HtTileUser tu;
@@ -325,8 +333,25 @@ k_hist_update_tmem_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
       if ((g & 1) != grp) continue;
       const int row0 = off[b] + (t - tu.lo) * HT_TILE, row_end = off[b + 1];
       // ---- softmax over the links of this thread's heads, P over its own scores
+      float rstd_r = 1.f, mu_r = 0.f;
+      if (LN && row0 + (int)r < row_end) {
+        const float2 st = __ldg(p.stats_in + row0 + r);
+        rstd_r = st.x; mu_r = st.y;
+      }
       if (!mbar_wait(&s_full[grp], i_ph, p.err, 32)) { ok = false; break; }
       tc_fence_after();
+      if (LN && b != ck_user && (ck_user < 0 || !p.shared)) {
+        // these scores exist, so every warp of the group is past the softmax of its last tile (its U was needed first): nobody
+        // still reads the last user's sums.  Every warp of a part writes the same values.
+        const float* src = p.cK + (int64_t)(p.shared ? 0 : b) * (NG * 128) + part * 64;
+#pragma unroll
+        for (int c = 0; c < NG; ++c) {
+          ck_s[c * 128 + part * 64 + lane] = src[c * 128 + lane];
+          ck_s[c * 128 + part * 64 + 32 + lane] = src[c * 128 + 32 + lane];
+        }
+        __syncwarp();
+      }
+      ck_user = b;
 #pragma unroll
       for (int c = 0; c < NG; ++c) {
         float v[64];
@@ -334,6 +359,17 @@ k_hist_update_tmem_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         tmem_ld_32x32(src, *reinterpret_cast<float(*)[32]>(&v[0]));
         tmem_ld_32x32(src + 32, *reinterpret_cast<float(*)[32]>(&v[32]));
         tmem_wait_ld();
+        if (LN) {
+          // s = rstd (raw - mu rowsum(K2)): the LayerNorm of the row, exact for the bf16 operands
+          const float4* ck = reinterpret_cast<const float4*>(ck_s + c * 128 + part * 64);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const float4 k = ck[j];
+            float2* w = reinterpret_cast<float2*>(&v[4 * j]);
+            w[0] = __fmul2_rn(__ffma2_rn(make_float2(-mu_r, -mu_r), make_float2(k.x, k.y), w[0]), make_float2(rstd_r, rstd_r));
+            w[1] = __fmul2_rn(__ffma2_rn(make_float2(-mu_r, -mu_r), make_float2(k.z, k.w), w[1]), make_float2(rstd_r, rstd_r));
+          }
+        }
 #pragma unroll
         for (int h = 0; h < 64 / ELL; ++h) {
           float2* w = reinterpret_cast<float2*>(&v[h * ELL]);
@@ -483,7 +519,7 @@ k_hist_update_tmem_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   }
 }
 
-template <int NG, int ELL>
+template <int NG, int ELL, bool LN>
 static lime_status launch_ht(const HistUpdateArgs& a, cudaStream_t st, const char* name) {
   CUtensorMap tmX, tmK2, tmG, tmU, tmWo;
   const uint64_t users = a.shared ? 1 : (uint64_t)a.B, HL = NG * 128;
@@ -494,26 +530,34 @@ static lime_status launch_ht(const HistUpdateArgs& a, cudaStream_t st, const cha
     return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
   HistUpdateTmemParams p;
   p.out = (__nv_bfloat16*)a.hist_out; p.off = a.off; p.tile_start = a.tile_start; p.B = a.B; p.silu = a.silu;
-  p.shared = a.shared; p.out_ln = a.out_ln; p.ln_eps = a.ln_eps; p.err = a.err;
+  p.cK = a.cK; p.stats_in = a.stats_in; p.shared = a.shared; p.out_ln = a.out_ln; p.ln_eps = a.ln_eps; p.err = a.err;
   const int grid = a.n_tile_upper < kSMs ? a.n_tile_upper : kSMs;
   if (grid < 1) return LIME_OK;
   static bool smem_set[kMaxDeviceOrdinals] = {};
-  const lime_status es = ensure_dynamic_smem((const void*)k_hist_update_tmem_tc<NG, ELL>, (int)HT_SMEM, smem_set);
+  const lime_status es = ensure_dynamic_smem((const void*)k_hist_update_tmem_tc<NG, ELL, LN>, (int)HT_SMEM, smem_set);
   if (es != LIME_OK) return es;
   ProfScope _p(name, st);
-  launch_pdl(k_hist_update_tmem_tc<NG, ELL>, dim3(grid), dim3(HT_THREADS), HT_SMEM, st, tmX, tmK2, tmG, tmU, tmWo, p);
+  launch_pdl(k_hist_update_tmem_tc<NG, ELL, LN>, dim3(grid), dim3(HT_THREADS), HT_SMEM, st, tmX, tmK2, tmG, tmU, tmWo, p);
   LIME_LAUNCH_CHECK(name);
   return LIME_OK;
 }
 
-bool hist_update_tmem_supported(int HL, int ell) {
-  return (HL == 128 && (ell == 16 || ell == 32)) || (HL == 256 && (ell == 32 || ell == 64));
+bool hist_update_tmem_supported(int dtype, int d, int f, int H, int ell, int phi, int gated_mlp) {
+  const int HL = H * ell;
+  return dtype == LIME_BF16 && d == HT_D && f == HT_F && ((HL == 128 && (ell == 16 || ell == 32)) || (HL == 256 && (ell == 32 || ell == 64))) &&
+         (phi == LIME_PHI_SOFTMAX || phi == LIME_PHI_SILU) && gated_mlp != 0;
 }
 
-lime_status launch_hist_update_tmem(const HistUpdateArgs& a, int HL, cudaStream_t st) {
+template <int NG, int ELL>
+static lime_status launch_ht_ln(const HistUpdateArgs& a, cudaStream_t st, const char* name) {
+  return a.ln ? launch_ht<NG, ELL, true>(a, st, name) : launch_ht<NG, ELL, false>(a, st, name);
+}
+
+lime_status launch_hist_update_tmem(const HistUpdateArgs& a, int H, cudaStream_t st) {
   if (a.total == 0) return LIME_OK;
-  if (HL == 128) return a.ell == 16 ? launch_ht<1, 16>(a, st, "k_hist_update_tc") : launch_ht<1, 32>(a, st, "k_hist_update_tc");
-  return a.ell == 32 ? launch_ht<2, 32>(a, st, "k_hist_update2_tc") : launch_ht<2, 64>(a, st, "k_hist_update2_tc");
+  if (a.ln && (a.stats_in == nullptr || a.cK == nullptr)) return LIME_INVALID_ARG;
+  if (H * a.ell == 128) return a.ell == 16 ? launch_ht_ln<1, 16>(a, st, "k_hist_update_tc") : launch_ht_ln<1, 32>(a, st, "k_hist_update_tc");
+  return a.ell == 32 ? launch_ht_ln<2, 32>(a, st, "k_hist_update2_tc") : launch_ht_ln<2, 64>(a, st, "k_hist_update2_tc");
 }
 
 }  // namespace lime

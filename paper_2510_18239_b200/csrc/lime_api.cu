@@ -88,7 +88,7 @@ static int pick_chunk(int64_t total_tokens, int row_blocks, int lo, int hi = 204
 // built for d = d_ff = 256, 0 = the generic CUDA-core path.
 static int tensor_core_mode(const lime_config& g, int d_ff) {
   if (link_attn_tc_supported(g.dtype, g.d, g.H, g.ell, g.phi) &&
-      (hist_update_tc_supported(g.dtype, g.d, d_ff, g.H, g.ell, g.phi, g.gated_mlp) ||
+      (hist_update_tmem_supported(g.dtype, g.d, d_ff, g.H, g.ell, g.phi, g.gated_mlp) ||
        hist_update2_tc_supported(g.dtype, g.d, d_ff, g.H, g.ell, g.phi, g.gated_mlp)))
     return 1;
   if (link_attn_d256_tc_supported(g.dtype, g.d, g.H, g.ell, g.phi) &&
@@ -241,8 +241,8 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
   la.ln = hist_ln; la.ln_eps = c->ln_eps; la.silu = g.phi == LIME_PHI_SILU; la.part_m = w.part_m; la.part_s = w.part_s; la.part_acc = w.part_acc; la.Ohat = w.Ohat;
   la.err = c->dev_err;
   // the attention kernel forms the LayerNorm statistics of every history row anyway; the history update reuses them
-  const bool one_block_update = c->tc_mode == 1 && hist_update_tc_supported(g.dtype, g.d, c->d_ff, g.H, g.ell, g.phi, g.gated_mlp);
-  const bool pass_stats = hist_ln && hist_out && one_block_update && total > 0;
+  const bool two_tiles = c->tc_mode == 1 && hist_update_tmem_supported(g.dtype, g.d, c->d_ff, g.H, g.ell, g.phi, g.gated_mlp);
+  const bool pass_stats = hist_ln && hist_out && two_tiles && total > 0;
   la.stats_out = pass_stats ? w.row_stats : nullptr;
   if ((s = c->tc_mode == 2 ? launch_link_attn_d256_tc(la, st) : launch_link_attn_tc(la, st)) != LIME_OK) return s;
   if (c->side256) {
@@ -272,7 +272,7 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
     hu.n_tile_upper = w.n_tile_upper; hu.ell = g.ell; hu.shared = ops.shared; hu.ln = hist_ln; hu.ln_eps = c->ln_eps;
     hu.out_ln = out_ln; hu.silu = g.phi == LIME_PHI_SILU; hu.err = c->dev_err;
     hu.stats_in = pass_stats ? w.row_stats : nullptr;
-    if (one_block_update) s = launch_hist_update_tc(hu, st);
+    if (two_tiles) s = launch_hist_update_tmem(hu, g.H, st);
     else s = launch_hist_update2_tc(hu, g.H, st);
     if (s != LIME_OK) return s;
   }

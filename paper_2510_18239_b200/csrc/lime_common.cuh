@@ -365,12 +365,9 @@ struct HistUpdateArgs {
   const float2* stats_in;               // nullable, ln only: {rstd, mean} of every row read, as left by the attention kernel
   int* err;
 };
-bool hist_update_tc_supported(int dtype, int d, int f, int H, int ell, int phi, int gated_mlp);
-lime_status launch_hist_update_tc(const HistUpdateArgs& a, cudaStream_t st);
-// the same for rows LayerNorm-ed already (a.ln must be 0), HL = H * ell in {128, 256}
-bool hist_update_tmem_supported(int HL, int ell);
-lime_status launch_hist_update_tmem(const HistUpdateArgs& a, int HL, cudaStream_t st);
-// same step for H * ell in {256, 384, 512} (link-side operands streamed per tile, k_hist_update2_tc.cu)
+bool hist_update_tmem_supported(int dtype, int d, int f, int H, int ell, int phi, int gated_mlp);     // H * ell = 128 or 256
+lime_status launch_hist_update_tmem(const HistUpdateArgs& a, int H, cudaStream_t st);                 // a.ln: with stats_in and cK
+// same step for other H * ell up to 512 (link-side operands streamed per tile, k_hist_update2_tc.cu)
 bool hist_update2_tc_supported(int dtype, int d, int f, int H, int ell, int phi, int gated_mlp);
 lime_status launch_hist_update2_tc(const HistUpdateArgs& a, int H, cudaStream_t st);
 

@@ -254,7 +254,8 @@ def test_link_contextualisation_with_one_hidden_layer(d, ell, w0, d_c, B):
 
 @pytest.mark.parametrize("d,H,ell", [(128, 4, 32), (128, 8, 16), (128, 4, 64), (128, 8, 32), (256, 4, 32), (256, 8, 64)])
 @pytest.mark.parametrize("lengths", [[1], [95, 96, 97, 0, 127, 128, 129, 191, 193, 257, 289], [4500, 3, 700], [130] * 160])
-@pytest.mark.parametrize("phi,per_user", [("softmax", True), ("silu", False)])
-def test_attention_over_token_tiles(d, H, ell, lengths, phi, per_user):
-    """Histories around the 96- and 128-token tiles, one of several chunks, more users than CTAs."""
-    _encode_against_oracle(synth.BF16, d, H, ell, 2, lengths, phi, False, per_user, 6e-2, 4e-2 if phi == "silu" else 2.5e-2)
+@pytest.mark.parametrize("phi,raw,per_user", [("softmax", False, True), ("silu", False, False), ("softmax", True, False), ("silu", True, True)])
+def test_attention_over_token_tiles(d, H, ell, lengths, phi, raw, per_user):
+    """Histories around the 96- and 128-token tiles, one of several chunks, more users than CTAs; rows as stored and
+    LayerNorm-ed by the lookup."""
+    _encode_against_oracle(synth.BF16, d, H, ell, 2, lengths, phi, raw, per_user, 6e-2, 4e-2 if phi == "silu" else 2.5e-2)
