@@ -7,8 +7,12 @@
 // time (the accumulator becomes the A fragment of the second layer's k-step) and keeps the 128-wide second layer in its
 // accumulators, so no activation touches memory.  A tcgen05 version would have to send every hidden block through TMEM, the
 // register file and shared memory again, and the batches served (tens of thousands of candidates) are a single wave.
-// The first layer's input is not folded through the link states: O is formed per candidate (four products) and enters as a
-// bf16 value and its remainder, so it keeps the accuracy of the fp32 mix and needs no per-user operand.
+// The first layer's input is not folded through the link states: O is formed per candidate (four products), so it needs no per-user
+// operand.  O and both hidden layers enter their products as a bf16 value and its bf16 remainder.  Error of the logits against
+// fp64 from the same link states (16 links, widths 512, 128, 64, four seeds): 2.0e-6 .. 5.3e-6; rounded once instead, the hidden
+// layers put 1.7e-3 .. 3.0e-3 into it (the CUDA-core kernel for other widths: 2.3e-7 .. 5.6e-7; a third piece leaves 0.9e-6 ..
+// 2.3e-6, what the tensor cores' sums add, and costs 18 us more).  25,600 candidates: 35 us a launch with one rounding, 44 with two
+// pieces.
 // Weights are read as stored ([in x out], ldmatrix.trans).  Chunk c (16 bytes) of row r sits at c ^ s(r), s(r) = (r & 7) ^
 // ((r >> 3 & 3) << 1): free of conflicts both for eight consecutive rows and for the rows 8 i, 8 i + 1 (i = 0..3) that the
 // permuted contraction over T needs (thread t of a quad holds features 8 t .. 8 t + 7 of a candidate row: one 16-byte load).
@@ -18,6 +22,7 @@
 namespace lime {
 
 constexpr int M3_D = 32, M3_N1 = 128, M3_N2 = 64, M3_WARPS = 8, M3_THREADS = M3_WARPS * 32;
+constexpr int M3_TERMS = 2;      // bf16 pieces of a value that was fp32: the mix, the first and the second hidden layer
 
 struct ScoreMlp3Params {
   const __nv_bfloat16* LS; const __nv_bfloat16* W; const __nv_bfloat16* T;
@@ -32,6 +37,15 @@ __device__ __forceinline__ uint32_t m3_at(int r, int c, int pitch) { return (uin
 __device__ __forceinline__ uint32_t m3_pack(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&v);
+}
+// two fp32 values as M3_TERMS packed bf16 pairs: the values, their remainders
+__device__ __forceinline__ void m3_split(float x, float y, uint32_t (&out)[M3_TERMS]) {
+#pragma unroll
+  for (int k = 0; k < M3_TERMS; ++k) {
+    out[k] = m3_pack(x, y);
+    x -= __uint_as_float(out[k] << 16);
+    y -= __uint_as_float(out[k] & 0xffff0000u);
+  }
 }
 __device__ __forceinline__ void m3_mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
@@ -173,18 +187,18 @@ k_score_mlp3(const ScoreMlp3Params p) {
       if (u1 >= s1 || b + 1 >= p.B) break;
       ++b;
     }
-    // O as A fragments: value and remainder
-    uint32_t oh[2][2][4], ol[2][2][4];
+    // O as A fragments
+    uint32_t of[M3_TERMS][2][2][4];
 #pragma unroll
     for (int m = 0; m < 2; ++m)
 #pragma unroll
       for (int ks = 0; ks < 2; ++ks)
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          const float x = o[m][2 * ks + (r >> 1)][(r & 1) * 2], y = o[m][2 * ks + (r >> 1)][(r & 1) * 2 + 1];
-          const uint32_t h = m3_pack(x, y);
-          oh[m][ks][r] = h;
-          ol[m][ks][r] = m3_pack(x - __uint_as_float(h << 16), y - __uint_as_float(h & 0xffff0000u));
+          uint32_t v[M3_TERMS];
+          m3_split(o[m][2 * ks + (r >> 1)][(r & 1) * 2], o[m][2 * ks + (r >> 1)][(r & 1) * 2 + 1], v);
+#pragma unroll
+          for (int k = 0; k < M3_TERMS; ++k) of[k][m][ks][r] = v[k];
         }
     if (!weights_in) {
       asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -217,7 +231,9 @@ k_score_mlp3(const ScoreMlp3Params p) {
 #pragma unroll
         for (int m = 0; m < 2; ++m)
 #pragma unroll
-          for (int n = 0; n < 2; ++n) { m3_mma(h[m][n], oh[m][ks], w[2 * n], w[2 * n + 1]); m3_mma(h[m][n], ol[m][ks], w[2 * n], w[2 * n + 1]); }
+          for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int k = 0; k < M3_TERMS; ++k) m3_mma(h[m][n], of[k][m][ks], w[2 * n], w[2 * n + 1]);
       }
 #pragma unroll
       for (int s = 0; s < 2; ++s) {
@@ -232,17 +248,24 @@ k_score_mlp3(const ScoreMlp3Params p) {
           for (int n = 0; n < 2; ++n) m3_mma(h[m][n], a, w[2 * n], w[2 * n + 1]);
         }
       }
-      uint32_t a[2][4];
+      uint32_t a[M3_TERMS][2][4];
 #pragma unroll
       for (int m = 0; m < 2; ++m)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) a[m][r] = m3_pack(fmaxf(h[m][r >> 1][(r & 1) * 2], 0.f), fmaxf(h[m][r >> 1][(r & 1) * 2 + 1], 0.f));
+        for (int r = 0; r < 4; ++r) {
+          uint32_t v[M3_TERMS];
+          m3_split(fmaxf(h[m][r >> 1][(r & 1) * 2], 0.f), fmaxf(h[m][r >> 1][(r & 1) * 2 + 1], 0.f), v);
+#pragma unroll
+          for (int k = 0; k < M3_TERMS; ++k) a[k][m][r] = v[k];
+        }
 #pragma unroll
       for (int n = 0; n < M3_N1 / 8; n += 2) {
         uint32_t w[4];
         m3_ldsm_t(w, sb + lay.w1 + m3_at(hb * 16 + (lane & 15), n + (lane >> 4), M3_N1 * 2));
 #pragma unroll
-        for (int m = 0; m < 2; ++m) { m3_mma(acc[m][n], a[m], w[0], w[1]); m3_mma(acc[m][n + 1], a[m], w[2], w[3]); }
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+          for (int k = 0; k < M3_TERMS; ++k) { m3_mma(acc[m][n], a[k][m], w[0], w[1]); m3_mma(acc[m][n + 1], a[k][m], w[2], w[3]); }
       }
     }
     // third layer
@@ -255,18 +278,24 @@ k_score_mlp3(const ScoreMlp3Params p) {
     }
 #pragma unroll
     for (int ks = 0; ks < M3_N1 / 16; ++ks) {
-      uint32_t a[2][4];
+      uint32_t a[M3_TERMS][2][4];
 #pragma unroll
       for (int m = 0; m < 2; ++m)
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
-          a[m][r] = m3_pack(fmaxf(acc[m][2 * ks + (r >> 1)][(r & 1) * 2], 0.f), fmaxf(acc[m][2 * ks + (r >> 1)][(r & 1) * 2 + 1], 0.f));
+        for (int r = 0; r < 4; ++r) {
+          uint32_t v[M3_TERMS];
+          m3_split(fmaxf(acc[m][2 * ks + (r >> 1)][(r & 1) * 2], 0.f), fmaxf(acc[m][2 * ks + (r >> 1)][(r & 1) * 2 + 1], 0.f), v);
+#pragma unroll
+          for (int k = 0; k < M3_TERMS; ++k) a[k][m][r] = v[k];
+        }
 #pragma unroll
       for (int n = 0; n < M3_N2 / 8; n += 2) {
         uint32_t w[4];
         m3_ldsm_t(w, sb + lay.w2 + m3_at(ks * 16 + (lane & 15), n + (lane >> 4), M3_N2 * 2));
 #pragma unroll
-        for (int m = 0; m < 2; ++m) { m3_mma(z[m][n], a[m], w[0], w[1]); m3_mma(z[m][n + 1], a[m], w[2], w[3]); }
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+          for (int k = 0; k < M3_TERMS; ++k) { m3_mma(z[m][n], a[k][m], w[0], w[1]); m3_mma(z[m][n + 1], a[k][m], w[2], w[3]); }
       }
     }
     // output layer: rows g, g + 8 (values 0-1, 2-3) of each half

@@ -259,3 +259,21 @@ def test_attention_over_token_tiles(d, H, ell, lengths, phi, raw, per_user):
     """Histories around the 96- and 128-token tiles, one of several chunks, more users than CTAs; rows as stored and
     LayerNorm-ed by the lookup."""
     _encode_against_oracle(synth.BF16, d, H, ell, 2, lengths, phi, raw, per_user, 6e-2, 4e-2 if phi == "silu" else 2.5e-2)
+
+
+@pytest.mark.parametrize("ell,w0", [(8, 64), (16, 512), (32, 128)])
+def test_three_layer_interaction_network_keeps_its_hidden_layers(ell, w0):
+    """The mix and both hidden layers enter each product as a bf16 value and its bf16 remainder, a relative 2^-17 of every term:
+    3 x 2^-16 of the norm of the logits bounds the three products; one rounding to bf16 is 2^-9."""
+    Bd = _lib()
+    d, dtype, B, C = 32, synth.BF16, 4, 150
+    r = np.random.default_rng(ell + w0)
+    LS, W, T = (synth.to_storage(x, dtype) for x in (r.normal(size=(B, ell, d)), O.softmax_rows(r.normal(size=(B * C, ell)) * 1.5), r.normal(size=(B * C, d))))
+    lime = Bd.Lime(d, 4, ell, 1, dtype=Bd.LIME_BF16)
+    layers = synth.ffn_weights(5, "head", (2 * d, w0, 128, 64, 1), dtype)
+    lime.set_head([(Bd.to_device(w, dtype), torch.from_numpy(b).cuda()) for w, b in layers])
+    got = Hh.to_f64(lime.score_candidates_head(Bd.to_device(LS, dtype), Bd.to_device(W, dtype), Bd.to_device(T, dtype), C=C))
+    L64 = [(synth.storage_to_f64(w, dtype), b.astype(np.float64)) for w, b in layers]
+    W64, T64, LS64 = (synth.storage_to_f64(x, dtype) for x in (W, T, LS))
+    want = np.concatenate([O.score_candidates_head(W64[b * C:(b + 1) * C], LS64[b], T64[b * C:(b + 1) * C], L64) for b in range(B)])
+    assert np.linalg.norm(got - want) <= 3 * 2.0 ** -16 * np.linalg.norm(want), np.linalg.norm(got - want) / np.linalg.norm(want)
