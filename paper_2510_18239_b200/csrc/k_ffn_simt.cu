@@ -5,8 +5,8 @@
 // concatenation and are split over it, so neither input row is ever formed:
 //   (L_l (+) E^C_b) W_0 = (L W_0[:d])_l + E^C_b W_0[d:]          the first term is weights only (formed at set-up)
 //   [O_c | T_c] W_0     = sum_l W[c,l] (LS_b W_0[:d])_l + T_c W_0[d:]          LSW_b = LS_b W_0[:d] once per user
-// The bf16 one-hidden-layer interaction network on dense candidate streams runs on tensor cores (k_score_head_tc.cu);
-// everything else (fp32 storage, deeper networks, ragged candidate lists, candidates taken by id) runs here.
+// On tensor cores instead: the bf16 one-hidden-layer interaction network on dense streams or a fixed number of ids per user
+// (k_score_head_tc.cu), one three-layer network at d = 32 (k_score_mlp3.cu), Eq. 2 with one hidden layer (k_link_ctx_mma.cu).
 #include "lime_common.cuh"
 
 namespace lime {
@@ -14,14 +14,12 @@ namespace lime {
 // ----------------------------------------------------------------------------- Y[r, :] = X[r, :] . W (+ b)
 // Small dense product with fp32 accumulation.  A block takes FR_ROWS rows of X and FR_COLS output columns; the rows sit in
 // shared memory, the block's slice of W is staged there too in pieces of FR_KC contraction indices (read once, coalesced
-// over the columns), and a thread forms FR_ROWS / 4 x 1 outputs per piece from shared memory only.  Outputs: fp32 [M x N]
-// and / or bf16 transposed per group of `group` rows ([M/group][N][group], the K-major operand layout of
-// k_score_head_tc.cu).
+// over the columns), and a thread forms FR_ROWS / 4 x 1 outputs per piece from shared memory only.
 constexpr int FR_ROWS = 32, FR_COLS = 32, FR_KC = 64, FR_THREADS = 128;      // thread (ty, tx): rows ty*8..ty*8+7, column tx
 template <typename TX, typename TW>
 __global__ void __launch_bounds__(FR_THREADS)
 k_rows_times_w(const TX* __restrict__ X, int64_t M, int K, const TW* __restrict__ W, int ldw, int N, const float* __restrict__ bias,
-               float* __restrict__ Y, __nv_bfloat16* __restrict__ Yt, int group) {
+               float* __restrict__ Y) {
   extern __shared__ float fr_sm[];
   float* xs = fr_sm;                                 // [FR_ROWS][K + 1]
   float* wsm = xs + FR_ROWS * (K + 1);               // [FR_KC][FR_COLS]
@@ -57,15 +55,13 @@ k_rows_times_w(const TX* __restrict__ X, int64_t M, int K, const TW* __restrict_
     for (int r = 0; r < RPT; ++r) {
       const int rr = ty * RPT + r;
       if (rr >= nr) break;
-      const int64_t row = r0 + rr;
-      if (Y) Y[row * N + col] = acc[r];
-      if (Yt) Yt[((row / group) * N + col) * group + (row % group)] = __float2bfloat16_rn(acc[r]);
+      Y[(r0 + rr) * N + col] = acc[r];
     }
   }
 }
 
 lime_status launch_rows_times_w(const void* X, int x_dtype, int64_t M, int K, const void* W, int w_dtype, int ldw, int N,
-                                const float* bias, float* Y, void* Yt, int group, const char* name, cudaStream_t st) {
+                                const float* bias, float* Y, const char* name, cudaStream_t st) {
   if (M == 0 || N == 0) return LIME_OK;
   const size_t smem = sizeof(float) * (FR_ROWS * ((size_t)K + 1) + FR_KC * FR_COLS);
   if (smem > 200 * 1024) return LIME_UNSUPPORTED_SHAPE;
@@ -74,8 +70,7 @@ lime_status launch_rows_times_w(const void* X, int x_dtype, int64_t M, int K, co
 #define LIME_RTW(TX, TW)                                                                                                  \
   do {                                                                                                                    \
     LIME_CUDA(cudaFuncSetAttribute(k_rows_times_w<TX, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));       \
-    k_rows_times_w<TX, TW><<<grid, FR_THREADS, smem, st>>>((const TX*)X, M, K, (const TW*)W, ldw, N, bias, Y,              \
-                                                          (__nv_bfloat16*)Yt, group);                                      \
+    k_rows_times_w<TX, TW><<<grid, FR_THREADS, smem, st>>>((const TX*)X, M, K, (const TW*)W, ldw, N, bias, Y);            \
   } while (0)
   if (x_dtype == LIME_F32 && w_dtype == LIME_F32) LIME_RTW(float, float);
   else if (x_dtype == LIME_F32) LIME_RTW(float, __nv_bfloat16);

@@ -29,7 +29,8 @@ struct GemmParams {
   int d, f, plain_v;                // output widths; plain_v: the third segment is V[T] (d columns) instead of G2 | U2
   __nv_bfloat16 *Q2, *K2, *G2t, *U2t, *V2t;
   float *cQ, *cK;                   // row sums of Q2 / K2 (only with d = 128: one n-tile per row)
-  // ROWS_T: out[(row / group) * n_cols + col][row % group] for col < n_cols (bf16): the product transposed per group of rows
+  // ROWS_T: out[(row / group) * n_cols + col][k * group + row % group] for col < n_cols, k < TERMS (bf16): the product transposed
+  // per group of rows, as TERMS pieces (the value, its remainder, ..)
   __nv_bfloat16* out_t;
   int group, n_cols;
   int* err;
@@ -40,7 +41,7 @@ __device__ __forceinline__ uint32_t gm_pack(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-template <int EPI, int NT>
+template <int EPI, int NT, int TERMS>
 __global__ void __launch_bounds__(GM_THREADS, 1)
 k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmParams p) {
   using namespace tc;
@@ -220,7 +221,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
       } else if (EPI == GM_EPI_ROWS_T) {
         const int64_t u = row / p.group;
         const int l = (int)(row % p.group);
-        __nv_bfloat16* dst = p.out_t + (u * p.n_cols + (int64_t)nt * NT) * p.group + l;
+        const int ld = TERMS * p.group;
+        __nv_bfloat16* dst = p.out_t + (u * p.n_cols + (int64_t)nt * NT) * ld + l;
 #pragma unroll
         for (int c = cb; c < ce; c += 16) {
           float v[16];
@@ -229,7 +231,15 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
           if (valid) {
 #pragma unroll
             for (int j = 0; j < 16; ++j)
-              if (nt * NT + c + j < p.n_cols) dst[(int64_t)(c + j) * p.group] = __float2bfloat16_rn(v[j]);
+              if (nt * NT + c + j < p.n_cols) {
+                __nv_bfloat16* at = dst + (c + j) * ld;
+#pragma unroll
+                for (int k = 0; k < TERMS; ++k, at += p.group) {
+                  const __nv_bfloat16 piece = __float2bfloat16_rn(v[j]);
+                  *at = piece;
+                  v[j] -= __bfloat162float(piece);
+                }
+              }
           }
         }
       }
@@ -248,13 +258,13 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   }
 }
 
-template <int EPI, int NT>
+template <int EPI, int NT, int TERMS = 1>
 static lime_status launch_gemm(const void* A, int64_t M, int K, const void* Bt, int n_rows_b, int n_tiles, GemmParams p,
                                const char* name, cudaStream_t st) {
   if (M == 0) return LIME_OK;
   CUtensorMap tmA, tmB;
   if (!make_tmap_bf16_sw128(&tmA, A, (uint64_t)M, (uint64_t)K, (uint64_t)K, 128) ||
-      !make_tmap_bf16_sw128(&tmB, Bt, (uint64_t)n_rows_b, (uint64_t)K, (uint64_t)K, 128))
+      !make_tmap_bf16_sw128(&tmB, Bt, (uint64_t)n_rows_b, (uint64_t)K, (uint64_t)K, NT))
     return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
   constexpr size_t stage = GM_SUB + (size_t)NT * 128;
   const int64_t m_tiles = (M + 127) / 128;
@@ -264,12 +274,12 @@ static lime_status launch_gemm(const void* A, int64_t M, int K, const void* Bt, 
   constexpr size_t smem = GM_MAX_STAGES * stage + (EPI == GM_EPI_PREP ? 8 * GM_PATCH : 0) + 256 + 1024;
   static_assert(smem <= 232448, "shared memory budget of one CTA");
   static bool smem_set[kMaxDeviceOrdinals] = {};
-  const lime_status es = ensure_dynamic_smem((const void*)k_gemm_tc<EPI, NT>, (int)smem, smem_set);
+  const lime_status es = ensure_dynamic_smem((const void*)k_gemm_tc<EPI, NT, TERMS>, (int)smem, smem_set);
   if (es != LIME_OK) return es;
   ProfScope _p(name, st);
   const int64_t tiles = m_tiles * n_tiles;
   const unsigned grid = (unsigned)(tiles < kSMs ? tiles : kSMs);
-  launch_pdl(k_gemm_tc<EPI, NT>, dim3(grid), dim3(GM_THREADS), smem, st, tmA, tmB, p);
+  launch_pdl(k_gemm_tc<EPI, NT, TERMS>, dim3(grid), dim3(GM_THREADS), smem, st, tmA, tmB, p);
   LIME_LAUNCH_CHECK(name);
   return LIME_OK;
 }
@@ -286,13 +296,17 @@ lime_status launch_gemm_prep(const LinkGemmArgs& a, cudaStream_t st) {
   return launch_gemm<GM_EPI_PREP, 128>(a.A, a.M, a.K, a.Bt, cols_all, n_tiles, p, "k_gemm_tc_prep", st);
 }
 
-// A [M x K] . Bt^T with Bt [n_cols x K] (bf16, K a multiple of 64): the product as bf16, transposed per group of `group`
-// consecutive rows: out_t [M / group][n_cols][group]
-lime_status launch_gemm_rows_t(const void* A, int64_t M, int K, const void* Bt, int n_cols, int group, void* out_t, int* err,
+// A [M x K] . Bt^T with Bt [n_cols x K] (bf16, K a multiple of 64): the product as `terms` bf16 pieces a value, transposed per
+// group of `group` consecutive rows: out_t [M / group][n_cols][terms][group]
+lime_status launch_gemm_rows_t(const void* A, int64_t M, int K, const void* Bt, int n_cols, int group, int terms, void* out_t, int* err,
                                const char* name, cudaStream_t st) {
-  if (K % 64 || K < 64 || n_cols < 1 || group < 1) return LIME_UNSUPPORTED_SHAPE;
+  if (K % 64 || K < 64 || n_cols < 1 || group < 1 || terms < 1 || terms > 3) return LIME_UNSUPPORTED_SHAPE;
   GemmParams p{};
   p.out_t = (__nv_bfloat16*)out_t; p.group = group; p.n_cols = n_cols; p.err = err;
+  // several pieces: what a thread stores is most of the time, so narrow tiles spread it over more CTAs (2048 rows x 96 columns, three
+  // pieces: 8.5 us, 29 in tiles of 128 columns; one piece, 128 columns: 11)
+  if (terms == 3) return launch_gemm<GM_EPI_ROWS_T, 32, 3>(A, M, K, Bt, n_cols, (n_cols + 31) / 32, p, name, st);
+  if (terms == 2) return launch_gemm<GM_EPI_ROWS_T, 32, 2>(A, M, K, Bt, n_cols, (n_cols + 31) / 32, p, name, st);
   return launch_gemm<GM_EPI_ROWS_T, 128>(A, M, K, Bt, n_cols, (n_cols + 127) / 128, p, name, st);
 }
 

@@ -15,6 +15,10 @@
 // rows 4 g .. 4 g + 3 of the tile by the gather form of the copy (one row high box, four row indices), both operands in the
 // swizzle their MMA expects.  An id outside the caches fetches row 0 and its slot scores 0.  (64 users x 500 candidates by id,
 // d = 256, ell = 32, n1 = 96: 308 us on the CUDA-core scorer before.)
+// LSW comes as `terms` bf16 pieces per value (the value, its remainder, ..), each a block of ell columns of the contraction against
+// the same weight rows.  Dense streams take one.  By id it is three, two where three do not fit: the CUDA-core scorer, which
+// serves all other candidate forms and served this one, keeps LSW in fp32 (error of the logits against fp64, 32 users x 500 by id,
+// d = 256, ell = 32, n1 = 96, two seeds: 2.8e-7 and 2.0e-7 there, 1.7e-4 and 1.6e-4 with one piece, 2.8e-7 and 3.8e-7 with three).
 #include "lime_common.cuh"
 #include "tc_common.cuh"
 
@@ -32,7 +36,7 @@ struct ScoreHeadParams {
   const float* b2;       // [1] or NULL
   int B, C, d, n1;
   int tiles_per_user, n_tiles;
-  int stages, lsw_bufs;
+  int stages, lsw_bufs, terms;
   int* err;
 };
 
@@ -51,7 +55,7 @@ k_score_head_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__
   const uint32_t t_bytes = (uint32_t)KB * SH_TILE * 128;
   constexpr uint32_t w_bytes = (uint32_t)SH_TILE * ELL * 2;
   const uint32_t stage_bytes = t_bytes + w_bytes;
-  const uint32_t lsw_bytes = ((uint32_t)n1 * ELL * 2 + 1023u) & ~1023u;
+  const uint32_t lsw_bytes = ((uint32_t)n1 * ELL * 2 * p.terms + 1023u) & ~1023u;
   const uint32_t w1b_bytes = (uint32_t)KB * n1 * 128;
   const int S = p.stages, LB = p.lsw_bufs;
 
@@ -133,8 +137,8 @@ k_score_head_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__
           const int lb = un % LB;
           if (!all(mbar_wait_spin(&lsw_empty[lb], ((uint32_t)(un / LB) & 1u) ^ 1u, p.err, 101))) { ok = false; break; }
           if (lane == 0) {
-            mbar_arrive_expect_tx(&lsw_full[lb], (uint32_t)n1 * ELL * 2);
-            for (int kb = 0; kb < WKB; ++kb)
+            mbar_arrive_expect_tx(&lsw_full[lb], (uint32_t)n1 * ELL * 2 * p.terms);
+            for (int kb = 0; kb < WKB * p.terms; ++kb)
               tma_load_2d_hint(lsw_base + (size_t)lb * lsw_bytes + (size_t)kb * n1 * W_ROW, &tmLSW, kb * WK, b * n1, &lsw_full[lb], pol_keep);
           }
           ++un;
@@ -196,11 +200,10 @@ k_score_head_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__
                         make_sdesc_k_sw128(smem_u32(w1b_base) + (uint32_t)kb * n1 * 128 + k * 32), idesc, (kb | k) != 0 ? 1u : 0u);
         }
         // + W_tile . LSW_b  (contraction over the links)
-#pragma unroll
-        for (int kb = 0; kb < WKB; ++kb) {
+        for (int kb = 0; kb < WKB * p.terms; ++kb) {
 #pragma unroll
           for (int k = 0; k < WK / 16; ++k)
-            mma_bf16_ss(d_tmem, make_sdesc_k_sw(a0 + t_bytes + (uint32_t)kb * SH_TILE * W_ROW + k * 32, W_ROW),
+            mma_bf16_ss(d_tmem, make_sdesc_k_sw(a0 + t_bytes + (uint32_t)(kb % WKB) * SH_TILE * W_ROW + k * 32, W_ROW),
                         make_sdesc_k_sw(lsw_addr + (uint32_t)kb * n1 * W_ROW + k * 32, W_ROW), idesc, 1u);
         }
         mma_commit(&empty[s]);
@@ -260,18 +263,24 @@ k_score_head_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__
 }
 
 // Shared-memory plan: S stages of (candidate tile + weight rows), one or two LSW buffers, W_1b, constants, barriers.
-static bool score_head_plan(int ell, int d, int n1, int* stages, int* lsw_bufs, size_t* smem_bytes) {
+struct ScoreHeadPlan {
+  int stages, lsw_bufs, terms;
+  size_t smem;
+};
+static bool score_head_plan(int ell, int d, int n1, bool by_id, ScoreHeadPlan* plan) {
   const size_t stage = (size_t)(d / 64) * SH_TILE * 128 + (size_t)SH_TILE * ell * 2;
-  const size_t lsw = ((size_t)n1 * ell * 2 + 1023) & ~(size_t)1023;
   const size_t w1b = ((size_t)(d / 64) * n1 * 128 + 1023) & ~(size_t)1023;
   const size_t fixed = 1024 + (2 * 256 + 4) * 4 + (2 * SH_MAX_STAGES + 9) * 8 + 16;
   const size_t budget = 226 * 1024;
-  for (int lb = 2; lb >= 1; --lb) {
-    if (fixed + w1b + lb * lsw + 2 * stage > budget) continue;
-    int S = (int)((budget - fixed - w1b - lb * lsw) / stage);
-    if (S > SH_MAX_STAGES) S = SH_MAX_STAGES;
-    *stages = S; *lsw_bufs = lb; *smem_bytes = fixed + w1b + lb * lsw + (size_t)S * stage;
-    return true;
+  for (int terms = by_id ? 3 : 1; terms >= (by_id ? 2 : 1); --terms) {
+    const size_t lsw = ((size_t)n1 * ell * 2 * terms + 1023) & ~(size_t)1023;
+    for (int lb = 2; lb >= 1; --lb) {
+      if (fixed + w1b + lb * lsw + 2 * stage > budget) continue;
+      int S = (int)((budget - fixed - w1b - lb * lsw) / stage);
+      if (S > SH_MAX_STAGES) S = SH_MAX_STAGES;
+      *plan = ScoreHeadPlan{S, lb, terms, fixed + w1b + lb * lsw + (size_t)S * stage};
+      return true;
+    }
   }
   return false;
 }
@@ -282,23 +291,27 @@ bool score_head_tc_supported(const ScoreArgs& a, int n1) {
   if (a.d % 64 != 0 || a.d > 512) return false;
   if (n1 % 16 != 0 || n1 < 16 || n1 > 256) return false;
   if (a.C <= 0 || a.total != (int64_t)a.B * a.C) return false;
-  int S, lb;
-  size_t smem;
-  return score_head_plan(a.ell, a.d, n1, &S, &lb, &smem);
+  ScoreHeadPlan plan;
+  return score_head_plan(a.ell, a.d, n1, a.cand_ids != nullptr, &plan);
+}
+
+int score_head_tc_terms(const ScoreArgs& a, int n1) {
+  ScoreHeadPlan plan;
+  return score_head_plan(a.ell, a.d, n1, a.cand_ids != nullptr, &plan) ? plan.terms : 0;
 }
 
 template <int ELL, bool GATHER>
 static lime_status launch_score_head_tc_t(const ScoreArgs& a, const ScoreHeadArgs& h, int* err, cudaStream_t st) {
-  int S, lb;
-  size_t smem;
-  if (!score_head_plan(ELL, a.d, h.n1, &S, &lb, &smem)) return LIME_UNSUPPORTED_SHAPE;
+  ScoreHeadPlan plan;
+  if (!score_head_plan(ELL, a.d, h.n1, GATHER, &plan)) return LIME_UNSUPPORTED_SHAPE;
+  const uint64_t lsw_cols = (uint64_t)ELL * plan.terms;
   constexpr int WK = ELL > 64 ? 64 : ELL;
   CUtensorMap tmT, tmW, tmLSW, tmW1b;
   const uint64_t rows = (uint64_t)(GATHER ? a.corpus_rows : a.total);
   const uint32_t box = GATHER ? 1 : SH_TILE;
   if (!make_tmap_bf16_sw128(&tmT, a.T, rows, (uint64_t)a.d, (uint64_t)a.d, box) ||
       !make_tmap_bf16_kmajor(&tmW, a.W, rows, ELL, ELL, box, WK) ||
-      !make_tmap_bf16_kmajor(&tmLSW, h.LSWt, (uint64_t)a.B * h.n1, ELL, ELL, (uint32_t)h.n1, WK) ||
+      !make_tmap_bf16_kmajor(&tmLSW, h.LSWt, (uint64_t)a.B * h.n1, lsw_cols, lsw_cols, (uint32_t)h.n1, WK) ||
       !make_tmap_bf16_sw128(&tmW1b, h.W1bT, (uint64_t)h.n1, (uint64_t)a.d, (uint64_t)a.d, (uint32_t)h.n1))
     return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
   ScoreHeadParams p;
@@ -306,13 +319,13 @@ static lime_status launch_score_head_tc_t(const ScoreArgs& a, const ScoreHeadArg
   p.logits = a.logits; p.b1 = h.b1; p.w2 = h.w2; p.b2 = h.b2; p.B = a.B; p.C = a.C; p.d = a.d; p.n1 = h.n1;
   p.tiles_per_user = (a.C + SH_TILE - 1) / SH_TILE;
   p.n_tiles = p.tiles_per_user * a.B;
-  p.stages = S; p.lsw_bufs = lb; p.err = err;
+  p.stages = plan.stages; p.lsw_bufs = plan.lsw_bufs; p.terms = plan.terms; p.err = err;
   const int grid = p.n_tiles < kSMs ? p.n_tiles : kSMs;
   static bool smem_set[kMaxDeviceOrdinals] = {};
   const lime_status es = ensure_dynamic_smem((const void*)k_score_head_tc<ELL, GATHER>, 227 * 1024, smem_set);      // `smem` differs by d
   if (es != LIME_OK) return es;
   ProfScope _p("k_score_head_tc", st);
-  launch_pdl(k_score_head_tc<ELL, GATHER>, dim3(grid), dim3(SH_THREADS), smem, st, tmT, tmW, tmLSW, tmW1b, p);
+  launch_pdl(k_score_head_tc<ELL, GATHER>, dim3(grid), dim3(SH_THREADS), plan.smem, st, tmT, tmW, tmLSW, tmW1b, p);
   LIME_LAUNCH_CHECK("k_score_head_tc");
   return LIME_OK;
 }

@@ -874,8 +874,8 @@ lime_status lime_set_context_mlp(lime_ctx* ctx, int32_t d_c, const lime_ffn* mlp
   c->have_ctx_mlp = false;
   LIME_CUDA(cudaMalloc(&c->ctx_first, sizeof(float) * (size_t)g.ell * w0));
   // weights-only part of the first layer: (L W_0[:d]) + b_0
-  lime_status s = launch_rows_times_w(c->w.links, g.dtype, g.ell, g.d, mlp->W[0], g.dtype, w0, w0, mlp->b[0], c->ctx_first, nullptr,
-                                      1, "k_ctx_first", static_cast<cudaStream_t>(stream));
+  lime_status s = launch_rows_times_w(c->w.links, g.dtype, g.ell, g.d, mlp->W[0], g.dtype, w0, w0, mlp->b[0], c->ctx_first,
+                                      "k_ctx_first", static_cast<cudaStream_t>(stream));
   if (s != LIME_OK) return s;
   c->ctx_mlp = *mlp;
   c->ctx_dc = d_c;
@@ -950,27 +950,24 @@ lime_status lime_score_candidates_head(lime_ctx* ctx, const void* link_states, i
   char* base = reinterpret_cast<char*>(align_up(reinterpret_cast<uintptr_t>(ws)));
   const size_t n = (size_t)B * c->ell_c * w0;
   if ((size_t)(base - static_cast<char*>(ws)) + align_up(n * 4) + align_up(n * 2) > ws_bytes) return LIME_WORKSPACE_TOO_SMALL;
-  float* LSW = reinterpret_cast<float*>(base);
-  void* LSWt = base + align_up(n * 4);
+  float* LSW = reinterpret_cast<float*>(base);       // [B][ell][w0], or its bf16 pieces (three at most: the same 6 n bytes)
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ScoreArgs a{};
   a.LS = link_states; a.W = cand_w; a.T = cand_emb; a.dtype = g.dtype; a.B = B; a.ell = c->ell_c; a.d = g.d;
   a.cand_off = cand_off; a.C = C; a.total = total_cands; a.cand_ids = cand_ids; a.logits = logits;
   a.corpus_rows = cand_ids ? corpus_rows : 0; a.dev_flag = cand_ids ? dev_flag : nullptr;
   if (score_mlp3_supported(a, f)) return launch_score_mlp3(a, f, st);
-  const bool tc = f.n_hidden == 1 && c->head_W1bT && score_head_tc_supported(a, w0);
   // per user: LSW_b = LS_b W_0[:d]  (the O half of the first layer applied to the link states, so O is never formed)
   lime_status s;
-  if (tc && c->head_W1aT && g.d % 64 == 0)      // on tensor cores when the scorer is (link states and W_0 are bf16)
-    s = launch_gemm_rows_t(link_states, (int64_t)B * c->ell_c, g.d, c->head_W1aT, w0, c->ell_c, LSWt, c->dev_err, "k_gemm_tc_lsw", st);
-  else
-    s = launch_rows_times_w(link_states, g.dtype, (int64_t)B * c->ell_c, g.d, f.W[0], g.dtype, w0, w0, nullptr,
-                            tc ? nullptr : LSW, tc ? LSWt : nullptr, c->ell_c, "k_head_lsw", st);
-  if (s != LIME_OK) return s;
-  if (tc) {
-    ScoreHeadArgs h{LSWt, c->head_W1bT, f.b[0], c->head_w2, f.b[1], w0};
+  if (f.n_hidden == 1 && c->head_W1bT && score_head_tc_supported(a, w0)) {
+    s = launch_gemm_rows_t(link_states, (int64_t)B * c->ell_c, g.d, c->head_W1aT, w0, c->ell_c, score_head_tc_terms(a, w0), base, c->dev_err,
+                           "k_gemm_tc_lsw", st);
+    if (s != LIME_OK) return s;
+    ScoreHeadArgs h{base, c->head_W1bT, f.b[0], c->head_w2, f.b[1], w0};
     return launch_score_head_tc(a, h, c->dev_err, st);
   }
+  s = launch_rows_times_w(link_states, g.dtype, (int64_t)B * c->ell_c, g.d, f.W[0], g.dtype, w0, w0, nullptr, LSW, "k_head_lsw", st);
+  if (s != LIME_OK) return s;
   const char* W0t = static_cast<const char*>(f.W[0]) + (size_t)g.d * w0 * elem_size(g.dtype);
   return launch_score_head_simt(a, LSW, W0t, f.b[0], w0, ffn_tail(f, 1), st);
 }

@@ -276,9 +276,9 @@ struct FfnArgs {
   const void* W[LIME_FFN_MAX_HIDDEN + 1];
   const float* b[LIME_FFN_MAX_HIDDEN + 1];
 };
-// Y = X . W (+ bias) for a few rows: fp32 [M x N] and / or bf16 transposed per group of rows [M/group][N][group]
+// Y = X . W (+ bias) for a few rows: fp32 [M x N]
 lime_status launch_rows_times_w(const void* X, int x_dtype, int64_t M, int K, const void* W, int w_dtype, int ldw, int N,
-                                const float* bias, float* Y, void* Yt, int group, const char* name, cudaStream_t st);
+                                const float* bias, float* Y, const char* name, cudaStream_t st);
 lime_status launch_link_ctx_mlp(int dtype, const float* first, const void* user_ctx, int d_c, const void* W0c, int w0, int B,
                                 int ell, const FfnArgs& f, float* out, cudaStream_t st);
 // the same with one hidden layer on tensor cores (k_link_ctx_mma.cu)
@@ -293,6 +293,7 @@ struct ScoreHeadArgs {
   const void* LSWt; const void* W1bT; const float* b1; const float* w2; const float* b2; int n1;
 };
 bool score_head_tc_supported(const ScoreArgs& a, int n1);
+int score_head_tc_terms(const ScoreArgs& a, int n1);      // bf16 pieces per value of LSWt [B][n1][terms][ell]
 lime_status launch_score_head_tc(const ScoreArgs& a, const ScoreHeadArgs& h, int* err, cudaStream_t st);
 
 // three hidden layers (w0 <= 512, 128, 64) at d = 32, any candidate form (k_score_mlp3.cu)
@@ -319,9 +320,9 @@ struct LinkGemmArgs {
   int* err;
 };
 lime_status launch_gemm_prep(const LinkGemmArgs& a, cudaStream_t st);
-// A [M x K] . Bt^T, Bt [n_cols x K] (bf16, K % 64 == 0, 16-byte aligned): bf16 result transposed per group of rows,
-// out_t [M / group][n_cols][group]
-lime_status launch_gemm_rows_t(const void* A, int64_t M, int K, const void* Bt, int n_cols, int group, void* out_t, int* err,
+// A [M x K] . Bt^T, Bt [n_cols x K] (bf16, K % 64 == 0, 16-byte aligned): `terms` bf16 pieces per value, transposed per group
+// of rows: out_t [M / group][n_cols][terms][group]
+lime_status launch_gemm_rows_t(const void* A, int64_t M, int K, const void* Bt, int n_cols, int group, int terms, void* out_t, int* err,
                                const char* name, cudaStream_t st);
 
 // GatedMLP on link rows fused with its consumers (k_link_mlp_tc.cu); d = d_ff in {128, 256}

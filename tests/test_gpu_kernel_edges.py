@@ -277,3 +277,26 @@ def test_three_layer_interaction_network_keeps_its_hidden_layers(ell, w0):
     W64, T64, LS64 = (synth.storage_to_f64(x, dtype) for x in (W, T, LS))
     want = np.concatenate([O.score_candidates_head(W64[b * C:(b + 1) * C], LS64[b], T64[b * C:(b + 1) * C], L64) for b in range(B)])
     assert np.linalg.norm(got - want) <= 3 * 2.0 ** -16 * np.linalg.norm(want), np.linalg.norm(got - want) / np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("d,ell,n1", [(256, 32, 96), (64, 128, 16), (128, 64, 224)])
+def test_interaction_head_by_id_is_as_exact_as_by_list(d, ell, n1):
+    """A fixed number of ids per user (tensor cores) and the same ids as lists (fp32 on CUDA cores) are the same candidates: the
+    per-user product enters as three bf16 pieces, or as two where three do not fit (the last shape), 2^-17 of each term."""
+    Bd = _lib()
+    dtype, B, C, V = synth.BF16, 3, 200, 300
+    r = np.random.default_rng(d + n1)
+    LS, W, T = (synth.to_storage(x, dtype) for x in (r.normal(size=(B, ell, d)), O.softmax_rows(r.normal(size=(V, ell))), r.normal(size=(V, d))))
+    lime = Bd.Lime(d, 4, ell, 1, dtype=Bd.LIME_BF16)
+    layers = synth.ffn_weights(5, "head", (2 * d, n1, 1), dtype)
+    lime.set_head([(Bd.to_device(w, dtype), torch.from_numpy(b).cuda()) for w, b in layers])
+    ids = r.integers(0, V, size=B * C).astype(np.int32)
+    on_device = [Bd.to_device(x, dtype) for x in (LS, W, T)]
+    got = [Hh.to_f64(lime.score_candidates_head(*on_device, cand_ids=torch.from_numpy(ids).cuda(), **form))
+           for form in (dict(C=C), dict(C=0, total_cands=B * C, cand_off=torch.arange(0, B * C + 1, C, dtype=torch.int32, device="cuda")))]
+    Bd.lime_device_status(lime.ctx)
+    L64 = [(synth.storage_to_f64(w, dtype), b.astype(np.float64)) for w, b in layers]
+    W64, T64, LS64 = (synth.storage_to_f64(x, dtype) for x in (W, T, LS))
+    want = np.concatenate([O.score_candidates_head(W64[ids[b * C:(b + 1) * C]], LS64[b], T64[ids[b * C:(b + 1) * C]], L64) for b in range(B)])
+    for x in got:
+        assert np.linalg.norm(x - want) <= 2.0 ** -16 * np.linalg.norm(want), np.linalg.norm(x - want) / np.linalg.norm(want)
