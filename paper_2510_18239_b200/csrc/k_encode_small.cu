@@ -15,7 +15,7 @@
 // bf16 remainder (two products, fp32-level accuracy; the weights are exact as they are stored).  Rounded once instead, they
 // alone would double the error of the link states (1.1 against 0.5 % of their norm).
 // A layer's six weights (12 KB) come in by cp.async a layer ahead.  Histories beyond the shared-memory capacity stay in
-// global memory (`scratch`), 16 rows of it at a time in a patch per warp.
+// global memory (`scratch`), 16 rows of it at a time in a patch per warp; the longest of a batch take a cluster of blocks each.
 // Rows of 64 bytes sit at pitch 64 with 16-byte chunk c at c ^ ((row >> 1) & 3): 16-byte reads of whole rows and ldmatrix
 // reads of one chunk of eight rows are both free of bank conflicts.  Where both operands are read as whole rows the
 // contraction over the 32 features is permuted so that thread t of a quad holds features 8 t .. 8 t + 7 (one 16-byte read
@@ -26,6 +26,13 @@
 namespace lime {
 
 constexpr int ES_D = 32, ES_WARPS = 8, ES_THREADS = ES_WARPS * 32;
+constexpr int ES_CAP = 1024;     // history rows a block keeps in shared memory
+// Histories over 2048 tokens are shared out over a cluster of eight blocks, in a launch of their own, at most fifteen of them (the
+// clusters that run at once; the line doubles until that holds).  One user of n tokens among 99 of 100, three layers, one block /
+// a cluster / the generic kernels, which split by token: n = 2000 183 / 84 / 776 us, 8000 701 / 127 / 925, 32000 2776 / 401 / 1592,
+// 150000 12971 / 1619 / 3860.  With 32 users of 2000 a block each is the better (184 against 214 us): what a layer's exchange
+// costs a cluster (about 14 us) wants a long history.
+constexpr int ES_LONG = 2048, ES_CLUSTER = 8, ES_CLUSTERS = 15;
 
 template <int H_, int ELL_>
 struct EsCfg {
@@ -57,6 +64,7 @@ struct EncodeSmallParams {
   const __nv_bfloat16* w[LIME_MAX_LAYERS][6];                   // W_Q, W_K, W_V (NULL: identity), W_g, W_u, W_o, as stored
   __nv_bfloat16* scratch;                                       // [total x d]
   __nv_bfloat16* link_states; float* lp;                        // exactly one is wanted
+  int B, clustered, skip_long;                                  // clustered: cluster k takes the k-th long user, else block b user b
   int n_layers, cap, ln, hist_ln, silu;                         // cap: history rows shared memory holds
   float eps, scale;                                             // scale of the scores (times log2 e with the softmax)
 };
@@ -138,19 +146,33 @@ __device__ __forceinline__ void es_ln(float (&c)[4][4], int i, float eps) {
   for (int n = 0; n < 4; ++n) { c[n][i] *= rstd; c[n][i + 1] *= rstd; }
 }
 
+// all blocks of the cluster, or the one block of a user that has no cluster
+__device__ __forceinline__ void es_sync(bool clustered) {
+  if (clustered) cluster_sync_all();
+  else __syncthreads();
+}
+
 template <class G>
 __global__ void __launch_bounds__(ES_THREADS)
 k_encode_small(const EncodeSmallParams p) {
   constexpr int H = G::H, ELL = G::ELL, HL = G::HL, LMT = G::LMT, MT = G::MT, TG = G::TG;
   extern __shared__ __align__(128) uint8_t sm[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-  const int b = blockIdx.x;
   uint8_t* const X = sm + G::OFF_X;
   uint8_t* const patch = sm + G::OFF_PATCH + warp * 1024;
   int* const next_tile = reinterpret_cast<int*>(sm + G::OFF_NEXT);
   pdl_launch_dependents();
   pdl_wait();
-  const int tok0 = p.off[b], n = p.off[b + 1] - tok0;
+  // a long user belongs to a cluster of blocks, each with a share of the history; the link rows are done by every block of it, from
+  // the shares' accumulators
+  const bool clustered = p.clustered != 0;
+  const int rank = clustered ? (int)blockIdx.x % ES_CLUSTER : 0, CL = clustered ? ES_CLUSTER : 1;
+  const int b = clustered ? nth_long_user(p.off, p.B, ES_LONG, ES_CLUSTERS, (int)blockIdx.x / ES_CLUSTER, next_tile) : (int)blockIdx.x;
+  if (b < 0) return;
+  const int user0 = p.off[b], user_n = p.off[b + 1] - user0;
+  if (p.skip_long && user_n > ES_LONG && user_n > long_user_line(p.off, p.B, ES_LONG, ES_CLUSTERS, next_tile)) return;
+  const int share = ((user_n + CL - 1) / CL + 15) & ~15, first = min(user_n, rank * share);
+  const int tok0 = user0 + first, n = min(user_n, first + share) - first;
   const bool resident = n <= p.cap;
   const int n_tiles = (n + 15) >> 4;
 
@@ -378,27 +400,41 @@ k_encode_small(const EncodeSmallParams p) {
         pm[0] = mx0; pm[8] = mx1; ps[0] = l0; ps[8] = l1;
       }
     }
-    __syncthreads();
+    es_sync(clustered);
     // ---- merge the shares, normalise: Ohat[l, h * 32 + i]
     for (int i = tid; i < HL * 4; i += ES_THREADS) {
       const int r = i >> 2, c = i & 3, h = r / ELL, l = r % ELL;
-      const float* pm = reinterpret_cast<const float*>(sm + G::OFF_PM) + r;
-      const float* ps = reinterpret_cast<const float*>(sm + G::OFF_PS) + r;
       float M = -INFINITY, S = 0.f, acc[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) acc[k] = 0.f;
+      auto highest = [&](const uint8_t* at) {
+        const float* pm = reinterpret_cast<const float*>(at + G::OFF_PM) + r;
 #pragma unroll
-      for (int s = 0; s < TG; ++s) M = fmaxf(M, pm[s * HL]);
+        for (int s = 0; s < TG; ++s) M = fmaxf(M, pm[s * HL]);
+      };
+      auto add = [&](const uint8_t* at) {
+        const float* pm = reinterpret_cast<const float*>(at + G::OFF_PM) + r;
+        const float* ps = reinterpret_cast<const float*>(at + G::OFF_PS) + r;
 #pragma unroll
-      for (int s = 0; s < TG; ++s) {
-        const float w = p.silu ? 1.f : (M == -INFINITY ? 0.f : es_ex2(pm[s * HL] - M));
-        S = fmaf(w, ps[s * HL], S);
-        const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(sm + G::OFF_PART) + (s * HL + r) * G::PART_LD + c * 8);
-        const float4 x = src[0], y = src[1];
-        acc[0] = fmaf(w, x.x, acc[0]); acc[1] = fmaf(w, x.y, acc[1]); acc[2] = fmaf(w, x.z, acc[2]); acc[3] = fmaf(w, x.w, acc[3]);
-        acc[4] = fmaf(w, y.x, acc[4]); acc[5] = fmaf(w, y.y, acc[5]); acc[6] = fmaf(w, y.z, acc[6]); acc[7] = fmaf(w, y.w, acc[7]);
+        for (int s = 0; s < TG; ++s) {
+          const float w = p.silu ? 1.f : (M == -INFINITY ? 0.f : es_ex2(pm[s * HL] - M));
+          S = fmaf(w, ps[s * HL], S);
+          const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(at + G::OFF_PART) + (s * HL + r) * G::PART_LD + c * 8);
+          const float4 x = src[0], y = src[1];
+          acc[0] = fmaf(w, x.x, acc[0]); acc[1] = fmaf(w, x.y, acc[1]); acc[2] = fmaf(w, x.z, acc[2]); acc[3] = fmaf(w, x.w, acc[3]);
+          acc[4] = fmaf(w, y.x, acc[4]); acc[5] = fmaf(w, y.y, acc[5]); acc[6] = fmaf(w, y.z, acc[6]); acc[7] = fmaf(w, y.w, acc[7]);
+        }
+      };
+      if (!clustered) {
+        highest(sm);
+        add(sm);
+      } else {
+#pragma unroll
+        for (int q = 0; q < ES_CLUSTER; ++q) highest(cluster_peer(static_cast<const uint8_t*>(sm), q));
+#pragma unroll 4
+        for (int q = 0; q < ES_CLUSTER; ++q) add(cluster_peer(static_cast<const uint8_t*>(sm), q));
       }
-      const float inv = n > 0 ? 1.0f / (p.silu ? (float)n : S) : 0.f;
+      const float inv = user_n > 0 ? 1.0f / (p.silu ? (float)user_n : S) : 0.f;
       uint32_t hi[4], lo[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) es_split(acc[2 * k] * inv, acc[2 * k + 1] * inv, hi[k], lo[k]);
@@ -406,7 +442,7 @@ k_encode_small(const EncodeSmallParams p) {
       *reinterpret_cast<uint4*>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
       *reinterpret_cast<uint4*>(dst + G::LROWS * H * 64) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
     }
-    __syncthreads();
+    es_sync(clustered);                                         // (of a cluster: the peers have read this block's accumulators)
     // ---- GatedMLP on the link rows: warps 0..3 take eight columns each of O and of the hidden layer, warps 0 .. LMT - 1 the
     // rows of T
     if (warp < 4) {
@@ -591,7 +627,7 @@ k_encode_small(const EncodeSmallParams p) {
     }
   }
   // L^P, as the link states (or for the projection that follows)
-  if (warp < LMT) {
+  if (warp < LMT && rank == 0) {
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -620,13 +656,36 @@ static lime_status launch_es(const EncodeSmallArgs& a, cudaStream_t st) {
   }
   p.scratch = (__nv_bfloat16*)a.scratch; p.link_states = (__nv_bfloat16*)a.link_states; p.lp = a.lp;
   p.n_layers = a.n_layers; p.ln = a.ln; p.hist_ln = a.hist_ln; p.silu = a.silu; p.eps = a.eps; p.scale = a.silu ? 1.0f : a.scale * 1.4426950408889634f;
-  // rows in shared memory: up to 1024 (64 KB) - the host knows the total only, and two blocks an SM matter more than
-  // keeping the rare longer history on chip
-  p.cap = (int)(a.total < 1024 ? a.total : 1024);
+  p.B = a.B; p.skip_long = 0;
+  p.cap = (int)(a.total < ES_CAP ? a.total : ES_CAP);
   const int smem = G::OFF_X + ((p.cap + 15) & ~15) * 64;
   static bool smem_set[kMaxDeviceOrdinals] = {};
-  lime_status s = ensure_dynamic_smem((const void*)k_encode_small<G>, G::OFF_X + 1024 * 64, smem_set);
+  lime_status s = ensure_dynamic_smem((const void*)k_encode_small<G>, G::OFF_X + ES_CAP * 64, smem_set);
   if (s != LIME_OK) return s;
+  // as many clusters as the total allows long users, which find theirs or leave; no launch where it allows none
+  int64_t longs = a.total / (ES_LONG + 1);
+  if (longs > a.B) longs = a.B;
+  if (longs > ES_CLUSTERS) longs = ES_CLUSTERS;
+  if (longs > 0) {
+    p.clustered = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)longs * ES_CLUSTER);
+    cfg.blockDim = dim3(ES_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = ES_CLUSTER; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    ProfScope _p("k_encode_small", st);
+    cudaLaunchKernelEx(&cfg, k_encode_small<G>, p);
+    LIME_LAUNCH_CHECK("k_encode_small");
+  }
+  p.clustered = 0;
+  p.skip_long = longs > 0;
   ProfScope _p("k_encode_small", st);
   launch_pdl(k_encode_small<G>, dim3((unsigned)a.B), dim3(ES_THREADS), (size_t)smem, st, p);
   LIME_LAUNCH_CHECK("k_encode_small");

@@ -44,6 +44,54 @@ __device__ __forceinline__ int upper_user(const int32_t* __restrict__ start, int
   return lo;
 }
 
+// Which users get a cluster of blocks each: those of more than `base` tokens, the line doubling until at most `most` are left.  The
+// host knows the total length only, so the blocks find the line.  Every thread of the block calls these; `word` is a word of its
+// shared memory (a static one would not fit beside all of it taken dynamically).
+__device__ __forceinline__ int long_user_line(const int32_t* __restrict__ off, int B, int base, int most, int* word) {
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 32) {
+    int line = base;
+    for (;; line *= 2) {
+      int n = 0;
+      for (int b = lane; b < B; b += 32) n += off[b + 1] - off[b] > line;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+      if (n <= most || line > (1 << 29)) break;
+    }
+    if (lane == 0) *word = line;
+  }
+  __syncthreads();
+  const int line = *word;
+  __syncthreads();
+  return line;
+}
+// the k-th of those users (from 0); -1: there are not that many
+__device__ __forceinline__ int nth_long_user(const int32_t* __restrict__ off, int B, int base, int most, int k, int* word) {
+  const int line = long_user_line(off, B, base, most, word), lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) *word = -1;
+  __syncthreads();
+  if (threadIdx.x < 32)
+    for (int b0 = 0; b0 < B && k >= 0; b0 += 32) {
+      const int b = min(b0 + lane, B - 1);
+      const unsigned m = __ballot_sync(0xffffffffu, b0 + lane < B && off[b + 1] - off[b] > line);
+      if (((m >> lane) & 1u) && __popc(m & ((1u << lane) - 1u)) == k) *word = b;
+      k -= __popc(m);
+    }
+  __syncthreads();
+  return *word;
+}
+// barrier of all threads of a cluster; what they wrote before it is visible behind it, to the cluster
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the same shared-memory address in block `rank` of the cluster, as a generic pointer
+template <typename T>
+__device__ __forceinline__ const T* cluster_peer(const T* p, int rank) {
+  uint64_t r;
+  asm volatile("mapa.u64 %0, %1, %2;" : "=l"(r) : "l"((uint64_t)p), "r"(rank));
+  return reinterpret_cast<const T*>(r);
+}
+
 // ----------------------------------------------------------------------------- context
 struct Ctx {
   lime_config cfg;

@@ -300,3 +300,42 @@ def test_interaction_head_by_id_is_as_exact_as_by_list(d, ell, n1):
     want = np.concatenate([O.score_candidates_head(W64[ids[b * C:(b + 1) * C]], LS64[b], T64[ids[b * C:(b + 1) * C]], L64) for b in range(B)])
     for x in got:
         assert np.linalg.norm(x - want) <= 2.0 ** -16 * np.linalg.norm(want), np.linalg.norm(x - want) / np.linalg.norm(want)
+
+
+# SiLU weights are not normalised: stacked layers grow and with them the error of the stored rows
+@pytest.mark.parametrize("H,ell", [(4, 16), (2, 8), (4, 32)])
+@pytest.mark.parametrize("lengths", [[2049, 20], [15, 2048, 0, 2049, 20, 2500] + [30] * 5, [9000] + [40] * 9, [2100] * 16 + [0] * 20 + [4200]])
+@pytest.mark.parametrize("phi,raw,per_user", [("softmax", False, True), ("silu", False, False)])
+def test_narrow_encode_of_long_histories(H, ell, lengths, phi, raw, per_user):
+    """d = 32: users of more than 2048 tokens take a cluster of eight blocks, the others one; shares in shared memory and not; more
+    such users than clusters, so that the line doubles."""
+    _encode_against_oracle(synth.BF16, 32, H, ell, 3, lengths, phi, raw, per_user, 6e-2, 4e-2 if phi == "silu" else 1.5e-2)
+
+
+@pytest.mark.parametrize("dtype,d,H,ell", [(synth.BF16, 32, 4, 16)])
+def test_one_long_history_among_short_ones_is_split(dtype, d, H, ell):
+    """One user with 20,000 tokens among 399 with 50, against 400 users of 99 or 100 (the same rows): the long one must not be left to
+    one block (26 times the time of the even batch where it was, 4.4 times on a cluster)."""
+    Bd = _lib()
+    dt = Bd.LIME_F32 if dtype == synth.F32 else Bd.LIME_BF16
+    lime = Bd.Lime(d, H, ell, 2, dtype=dt)
+    g = torch.Generator("cuda").manual_seed(1)
+    td = torch.float32 if dtype == synth.F32 else torch.bfloat16
+    rand = lambda *shape, std: (torch.randn(shape, generator=g, device="cuda") * std).to(td)
+    weights = [{k: rand(d, d, std=d ** -0.5) for k in ("Wq", "Wk", "Wv", "Wg", "Wu", "Wo")} for _ in range(2)]
+    links, hist = rand(ell, d, std=1.0), rand(20000 + 399 * 50, d, std=1.0)
+    lime.set_weights(links, weights)
+
+    def best(lengths):
+        off = lime.lengths_to_offsets(torch.tensor(lengths, dtype=torch.int32, device="cuda"))
+        times = []
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            lime.encode_user_normalized(hist, off)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        return min(times)
+    skewed, even = best([20000] + [50] * 399), best([100] * 350 + [99] * 50)
+    assert skewed <= 15 * even, (skewed, even)
