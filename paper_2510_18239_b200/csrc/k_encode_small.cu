@@ -13,7 +13,12 @@
 //   rows   P = softmax_h(X . K2^T), U = SiLU(P G2) * (P U2), X <- LN(U W_o)   the other warps at once, then all; 16 rows at a time
 // The link rows are few and everything depends on them, so their activations enter each product as a bf16 value and its
 // bf16 remainder (two products, fp32-level accuracy; the weights are exact as they are stored).  Rounded once instead, they
-// alone would double the error of the link states (1.1 against 0.5 % of their norm).
+// alone would double the error of the link states (1.1 against 0.5 % of their norm).  Two more splits hold the error at that of the
+// generic kernels, which keep link rows, probabilities and the first layer's LayerNorm in fp32 and round the history's K, V, Q, O, U:
+// with SiLU, whose probabilities are not normalised, Q2, K2 and the probabilities; with rows that arrive raw, the normalised rows of
+// the first layer.  Error of the link states against fp64, four heads of 16 links, three layers, 64 users of 10..256 tokens, rms over
+// them (generic kernels; rounded once): softmax 0.91 % (1.14), SiLU 1.4 (1.9; 2.1), raw rows softmax 0.55 (0.66; 0.91), raw rows SiLU
+// 0.91 (1.4; 2.1).
 // A layer's six weights (12 KB) come in by cp.async a layer ahead.  Histories beyond the shared-memory capacity stay in
 // global memory (`scratch`), 16 rows of it at a time in a patch per warp; the longest of a batch take a cluster of blocks each.
 // Rows of 64 bytes sit at pitch 64 with 16-byte chunk c at c ^ ((row >> 1) & 3): 16-byte reads of whole rows and ldmatrix
@@ -52,9 +57,10 @@ struct EsCfg {
   static constexpr int OFF_THAT = OFF_OHAT + 2 * LROWS * H * 64;
   static constexpr int OFF_O = OFF_THAT + 2 * LROWS * 64;
   static constexpr int OFF_U = OFF_O + 2 * LROWS * 64;
-  static constexpr int OFF_NEXT = OFF_U + 2 * LROWS * 64;      // tile counter
-  static constexpr int OFF_PATCH = OFF_NEXT + 16;              // [warps][16 x 64 bytes]
-  static constexpr int OFF_X = OFF_PATCH + ES_WARPS * 1024;
+  static constexpr int OFF_LO = OFF_U + 2 * LROWS * 64;        // SiLU: remainders of Q2, K2
+  static constexpr int OFF_NEXT = OFF_LO + 2 * HL * 64;        // tile counter
+  static constexpr int OFF_PATCH = OFF_NEXT + 16;              // [warps][16 x 64 bytes], the same for the remainders of raw rows
+  static constexpr int OFF_X = OFF_PATCH + 2 * ES_WARPS * 1024;
   static_assert(HL % 16 == 0 && MT <= ES_WARPS && ES_WARPS % MT == 0, "split of the stacked rows over the warps");
 };
 
@@ -65,7 +71,7 @@ struct EncodeSmallParams {
   __nv_bfloat16* scratch;                                       // [total x d]
   __nv_bfloat16* link_states; float* lp;                        // exactly one is wanted
   int B, clustered, skip_long;                                  // clustered: cluster k takes the k-th long user, else block b user b
-  int n_layers, cap, ln, hist_ln, silu;                         // cap: history rows shared memory holds
+  int n_layers, cap, ln;                                        // cap: history rows shared memory holds
   float eps, scale;                                             // scale of the scores (times log2 e with the softmax)
 };
 
@@ -97,6 +103,8 @@ __device__ __forceinline__ void es_split(float x, float y, uint32_t& hi, uint32_
   hi = es_pack(x, y);
   lo = es_pack(x - es_lo(hi), y - es_hi(hi));
 }
+// the remainders alone
+__device__ __forceinline__ uint32_t es_rest(float x, float y, uint32_t hi) { return es_pack(x - es_lo(hi), y - es_hi(hi)); }
 // both k-steps of a 32-feature contraction in the permuted order: rows g and g + 8 of A, one row of B
 __device__ __forceinline__ void es_mma32(float (&c)[4], const uint4& a, const uint4& a8, const uint4& b) {
   es_mma(c, a.x, a8.x, a.y, a8.y, b.x, b.y);
@@ -152,7 +160,8 @@ __device__ __forceinline__ void es_sync(bool clustered) {
   else __syncthreads();
 }
 
-template <class G>
+// RAW: the rows arrive without their LayerNorm, and the first layer takes the normalised ones as value and remainder
+template <class G, bool SILU, bool RAW>
 __global__ void __launch_bounds__(ES_THREADS)
 k_encode_small(const EncodeSmallParams p) {
   constexpr int H = G::H, ELL = G::ELL, HL = G::HL, LMT = G::LMT, MT = G::MT, TG = G::TG;
@@ -192,26 +201,34 @@ k_encode_small(const EncodeSmallParams p) {
   };
   load_weights(0);
 
-  // history rows -> shared memory (or, too long for it, -> scratch), LayerNorm-ed on the way where they arrive raw
-  {
+  // LayerNorm of a row that a quad holds eight features each of: packed values, and their remainders
+  auto ln_row = [&](const uint4& v, uint4& hi, uint4& lo) {
+    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+    float s = 0.f, q = 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s += es_lo(u[k]) + es_hi(u[k]);
+    const float mu = es_quad_sum(s) * (1.0f / ES_D);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) { const float x = es_lo(u[k]) - mu, y = es_hi(u[k]) - mu; q = fmaf(x, x, q); q = fmaf(y, y, q); }
+    const float rstd = rsqrtf(es_quad_sum(q) * (1.0f / ES_D) + p.eps);
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) es_split((es_lo(u[k]) - mu) * rstd, (es_hi(u[k]) - mu) * rstd, h[k], l[k]);
+    hi = make_uint4(h[0], h[1], h[2], h[3]);
+    lo = make_uint4(l[0], l[1], l[2], l[3]);
+  };
+  // history rows -> shared memory, or to scratch where they are too many (raw ones stay where they are until the first update)
+  uint8_t* const XL = X + ((p.cap + 15) & ~15) * 64;            // remainders of raw rows
+  if (!RAW || resident) {
     __nv_bfloat16* const big = p.scratch + (int64_t)tok0 * ES_D;
     for (int i = tid; i < n_tiles * 64; i += ES_THREADS) {
       const int row = i >> 2, c = i & 3;
-      uint4 v = make_uint4(0, 0, 0, 0);
+      uint4 v = make_uint4(0, 0, 0, 0), rest = v;
       if (row < n) v = __ldg(reinterpret_cast<const uint4*>(p.hist + (int64_t)(tok0 + row) * ES_D) + c);
-      if (p.hist_ln) {
-        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-        float s = 0.f, q = 0.f;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) s += es_lo(u[k]) + es_hi(u[k]);
-        const float mu = es_quad_sum(s) * (1.0f / ES_D);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) { const float x = es_lo(u[k]) - mu, y = es_hi(u[k]) - mu; q = fmaf(x, x, q); q = fmaf(y, y, q); }
-        const float rstd = rsqrtf(es_quad_sum(q) * (1.0f / ES_D) + p.eps);
-        uint32_t o[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) o[k] = es_pack((es_lo(u[k]) - mu) * rstd, (es_hi(u[k]) - mu) * rstd);
-        if (row < n) v = make_uint4(o[0], o[1], o[2], o[3]);
+      if constexpr (RAW) {
+        ln_row(v, v, rest);
+        if (row >= n) v = rest = make_uint4(0, 0, 0, 0);
+        *reinterpret_cast<uint4*>(XL + es_sw(row, c)) = rest;
       }
       if (resident) *reinterpret_cast<uint4*>(X + es_sw(row, c)) = v;
       else if (row < n) *(reinterpret_cast<uint4*>(big + (int64_t)row * ES_D) + c) = v;
@@ -234,21 +251,35 @@ k_encode_small(const EncodeSmallParams p) {
       *reinterpret_cast<__nv_bfloat16*>(dst + G::LROWS * 64) = __float2bfloat16_rn(x - __bfloat162float(hi));
     }
   }
-  // 16 rows of the history as a swizzled tile in shared memory
-  auto tile = [&](int r0) -> uint8_t* {
+  // 16 rows of the history as a swizzled tile in shared memory; of raw rows (`first`) the remainders lie at rest(tile)
+  auto tile = [&](int r0, bool first) -> uint8_t* {
     if (resident) return X + r0 * 64;
-    const __nv_bfloat16* src = p.scratch + (int64_t)(tok0 + r0) * ES_D;
-    const int row = lane >> 1;
+    const __nv_bfloat16* src = (first ? p.hist : p.scratch) + (int64_t)(tok0 + r0) * ES_D;
     __syncwarp();
+    if (first) {
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int c = (lane & 1) * 2 + k;
-      const uint4 v = r0 + row < n ? *(reinterpret_cast<const uint4*>(src + row * ES_D) + c) : make_uint4(0, 0, 0, 0);
-      *reinterpret_cast<uint4*>(patch + es_sw(row, c)) = v;
+      for (int k = 0; k < 2; ++k) {                             // four lanes a row
+        const int row = k * 8 + g;
+        uint4 v = make_uint4(0, 0, 0, 0), rest;
+        if (r0 + row < n) v = __ldg(reinterpret_cast<const uint4*>(src + row * ES_D) + t);
+        ln_row(v, v, rest);
+        if (r0 + row >= n) v = rest = make_uint4(0, 0, 0, 0);
+        *reinterpret_cast<uint4*>(patch + es_sw(row, t)) = v;
+        *reinterpret_cast<uint4*>(patch + ES_WARPS * 1024 + es_sw(row, t)) = rest;
+      }
+    } else {
+      const int row = lane >> 1;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int c = (lane & 1) * 2 + k;
+        const uint4 v = r0 + row < n ? *(reinterpret_cast<const uint4*>(src + row * ES_D) + c) : make_uint4(0, 0, 0, 0);
+        *reinterpret_cast<uint4*>(patch + es_sw(row, c)) = v;
+      }
     }
     __syncwarp();
     return patch;
   };
+  auto rest = [&](uint8_t* xt) { return resident ? XL + (xt - X) : xt + ES_WARPS * 1024; };
 
   float lp[4][4];                                              // running sum of T (warps 0 .. LMT - 1)
 #pragma unroll
@@ -257,7 +288,7 @@ k_encode_small(const EncodeSmallParams p) {
     for (int e = 0; e < 4; ++e) lp[i][e] = 0.f;
 
   for (int j = 0; j < p.n_layers; ++j) {
-    const bool last = j + 1 == p.n_layers;
+    const bool last = j + 1 == p.n_layers, raw = RAW && j == 0;
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     const uint8_t* W = sm + G::OFF_W + (j & 1) * (6 * 2048);
@@ -320,12 +351,25 @@ k_encode_small(const EncodeSmallParams p) {
               }
             }
           }
-          uint8_t* dst = sm + G::OFF_OPS + op * (HL * 64);
           const int r = h * ELL + m * 16 + g;
+          auto store = [&](uint8_t* dst) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            *reinterpret_cast<uint32_t*>(dst + es_sw(r, i) + t * 4) = es_pack(d[i][0] * sc, d[i][1] * sc);
-            if (ELL > 8) *reinterpret_cast<uint32_t*>(dst + es_sw(r + 8, i) + t * 4) = es_pack(d[i][2] * sc, d[i][3] * sc);
+            for (int i = 0; i < 4; ++i) {
+              *reinterpret_cast<uint32_t*>(dst + es_sw(r, i) + t * 4) = es_pack(d[i][0], d[i][1]);
+              if (ELL > 8) *reinterpret_cast<uint32_t*>(dst + es_sw(r + 8, i) + t * 4) = es_pack(d[i][2], d[i][3]);
+            }
+          };
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) d[i][e] *= sc;
+          store(sm + G::OFF_OPS + op * (HL * 64));
+          if (SILU && op < 2) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) d[i][e] -= __bfloat162float(__float2bfloat16_rn(d[i][e]));
+            store(sm + G::OFF_LO + op * (HL * 64));
           }
         }
       }
@@ -336,22 +380,26 @@ k_encode_small(const EncodeSmallParams p) {
     {
       const int m = warp % MT, tg = warp / MT;
       const uint4 qa = es_lds(sm + G::OFF_OPS + es_sw(m * 16 + g, t)), qa8 = es_lds(sm + G::OFF_OPS + es_sw(m * 16 + g + 8, t));
+      uint4 ql = make_uint4(0, 0, 0, 0), ql8 = ql;
+      if (SILU) { ql = es_lds(sm + G::OFF_LO + es_sw(m * 16 + g, t)); ql8 = es_lds(sm + G::OFF_LO + es_sw(m * 16 + g + 8, t)); }
       float o[4][4], mx0 = -INFINITY, mx1 = -INFINITY, l0 = 0.f, l1 = 0.f;
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int e = 0; e < 4; ++e) o[i][e] = 0.f;
       for (int tt = tg; tt < n_tiles; tt += TG) {
-        const uint8_t* xt = tile(tt * 16);
+        uint8_t* const xt = tile(tt * 16, raw);
         float s[2][4];
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
 #pragma unroll
           for (int e = 0; e < 4; ++e) s[i][e] = 0.f;
           es_mma32(s[i], qa, qa8, es_lds(xt + es_sw(i * 8 + g, t)));
+          if (SILU) es_mma32(s[i], ql, ql8, es_lds(xt + es_sw(i * 8 + g, t)));
+          if (raw) es_mma32(s[i], qa, qa8, es_lds(rest(xt) + es_sw(i * 8 + g, t)));
         }
         const int left = n - tt * 16;                          // valid tokens of the tile
-        if (p.silu) {
+        if (SILU) {
 #pragma unroll
           for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -385,6 +433,16 @@ k_encode_small(const EncodeSmallParams p) {
           es_ldsm_t(r, es_addr(xt + es_sw((lane & 15), c0 + (lane >> 4))));
           es_mma(o[c0], a0, a1, a2, a3, r[0], r[1]);
           es_mma(o[c0 + 1], a0, a1, a2, a3, r[2], r[3]);
+          if (SILU) {
+            const uint32_t l0 = es_rest(s[0][0], s[0][1], a0), l1 = es_rest(s[0][2], s[0][3], a1), l2 = es_rest(s[1][0], s[1][1], a2), l3 = es_rest(s[1][2], s[1][3], a3);
+            es_mma(o[c0], l0, l1, l2, l3, r[0], r[1]);
+            es_mma(o[c0 + 1], l0, l1, l2, l3, r[2], r[3]);
+          }
+          if (raw) {
+            es_ldsm_t(r, es_addr(rest(xt) + es_sw((lane & 15), c0 + (lane >> 4))));
+            es_mma(o[c0], a0, a1, a2, a3, r[0], r[1]);
+            es_mma(o[c0 + 1], a0, a1, a2, a3, r[2], r[3]);
+          }
         }
       }
       float* part = reinterpret_cast<float*>(sm + G::OFF_PART) + (tg * HL + m * 16 + g) * G::PART_LD + 2 * t;
@@ -417,7 +475,7 @@ k_encode_small(const EncodeSmallParams p) {
         const float* ps = reinterpret_cast<const float*>(at + G::OFF_PS) + r;
 #pragma unroll
         for (int s = 0; s < TG; ++s) {
-          const float w = p.silu ? 1.f : (M == -INFINITY ? 0.f : es_ex2(pm[s * HL] - M));
+          const float w = SILU ? 1.f : (M == -INFINITY ? 0.f : es_ex2(pm[s * HL] - M));
           S = fmaf(w, ps[s * HL], S);
           const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(at + G::OFF_PART) + (s * HL + r) * G::PART_LD + c * 8);
           const float4 x = src[0], y = src[1];
@@ -434,7 +492,7 @@ k_encode_small(const EncodeSmallParams p) {
 #pragma unroll 4
         for (int q = 0; q < ES_CLUSTER; ++q) add(cluster_peer(static_cast<const uint8_t*>(sm), q));
       }
-      const float inv = user_n > 0 ? 1.0f / (p.silu ? (float)user_n : S) : 0.f;
+      const float inv = user_n > 0 ? 1.0f / (SILU ? (float)user_n : S) : 0.f;
       uint32_t hi[4], lo[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) es_split(acc[2 * k] * inv, acc[2 * k + 1] * inv, hi[k], lo[k]);
@@ -530,8 +588,10 @@ k_encode_small(const EncodeSmallParams p) {
       if (lane == 0) tt = atomicAdd(next_tile, 1);
       tt = __shfl_sync(0xffffffffu, tt, 0);
       if (tt >= n_tiles) break;
-      uint8_t* xt = tile(tt * 16);
+      uint8_t* const xt = tile(tt * 16, raw);
       const uint4 a = es_lds(xt + es_sw(g, t)), a8 = es_lds(xt + es_sw(g + 8, t));
+      uint4 ar = make_uint4(0, 0, 0, 0), ar8 = ar;
+      if (raw) { ar = es_lds(rest(xt) + es_sw(g, t)); ar8 = es_lds(rest(xt) + es_sw(g + 8, t)); }
       float gt[4][4], up[4][4];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
@@ -548,8 +608,10 @@ k_encode_small(const EncodeSmallParams p) {
 #pragma unroll
           for (int e = 0; e < 4; ++e) s[i][e] = 0.f;
           es_mma32(s[i], a, a8, es_lds(K2 + es_sw((q + i) * 8 + g, t)));
+          if (SILU) es_mma32(s[i], a, a8, es_lds(sm + G::OFF_LO + HL * 64 + es_sw((q + i) * 8 + g, t)));
+          if (raw) es_mma32(s[i], ar, ar8, es_lds(K2 + es_sw((q + i) * 8 + g, t)));
         }
-        if (p.silu) {
+        if (SILU) {
 #pragma unroll
           for (int i = 0; i < NTG; ++i)
 #pragma unroll
@@ -580,16 +642,22 @@ k_encode_small(const EncodeSmallParams p) {
           const uint32_t a0 = es_pack(s[2 * ks][0], s[2 * ks][1]), a1 = es_pack(s[2 * ks][2], s[2 * ks][3]);
           const uint32_t a2 = es_pack(s[2 * ks + 1][0], s[2 * ks + 1][1]), a3 = es_pack(s[2 * ks + 1][2], s[2 * ks + 1][3]);
           const int r = (q + 2 * ks) * 8 + (lane & 15);
+          auto mix = [&](uint32_t b0, uint32_t b1, uint32_t b2, uint32_t b3) {
 #pragma unroll
-          for (int c0 = 0; c0 < 4; c0 += 2) {
-            uint32_t w[4];
-            es_ldsm_t(w, es_addr(G2 + es_sw(r, c0 + (lane >> 4))));
-            es_mma(gt[c0], a0, a1, a2, a3, w[0], w[1]);
-            es_mma(gt[c0 + 1], a0, a1, a2, a3, w[2], w[3]);
-            es_ldsm_t(w, es_addr(G2 + HL * 64 + es_sw(r, c0 + (lane >> 4))));
-            es_mma(up[c0], a0, a1, a2, a3, w[0], w[1]);
-            es_mma(up[c0 + 1], a0, a1, a2, a3, w[2], w[3]);
-          }
+            for (int c0 = 0; c0 < 4; c0 += 2) {
+              uint32_t w[4];
+              es_ldsm_t(w, es_addr(G2 + es_sw(r, c0 + (lane >> 4))));
+              es_mma(gt[c0], b0, b1, b2, b3, w[0], w[1]);
+              es_mma(gt[c0 + 1], b0, b1, b2, b3, w[2], w[3]);
+              es_ldsm_t(w, es_addr(G2 + HL * 64 + es_sw(r, c0 + (lane >> 4))));
+              es_mma(up[c0], b0, b1, b2, b3, w[0], w[1]);
+              es_mma(up[c0 + 1], b0, b1, b2, b3, w[2], w[3]);
+            }
+          };
+          mix(a0, a1, a2, a3);
+          if (SILU)
+            mix(es_rest(s[2 * ks][0], s[2 * ks][1], a0), es_rest(s[2 * ks][2], s[2 * ks][3], a1), es_rest(s[2 * ks + 1][0], s[2 * ks + 1][1], a2),
+                es_rest(s[2 * ks + 1][2], s[2 * ks + 1][3], a3));
         }
       }
       uint32_t u[4][2];
@@ -646,8 +714,8 @@ bool encode_small_supported(int dtype, int d, int d_ff, int H, int ell, int gate
   return dtype == LIME_BF16 && d == ES_D && d_ff == ES_D && gated_mlp && es_shape(H, ell);
 }
 
-template <class G>
-static lime_status launch_es(const EncodeSmallArgs& a, cudaStream_t st) {
+template <class G, bool SILU, bool RAW>
+static lime_status launch_es_t(const EncodeSmallArgs& a, cudaStream_t st) {
   EncodeSmallParams p;
   p.hist = (const __nv_bfloat16*)a.hist; p.off = a.off; p.links = a.links; p.links_per_user = a.links_per_user;
   for (int j = 0; j < a.n_layers; ++j) {
@@ -655,12 +723,13 @@ static lime_status launch_es(const EncodeSmallArgs& a, cudaStream_t st) {
     for (int m = 0; m < 6; ++m) p.w[j][m] = (const __nv_bfloat16*)w[m];
   }
   p.scratch = (__nv_bfloat16*)a.scratch; p.link_states = (__nv_bfloat16*)a.link_states; p.lp = a.lp;
-  p.n_layers = a.n_layers; p.ln = a.ln; p.hist_ln = a.hist_ln; p.silu = a.silu; p.eps = a.eps; p.scale = a.silu ? 1.0f : a.scale * 1.4426950408889634f;
+  p.n_layers = a.n_layers; p.ln = a.ln; p.eps = a.eps; p.scale = SILU ? 1.0f : a.scale * 1.4426950408889634f;
   p.B = a.B; p.skip_long = 0;
-  p.cap = (int)(a.total < ES_CAP ? a.total : ES_CAP);
-  const int smem = G::OFF_X + ((p.cap + 15) & ~15) * 64;
+  constexpr int row_bytes = RAW ? 128 : 64, most = (232448 - G::OFF_X) / row_bytes / 16 * 16, cap = most < ES_CAP ? most : ES_CAP;
+  p.cap = (int)(a.total < cap ? a.total : cap);
+  const int smem = G::OFF_X + ((p.cap + 15) & ~15) * row_bytes;
   static bool smem_set[kMaxDeviceOrdinals] = {};
-  lime_status s = ensure_dynamic_smem((const void*)k_encode_small<G>, G::OFF_X + ES_CAP * 64, smem_set);
+  lime_status s = ensure_dynamic_smem((const void*)k_encode_small<G, SILU, RAW>, G::OFF_X + cap * row_bytes, smem_set);
   if (s != LIME_OK) return s;
   // as many clusters as the total allows long users, which find theirs or leave; no launch where it allows none
   int64_t longs = a.total / (ES_LONG + 1);
@@ -681,15 +750,21 @@ static lime_status launch_es(const EncodeSmallArgs& a, cudaStream_t st) {
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     ProfScope _p("k_encode_small", st);
-    cudaLaunchKernelEx(&cfg, k_encode_small<G>, p);
+    cudaLaunchKernelEx(&cfg, k_encode_small<G, SILU, RAW>, p);
     LIME_LAUNCH_CHECK("k_encode_small");
   }
   p.clustered = 0;
   p.skip_long = longs > 0;
   ProfScope _p("k_encode_small", st);
-  launch_pdl(k_encode_small<G>, dim3((unsigned)a.B), dim3(ES_THREADS), (size_t)smem, st, p);
+  launch_pdl(k_encode_small<G, SILU, RAW>, dim3((unsigned)a.B), dim3(ES_THREADS), (size_t)smem, st, p);
   LIME_LAUNCH_CHECK("k_encode_small");
   return LIME_OK;
+}
+
+template <class G>
+static lime_status launch_es(const EncodeSmallArgs& a, cudaStream_t st) {
+  if (a.silu) return a.hist_ln ? launch_es_t<G, true, true>(a, st) : launch_es_t<G, true, false>(a, st);
+  return a.hist_ln ? launch_es_t<G, false, true>(a, st) : launch_es_t<G, false, false>(a, st);
 }
 
 lime_status launch_encode_small(const EncodeSmallArgs& a, cudaStream_t st) {
