@@ -18,6 +18,11 @@
 namespace lime {
 
 constexpr int EF_D = 64, EF_THREADS = 256, EF_TILE = 128;
+// A user whose share would be over 2048 tokens takes a cluster of sixteen blocks, in a launch of their own, at most seven of them (the
+// clusters that run at once; the line doubles until that holds).  One user of n tokens among 99 of 100, two layers, without it /
+// with it / the generic kernels, which split by token: n = 2000 351 / 353 / 395 us, 4000 680 / 105 / 442, 32000 2985 / 466 / 886,
+// 150000 3645 / 2050 / 2035; 200000 among 399 of 50: 9817 / 2820 / 2612.
+constexpr int EF_LONG = 2048, EF_LONG_CLUSTER = 16, EF_LONG_CLUSTERS = 7;
 constexpr int EF_LD = 68;                                        // floats per row of operands read along the contraction: spreads the banks
 
 template <int H_, int ELL_>
@@ -55,6 +60,7 @@ struct EncodeF32Params {
   const float* w[LIME_MAX_LAYERS][6];                            // W_Q, W_K, W_V (NULL: identity), W_g, W_u, W_o
   float* scratch;                                                // [total x d]: histories beyond shared memory
   float* out;                                                    // L^P
+  int B, longer_than, skip_long;                                 // a user has to be longer than that to be a long one
   int n_layers, cluster, cap, ln, hist_ln, silu;                 // cap: history rows a block holds
   float eps, scale;                                              // scale times log2 e with the softmax
   int* err;
@@ -258,27 +264,36 @@ __device__ __forceinline__ void ef_update_tile(float* fs, float* x, int ld, int 
   }
 }
 
-template <class G>
+// LONG: cluster k takes the k-th long user, and the blocks read each other's message in place (pushed, sixteen slots would not fit
+// beside the operands); without it cluster b takes user b and a long user is left out.
+template <class G, bool LONG>
 __global__ void __launch_bounds__(EF_THREADS, 1)
 k_encode_f32(const EncodeF32Params p) {
   constexpr int ELL = G::ELL, HL = G::HL, DH = G::DH, D = EF_D;
   extern __shared__ __align__(128) float fs[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int CL = p.cluster, b = blockIdx.x / CL, rank = blockIdx.x % CL;
+  const int CL = LONG ? EF_LONG_CLUSTER : p.cluster, rank = blockIdx.x % CL;
   const int c = tid & 63, kq = tid >> 6, k0 = kq * 16;           // link rows: output column, quarter of the contraction
   float* const ex = fs + G::EX;
-  float* const X = ex + 2 * CL * G::MSG;
+  float* const X = ex + (LONG ? 1 : 2 * CL) * G::MSG;
   uint64_t* const bar = reinterpret_cast<uint64_t*>(fs + G::BAR);
   const uint32_t msg_bytes = (uint32_t)(CL - 1) * G::MSG * 4;
-  if (tid == 0) {
+  if (!LONG && tid == 0) {
     tc::mbar_init(bar, 1);
     tc::mbar_arrive_expect_tx(bar, msg_bytes);
     tc::fence_barrier_init();
   }
-  if (CL > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  if (!LONG && CL > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   pdl_launch_dependents();
   pdl_wait();
+  int* const word = reinterpret_cast<int*>(fs + G::MX);
+  const int b = LONG ? nth_long_user(p.off, p.B, p.longer_than, EF_LONG_CLUSTERS, blockIdx.x / CL, word) : (int)blockIdx.x / CL;
+  if (LONG && b < 0) return;                                     // the whole cluster
   const int u0 = p.off[b], un = p.off[b + 1] - u0;
+  if (!LONG && p.skip_long && un > p.longer_than && un > long_user_line(p.off, p.B, p.longer_than, EF_LONG_CLUSTERS, word)) {
+    if (CL > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    return;
+  }
   const int share = (un + CL - 1) / CL, tok0 = u0 + min(un, rank * share), n = min(un, (rank + 1) * share) - min(un, rank * share);
   const bool resident = share <= p.cap;
   float* const rows = resident ? X : p.scratch + (int64_t)tok0 * D;    // the block's history
@@ -422,7 +437,7 @@ k_encode_f32(const EncodeF32Params p) {
     for (int r = 0; r < RPT; ++r)
       *reinterpret_cast<float4*>(fs + G::PART + (grp * HL + rg * RPT + r) * D + cg * 4) = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
     // the message: accumulator, maxima, sums of this share -> slot `rank` here and in every peer
-    float* const slot = ex + ((j & 1) * CL + rank) * G::MSG;
+    float* const slot = LONG ? ex : ex + ((j & 1) * CL + rank) * G::MSG;
     // weights of what follows
     float wk[16];
     if (!last) ef_wrow(wk, p.w[j][0], k0, c);
@@ -434,8 +449,9 @@ k_encode_f32(const EncodeF32Params p) {
       *reinterpret_cast<float4*>(slot + i * 4) = make_float4((x.x + y.x) + (z.x + w.x), (x.y + y.y) + (z.y + w.y), (x.z + y.z) + (z.z + w.z), (x.w + y.w) + (z.w + w.w));
     }
     if (tid < 2 * HL) slot[HL * D + tid] = fs[G::RUN + tid];      // maxima, sums
-    __syncthreads();
-    if (CL > 1) {
+    if (LONG) cluster_sync_all();
+    else __syncthreads();
+    if (!LONG && CL > 1) {
       if (j == 0) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // the peers run
       const uint32_t at = (uint32_t)__cvta_generic_to_shared(slot), ba = (uint32_t)__cvta_generic_to_shared(bar);
       for (int i = tid; i < G::MSG / 4; i += EF_THREADS) {
@@ -447,21 +463,25 @@ k_encode_f32(const EncodeF32Params p) {
     // ---- merge the shares: Ohat [(h, l)][64]
     for (int i = tid; i < HL * D / 4; i += EF_THREADS) {
       const int r = i / (D / 4);
-      const float* msg = ex + (j & 1) * CL * G::MSG;
       float M = -INFINITY, S = 0.f;
       float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int q = 0; q < CL; ++q) M = fmaxf(M, msg[q * G::MSG + HL * D + r]);
+      auto msg = [&](int q) -> const float* {
+        if constexpr (LONG) return cluster_peer(static_cast<const float*>(ex), q);
+        else return ex + ((j & 1) * CL + q) * G::MSG;
+      };
+      for (int q = 0; q < CL; ++q) M = fmaxf(M, msg(q)[HL * D + r]);
       for (int q = 0; q < CL; ++q) {
-        const float m = msg[q * G::MSG + HL * D + r], w = m == -INFINITY ? 0.f : ef_ex2(m - M);
-        S = fmaf(w, msg[q * G::MSG + HL * D + HL + r], S);
-        const float4 x = ef_ld4(msg + q * G::MSG + i * 4);
+        const float m = msg(q)[HL * D + r], w = m == -INFINITY ? 0.f : ef_ex2(m - M);
+        S = fmaf(w, msg(q)[HL * D + HL + r], S);
+        const float4 x = ef_ld4(msg(q) + i * 4);
         o.x = fmaf(w, x.x, o.x); o.y = fmaf(w, x.y, o.y); o.z = fmaf(w, x.z, o.z); o.w = fmaf(w, x.w, o.w);
       }
       const float inv = un > 0 ? 1.0f / (p.silu ? (float)un : S) : 0.f;
       *reinterpret_cast<float4*>(fs + G::OHAT + i * 4) = make_float4(o.x * inv, o.y * inv, o.z * inv, o.w * inv);
     }
-    __syncthreads();
-    if (tid == 0 && !last) tc::mbar_arrive_expect_tx(bar, msg_bytes);     // every thread has seen this layer's messages
+    if (LONG) cluster_sync_all();                                 // the peers have read this block's message
+    else __syncthreads();
+    if (!LONG && tid == 0 && !last) tc::mbar_arrive_expect_tx(bar, msg_bytes);     // every thread has seen this layer's messages
     // ---- what the history update multiplies with (K, V of this layer still in their rows): K2, [G2 | U2], W_o
     if (!last) {
       ef_quarter<ELL, 2>({red_at(2), red_at(3)}, fs + G::ROW_C, {&wb, &wc}, k0, c);
@@ -529,32 +549,50 @@ static lime_status launch_ef(EncodeF32Params p, int B, int64_t total, cudaStream
          (((int64_t)B * cl * 2 <= 144 && total / ((int64_t)B * cl * 2) >= 48) || 2 * total / ((int64_t)B * cl) > (kSmem - fixed_bytes(cl)) / kRow))
     cl *= 2;
   p.cluster = cl;
+  p.B = B;
+  p.longer_than = EF_LONG * cl;
   // the host knows the mean length only: room for twice the mean share, 256 rows at least, where shared memory has it
   const int64_t fixed = fixed_bytes(cl), most = (kSmem - fixed) / kRow;
   int64_t cap = 2 * total / ((int64_t)B * cl) + 1;
   if (cap < 256) cap = 256;
   if (cap > total) cap = total;
   p.cap = (int)(cap < most ? cap : most);
-  const size_t smem = (size_t)(fixed + p.cap * kRow);
+  auto launch = [&](void (*kernel)(EncodeF32Params), bool (&smem_set)[kMaxDeviceOrdinals], int64_t blocks, int cluster, size_t smem, const EncodeF32Params& q) -> lime_status {
+    const lime_status s = ensure_dynamic_smem((const void*)kernel, (int)kSmem, smem_set);
+    if (s != LIME_OK) return s;
+    if (cluster > 8) LIME_CUDA(cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(EF_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    ProfScope _p("k_encode_f32", st);
+    cudaLaunchKernelEx(&cfg, kernel, q);
+    LIME_LAUNCH_CHECK("k_encode_f32");
+    return LIME_OK;
+  };
+  // as many clusters of sixteen as the total allows long users, which find theirs or leave; no launch where it allows none
+  int64_t longs = total / (p.longer_than + 1);
+  if (longs > B) longs = B;
+  if (longs > EF_LONG_CLUSTERS) longs = EF_LONG_CLUSTERS;
+  p.skip_long = longs > 0;
+  if (longs > 0) {
+    EncodeF32Params q = p;
+    constexpr int64_t long_fixed = (int64_t)(G::EX + G::MSG) * 4;
+    q.cap = (int)((kSmem - long_fixed) / kRow);
+    static bool long_smem_set[kMaxDeviceOrdinals] = {};
+    const lime_status s = launch(k_encode_f32<G, true>, long_smem_set, longs * EF_LONG_CLUSTER, EF_LONG_CLUSTER, (size_t)(long_fixed + q.cap * kRow), q);
+    if (s != LIME_OK) return s;
+  }
   static bool smem_set[kMaxDeviceOrdinals] = {};
-  lime_status s = ensure_dynamic_smem((const void*)k_encode_f32<G>, 232448, smem_set);
-  if (s != LIME_OK) return s;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)B * cl);
-  cfg.blockDim = dim3(EF_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = cl; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  ProfScope _p("k_encode_f32", st);
-  cudaLaunchKernelEx(&cfg, k_encode_f32<G>, p);
-  LIME_LAUNCH_CHECK("k_encode_f32");
-  return LIME_OK;
+  return launch(k_encode_f32<G, false>, smem_set, (int64_t)B * cl, cl, (size_t)(fixed + p.cap * kRow), p);
 }
 
 lime_status launch_encode_f32(const EncodeSmallArgs& a, int* err, cudaStream_t st) {

@@ -96,8 +96,9 @@ static int tensor_core_mode(const lime_config& g, int d_ff) {
     return 2;
   return 0;
 }
-// One block (or cluster) per user serves histories of ordinary length; a few very long ones leave most SMs idle and take the generic
-// kernels, which split them.
+// One launch for the whole encode, a block or a cluster per user, up to 2048 tokens a user on average (at that mean, 32 users: d = 32
+// 178 us, generic kernels 1601; fp32 174 us, 815).  Single users may be far longer: these are given more blocks on the device, which
+// knows the lengths (k_encode_small.cu, k_encode_f32.cu).
 static bool encode_small_wanted(const Ctx* c, int32_t B, int64_t total) {
   const lime_config& g = c->cfg;
   return (encode_small_supported(g.dtype, g.d, c->d_ff, g.H, g.ell, g.gated_mlp) ||

@@ -312,10 +312,10 @@ def test_narrow_encode_of_long_histories(H, ell, lengths, phi, raw, per_user):
     _encode_against_oracle(synth.BF16, 32, H, ell, 3, lengths, phi, raw, per_user, 6e-2, 4e-2 if phi == "silu" else 1.5e-2)
 
 
-@pytest.mark.parametrize("dtype,d,H,ell", [(synth.BF16, 32, 4, 16)])
+@pytest.mark.parametrize("dtype,d,H,ell", [(synth.BF16, 32, 4, 16), (synth.F32, 64, 2, 8)])
 def test_one_long_history_among_short_ones_is_split(dtype, d, H, ell):
     """One user with 20,000 tokens among 399 with 50, against 400 users of 99 or 100 (the same rows): the long one must not be left to
-    one block (26 times the time of the even batch where it was, 4.4 times on a cluster)."""
+    one block (26 and 29 times the time of the even batch where it was; 4.4 and 3.0 times on a cluster)."""
     Bd = _lib()
     dt = Bd.LIME_F32 if dtype == synth.F32 else Bd.LIME_BF16
     lime = Bd.Lime(d, H, ell, 2, dtype=dt)
@@ -378,3 +378,11 @@ def test_narrow_encode_is_as_exact_as_the_generic_kernels(phi, raw):
             LP, _ = O.encode_user(O.gather_history(table64, inp["hist_ids"][offh[b]:offh[b + 1]]), links64, layers, cfg)
             sums += [((x[b] - LP) ** 2).sum() / (LP ** 2).sum() for x in (one, generic)]
     assert sums[0] ** 0.5 <= 1.1 * sums[1] ** 0.5, sums ** 0.5
+
+
+@pytest.mark.parametrize("H,ell", [(2, 8), (4, 8), (2, 16)])
+@pytest.mark.parametrize("lengths", [[9000] + [10] * 89, [2049, 2048, 0, 2100, 5] + [20] * 200, [2100] * 9 + [20] * 150 + [4300]])
+@pytest.mark.parametrize("phi,raw,per_user", [("softmax", True, True), ("silu", False, False)])
+def test_fp32_encode_of_long_histories(H, ell, lengths, phi, raw, per_user):
+    """fp32 at d = 64: a share of more than 2048 tokens moves the user to a cluster of sixteen blocks, seven users at most."""
+    _encode_against_oracle(synth.F32, 64, H, ell, 3, lengths, phi, raw, per_user, 1e-4, 1e-5)
