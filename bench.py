@@ -65,12 +65,12 @@ def kernel_models(wl: synth.Workload, total_tokens: int, cand_heads: int = 1):
         "k_precompute": dict(bytes=BC * es * (d + ell * cand_heads)),
         # fused tensor-core layer kernels: history rows read once per direction, written once by the update
         "k_link_attn_tc": dict(bytes=n * N * d * es, flops=n * 4.0 * HL * d * N, pipe="tensor"),
-        "k_hist_update_tc": dict(bytes=(n - 1) * 2.0 * N * d * es, flops=(n - 1) * 2.0 * N * (HL * d + 2 * HL * f + f * d),
+        "k_link_attn_tmem_tc": dict(bytes=n * N * d * es, flops=n * 4.0 * HL * d * N, pipe="tensor"),
+        "k_hist_update_tmem_tc": dict(bytes=(n - 1) * 2.0 * N * d * es, flops=(n - 1) * 2.0 * N * (HL * d + 2 * HL * f + f * d),
                                  pipe="tensor"),
         "k_hist_update2_tc": dict(bytes=(n - 1) * 2.0 * N * d * es, flops=(n - 1) * 2.0 * N * (HL * d + 2 * HL * f + f * d),
                                   pipe="tensor"),
-        # d = 256 kernels: folded scores against the stored rows, values mixed head by head, GatedMLP weights as they stand
-        "k_link_attn_d256_tc": dict(bytes=n * N * d * es, flops=n * 4.0 * HL * d * N, pipe="tensor"),
+        # d = 256: folded scores against the stored rows, values mixed head by head, GatedMLP weights as they stand
         "k_hist_update_d256_tc": dict(bytes=(n - 1) * 2.0 * N * d * es,
                                       flops=(n - 1) * 2.0 * N * (HL * d + ell * d + 2 * d * f + f * d), pipe="tensor"),
         # link-side GEMMs (rows = users x links): PREP (layers 2..n: folded queries / keys and values or gate / up operands)
@@ -268,15 +268,15 @@ NCU_TRAFFIC = {
     # dense scorer: 169.9 MB read + 3.5 MB written
     ("k_score_tc", "bf16_baseline", 256, 2048): {"bytes": 173.5e6, "source": "k_score_tc.cu", "sha": "af919608f4657e09"},
     # XOR-layer kernels: average per launch
-    ("k_link_attn_tc", "bf16_baseline", 256, 2048): {"bytes": 37.8e6, "source": "k_link_attn_tmem_tc.cu", "sha": "74a161f19f4064a1"},
-    ("k_hist_update_tc", "bf16_baseline", 256, 2048): {"bytes": 33.8e6, "source": "k_hist_update_tmem_tc.cu", "sha": "bbde8b584842ab94"},
+    ("k_link_attn_tmem_tc", "bf16_baseline", 256, 2048): {"bytes": 37.8e6, "source": "k_link_attn_tmem_tc.cu", "sha": "74a161f19f4064a1"},
+    ("k_hist_update_tmem_tc", "bf16_baseline", 256, 2048): {"bytes": 33.8e6, "source": "k_hist_update_tmem_tc.cu", "sha": "bbde8b584842ab94"},
     # scorer by id over packed corpus records: 174.5 MB read + 4.1 MB written per launch
     ("k_score_gather_tc", "bf16_baseline", 256, 2048): {"bytes": 178.6e6, "source": "k_score_gather_tc.cu", "sha": "580e539a2d79f57c"},
     # scorer through the interaction network (--head 96): 169.4 MB read + 4.4 MB written per launch
     ("k_score_head_tc", "bf16_baseline", 256, 2048): {"bytes": 173.8e6, "source": "k_score_head_tc.cu", "sha": "614556b96c1342b2"},
     # d = 256 kernels: captured on 128 users of the same model and length mix (327,680 tokens) and scaled by the tokens of
     # a launch (persistent kernels, identical tiles: traffic grows in proportion): bytes per token, average of the layers
-    ("k_link_attn_d256_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 578.7, "source": "k_link_attn_tmem_tc.cu", "sha": "74a161f19f4064a1"},
+    ("k_link_attn_tmem_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 578.7, "source": "k_link_attn_tmem_tc.cu", "sha": "74a161f19f4064a1"},
     ("k_hist_update_d256_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 846.5, "source": "k_hist_update_d256_tc.cu", "sha": "b0e365c3aee6d1d3"},
 }
 

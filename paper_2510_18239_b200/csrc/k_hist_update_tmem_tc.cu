@@ -520,7 +520,7 @@ k_hist_update_tmem_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
 }
 
 template <int NG, int ELL, bool LN>
-static lime_status launch_ht(const HistUpdateArgs& a, cudaStream_t st, const char* name) {
+static lime_status launch_ht(const HistUpdateArgs& a, cudaStream_t st) {
   CUtensorMap tmX, tmK2, tmG, tmU, tmWo;
   const uint64_t users = a.shared ? 1 : (uint64_t)a.B, HL = NG * 128;
   if (!make_tmap_bf16_sw128(&tmX, a.hist_in, (uint64_t)a.total, HT_D, HT_D, HT_TILE) ||
@@ -536,9 +536,9 @@ static lime_status launch_ht(const HistUpdateArgs& a, cudaStream_t st, const cha
   static bool smem_set[kMaxDeviceOrdinals] = {};
   const lime_status es = ensure_dynamic_smem((const void*)k_hist_update_tmem_tc<NG, ELL, LN>, (int)HT_SMEM, smem_set);
   if (es != LIME_OK) return es;
-  ProfScope _p(name, st);
+  ProfScope _p("k_hist_update_tmem_tc", st);
   launch_pdl(k_hist_update_tmem_tc<NG, ELL, LN>, dim3(grid), dim3(HT_THREADS), HT_SMEM, st, tmX, tmK2, tmG, tmU, tmWo, p);
-  LIME_LAUNCH_CHECK(name);
+  LIME_LAUNCH_CHECK("k_hist_update_tmem_tc");
   return LIME_OK;
 }
 
@@ -549,15 +549,15 @@ bool hist_update_tmem_supported(int dtype, int d, int f, int H, int ell, int phi
 }
 
 template <int NG, int ELL>
-static lime_status launch_ht_ln(const HistUpdateArgs& a, cudaStream_t st, const char* name) {
-  return a.ln ? launch_ht<NG, ELL, true>(a, st, name) : launch_ht<NG, ELL, false>(a, st, name);
+static lime_status launch_ht_ln(const HistUpdateArgs& a, cudaStream_t st) {
+  return a.ln ? launch_ht<NG, ELL, true>(a, st) : launch_ht<NG, ELL, false>(a, st);
 }
 
 lime_status launch_hist_update_tmem(const HistUpdateArgs& a, int H, cudaStream_t st) {
   if (a.total == 0) return LIME_OK;
   if (a.ln && (a.stats_in == nullptr || a.cK == nullptr)) return LIME_INVALID_ARG;
-  if (H * a.ell == 128) return a.ell == 16 ? launch_ht_ln<1, 16>(a, st, "k_hist_update_tc") : launch_ht_ln<1, 32>(a, st, "k_hist_update_tc");
-  return a.ell == 32 ? launch_ht_ln<2, 32>(a, st, "k_hist_update2_tc") : launch_ht_ln<2, 64>(a, st, "k_hist_update2_tc");
+  if (H * a.ell == 128) return a.ell == 16 ? launch_ht_ln<1, 16>(a, st) : launch_ht_ln<1, 32>(a, st);
+  return a.ell == 32 ? launch_ht_ln<2, 32>(a, st) : launch_ht_ln<2, 64>(a, st);
 }
 
 }  // namespace lime

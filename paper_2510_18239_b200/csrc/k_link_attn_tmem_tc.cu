@@ -582,7 +582,7 @@ int link_attn_d256_groups(int n_chunk_upper, int H, int ell) {
 }
 
 template <class G>
-static lime_status launch_link_attn_tmem(const LinkAttnArgs& a, cudaStream_t st, const char* name, bool (&smem_set)[kMaxDeviceOrdinals]) {
+static lime_status launch_link_attn_tmem(const LinkAttnArgs& a, cudaStream_t st, bool (&smem_set)[kMaxDeviceOrdinals]) {
   if (a.n_chunk_upper <= 0 || a.total == 0) return LIME_OK;   // no history: the merge step writes zeros
   if (a.ln) return LIME_INVALID_ARG;                           // rows must arrive LayerNorm-ed
   CUtensorMap tmX, tmQ2;
@@ -600,19 +600,19 @@ static lime_status launch_link_attn_tmem(const LinkAttnArgs& a, cudaStream_t st,
   if (!G::STRIDED && a.n_groups * p.RB != grid) return LIME_INVALID_ARG;      // the schedule was dealt for another grid
   lime_status es = ensure_dynamic_smem((const void*)k_link_attn_tmem_tc<G>, (int)G::SMEM, smem_set);
   if (es != LIME_OK) return es;
-  ProfScope _p(name, st);
+  ProfScope _p("k_link_attn_tmem_tc", st);
   launch_pdl(k_link_attn_tmem_tc<G>, dim3(grid), dim3(G::THREADS), G::SMEM, st, tmX, tmQ2, p);
-  LIME_LAUNCH_CHECK(name);
+  LIME_LAUNCH_CHECK("k_link_attn_tmem_tc");
   return LIME_OK;
 }
 
 lime_status launch_link_attn_d128_tmem(const LinkAttnArgs& a, cudaStream_t st) {
   static bool smem_set[kMaxDeviceOrdinals] = {};
-  return launch_link_attn_tmem<LtD128>(a, st, "k_link_attn_tc", smem_set);
+  return launch_link_attn_tmem<LtD128>(a, st, smem_set);
 }
 lime_status launch_link_attn_d256_tc(const LinkAttnArgs& a, cudaStream_t st) {
   static bool smem_set[kMaxDeviceOrdinals] = {};
-  return launch_link_attn_tmem<LtD256>(a, st, "k_link_attn_d256_tc", smem_set);
+  return launch_link_attn_tmem<LtD256>(a, st, smem_set);
 }
 
 }  // namespace lime
