@@ -1,5 +1,5 @@
 // History update of one XOR layer on tcgen05 for more stacked (head, link) rows than one SM can keep resident
-// (H * ell = 384 or 512 at d = d_ff = 128, e.g. 8 heads x 64 links):
+// (H * ell = 512 at d = d_ff = 128: 8 heads x 64 links or 16 x 32):
 //
 //   S'[t,:] = GatedMLP( O[S]_t ),   O[S]_t = concat_h softmax_l( Q[S]_{t,h} K[T]_{l,h}^T * scale ) V[T]_{l,h}     (Eq. 7, Eq. 5)
 //
@@ -20,6 +20,7 @@
 namespace lime {
 
 constexpr int H2_D = 128, H2_F = 128, H2_TILE = 128;
+constexpr int H2_HL = 512, H2_NG = H2_HL / 128;         // stacked rows, groups of them
 constexpr int H2_ROW_WARPS = 8, H2_THREADS = 64 + 32 * H2_ROW_WARPS;
 constexpr uint32_t H2_SUB = 128 * 128;                  // bytes of one [128 rows x 64 bf16] swizzled sub-tile
 constexpr uint32_t H2_OFF_X = 0;                        // token tile: 2 K-blocks
@@ -29,8 +30,8 @@ constexpr uint32_t H2_OFF_WO = H2_OFF_GU + 4 * H2_SUB;  // [d x f]: 2 K-blocks
 constexpr uint32_t H2_OFF_PU = H2_OFF_WO + 2 * H2_SUB;  // P_c, then U: 2 K-blocks
 constexpr uint32_t H2_OFF_STATS = H2_OFF_PU + 2 * H2_SUB;    // 2 (tile parity) x 128 float2 {rstd, mu}
 constexpr uint32_t H2_OFF_EXCH = H2_OFF_STATS + 2 * 128 * 8; // pair exchange: [2 tile parities][2 halves][128] float2 {mean, M2}
-constexpr uint32_t H2_OFF_CK = H2_OFF_EXCH + 4 * 128 * 8;    // the current user's HL key row sums (up to 512 floats)
-constexpr uint32_t H2_OFF_BAR = H2_OFF_CK + 512 * 4;
+constexpr uint32_t H2_OFF_CK = H2_OFF_EXCH + 4 * 128 * 8;    // the current user's key row sums
+constexpr uint32_t H2_OFF_BAR = H2_OFF_CK + H2_HL * 4;
 constexpr int H2_IDX_CAP = 1025;                            // users + 1 whose offsets are staged in shared memory (the
 constexpr uint32_t H2_OFF_IDX = H2_OFF_BAR + 256;           // search for a tile's user is a chain of dependent reads:
 constexpr uint32_t H2_SMEM = H2_OFF_IDX + 2 * H2_IDX_CAP * 4 + 8;   // microseconds from global memory)
@@ -38,10 +39,10 @@ static_assert(H2_SMEM <= 232448, "shared memory budget of one CTA");
 
 struct HistUpdate2Params {
   __nv_bfloat16* out;            // [total x d]
-  const float* cK;               // [users x HL] row sums of K2
+  const float* cK;               // [users x 512] row sums of K2
   const int32_t* off;            // [B+1]
   const int32_t* tile_start;     // [B+1] prefix of per-user tile counts (tile = 128 tokens)
-  int B, HL, NG, shared, out_ln; // NG = HL / 128 groups
+  int B, shared, out_ln;
   int silu;                      // 1: P = SiLU(scores) / ell (Algorithm 2) instead of the per-head softmax
   float ln_eps;
   int* err;
@@ -116,7 +117,7 @@ k_hist_update2_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 19);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int NG = p.NG;
+  constexpr int NG = H2_NG;
 
   if (threadIdx.x == 0) {
     mbar_init(x_full, 1); mbar_init(x_empty, 1 + H2_ROW_WARPS);
@@ -174,7 +175,7 @@ k_hist_update2_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant
           if (q > 0 && !mbar_wait(k2_empty, (uint32_t)(q - 1) & 1u, p.err, 11)) { ok = false; break; }
           mbar_arrive_expect_tx(k2_full, 2 * H2_SUB);
           for (int kb = 0; kb < 2; ++kb)
-            tma_load_2d_hint(smem + H2_OFF_K2 + kb * H2_SUB, &tmK2, kb * 64, urow * p.HL + c * 128, k2_full, pol_keep);
+            tma_load_2d_hint(smem + H2_OFF_K2 + kb * H2_SUB, &tmK2, kb * 64, urow * H2_HL + c * 128, k2_full, pol_keep);
           if (q > 0 && !mbar_wait(ops_empty, (uint32_t)(q - 1) & 1u, p.err, 13)) { ok = false; break; }
           mbar_arrive_expect_tx(ops_full, 4 * H2_SUB);
           for (int kb = 0; kb < 2; ++kb) {
@@ -218,7 +219,7 @@ k_hist_update2_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         if (!mbar_wait(x_full, (uint32_t)g & 1u, p.err, 23)) break;
         const int u0 = g * (NG + 1);
         // 1. scores of the first group (its buffer last held the scores of the previous tile's last group: consumed)
-        if (!issue_scores(q, u0, NG == 1)) { ok = false; break; }
+        if (!issue_scores(q, u0, false)) { ok = false; break; }
         for (int c = 0; c < NG && ok; ++c, ++q) {
           if (c + 1 < NG) {
             // 1'. scores of the next group, under this group's softmax; for c = 0 the buffer last held S' of the previous tile
@@ -240,9 +241,8 @@ k_hist_update2_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant
           if (c == NG - 1) mma_commit(gu_full);
         }
         if (!ok) break;
-        // 5. S'(g) = U(g) . W_o, into the buffer after the last group's (with one group that one last held S'(g-1))
+        // 5. S'(g) = U(g) . W_o, into the buffer after the last group's
         if (!mbar_wait(u_ready, (uint32_t)g & 1u, p.err, 25)) break;
-        if (NG == 1 && g > 0 && !mbar_wait(sp_free, (uint32_t)(g - 1) & 1u, p.err, 26)) break;
         tc_fence_after();
         for (int kk = 0; kk < 8; ++kk) {
           const uint32_t o = (uint32_t)(kk >> 2) * H2_SUB + (uint32_t)(kk & 3) * 32;
@@ -310,8 +310,8 @@ k_hist_update2_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         if (b != ck_user && (ck_user < 0 || !p.shared)) {
           // every warp has passed the rendezvous, i.e. finished the previous tile: nobody still reads the old sums.
           // Warps of a half write identical values.
-          for (int i = half * 64 + lane; i < p.HL; i += 128) ck_all[i] = p.cK[(int64_t)(p.shared ? 0 : b) * p.HL + i];
-          for (int i = half * 64 + 32 + lane; i < p.HL; i += 128) ck_all[i] = p.cK[(int64_t)(p.shared ? 0 : b) * p.HL + i];
+          for (int i = half * 64 + lane; i < H2_HL; i += 128) ck_all[i] = p.cK[(int64_t)(p.shared ? 0 : b) * H2_HL + i];
+          for (int i = half * 64 + 32 + lane; i < H2_HL; i += 128) ck_all[i] = p.cK[(int64_t)(p.shared ? 0 : b) * H2_HL + i];
           __syncwarp();
         }
         ck_user = b;
@@ -480,24 +480,23 @@ k_hist_update2_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant
 }
 
 bool hist_update2_tc_supported(int dtype, int d, int f, int H, int ell, int phi, int gated_mlp) {
-  const int HL = H * ell;
-  return dtype == LIME_BF16 && d == H2_D && f == H2_F && HL % 128 == 0 && HL >= 384 && HL <= 512 && (ell == 32 || ell == 64) &&
+  return dtype == LIME_BF16 && d == H2_D && f == H2_F && H * ell == H2_HL && (ell == 32 || ell == 64) &&
          (phi == LIME_PHI_SOFTMAX || phi == LIME_PHI_SILU) && gated_mlp != 0;
 }
 
 template <int ELL>
-static lime_status launch_hu2(const HistUpdateArgs& a, int HL, cudaStream_t st) {
+static lime_status launch_hu2(const HistUpdateArgs& a, cudaStream_t st) {
   CUtensorMap tmX, tmK2, tmG, tmU, tmWo;
   const uint64_t users = a.shared ? 1 : (uint64_t)a.B;
   if (!make_tmap_bf16_sw128(&tmX, a.hist_in, (uint64_t)a.total, H2_D, H2_D, H2_TILE) ||
-      !make_tmap_bf16_sw128(&tmK2, a.K2, users * HL, H2_D, H2_D, 128) ||
-      !make_tmap_bf16_sw128(&tmG, a.G2t, users * H2_F, (uint64_t)HL, (uint64_t)HL, 128) ||
-      !make_tmap_bf16_sw128(&tmU, a.U2t, users * H2_F, (uint64_t)HL, (uint64_t)HL, 128) ||
+      !make_tmap_bf16_sw128(&tmK2, a.K2, users * H2_HL, H2_D, H2_D, 128) ||
+      !make_tmap_bf16_sw128(&tmG, a.G2t, users * H2_F, H2_HL, H2_HL, 128) ||
+      !make_tmap_bf16_sw128(&tmU, a.U2t, users * H2_F, H2_HL, H2_HL, 128) ||
       !make_tmap_bf16_sw128(&tmWo, a.WoT, H2_D, H2_F, H2_F, 128))
     return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
   HistUpdate2Params p;
-  p.out = (__nv_bfloat16*)a.hist_out; p.cK = a.cK; p.off = a.off; p.tile_start = a.tile_start; p.B = a.B; p.HL = HL;
-  p.NG = HL / 128; p.shared = a.shared; p.silu = a.silu; p.out_ln = a.out_ln; p.ln_eps = a.ln_eps; p.err = a.err;
+  p.out = (__nv_bfloat16*)a.hist_out; p.cK = a.cK; p.off = a.off; p.tile_start = a.tile_start; p.B = a.B;
+  p.shared = a.shared; p.silu = a.silu; p.out_ln = a.out_ln; p.ln_eps = a.ln_eps; p.err = a.err;
   int grid = a.n_tile_upper < kSMs ? a.n_tile_upper : kSMs;
   if (grid < 1) return LIME_OK;
   static bool smem_ln[kMaxDeviceOrdinals] = {}, smem_plain[kMaxDeviceOrdinals] = {};
@@ -511,11 +510,11 @@ static lime_status launch_hu2(const HistUpdateArgs& a, int HL, cudaStream_t st) 
   return LIME_OK;
 }
 
-lime_status launch_hist_update2_tc(const HistUpdateArgs& a, int H, cudaStream_t st) {
+lime_status launch_hist_update2_tc(const HistUpdateArgs& a, cudaStream_t st) {
   if (a.total == 0) return LIME_OK;
   switch (a.ell) {
-    case 32: return launch_hu2<32>(a, H * a.ell, st);
-    case 64: return launch_hu2<64>(a, H * a.ell, st);
+    case 32: return launch_hu2<32>(a, st);
+    case 64: return launch_hu2<64>(a, st);
   }
   return LIME_UNSUPPORTED_SHAPE;
 }

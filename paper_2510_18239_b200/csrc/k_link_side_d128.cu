@@ -41,7 +41,7 @@ struct LinkSide128Params {
   const __nv_bfloat16* Ohat; const float *part_m, *part_s, *part_acc; const int32_t* chunk_start;
   const __nv_bfloat16 *WpostT, *WoT, *WprepT;                    // WprepT nullable: no operands
   int need_hist, lp_accumulate, ln;
-  float *T_out, *LP;
+  float* LP;
   __nv_bfloat16 *link_states, *Q2, *K2, *G2t, *U2t;
   float eps;
   int* err;
@@ -252,12 +252,11 @@ k_link_side_d128(const LinkSide128Params p) {
   }
   __syncthreads();
   tc::mbar_wait(&bars[2], 0, p.err, 91);
-  // T of this block's columns leaves: fp32 rows, the running sum of Eq. 8, the link states
+  // T of this block's columns leaves: the running sum of Eq. 8, the link states
   for (int i = tid; i < rows * 8; i += L1_THREADS) {
     const int lr = i >> 3, c = rank * 32 + (i & 7) * 4;
     float4 v = *reinterpret_cast<const float4*>(Ts + lr * G::T_LD + c);
     const int64_t o = (int64_t)(row_first + lr) * D + c;
-    if (p.T_out) *reinterpret_cast<float4*>(p.T_out + o) = v;
     if (p.LP) {
       if (p.lp_accumulate) {
         const float4 x = *reinterpret_cast<const float4*>(p.LP + o);
@@ -361,7 +360,7 @@ lime_status launch_link_side_d128(const LinkSide128Args& a, cudaStream_t st) {
   typedef const __nv_bfloat16* B16;
   p.users = a.users; p.ell = a.ell; p.Ohat = (B16)a.Ohat; p.part_m = a.part_m; p.part_s = a.part_s; p.part_acc = a.part_acc;
   p.chunk_start = a.chunk_start; p.WpostT = (B16)a.WpostT; p.WoT = (B16)a.WoT; p.WprepT = (B16)a.WprepT;
-  p.need_hist = a.need_hist; p.lp_accumulate = a.lp_accumulate; p.ln = a.ln; p.T_out = a.T_out; p.LP = a.LP;
+  p.need_hist = a.need_hist; p.lp_accumulate = a.lp_accumulate; p.ln = a.ln; p.LP = a.LP;
   p.link_states = (__nv_bfloat16*)a.link_states; p.Q2 = (__nv_bfloat16*)a.Q2; p.K2 = (__nv_bfloat16*)a.K2;
   p.G2t = (__nv_bfloat16*)a.G2t; p.U2t = (__nv_bfloat16*)a.U2t; p.eps = a.eps; p.err = a.err;
   switch (link_side_d128_rows((int64_t)a.users * a.ell)) {

@@ -5,7 +5,7 @@
 //
 // What bounds it: the rate at which HBM serves random rows.  Rows by id arrive in pieces of 2 d and 2 ell bytes; the
 // memory system opens about 16.5 G different 256-byte blocks a second whatever fetches them, so the kernel's part is to
-// keep enough rows in flight and to add no latency of its own.  A warp takes 16 MT consecutive slots, reads its rows from
+// keep enough rows in flight and to add no latency of its own.  A warp takes 16 consecutive slots, reads its rows from
 // global memory straight into the A fragments of mma.m16n8k16 (no shared memory, no barrier, no tensor memory to allocate:
 // the first row is requested two dependent reads after the launch) and forms A = T_rows . LS^T; the ell-term dot with the
 // weight row follows in registers.  The tensor work (2 ell d per candidate against 2 d + 2 ell bytes) is far below what
@@ -32,7 +32,7 @@ struct ScoreRowsParams {
   int ldt, ldw;            // row pitches in elements
   int rows;                // rows of W and T
   int total;               // slots
-  int B, C, n_groups;      // groups of 16 * MT slots
+  int B, C, n_groups;      // groups of 16 slots (8 with fp32 storage)
 };
 
 __device__ __forceinline__ uint4 sr_ld_stream(const void* p) {
@@ -67,10 +67,10 @@ __device__ __forceinline__ int sr_find_user(const int32_t* __restrict__ off, int
   return lo;
 }
 
-template <int D, int ELL, int MT>
+template <int D, int ELL>
 __global__ void __launch_bounds__(SR_WARPS * 32, sr_blocks(D, ELL))
 k_score_rows(const ScoreRowsParams p) {
-  constexpr int NT = ELL / 8, NL = ELL / 4, KJ = D / 32, RW = 2 * MT;    // n-tiles, links per thread, 32-column chunks, rows per thread
+  constexpr int NT = ELL / 8, NL = ELL / 4, KJ = D / 32;    // n-tiles, links per thread, 32-column chunks
   pdl_launch_dependents();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
@@ -81,7 +81,7 @@ k_score_rows(const ScoreRowsParams p) {
   // this kernel fit beside it: 100 lists of 20..1500 ids, the batch 142 -> 134 us.  The tcgen05 scorers do not gain: their CTAs
   // take a whole SM, so those that wait for one of the busy SMs start late whatever the others have prefetched)
   for (int grp = g_begin + warp; grp < min(g_end, g_begin + SR_AHEAD * SR_WARPS); grp += SR_WARPS) {
-    const int slot = grp * (16 * MT) + (lane & 15);
+    const int slot = grp * 16 + (lane & 15);
     const int id = slot < p.total ? (p.ids != nullptr ? __ldcg(p.ids + slot) : slot) : -1;
     if (id >= 0 && id < p.rows) {
       const char* row = reinterpret_cast<const char*>(p.T + (int64_t)id * p.ldt);
@@ -92,11 +92,11 @@ k_score_rows(const ScoreRowsParams p) {
   pdl_wait();
   int b = -1;
   for (int grp = g_begin + warp; grp < g_end; grp += SR_WARPS) {
-    const int s0 = grp * (16 * MT);
-    const int s1 = min(s0 + 16 * MT, p.total);
+    const int s0 = grp * 16;
+    const int s1 = min(s0 + 16, p.total);
     // one row index per slot
     int row = s0 + lane;
-    bool in = (MT == 2 || lane < 16) && row < s1;
+    bool in = lane < 16 && row < s1;
     if (p.ids != nullptr) {
       const int32_t id = in ? __ldg(p.ids + row) : 0;
       const bool good = id >= 0 && id < p.rows;
@@ -106,10 +106,10 @@ k_score_rows(const ScoreRowsParams p) {
     }
     const unsigned live = __ballot_sync(0xffffffffu, in);
     // T rows as A fragments (all chunks requested at once), weight pieces
-    uint4 a[RW][KJ];
-    uint32_t w[RW][NL / 2];
+    uint4 a[2][KJ];
+    uint32_t w[2][NL / 2];
 #pragma unroll
-    for (int i = 0; i < RW; ++i) {
+    for (int i = 0; i < 2; ++i) {
       const int r = g + 8 * i;
       const int rr = __shfl_sync(0xffffffffu, row, r);
       const bool on = (live >> r) & 1u;
@@ -137,48 +137,44 @@ k_score_rows(const ScoreRowsParams p) {
     for (;;) {
       const int u_end = p.cand_off == nullptr ? (b + 1) * p.C : __ldg(p.cand_off + b + 1);
       if (u_end > s0) {
-        float acc[MT][NT][4];
+        float acc[NT][4];
 #pragma unroll
-        for (int m = 0; m < MT; ++m)
+        for (int n = 0; n < NT; ++n)
 #pragma unroll
-          for (int n = 0; n < NT; ++n)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[m][n][e] = 0.f;
+          for (int e = 0; e < 4; ++e) acc[n][e] = 0.f;
         const __nv_bfloat16* ls = p.LS + (int64_t)b * (ELL * D) + (int64_t)((g >> 1) * NL + (g & 1)) * D + t * 8;
 #pragma unroll
         for (int j = 0; j < KJ; ++j) {
-constexpr int NB = NT < 4 ? NT : 4;
+          constexpr int NB = NT < 4 ? NT : 4;
 #pragma unroll
           for (int n0 = 0; n0 < NT; n0 += NB) {
             uint4 bf[NB];
 #pragma unroll
             for (int n = 0; n < NB; ++n) bf[n] = sr_ld_keep(ls + (2 * (n0 + n)) * D + j * 32);
 #pragma unroll
-            for (int n = 0; n < NB; ++n)
-#pragma unroll
-              for (int m = 0; m < MT; ++m) {
-                sr_mma(acc[m][n0 + n], a[2 * m][j].x, a[2 * m + 1][j].x, a[2 * m][j].y, a[2 * m + 1][j].y, bf[n].x, bf[n].y);
-                sr_mma(acc[m][n0 + n], a[2 * m][j].z, a[2 * m + 1][j].z, a[2 * m][j].w, a[2 * m + 1][j].w, bf[n].z, bf[n].w);
-              }
+            for (int n = 0; n < NB; ++n) {
+              sr_mma(acc[n0 + n], a[0][j].x, a[1][j].x, a[0][j].y, a[1][j].y, bf[n].x, bf[n].y);
+              sr_mma(acc[n0 + n], a[0][j].z, a[1][j].z, a[0][j].w, a[1][j].w, bf[n].z, bf[n].w);
+            }
           }
         }
         // dot with the weights: links t * NL + 2 n + {0, 1} of rows g (c0, c1) and g + 8 (c2, c3)
-        float v[RW];
+        float v[2];
 #pragma unroll
-        for (int i = 0; i < RW; ++i) {
+        for (int i = 0; i < 2; ++i) {
           float s = 0.f;
 #pragma unroll
           for (int n = 0; n < NT; ++n) {
             const uint32_t u = w[i][n];
-            s = fmaf(__uint_as_float(u << 16), acc[i >> 1][n][(i & 1) * 2], s);
-            s = fmaf(__uint_as_float(u & 0xffff0000u), acc[i >> 1][n][(i & 1) * 2 + 1], s);
+            s = fmaf(__uint_as_float(u << 16), acc[n][i * 2], s);
+            s = fmaf(__uint_as_float(u & 0xffff0000u), acc[n][i * 2 + 1], s);
           }
           s += __shfl_xor_sync(0xffffffffu, s, 1);
           s += __shfl_xor_sync(0xffffffffu, s, 2);
           v[i] = s;
         }
-        // lane (g, t) keeps row g + 8 t
-        const float mine = RW == 4 ? (t == 0 ? v[0] : t == 1 ? v[1] : t == 2 ? v[2] : v[RW - 1]) : (t == 0 ? v[0] : v[1]);
+        // lanes t = 0, 1 keep row g + 8 t
+        const float mine = t == 0 ? v[0] : v[1];
         const int slot = s0 + g + 8 * t;
         const int u_begin = p.cand_off == nullptr ? b * p.C : __ldg(p.cand_off + b);
         if (slot >= u_begin && slot < u_end) out = mine;
@@ -187,7 +183,7 @@ constexpr int NB = NT < 4 ? NT : 4;
       ++b;
     }
     const int slot = s0 + g + 8 * t;
-    if ((MT == 2 || t < 2) && slot < s1) p.logits[slot] = out;
+    if (t < 2 && slot < s1) p.logits[slot] = out;
   }
 }
 
@@ -436,16 +432,15 @@ bool score_rows_preferred(const ScoreArgs& a) {
 
 template <int D, int ELL>
 static lime_status launch_score_rows_t(const ScoreArgs& a, cudaStream_t st) {
-  constexpr int MT = 1;      // 32 slots per pass while rows, accumulators and weights fit in 128 registers
   ScoreRowsParams p;
   p.LS = (const __nv_bfloat16*)a.LS; p.W = (const __nv_bfloat16*)a.W; p.T = (const __nv_bfloat16*)a.T;
   p.cand_off = a.cand_off; p.ids = a.cand_ids; p.flag = a.dev_flag; p.logits = a.logits;
   p.ldt = a.ldt ? (int)a.ldt : D; p.ldw = a.ldw ? (int)a.ldw : ELL;
   p.rows = (int)(a.cand_ids ? a.corpus_rows : a.total); p.total = (int)a.total; p.B = a.B; p.C = a.C;
-  p.n_groups = (int)((a.total + 16 * MT - 1) / (16 * MT));
+  p.n_groups = (int)((a.total + 15) / 16);
   const int64_t blocks = (p.n_groups + SR_WARPS - 1) / SR_WARPS, cap = 2 * kSMs;
   ProfScope _p("k_score_rows", st);
-  launch_pdl(k_score_rows<D, ELL, MT>, dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(SR_WARPS * 32), 0, st, p);
+  launch_pdl(k_score_rows<D, ELL>, dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(SR_WARPS * 32), 0, st, p);
   LIME_LAUNCH_CHECK("k_score_rows");
   return LIME_OK;
 }

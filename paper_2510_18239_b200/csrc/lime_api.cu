@@ -274,7 +274,7 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
     hu.out_ln = out_ln; hu.silu = g.phi == LIME_PHI_SILU; hu.err = c->dev_err;
     hu.stats_in = pass_stats ? w.row_stats : nullptr;
     if (two_tiles) s = launch_hist_update_tmem(hu, g.H, st);
-    else s = launch_hist_update2_tc(hu, g.H, st);
+    else s = launch_hist_update2_tc(hu, st);
     if (s != LIME_OK) return s;
   }
   if (side1 != nullptr) {

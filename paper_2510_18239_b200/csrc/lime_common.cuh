@@ -416,9 +416,9 @@ struct HistUpdateArgs {
 };
 bool hist_update_tmem_supported(int dtype, int d, int f, int H, int ell, int phi, int gated_mlp);     // H * ell = 128 or 256
 lime_status launch_hist_update_tmem(const HistUpdateArgs& a, int H, cudaStream_t st);                 // a.ln: with stats_in and cK
-// same step for other H * ell up to 512 (link-side operands streamed per tile, k_hist_update2_tc.cu)
+// the same step for H * ell = 512 (link-side operands streamed per tile, k_hist_update2_tc.cu)
 bool hist_update2_tc_supported(int dtype, int d, int f, int H, int ell, int phi, int gated_mlp);
-lime_status launch_hist_update2_tc(const HistUpdateArgs& a, int H, cudaStream_t st);
+lime_status launch_hist_update2_tc(const HistUpdateArgs& a, cudaStream_t st);
 
 // ---- tensor-core XOR layer at d = d_ff = 256 (bf16; ell = 64 with H in {2, 4, 8}, ell = 32 with H in {4, 8}; history rows LayerNorm-ed already) ----
 bool link_attn_d256_tc_supported(int dtype, int d, int H, int ell, int phi);
@@ -446,7 +446,7 @@ struct LinkSide128Args {
   const void* Ohat; const float *part_m, *part_s, *part_acc; const int32_t* chunk_start;
   const void *WpostT, *WoT, *WprepT;                        // this layer's GatedMLP; next layer's operands (NULL: none wanted)
   int need_hist, lp_accumulate, ln;
-  float *T_out, *LP;                                        // nullable
+  float* LP;                                                // nullable
   void *link_states, *Q2, *K2, *G2t, *U2t;                  // link_states (nullable): bf16 L^P instead of LP
   float eps;
   int* err;
