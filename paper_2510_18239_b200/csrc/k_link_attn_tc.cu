@@ -63,7 +63,8 @@ struct LinkAttnParams {
   const int32_t* off;
   const int32_t* chunk_start;     // [B+1] prefix of per-user chunk counts
   const int32_t* chunk_user;      // [chunk items] user of each (user, chunk) item
-  int B, chunk, shared, ell, H;
+  const int32_t* chunk;           // tokens per chunk
+  int B, shared, ell, H;
   int silu;                       // attention activation: 0 softmax (online, log2 domain), 1 SiLU(s) / N(U) (Algorithm 2)
   int HL, RB;                     // stacked (head, link) rows in all, and 128-row blocks of them (one per work item)
   float ln_eps;
@@ -241,9 +242,10 @@ k_link_attn_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
   // item -> token range; identical in every role
   const int rb = (int)blockIdx.x % p.RB;
   const int ci_first = (int)blockIdx.x / p.RB, ci_step = (int)gridDim.x / p.RB, n_ci = n_items / p.RB;
+  const int chunk = __ldg(p.chunk);
   auto item_range = [&](int ci, int b, int& tok0, int& tok1) {
-    tok0 = off[b] + (ci - chunk_start[b]) * p.chunk;
-    tok1 = min(off[b + 1], tok0 + p.chunk);
+    tok0 = off[b] + (ci - chunk_start[b]) * chunk;
+    tok1 = min(off[b + 1], tok0 + chunk);
   };
 
   if (warp == 0) {

@@ -71,7 +71,8 @@ struct LinkAttnTmemParams {
   const int32_t* chunk_user;      // [chunk items] user of each (user, chunk) item
   const int32_t* group_start;     // [groups + 1] the items of a group of CTAs (one CTA per row block) are
   const int32_t* group_items;     //              group_items[group_start[j] .. group_start[j + 1]); unused when strided
-  int B, chunk, shared, ell, H;
+  const int32_t* chunk;           // tokens per chunk
+  int B, shared, ell, H;
   int silu;
   int HL, RB;                     // stacked (head, link) rows in all, and 128-row blocks of them (one per work item)
   float *part_m, *part_s, *part_acc;   // [items x HL], [items x HL], [items x HL x d]
@@ -146,7 +147,7 @@ struct LtItemWalk {
   }
   __device__ __forceinline__ int item(int ps) const { return ps < end ? (STRIDED ? ps : __ldg(items + ps)) : -1; }
   __device__ __forceinline__ void init(const LinkAttnTmemParams& p, int first, int last, int step_) {
-    items = p.group_items; chunk_user = p.chunk_user; chunk_start = p.chunk_start; off = p.off; chunk = p.chunk;
+    items = p.group_items; chunk_user = p.chunk_user; chunk_start = p.chunk_start; off = p.off; chunk = __ldg(p.chunk);
     pos = first; end = last; step = step_;
     ci = item(pos);
     ci1 = item(pos + step);

@@ -123,16 +123,31 @@ __device__ void balance_groups(const int32_t* __restrict__ off, int chunk, const
 
 // both work lists of the XOR layers in one launch: chunks of the links<-history attention, tiles of the history update
 __global__ void __launch_bounds__(1024)
-k_layer_schedules(const int32_t* __restrict__ off, int B, int chunk, int32_t* __restrict__ chunk_start, int tile,
+k_layer_schedules(const int32_t* __restrict__ off, int B, const ChunkRule rule, int32_t* __restrict__ chunk_out,
+                  int32_t* __restrict__ chunk_start, int tile,
                   int32_t* __restrict__ tile_start, int32_t* __restrict__ chunk_user, int32_t* __restrict__ merge_needed,
                   int G, int att_tile, int32_t* __restrict__ group_start, int32_t* __restrict__ group_items,
                   int32_t* __restrict__ scratch) {
   pdl_launch_dependents();     // simple kernel: the next one may set itself up beside it
   pdl_wait();                  // nothing is read or written before the previous kernel is complete
-  // does any user's attention output need the merge step (several chunks to combine, or no history: a zero row)?
-  __shared__ int any_merge;
-  if (threadIdx.x == 0) any_merge = 0;
+  __shared__ int any_merge, longest, short_items;
+  if (threadIdx.x == 0) { any_merge = 0; longest = 0; short_items = 0; }
   __syncthreads();
+  if (rule.short_tokens > 0) {
+    int n_max = 0, items = 0;
+    for (int b = threadIdx.x; b < B; b += blockDim.x) {
+      const int n = off[b + 1] - off[b];
+      n_max = max(n_max, n);
+      if (n > rule.short_tokens) items += (n + rule.short_tokens - 1) / rule.short_tokens;
+    }
+    n_max = __reduce_max_sync(0xffffffffu, n_max);
+    items = __reduce_add_sync(0xffffffffu, items);
+    if ((threadIdx.x & 31) == 0 && n_max > rule.short_tokens) { atomicMax(&longest, n_max); atomicAdd(&short_items, items); }
+    __syncthreads();
+  }
+  const int chunk = longest > 2 * rule.short_tokens && short_items <= rule.short_items ? rule.short_tokens : rule.tokens;
+  if (threadIdx.x == 0) *chunk_out = chunk;
+  // does any user's attention output need the merge step (several chunks to combine, or no history: a zero row)?
   for (int b = threadIdx.x; b < B; b += blockDim.x)
     if (off[b + 1] - off[b] <= 0 || off[b + 1] - off[b] > chunk) any_merge = 1;
   __syncthreads();
@@ -158,11 +173,11 @@ k_layer_schedules(const int32_t* __restrict__ off, int B, int chunk, int32_t* __
   }
 }
 
-lime_status launch_layer_schedules(const int32_t* off, int B, int chunk, int32_t* chunk_start, int tile, int32_t* tile_start,
+lime_status launch_layer_schedules(const int32_t* off, int B, const ChunkRule& chunk, int32_t* chunk_out, int32_t* chunk_start, int tile, int32_t* tile_start,
                                    int32_t* chunk_user, int32_t* merge_needed, const GroupSchedule& gs, cudaStream_t st) {
   if (gs.group_start != nullptr && (gs.n_groups < 1 || gs.n_groups > 160 || gs.att_tile < 1)) return LIME_INVALID_ARG;
   ProfScope _p("k_layer_schedules", st);
-  launch_pdl(k_layer_schedules, dim3(1), dim3(1024), 0, st, off, B, chunk, chunk_start, tile, tile_start, chunk_user, merge_needed,
+  launch_pdl(k_layer_schedules, dim3(1), dim3(1024), 0, st, off, B, chunk, chunk_out, chunk_start, tile, tile_start, chunk_user, merge_needed,
              gs.n_groups, gs.att_tile, gs.group_start, gs.group_items, gs.scratch);
   LIME_LAUNCH_CHECK("k_layer_schedules");
   return LIME_OK;

@@ -119,7 +119,9 @@ struct Workspace {
   float *cQ, *cK;
   float2* row_stats;   // LayerNorm {rstd, mean} of the history rows of the layer being processed
   void *That, *Ohat, *UTb;   // LN(T) [B*ell x d], merged attention rows [B*ell x H*d], GLU output [B*ell x d_ff] (bf16)
-  int chunk, n_chunk_upper, n_tile_upper;
+  ChunkRule chunk;
+  int32_t* chunk_dev;            // the length that k_layer_schedules chose
+  int n_chunk_upper, n_tile_upper;
   size_t bytes;
 };
 
@@ -144,9 +146,19 @@ static Workspace carve(const Ctx* c, void* base, int32_t B, int64_t total) {
   // At least 2048 tokens once the users alone make 64 work items: splitting histories of some hundred tokens then evens out less
   // than the merge of the partials costs (100 users of 250..1000 tokens, two layers: 105 -> 87 us with 32 links, 142 -> 113 us
   // with 64).  With fewer users the split is what occupies the SMs (16 users of 375..1500 tokens: 57 us, 64 us unsplit).
-  const int row_blocks = (g.H * g.ell + 127) / 128, lo = (int64_t)B * row_blocks >= 64 ? 2048 : 512;
-  w.chunk = c->tc_mode == 2 ? pick_chunk(total, row_blocks, lo, 4096) : (tc_link ? pick_chunk(total, row_blocks, lo) : pick_chunk(total, 1, 64));
-  w.n_chunk_upper = (int)((total + w.chunk - 1) / w.chunk + B);
+  // But 512 where few histories are longer, however many users there are: one user of 2000 or 4000 tokens among 64 of 100 takes 74
+  // and 76 us unsplit, 59 and 61 us split (with 64 links 80 -> 69, 85 -> 70 us; d = 256 187 -> 175, 204 -> 189 us).  Up to 64 such
+  // work items the split wins or is even (100 users, 8 of them of 2000: 79 -> 69 us, 20 of 1500: 78 -> 74 us; with 64 links 91 -> 82
+  // and 91 -> 93 us), beyond it loses (30 of 2000, 64 links: 114 -> 128 us; d = 256, 8 of 2000: 239 -> 246 us).
+  // Only the device knows the lengths: k_layer_schedules decides.
+  const int row_blocks = (g.H * g.ell + 127) / 128;
+  const bool many = tc_link && (int64_t)B * row_blocks >= 64;
+  w.chunk = ChunkRule{};
+  w.chunk.tokens = tc_link ? pick_chunk(total, row_blocks, many ? 2048 : 512, c->tc_mode == 2 ? 4096 : 2048) : pick_chunk(total, 1, 64);
+  if (many) { w.chunk.short_tokens = 512; w.chunk.short_items = 64 / row_blocks; }
+  w.chunk_dev = (int32_t*)take(4);
+  const int64_t split_items = (total + w.chunk.tokens - 1) / w.chunk.tokens;
+  w.n_chunk_upper = (int)((split_items > w.chunk.short_items ? split_items : w.chunk.short_items) + B);
   w.n_tile_upper = (int)((total + kHistTile - 1) / kHistTile + B);
   w.chunk_user = (int32_t*)take((size_t)w.n_chunk_upper * 4);
   if (c->tc_mode == 2) {
@@ -238,7 +250,7 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
   LinkAttnArgs la{};
   la.hist = hist_in; la.total = total; la.Q2 = ops.Q2; la.cQ = ops.cQ; la.off = off; la.chunk_start = w.chunk_start; la.chunk_user = w.chunk_user; la.B = B;
   la.group_start = w.groups.group_start; la.group_items = w.groups.group_items; la.n_groups = w.groups.n_groups;
-  la.chunk = w.chunk; la.n_chunk_upper = w.n_chunk_upper; la.ell = g.ell; la.d = g.d; la.H = g.H; la.shared = ops.shared;
+  la.chunk = w.chunk_dev; la.n_chunk_upper = w.n_chunk_upper; la.ell = g.ell; la.d = g.d; la.H = g.H; la.shared = ops.shared;
   la.ln = hist_ln; la.ln_eps = c->ln_eps; la.silu = g.phi == LIME_PHI_SILU; la.part_m = w.part_m; la.part_s = w.part_s; la.part_acc = w.part_acc; la.Ohat = w.Ohat;
   la.err = c->dev_err;
   // the attention kernel forms the LayerNorm statistics of every history row anyway; the history update reuses them
@@ -385,7 +397,7 @@ static lime_status xor_layer_impl(Ctx* c, int layer, const void* hist_in, const 
   const lime_config& g = c->cfg;
   lime_status s;
   if (!schedules_ready) {
-    if ((s = launch_layer_schedules(off, B, w.chunk, w.chunk_start, kHistTile, w.tile_start, w.chunk_user, w.merge_needed, w.groups, st)) != LIME_OK) return s;
+    if ((s = launch_layer_schedules(off, B, w.chunk, w.chunk_dev, w.chunk_start, kHistTile, w.tile_start, w.chunk_user, w.merge_needed, w.groups, st)) != LIME_OK) return s;
   }
   if (layer_on_tensor_cores(c, layer))
     return xor_layer_tc(c, layer, hist_in, off, B, total, links_in, links_shared, hist_out, links_out, w, st);
@@ -414,7 +426,7 @@ static lime_status xor_layer_impl(Ctx* c, int layer, const void* hist_in, const 
   al.QT = w.QT; al.qt_user_stride = links_shared ? 0 : (int64_t)g.ell * g.d;
   al.KS = w.K; al.VS = w.V; al.s_dtype = g.dtype; al.off = off; al.B = B; al.total = total;
   al.ell = g.ell; al.d = g.d; al.H = g.H; al.phi = g.phi; al.scale = c->attn_scale;
-  al.chunk = w.chunk; al.chunk_start = w.chunk_start; al.n_chunk_upper = w.n_chunk_upper;
+  al.chunk = w.chunk.tokens; al.chunk_start = w.chunk_start; al.n_chunk_upper = w.n_chunk_upper;
   al.part_m = w.part_m; al.part_s = w.part_s; al.part_acc = w.part_acc; al.AT = w.AT;
   if ((s = launch_attn_link_simt(al, st)) != LIME_OK) return s;
   if ((s = launch_attn_link_merge(al, st)) != LIME_OK) return s;
@@ -765,7 +777,7 @@ static lime_status encode_user_impl(lime_ctx* ctx, const void* hist, bool hist_n
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   lime_status s;
   const bool narrow = encode_small_wanted(c, B, total_tokens);
-  if (!narrow && (s = launch_layer_schedules(off, B, w.chunk, w.chunk_start, kHistTile, w.tile_start, w.chunk_user, w.merge_needed, w.groups, st)) != LIME_OK) return s;
+  if (!narrow && (s = launch_layer_schedules(off, B, w.chunk, w.chunk_dev, w.chunk_start, kHistTile, w.tile_start, w.chunk_user, w.merge_needed, w.groups, st)) != LIME_OK) return s;
   const int64_t BLd = (int64_t)B * g.ell * g.d;
   if (narrow) {
     EncodeSmallArgs a{};

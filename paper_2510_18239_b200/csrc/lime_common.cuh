@@ -207,7 +207,10 @@ struct GroupSchedule {
   int n_groups = 0, att_tile = 0;
   int32_t* group_start = nullptr; int32_t* group_items = nullptr; int32_t* scratch = nullptr;
 };
-lime_status launch_layer_schedules(const int32_t* off, int B, int chunk, int32_t* chunk_start, int tile, int32_t* tile_start,
+// How long the work items of the links <- history attention are: `tokens`, or `short_tokens` (0: never) where some history is over
+// twice as long as that and the histories longer than it make no more than `short_items` such chunks.
+struct ChunkRule { int tokens = 0, short_tokens = 0, short_items = 0; };
+lime_status launch_layer_schedules(const int32_t* off, int B, const ChunkRule& chunk, int32_t* chunk_out, int32_t* chunk_start, int tile, int32_t* tile_start,
                                    int32_t* chunk_user, int32_t* merge_needed, const GroupSchedule& gs, cudaStream_t st);
 
 // Y[r, n] (+)= epilogue( LN?(X[r, :]) . W[:, n] ) for up to three weight matrices sharing X.
@@ -389,7 +392,7 @@ lime_status launch_link_mlp_tc(const LinkMlpArgs& a, cudaStream_t st);
 struct LinkAttnArgs {
   const void* hist; int64_t total;          // [total x d] bf16
   const void* Q2; const float* cQ;          // folded link queries [users x H*ell x d] bf16 and their row sums
-  const int32_t* off; const int32_t* chunk_start; int B, chunk, n_chunk_upper;
+  const int32_t* off; const int32_t* chunk_start; const int32_t* chunk; int B, n_chunk_upper;   // chunk: tokens per work item
   const int32_t* chunk_user;                // [items] user of each (user, chunk) work item
   const int32_t* group_start; const int32_t* group_items; int n_groups;   // balanced deal of the items (d = 256 kernel)
   int ell, d, H, shared, ln; float ln_eps;

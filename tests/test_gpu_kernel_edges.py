@@ -386,3 +386,42 @@ def test_narrow_encode_is_as_exact_as_the_generic_kernels(phi, raw):
 def test_fp32_encode_of_long_histories(H, ell, lengths, phi, raw, per_user):
     """fp32 at d = 64: a share of more than 2048 tokens moves the user to a cluster of sixteen blocks, seven users at most."""
     _encode_against_oracle(synth.F32, 64, H, ell, 3, lengths, phi, raw, per_user, 1e-4, 1e-5)
+
+
+@pytest.mark.parametrize("d,H,ell", [(128, 4, 32), (128, 8, 32), (256, 8, 64)])
+@pytest.mark.parametrize("lengths", [[2000] + [20] * 80, [1025] * 2 + [512] * 70 + [0], [1024] + [30] * 70, [5000] * 3 + [513] * 7 + [40] * 60, [700] * 66])
+@pytest.mark.parametrize("phi,raw", [("softmax", False), ("silu", True)])
+def test_chunk_length_chosen_from_the_lengths(d, H, ell, lengths, phi, raw):
+    """64 work items and more: chunks of 512 tokens where few histories are longer and one is over 1024, of 2048 or 4096 otherwise;
+    the lines between them, up to the most chunks that are split."""
+    _encode_against_oracle(synth.BF16, d, H, ell, 2, lengths, phi, raw, False, 6e-2, 4e-2 if phi == "silu" else 2.5e-2)
+
+
+def test_one_long_history_is_split_among_many_users():
+    """One user of 4000 tokens among 99 of 100, against 100 users of 100 (d = 128): 1.46 times the time where a history is one work item
+    whenever the users are many, 1.16 times split."""
+    Bd = _lib()
+    d, H, ell = 128, 4, 32
+    lime = Bd.Lime(d, H, ell, 2, dtype=Bd.LIME_BF16)
+    g = torch.Generator("cuda").manual_seed(1)
+    rand = lambda *shape, std: (torch.randn(shape, generator=g, device="cuda") * std).to(torch.bfloat16)
+    weights = [{k: rand(d, d, std=d ** -0.5) for k in ("Wq", "Wk", "Wv", "Wg", "Wu", "Wo")} for _ in range(2)]
+    links = rand(ell, d, std=1.0)
+    lime.set_weights(links, weights)
+
+    def best(lengths):
+        hist = rand(sum(lengths), d, std=1.0)
+        off = lime.lengths_to_offsets(torch.tensor(lengths, dtype=torch.int32, device="cuda"))
+        times = []
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            a.record()
+            for _ in range(20):
+                lime.encode_user_normalized(hist, off)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        return min(times)
+    skewed, even = best([4000] + [100] * 99), best([100] * 100)
+    assert skewed <= 1.3 * even, (skewed, even)
