@@ -67,7 +67,14 @@ static cudaError_t weight_alloc(int device, void** p, size_t bytes, cudaStream_t
 }
 static void weight_free(int device, void* p) {
   if (p == nullptr) return;
-  cudaFree(p);                                          // waits for the device, as every lime_destroy does
+  // Memory of a pool is freed in stream order: cudaFree of it does not wait for kernels that may still read it, as that of a plain
+  // allocation does.  So this waits, on the device that owns it.
+  int current = device;
+  cudaGetDevice(&current);
+  if (current != device) cudaSetDevice(device);
+  cudaDeviceSynchronize();
+  cudaFree(p);
+  if (current != device) cudaSetDevice(current);
   WeightPool& w = g_weight_pool[device];
   std::lock_guard<std::mutex> hold(w.lock);
   if (--w.users == 0) cudaMemPoolTrimTo(w.pool, 0);

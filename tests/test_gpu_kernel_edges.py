@@ -425,3 +425,31 @@ def test_one_long_history_is_split_among_many_users():
         return min(times)
     skewed, even = best([4000] + [100] * 99), best([100] * 100)
     assert skewed <= 1.3 * even, (skewed, even)
+
+
+def test_destroy_waits_for_the_kernels_that_read_its_weight_copies():
+    """d = 256 with 32 links keeps its transposed weights in pool memory.  A context destroyed behind queued encodes must not give
+    them to the next one while they are read: same link states as when the device was idle."""
+    Bd = _lib()
+    d, H, ell, B, n = 256, 4, 32, 64, 600
+    g = torch.Generator("cuda").manual_seed(1)
+    rand = lambda *shape, std: (torch.randn(shape, generator=g, device="cuda") * std).to(torch.bfloat16)
+    hist = rand(B * n, d, std=1.0)
+    lengths = torch.full((B,), n, dtype=torch.int32, device="cuda")
+    models = [(rand(ell, d, std=1.0), [{k: rand(d, d, std=d ** -0.5) for k in ("Wq", "Wk", "Wv", "Wg", "Wu", "Wo")} for _ in range(2)]) for _ in range(2)]
+
+    def context(model):
+        lime = Bd.Lime(d, H, ell, 2, dtype=Bd.LIME_BF16)
+        lime.set_weights(*model)
+        return lime
+    lime = context(models[0])
+    off = lime.lengths_to_offsets(lengths)
+    want = lime.encode_user_normalized(hist, off).clone()
+    torch.cuda.synchronize()
+    for _ in range(3):
+        got = [lime.encode_user_normalized(hist, off).clone() for _ in range(20)]
+        lime.close()
+        other = context(models[1])               # takes the memory that was given back
+        assert all(torch.equal(x, want) for x in got)
+        del other
+        lime = context(models[0])
