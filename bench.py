@@ -268,16 +268,16 @@ NCU_TRAFFIC = {
     # dense scorer: 169.9 MB read + 3.5 MB written
     ("k_score_tc", "bf16_baseline", 256, 2048): {"bytes": 173.5e6, "source": "k_score_tc.cu", "sha": "af919608f4657e09"},
     # XOR-layer kernels: average per launch
-    ("k_link_attn_tmem_tc", "bf16_baseline", 256, 2048): {"bytes": 37.8e6, "source": "k_link_attn_tmem_tc.cu", "sha": "74a161f19f4064a1"},
-    ("k_hist_update_tmem_tc", "bf16_baseline", 256, 2048): {"bytes": 33.8e6, "source": "k_hist_update_tmem_tc.cu", "sha": "bbde8b584842ab94"},
+    ("k_link_attn_tmem_tc", "bf16_baseline", 256, 2048): {"bytes": 37.8e6, "source": "k_link_attn_tmem_tc.cu", "sha": "dbee6fc6fe3d5684"},
+    ("k_hist_update_tmem_tc", "bf16_baseline", 256, 2048): {"bytes": 33.8e6, "source": "k_hist_update_tmem_tc.cu", "sha": "2a2ce314fb1bfbf3"},
     # scorer by id over packed corpus records: 174.5 MB read + 4.1 MB written per launch
     ("k_score_gather_tc", "bf16_baseline", 256, 2048): {"bytes": 178.6e6, "source": "k_score_gather_tc.cu", "sha": "580e539a2d79f57c"},
-    # scorer through the interaction network (--head 96): 169.4 MB read + 4.4 MB written per launch
-    ("k_score_head_tc", "bf16_baseline", 256, 2048): {"bytes": 173.8e6, "source": "k_score_head_tc.cu", "sha": "614556b96c1342b2"},
+    # scorer through the interaction network (--head 96): 169.4 MB read + 5.0 MB written per launch
+    ("k_score_head_tc", "bf16_baseline", 256, 2048): {"bytes": 174.4e6, "source": "k_score_head_tc.cu", "sha": "345f4dcbe7ab9f5a"},
     # d = 256 kernels: captured on 128 users of the same model and length mix (327,680 tokens) and scaled by the tokens of
     # a launch (persistent kernels, identical tiles: traffic grows in proportion): bytes per token, average of the layers
-    ("k_link_attn_tmem_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 578.7, "source": "k_link_attn_tmem_tc.cu", "sha": "74a161f19f4064a1"},
-    ("k_hist_update_d256_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 846.5, "source": "k_hist_update_d256_tc.cu", "sha": "b0e365c3aee6d1d3"},
+    ("k_link_attn_tmem_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 604.7, "source": "k_link_attn_tmem_tc.cu", "sha": "dbee6fc6fe3d5684"},
+    ("k_hist_update_d256_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 944.7, "source": "k_hist_update_d256_tc.cu", "sha": "b0e365c3aee6d1d3"},
 }
 
 

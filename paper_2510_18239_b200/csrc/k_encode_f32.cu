@@ -538,7 +538,7 @@ bool encode_f32_supported(int dtype, int d, int d_ff, int H, int ell, int gated_
 
 template <class G>
 static lime_status launch_ef(EncodeF32Params p, int B, int64_t total, cudaStream_t st) {
-  // Blocks per user: as many as run at once (a block fills an SM, clusters of four fit 144 of them), a share of no less than
+  // Blocks per user: as many as run at once (a block fills an SM; clusters of two fit 148 of them, of four 132), a share of no less than
   // about 50 tokens (a smaller one does not pay for the exchange), at most the eight of a portable cluster; more where the
   // shares would not fit shared memory.
   constexpr int64_t kSmem = 232448, kRow = EF_LD * 4;
