@@ -270,8 +270,8 @@ NCU_TRAFFIC = {
     # XOR-layer kernels: average per launch
     ("k_link_attn_tmem_tc", "bf16_baseline", 256, 2048): {"bytes": 37.8e6, "source": "k_link_attn_tmem_tc.cu", "sha": "dbee6fc6fe3d5684"},
     ("k_hist_update_tmem_tc", "bf16_baseline", 256, 2048): {"bytes": 33.8e6, "source": "k_hist_update_tmem_tc.cu", "sha": "2a2ce314fb1bfbf3"},
-    # scorer by id over packed corpus records: 174.5 MB read + 4.1 MB written per launch
-    ("k_score_gather_tc", "bf16_baseline", 256, 2048): {"bytes": 178.6e6, "source": "k_score_gather_tc.cu", "sha": "580e539a2d79f57c"},
+    # scorer by id over packed corpus records: 174.5 MB read + 4.2 MB written per launch
+    ("k_score_gather_tc", "bf16_baseline", 256, 2048): {"bytes": 178.7e6, "source": "k_score_gather_tc.cu", "sha": "d1a45f59fe51066e"},
     # scorer through the interaction network (--head 96): 169.4 MB read + 5.0 MB written per launch
     ("k_score_head_tc", "bf16_baseline", 256, 2048): {"bytes": 174.4e6, "source": "k_score_head_tc.cu", "sha": "345f4dcbe7ab9f5a"},
     # d = 256 kernels: captured on 128 users of the same model and length mix (327,680 tokens) and scaled by the tokens of

@@ -130,28 +130,31 @@ k_layer_schedules(const int32_t* __restrict__ off, int B, const ChunkRule rule, 
                   int32_t* __restrict__ scratch) {
   pdl_launch_dependents();     // simple kernel: the next one may set itself up beside it
   pdl_wait();                  // nothing is read or written before the previous kernel is complete
-  __shared__ int any_merge, longest, short_items;
-  if (threadIdx.x == 0) { any_merge = 0; longest = 0; short_items = 0; }
-  __syncthreads();
+  int longest = 0, short_items = 0;
   if (rule.short_tokens > 0) {
-    int n_max = 0, items = 0;
+    __shared__ int warp_longest[32], warp_items[32];           // of the block's 32 warps
     for (int b = threadIdx.x; b < B; b += blockDim.x) {
       const int n = off[b + 1] - off[b];
-      n_max = max(n_max, n);
-      if (n > rule.short_tokens) items += (n + rule.short_tokens - 1) / rule.short_tokens;
+      longest = max(longest, n);
+      if (n > rule.short_tokens) short_items += (n + rule.short_tokens - 1) / rule.short_tokens;
     }
-    n_max = __reduce_max_sync(0xffffffffu, n_max);
-    items = __reduce_add_sync(0xffffffffu, items);
-    if ((threadIdx.x & 31) == 0 && n_max > rule.short_tokens) { atomicMax(&longest, n_max); atomicAdd(&short_items, items); }
+    longest = __reduce_max_sync(0xffffffffu, longest);
+    short_items = __reduce_add_sync(0xffffffffu, short_items);
+    if ((threadIdx.x & 31) == 0) { warp_longest[threadIdx.x >> 5] = longest; warp_items[threadIdx.x >> 5] = short_items; }
     __syncthreads();
+    longest = __reduce_max_sync(0xffffffffu, warp_longest[threadIdx.x & 31]);
+    short_items = __reduce_add_sync(0xffffffffu, warp_items[threadIdx.x & 31]);
   }
   const int chunk = longest > 2 * rule.short_tokens && short_items <= rule.short_items ? rule.short_tokens : rule.tokens;
-  if (threadIdx.x == 0) *chunk_out = chunk;
   // does any user's attention output need the merge step (several chunks to combine, or no history: a zero row)?
+  int merge = 0;
   for (int b = threadIdx.x; b < B; b += blockDim.x)
-    if (off[b + 1] - off[b] <= 0 || off[b + 1] - off[b] > chunk) any_merge = 1;
-  __syncthreads();
-  if (threadIdx.x == 0 && merge_needed != nullptr) *merge_needed = any_merge;
+    if (off[b + 1] - off[b] <= 0 || off[b + 1] - off[b] > chunk) merge = 1;
+  merge = __syncthreads_or(merge);
+  if (threadIdx.x == 0) {
+    *chunk_out = chunk;
+    if (merge_needed != nullptr) *merge_needed = merge;
+  }
   block_exclusive_scan(B, chunk_start, [&](int i) {
     int n = off[i + 1] - off[i];
     return n > 0 ? (n + chunk - 1) / chunk : 0;
