@@ -13,15 +13,18 @@
 //   O[:, head] = P_head [128 x ell] . V_head [ell x d_h]
 //   O * 1 / (row sum of the head) -> bf16
 //   per half hf of the hidden columns:   [gate | up] = O . [W_g | W_u][:, hf]  ->  U = SiLU(gate) * up (bf16)
-//                                        S' (+)= U . W_o[hf rows, :]
+//   S' = U . W_o
 //   S' -> (LayerNorm) -> bf16 -> global memory
 // Every contraction but the value mix is issued 256 columns wide: at 128 columns an MMA re-reads its A operand from
 // shared memory twice as often per flop, and shared-memory bandwidth (operands in, TMA writes, the row warps) is what
 // the tensor pipe waits for here.
 // TMEM (512 columns) as two regions.  A: scores of the first 256 stacked rows, then P of all of them (a thread's bf16 pairs
-// over its own scores: the first group's in the first half of its columns, the second's in the other), then [gate | up] of one
-// half, then U over the gates.  B: scores of the other 256 stacked rows, then O, then S'.  P and U are A operands there: no
-// shared memory, no proxy fence.  A takes the next tile's first scores right behind this tile's last contraction.
+// over its own scores: the first group's in the first half of its columns, the second's in the other), then [gate | up] of the
+// first half, then U of both halves.  B: scores of the other 256 stacked rows, then O, then [gate | up] of the second half, then S'.
+// P and U are A operands there: no shared memory, no proxy fence.  A takes the next tile's first scores right behind this tile's
+// last contraction.  Both halves' [gate | up] are issued back to back, so that the second is formed while the row warps work on the
+// first (one after the other in A, with S' begun in between: 266 us a launch of 128 users of 1024..4096 tokens, 64 links x 8 heads,
+// this way 242; 64 users of 100..1024, 32 links x 4 heads 42 -> 38 us).
 // Shared memory: X tile 64 KB (dead once the scores are formed, then O as bf16) and a ring of four 32 KB operand slabs
 // ([256 rows x 64 of the contraction index]) through which K2, V[T]^T, [W_g | W_u] and W_o stream from L2 in the order the MMA
 // issuer consumes them.  (16 KB slabs of 32 of the contraction index, 64-byte swizzle - half again as many in flight - were
@@ -32,7 +35,8 @@
 // Measured (1024 users of 1024..4096 tokens, 64 links x 8 heads): 27500 cycles a tile against 32000 with P and U in shared memory
 // (over the token tile, so that the softmax had to wait for every score), 11300 of them tensor time; 2.65 -> 2.41 ms a launch at
 // the 1 kW power cap, where the batch runs.  What is left: the chain of one tile (TMEM has no room for a second), of which the
-// slabs' arrival (640 KB a tile from L2) takes 6300 and the rows' way out 6500.
+// exponentials take 5400 and the rows' way out 7000.  The slabs (640 KB a tile from L2) are not what is waited for: with half the
+// bytes copied the launch took as long.
 #include "lime_common.cuh"
 #include "tc_common.cuh"
 
@@ -121,12 +125,13 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   uint64_t* p_ready = bars + 12;      // per tile: P in TMEM, scores consumed (16 warps)
   uint64_t* o_full = bars + 13;       // per tile: O complete in TMEM
   uint64_t* o_ready = bars + 14;      // per tile: O as bf16 in smem (16 warps)
-  uint64_t* gu_full = bars + 15;      // per (tile, half): [gate | up] complete
-  uint64_t* u_ready = bars + 16;      // per (tile, half): U in TMEM, [gate | up] read (16 warps)
-  uint64_t* sp_full = bars + 17;      // per tile: S' complete
-  uint64_t* sp_read = bars + 18;      // per tile: S' read out of TMEM (16 warps)
-  uint64_t* row_bar = bars + 19;      // [4] rendezvous of the four warps sharing a TMEM lane quarter
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 23);
+  uint64_t* gu_full = bars + 15;      // [2] per tile: [gate | up] of a half complete
+  uint64_t* gu_read = bars + 17;      // per tile: [gate | up] of the second half in registers (16 warps)
+  uint64_t* u_ready = bars + 18;      // [2] per tile: U of a half in TMEM (16 warps)
+  uint64_t* sp_full = bars + 20;      // per tile: S' complete
+  uint64_t* sp_read = bars + 21;      // per tile: S' read out of TMEM (16 warps)
+  uint64_t* row_bar = bars + 22;      // [4] rendezvous of the four warps sharing a TMEM lane quarter
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 26);
   static_assert(HC_RING == 4, "barrier table above");
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -144,7 +149,8 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     for (int i = 0; i < HC_RING; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
     mbar_init(x_full, 1); mbar_init(x_free, 1);
     mbar_init(&s_full[0], 1); mbar_init(&s_full[1], 1); mbar_init(p_ready, HC_ROW_WARPS);
-    mbar_init(o_full, 1); mbar_init(o_ready, HC_ROW_WARPS); mbar_init(gu_full, 1); mbar_init(u_ready, HC_ROW_WARPS);
+    mbar_init(o_full, 1); mbar_init(o_ready, HC_ROW_WARPS);
+    mbar_init(&gu_full[0], 1); mbar_init(&gu_full[1], 1); mbar_init(gu_read, HC_ROW_WARPS); mbar_init(&u_ready[0], HC_ROW_WARPS); mbar_init(&u_ready[1], HC_ROW_WARPS);
     mbar_init(sp_full, 1); mbar_init(sp_read, HC_ROW_WARPS);
     for (int i = 0; i < 4; ++i) mbar_init(&row_bar[i], HC_PARTS);
     fence_barrier_init();
@@ -210,14 +216,10 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
           tma_load_2d_hint(smem + HC_OFF_RING + s * HC_SLAB, &tmV, 0, urow * HC_D, &full[s], pol_keep);
           ++sl;
         }
-        // then per half of the hidden columns the gate and up columns of W_g / W_u (contraction over d) and that half's
-        // rows of W_o (all output columns)
-        for (int hf = 0; hf < 2 && ok; ++hf) {
-          if (hf == 1)
-            for (int kb = 0; kb < 2 && ok; ++kb) ok = slab(&tmWo, kb * 64, 0, 128, 2);             // S'(0): hidden columns 0..127
+        // then per half of the hidden columns the gate and up columns of W_g / W_u (contraction over d), and W_o
+        for (int hf = 0; hf < 2; ++hf)
           for (int kb = 0; kb < 4 && ok; ++kb) ok = slab(&tmWgu, kb * 64, hf * 128, HC_F + hf * 128, 2);
-        }
-        for (int kb = 0; kb < 2 && ok; ++kb) ok = slab(&tmWo, 128 + kb * 64, 0, 128, 2);           // S'(1): hidden columns 128..255
+        for (int kb = 0; kb < 4 && ok; ++kb) ok = slab(&tmWo, kb * 64, 0, 128, 2);
       }
       if (!ok || *(volatile int*)p.err != 0) {
         // giving up: let the copies already issued land (bounded) before this CTA's shared memory goes away
@@ -300,17 +302,18 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         }
         __syncwarp();
         next_slot();
-        // 3. GatedMLP on O (bf16 in the X / O buffer), the hidden columns in two halves
+        // 3. GatedMLP on O (bf16 in the X / O buffer), the hidden columns in two halves: the second's [gate | up] over O in B,
+        //    under the row warps' work on the first
         if (!wait(o_ready, (uint32_t)g & 1u, 25)) break;
-        for (int hf = 0; hf < 2 && ok; ++hf) {
-          // S' = U(0) . W_o[0..127, :] before the second half's [gate | up] is formed over it
-          if (hf == 1)
-            for (int kb = 0; kb < 2 && ok; ++kb) ok = slab_u(kb, kb == 0, nullptr);
+        for (int hf = 0; hf < 2; ++hf)
           for (int kb = 0; kb < 4 && ok; ++kb)
-            ok = slab_ss(A, kb, idesc_256, kb == 0, kb == 3 ? gu_full : nullptr, kb == 3 && hf == 1 ? x_free : nullptr);
-          if (ok) ok = wait(u_ready, (uint32_t)hf, 27);            // two phases a tile
+            ok = slab_ss(hf ? B : A, kb, idesc_256, kb == 0, kb == 3 ? &gu_full[hf] : nullptr, kb == 3 && hf == 1 ? x_free : nullptr);
+        // S' over the second half's [gate | up], once that is in registers: U(0) . W_o[0..127, :] under the work on it
+        for (int kb = 0; kb < 4 && ok; ++kb) {
+          if ((kb & 1) == 0 && !wait(&u_ready[kb >> 1], (uint32_t)g & 1u, 27)) ok = false;
+          if (kb == 0 && ok) ok = wait(gu_read, (uint32_t)g & 1u, 29);
+          if (ok) ok = slab_u(kb, kb == 0, kb == 3 ? sp_full : nullptr);
         }
-        for (int kb = 0; kb < 2 && ok; ++kb) ok = slab_u(kb, false, kb == 1 ? sp_full : nullptr);
       }
     }
   } else if (n > 0) {
@@ -408,25 +411,31 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(o_ready);
-      // ---- per half of the hidden columns: U = SiLU(gate) * up for this thread's 32 columns, over its own gates
+      // ---- per half of the hidden columns: U = SiLU(gate) * up for this thread's 32 columns, over its own gates and ups of the
+      //      first half
       for (int hf = 0; hf < 2 && ok; ++hf) {
-        if (!mbar_wait(gu_full, (uint32_t)hf, p.err, 34)) { ok = false; break; }          // two phases a tile
+        if (!mbar_wait(&gu_full[hf], (uint32_t)g & 1u, p.err, 34)) { ok = false; break; }
         tc_fence_after();
         float gt[32], up[32], pk[16];
-        tmem_ld_32x32(lane_addr + RA + part * 32, gt);
-        tmem_ld_32x32(lane_addr + RA + 128 + part * 32, up);
+        tmem_ld_32x32(lane_addr + (hf ? RB : RA) + part * 32, gt);
+        tmem_ld_32x32(lane_addr + (hf ? RB : RA) + 128 + part * 32, up);
         tmem_wait_ld();
+        if (hf == 1) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(gu_read);
+        }
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           const float2 hx = __fmul2_rn(make_float2(gt[2 * j], gt[2 * j + 1]), make_float2(0.5f, 0.5f));
           const float2 y = __fmul2_rn(__ffma2_rn(hx, make_float2(hc_tanh(hx.x), hc_tanh(hx.y)), hx), make_float2(up[2 * j], up[2 * j + 1]));
           pk[j] = __uint_as_float(hc_pack(y.x, y.y));
         }
-        tmem_st_32x16(lane_addr + RA + part * 32, pk);
+        tmem_st_32x16(lane_addr + RA + (uint32_t)hf * 128 + part * 32, pk);
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(u_ready);
+        if (lane == 0) mbar_arrive(&u_ready[hf]);
       }
       if (!ok) break;
       // ---- S': this thread's 64 columns of its row -> (LayerNorm) -> bf16 -> global, straight from registers
