@@ -54,7 +54,7 @@ constexpr uint32_t HC_OFF_PATCH = HC_OFF_RING + HC_RING * HC_SLAB;
 constexpr uint32_t HC_OFF_EXCH = HC_OFF_PATCH + HC_ROW_WARPS * HC_PATCH;   // [PARTS][128] float2
 constexpr uint32_t HC_OFF_INV = HC_OFF_EXCH + HC_PARTS * 128 * 8;     // [8 heads][128 rows] 1 / softmax row sum
 constexpr uint32_t HC_OFF_BAR = HC_OFF_INV + 8 * 128 * 4;
-constexpr int HC_IDX_CAP = 1025;                                // users + 1 whose offsets are staged in shared memory
+constexpr int HC_IDX_CAP = kEarlyUsers + 1;                     // users + 1 whose offsets are staged in shared memory
 constexpr uint32_t HC_OFF_IDX = HC_OFF_BAR + 512;
 constexpr uint32_t HC_SMEM = HC_OFF_IDX + 2 * HC_IDX_CAP * 4 + 8;
 static_assert(HC_SMEM <= 232448, "shared memory budget of one CTA");
@@ -66,6 +66,7 @@ struct HistUpdate256Params {
   int B, H, HL, shared, out_ln;
   int silu;                      // 1: P = SiLU(scores) / ell (Algorithm 2) instead of the per-head softmax
   float ln_eps;
+  BesideLinkSide beside;
   int* err;
 };
 
@@ -135,10 +136,6 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   static_assert(HC_RING == 4, "barrier table above");
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_tiles_all = p.tile_start[p.B];
-  const int t_begin = (int)(((int64_t)blockIdx.x * n_tiles_all) / gridDim.x);
-  const int t_end = (int)(((int64_t)(blockIdx.x + 1) * n_tiles_all) / gridDim.x);
-  const int n = t_end - t_begin;
   constexpr uint32_t V_ROW = ELL * 2;                        // bytes of a V[T]^T row (its swizzle span)
   constexpr uint32_t V_BYTES = HC_D * V_ROW;
   const int d_h = HC_D / p.H;
@@ -157,18 +154,27 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     prefetch_tmap(&tmX); prefetch_tmap(&tmK2); prefetch_tmap(&tmV); prefetch_tmap(&tmWgu); prefetch_tmap(&tmWo);
   }
   if (warp == 1) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
-  const int32_t* tile_start = p.tile_start;
-  const int32_t* off = p.off;
-  if (p.B + 1 <= HC_IDX_CAP) {
-    int32_t* idx = reinterpret_cast<int32_t*>(smem + HC_OFF_IDX);
-    for (int i = threadIdx.x; i <= p.B; i += HC_THREADS) { idx[i] = p.tile_start[i]; idx[HC_IDX_CAP + i] = p.off[i]; }
-    tile_start = idx;
-    off = idx + HC_IDX_CAP;
-  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // set-up done: the next kernel's CTAs may become resident; nothing an earlier kernel wrote is read before this wait (beside the
+  // link side: before everything up to the attention is complete, see lime_common.cuh)
+  pdl_launch_dependents();
+  if (!p.beside.early) pdl_wait();
+  const int n_tiles_all = __ldcg(p.tile_start + p.B);
+  const int t_begin = early_first_tile(blockIdx.x, gridDim.x, n_tiles_all, p.beside.late, p.beside.late_by);
+  const int t_end = early_first_tile(blockIdx.x + 1, gridDim.x, n_tiles_all, p.beside.late, p.beside.late_by);
+  const int n = t_end - t_begin;
+  const int32_t* tile_start = p.tile_start;
+  const int32_t* off = p.off;
+  if (p.B + 1 <= HC_IDX_CAP) {
+    int32_t* idx = reinterpret_cast<int32_t*>(smem + HC_OFF_IDX);
+    for (int i = threadIdx.x; i <= p.B; i += HC_THREADS) { idx[i] = __ldcg(p.tile_start + i); idx[HC_IDX_CAP + i] = __ldcg(p.off + i); }
+    tile_start = idx;
+    off = idx + HC_IDX_CAP;
+    __syncthreads();
+  }
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -513,6 +519,7 @@ k_hist_update_d256_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     tc_fence_after();
     tmem_dealloc(tmem_base, 512);
   }
+  if (p.beside.early) pdl_wait();                            // whoever waits for this kernel waits for the link side too
 }
 
 bool hist_update_d256_tc_supported(int dtype, int d, int f, int H, int ell, int phi, int gated_mlp) {
@@ -534,14 +541,14 @@ static lime_status launch_hist_update_d256_t(const HistUpdate256Args& a, cudaStr
     return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
   HistUpdate256Params p;
   p.out = (__nv_bfloat16*)a.hist_out; p.off = a.off; p.tile_start = a.tile_start; p.B = a.B; p.H = a.H; p.HL = HL;
-  p.shared = a.shared; p.silu = a.silu; p.out_ln = a.out_ln; p.ln_eps = a.ln_eps; p.err = a.err;
+  p.shared = a.shared; p.silu = a.silu; p.out_ln = a.out_ln; p.ln_eps = a.ln_eps; p.beside = a.beside; p.err = a.err;
   int grid = a.n_tile_upper < kSMs ? a.n_tile_upper : kSMs;
   if (grid < 1) return LIME_OK;
   static bool smem_set[kMaxDeviceOrdinals] = {};
   lime_status es = ensure_dynamic_smem((const void*)k_hist_update_d256_tc<ELL>, (int)HC_SMEM, smem_set);
   if (es != LIME_OK) return es;
   ProfScope _p("k_hist_update_d256_tc", st);
-  k_hist_update_d256_tc<ELL><<<grid, HC_THREADS, HC_SMEM, st>>>(tmX, tmK2, tmV, tmWgu, tmWo, p);
+  launch_pdl(k_hist_update_d256_tc<ELL>, dim3(grid), dim3(HC_THREADS), HC_SMEM, st, tmX, tmK2, tmV, tmWgu, tmWo, p);
   LIME_LAUNCH_CHECK("k_hist_update_d256_tc");
   return LIME_OK;
 }

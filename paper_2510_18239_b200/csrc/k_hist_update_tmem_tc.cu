@@ -44,7 +44,7 @@ constexpr uint32_t HT_OFF_PATCH = HT_OFF_RING + HT_RING * HT_SUB;
 constexpr uint32_t HT_OFF_EXCH = HT_OFF_PATCH + 2 * HT_GROUP_WARPS * HT_PATCH;      // [2 groups][PARTS][128] float2 {mean, M2}
 constexpr uint32_t HT_OFF_CK = HT_OFF_EXCH + 2 * HT_PARTS * 128 * 8;  // [2 groups][256] (LN) row sums of their user's K2
 constexpr uint32_t HT_OFF_BAR = HT_OFF_CK + 2 * 256 * 4;
-constexpr int HT_IDX_CAP = 1025;                              // users + 1 whose offsets are staged in shared memory (the
+constexpr int HT_IDX_CAP = kEarlyUsers + 1;                             // users + 1 whose offsets are staged in shared memory (the
 constexpr uint32_t HT_OFF_IDX = HT_OFF_BAR + 512;             // search for a tile's user is a chain of dependent reads)
 constexpr uint32_t HT_SMEM = HT_OFF_IDX + 2 * HT_IDX_CAP * 4 + 8;
 constexpr int HT_REGS_LAUNCH = 96, HT_REGS_CONTROL = 64, HT_REGS_ROWS = 104;     // registers a thread: at launch, after the split
@@ -60,6 +60,7 @@ struct HistUpdateTmemParams {
   int B, shared, out_ln;
   int silu;                      // 1: P = SiLU(scores) / ell (Algorithm 2) instead of the per-head softmax
   float ln_eps;
+  BesideLinkSide beside;
   int* err;
 };
 
@@ -156,18 +157,19 @@ k_hist_update_tmem_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  // set-up done: the next kernel's CTAs may become resident; nothing an earlier kernel wrote is read before this wait
+  // set-up done: the next kernel's CTAs may become resident; nothing an earlier kernel wrote is read before this wait (beside the
+  // link side: before everything up to the attention is complete, see lime_common.cuh)
   pdl_launch_dependents();
-  pdl_wait();
-  const int n_tiles_all = p.tile_start[p.B];
-  const int t_begin = (int)(((int64_t)blockIdx.x * n_tiles_all) / gridDim.x);
-  const int t_end = (int)(((int64_t)(blockIdx.x + 1) * n_tiles_all) / gridDim.x);
+  if (!p.beside.early) pdl_wait();
+  const int n_tiles_all = __ldcg(p.tile_start + p.B);
+  const int t_begin = early_first_tile(blockIdx.x, gridDim.x, n_tiles_all, p.beside.late, p.beside.late_by);
+  const int t_end = early_first_tile(blockIdx.x + 1, gridDim.x, n_tiles_all, p.beside.late, p.beside.late_by);
   const int n = t_end - t_begin;                              // tiles of this CTA, g = 0..n-1
   const int32_t* tile_start = p.tile_start;
   const int32_t* off = p.off;
   if (p.B + 1 <= HT_IDX_CAP) {
     int32_t* idx = reinterpret_cast<int32_t*>(smem + HT_OFF_IDX);
-    for (int i = threadIdx.x; i <= p.B; i += HT_THREADS) { idx[i] = p.tile_start[i]; idx[HT_IDX_CAP + i] = p.off[i]; }
+    for (int i = threadIdx.x; i <= p.B; i += HT_THREADS) { idx[i] = __ldcg(p.tile_start + i); idx[HT_IDX_CAP + i] = __ldcg(p.off + i); }
     tile_start = idx;
     off = idx + HT_IDX_CAP;
     __syncthreads();
@@ -335,7 +337,7 @@ k_hist_update_tmem_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
       // ---- softmax over the links of this thread's heads, P over its own scores
       float rstd_r = 1.f, mu_r = 0.f;
       if (LN && row0 + (int)r < row_end) {
-        const float2 st = __ldg(p.stats_in + row0 + r);
+        const float2 st = __ldcg(p.stats_in + row0 + r);
         rstd_r = st.x; mu_r = st.y;
       }
       if (!mbar_wait(&s_full[grp], i_ph, p.err, 32)) { ok = false; break; }
@@ -346,8 +348,8 @@ k_hist_update_tmem_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         const float* src = p.cK + (int64_t)(p.shared ? 0 : b) * (NG * 128) + part * 64;
 #pragma unroll
         for (int c = 0; c < NG; ++c) {
-          ck_s[c * 128 + part * 64 + lane] = src[c * 128 + lane];
-          ck_s[c * 128 + part * 64 + 32 + lane] = src[c * 128 + 32 + lane];
+          ck_s[c * 128 + part * 64 + lane] = __ldcg(src + c * 128 + lane);
+          ck_s[c * 128 + part * 64 + 32 + lane] = __ldcg(src + c * 128 + 32 + lane);
         }
         __syncwarp();
       }
@@ -517,6 +519,7 @@ k_hist_update_tmem_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     tc_fence_after();
     tmem_dealloc(tmem_base, 512);
   }
+  if (p.beside.early) pdl_wait();                             // whoever waits for this kernel waits for the link side too
 }
 
 template <int NG, int ELL, bool LN>
@@ -530,7 +533,7 @@ static lime_status launch_ht(const HistUpdateArgs& a, cudaStream_t st) {
     return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
   HistUpdateTmemParams p;
   p.out = (__nv_bfloat16*)a.hist_out; p.off = a.off; p.tile_start = a.tile_start; p.B = a.B; p.silu = a.silu;
-  p.cK = a.cK; p.stats_in = a.stats_in; p.shared = a.shared; p.out_ln = a.out_ln; p.ln_eps = a.ln_eps; p.err = a.err;
+  p.cK = a.cK; p.stats_in = a.stats_in; p.shared = a.shared; p.out_ln = a.out_ln; p.ln_eps = a.ln_eps; p.beside = a.beside; p.err = a.err;
   const int grid = a.n_tile_upper < kSMs ? a.n_tile_upper : kSMs;
   if (grid < 1) return LIME_OK;
   static bool smem_set[kMaxDeviceOrdinals] = {};

@@ -109,9 +109,10 @@ k_link_mlp_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   constexpr uint32_t COL_GU = 0, COL_OUT = 256;
-  // set-up done: the next kernel's CTAs may become resident; nothing an earlier kernel wrote is read before this wait
-  pdl_launch_dependents();
+  // set-up done; nothing an earlier kernel wrote is read before this wait.  The signal follows it: a history update that runs beside
+  // this kernel starts behind all that this one waits for (lime_common.cuh)
   pdl_wait();
+  pdl_launch_dependents();
 
   if (warp == 0) {
     if (lane == 0) {

@@ -133,8 +133,8 @@ k_link_side_d128(const LinkSide128Params p) {
     tc::fence_barrier_init();
   }
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  pdl_launch_dependents();
   pdl_wait();
+  pdl_launch_dependents();                                       // behind the wait: lime_common.cuh, the update beside the link side
 
   // ---- [gate | up], the part of head `rank`: warp = hidden columns warp * 8 .. (gate and up)
   {
@@ -329,6 +329,11 @@ k_link_side_d128(const LinkSide128Params p) {
 static int link_side_d128_rows(int64_t rows) { return rows <= 32 * 32 ? 32 : rows <= 32 * 64 ? 64 : 0; }
 bool link_side_d128_wanted(int d, int d_ff, int H, int ell, int64_t users) {
   return d == L1_D && d_ff == L1_D && H == L1_H && ell % 8 == 0 && link_side_d128_rows(users * ell) != 0;
+}
+
+int link_side_d128_blocks(int64_t rows) {
+  const int per = link_side_d128_rows(rows);
+  return per == 0 ? 0 : (int)((rows + per - 1) / per) * L1_CL;
 }
 
 template <class G>

@@ -150,8 +150,8 @@ k_link_side_d256(const LinkSide256Params p) {
     tc::fence_barrier_init();
   }
   l2_arrive();                                                   // this block runs and its barriers exist: it may be written to
-  pdl_launch_dependents();
   pdl_wait();
+  pdl_launch_dependents();                                       // behind the wait: lime_common.cuh, the update beside the link side
 
   // c (columns col, col + 1 of rows m * 16 + g and + 8) to this block's operand buffer at `off`, as value and remainder
   auto store_split = [&](uint32_t off, int m, int col, const float (&c)[4]) {
@@ -391,6 +391,10 @@ k_link_side_d256(const LinkSide256Params p) {
 // 1.76 ms here); 128-row tcgen05 tiles would be full from about 512 users on.
 bool link_side_d256_supported(int d, int d_ff, int H, int ell) { return d == LS2_D && d_ff == LS2_D && ell == LS2_ELL && (H == 4 || H == 8); }
 
+// one user per cluster while the clusters run at once (32 of four blocks do, whatever the SMs per GPC), two beyond
+static int link_side_d256_users(int users) { return users <= 32 ? 1 : 2; }
+int link_side_d256_blocks(int users) { const int per = link_side_d256_users(users); return (users + per - 1) / per * 4; }
+
 template <class G>
 static lime_status launch_ls2(const LinkSide256Params& p, cudaStream_t st) {
   static bool smem_set[kMaxDeviceOrdinals] = {};
@@ -426,8 +430,7 @@ lime_status launch_link_side_d256(const LinkSide256Args& a, cudaStream_t st) {
   p.need_hist = a.need_hist; p.lp_accumulate = a.lp_accumulate; p.ln = a.ln; p.T_out = a.T_out; p.LP = a.LP;
   p.link_states = (__nv_bfloat16*)a.link_states; p.Q2 = (__nv_bfloat16*)a.Q2; p.K2 = (__nv_bfloat16*)a.K2; p.V2t = (__nv_bfloat16*)a.V2t;
   p.scale = a.scale; p.eps = a.eps; p.err = a.err;
-  // one user per cluster while the clusters run at once (32 of four blocks do, whatever the SMs per GPC), two beyond
-  if (a.users <= 32) return a.H == 4 ? launch_ls2<Ls2Cfg<4, 1>>(p, st) : launch_ls2<Ls2Cfg<8, 1>>(p, st);
+  if (link_side_d256_users(a.users) == 1) return a.H == 4 ? launch_ls2<Ls2Cfg<4, 1>>(p, st) : launch_ls2<Ls2Cfg<8, 1>>(p, st);
   return a.H == 4 ? launch_ls2<Ls2Cfg<4, 2>>(p, st) : launch_ls2<Ls2Cfg<8, 2>>(p, st);
 }
 

@@ -111,6 +111,10 @@ static bool encode_small_wanted(const Ctx* c, int32_t B, int64_t total) {
   return (encode_small_supported(g.dtype, g.d, c->d_ff, g.H, g.ell, g.gated_mlp) ||
           encode_f32_supported(g.dtype, g.d, c->d_ff, g.H, g.ell, g.gated_mlp)) && total <= 2048ll * B;
 }
+// d = 128 with few link rows: the link side of a layer is one kernel (k_link_side_d128.cu)
+static bool few_link_rows(const Ctx* c, int64_t B) {
+  return c->tc_mode == 1 && link_side_d128_wanted(c->cfg.d, c->d_ff, c->cfg.H, c->cfg.ell, B);
+}
 constexpr int kHistTile = 128;  // tokens per block of the history<-links attention
 
 struct Workspace {
@@ -123,6 +127,7 @@ struct Workspace {
   float *part_m, *part_s, *part_acc;
   // tensor-core path: folded link-side operands (bf16) and their row sums
   void *Q2, *K2, *G2t, *U2t, *V2t;
+  void *K2b, *G2tb, *U2tb;       // few link rows: the history update's operands of every other layer
   float *cQ, *cK;
   float2* row_stats;   // LayerNorm {rstd, mean} of the history rows of the layer being processed
   void *That, *Ohat, *UTb;   // LN(T) [B*ell x d], merged attention rows [B*ell x H*d], GLU output [B*ell x d_ff] (bf16)
@@ -183,6 +188,8 @@ static Workspace carve(const Ctx* c, void* base, int32_t B, int64_t total) {
   w.Q2 = take((size_t)B * HL * g.d * 2); w.K2 = take((size_t)B * HL * g.d * 2);
   w.G2t = take((size_t)B * c->d_ff * HL * 2); w.U2t = take((size_t)B * c->d_ff * HL * 2);
   w.V2t = take((size_t)B * g.d * g.ell * 2);
+  const size_t second = few_link_rows(c, B) ? (size_t)B * HL * 2 : 0;
+  w.K2b = take(second * g.d); w.G2tb = take(second * c->d_ff); w.U2tb = take(second * c->d_ff);
   w.cQ = (float*)take((size_t)B * HL * 4); w.cK = (float*)take((size_t)B * HL * 4);
   w.row_stats = (float2*)take((size_t)total * 8);
   w.That = take((size_t)B * g.ell * g.d * 2); w.Ohat = take((size_t)B * g.ell * g.H * g.d * 2);
@@ -238,6 +245,15 @@ static lime_status make_link_operands(Ctx* c, int layer, const void* That, int64
   return launch_gemm_prep(gp, st);
 }
 
+// How the update of `tiles` tiles at most shares the SMs with a link side of `blocks` blocks, one per SM, each of which takes as long as
+// `late_by` eighths of a tile of the update: the update's blocks that find no free SM (those of the highest index) start that much later.
+static BesideLinkSide beside_link_side(int64_t blocks, int late_by, int tiles, int B) {
+  if (B > kEarlyUsers) return BesideLinkSide{};
+  const int last = blocks > 0 ? (int)((blocks - 1) % kSMs) + 1 : 0, grid = tiles < kSMs ? tiles : kSMs;      // blocks of its last wave
+  const int late = grid - (kSMs - last);
+  return BesideLinkSide{1, late > 0 ? late : 0, late_by};
+}
+
 // The streaming part of one XOR layer on tensor cores: links<-history attention, GatedMLP on the link rows with its
 // fused consumers (`mlp` carries the outputs wanted), and the history update.  `hist_ln`: apply LayerNorm to the rows
 // read (0 when they were stored normalised by the previous layer); `out_ln`: store LayerNorm(S').
@@ -264,13 +280,32 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
   const bool two_tiles = c->tc_mode == 1 && hist_update_tmem_supported(g.dtype, g.d, c->d_ff, g.H, g.ell, g.phi, g.gated_mlp);
   const bool pass_stats = hist_ln && hist_out && two_tiles && total > 0;
   la.stats_out = pass_stats ? w.row_stats : nullptr;
+  // The link side and the history update need nothing of each other: the update runs beside it (lime_common.cuh), which takes the
+  // shorter of the two off the layer where SMs are free and evens out the tiles where they are not.  Eighths of a tile that a block of
+  // the link side takes, by measurement (us a batch with 0 / 8 / 16 / 20 / 24 / 32 / 40, and with the update behind the link side):
+  // d = 128, three kernels: 256 users x 512, two layers 139.5 / 139.3 / 135.9 / 135.7 / 137.8 / 137.8 / 140.2, 140.3; 150 users of
+  // 100..1500, 64 links, four layers 345.9 / 345.4 / 331.2 / 343.4 / 343.8 / 343.8 / 355.2, 351.6 (a tile of 256 stacked rows takes
+  // longer); one kernel: 40 users of 100..1500 72.3 / 72.3 / 70.5 / 70.3 / 70.5 / 63.0 / 63.0, 74.3; 32 users of 2000..4000, 64 links
+  // 269.8 / 268.8 / 260.4 / 260.2 / 260.5 / 261.6 / 267.8, 276.2; d = 256, 32 links: 64 users of 100..1024, three layers 244.8 / 225.4 /
+  // 224.7 / 226.8 / 226.6 / 245.6 / 264.4, 245.8; 16 users 135.9 / 111.5 / 111.2 / 111.5 / 111.8 / 111.7 / 111.2, 143.5.
+  const int wide = g.H * g.ell > 128;
+  BesideLinkSide beside;
+  if (c->side256) beside = beside_link_side(link_side_d256_blocks(B), 14, w.n_tile_upper, B);
+  else if (side1 != nullptr) beside = beside_link_side(link_side_d128_blocks((int64_t)B * g.ell), wide ? 24 : 30, w.n_tile_upper, B);
+  else beside = beside_link_side(((int64_t)B * g.ell + 127) / 128, c->tc_mode == 2 ? 44 : wide ? 16 : 20, w.n_tile_upper, B);
   if ((s = c->tc_mode == 2 ? launch_link_attn_d256_tc(la, st) : launch_link_attn_tc(la, st)) != LIME_OK) return s;
   if (c->side256) {
     // merge, T^j and what follows from it - the next layer's operands included - in one kernel; `side` says what is wanted
     LinkSide256Args a = *side;
     a.Ohat = w.Ohat; a.part_m = w.part_m; a.part_s = w.part_s; a.part_acc = w.part_acc; a.chunk_start = w.chunk_start;
     if ((s = launch_link_side_d256(a, st)) != LIME_OK) return s;
-  } else if (side1 == nullptr) {
+  } else if (side1 != nullptr) {
+    // few link rows: merge, T^j and the next layer's operands in one kernel
+    LinkSide128Args a = *side1;
+    a.users = B; a.ell = g.ell; a.Ohat = w.Ohat; a.part_m = w.part_m; a.part_s = w.part_s; a.part_acc = w.part_acc;
+    a.chunk_start = w.chunk_start; a.WpostT = c->WpostT[layer]; a.WoT = c->WoT[layer]; a.ln = g.ln; a.eps = c->ln_eps; a.err = c->dev_err;
+    if ((s = launch_link_side_d128(a, st)) != LIME_OK) return s;
+  } else {
   if ((s = launch_link_attn_merge_norm(w.chunk_start, w.merge_needed, B, g.ell, g.d, g.H, w.part_m, w.part_s, w.part_acc, w.Ohat, st)) != LIME_OK)
     return s;
   // T^j = GatedMLP(O[T]) with W_V folded into the gate / up weights, and what the next step needs from it
@@ -282,7 +317,7 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
     HistUpdate256Args hu{};
     hu.hist_in = hist_in; hu.hist_out = hist_out; hu.total = total; hu.K2 = ops.K2; hu.V2t = ops.V2t; hu.WguT = c->WguT[layer];
     hu.WoT = c->WoT[layer]; hu.off = off; hu.tile_start = w.tile_start; hu.B = B; hu.n_tile_upper = w.n_tile_upper; hu.H = g.H; hu.ell = g.ell;
-    hu.shared = ops.shared; hu.out_ln = out_ln; hu.silu = g.phi == LIME_PHI_SILU; hu.ln_eps = c->ln_eps; hu.err = c->dev_err;
+    hu.shared = ops.shared; hu.out_ln = out_ln; hu.silu = g.phi == LIME_PHI_SILU; hu.ln_eps = c->ln_eps; hu.beside = beside; hu.err = c->dev_err;
     if ((s = launch_hist_update_d256_tc(hu, st)) != LIME_OK) return s;
   } else if (hist_out) {
     // history attends back over the links; scores, per-head softmax, value mix and GatedMLP in one fused kernel
@@ -291,17 +326,10 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
     hu.cK = ops.cK; hu.WoT = c->WoT[layer]; hu.off = off; hu.tile_start = w.tile_start; hu.B = B;
     hu.n_tile_upper = w.n_tile_upper; hu.ell = g.ell; hu.shared = ops.shared; hu.ln = hist_ln; hu.ln_eps = c->ln_eps;
     hu.out_ln = out_ln; hu.silu = g.phi == LIME_PHI_SILU; hu.err = c->dev_err;
-    hu.stats_in = pass_stats ? w.row_stats : nullptr;
+    hu.stats_in = pass_stats ? w.row_stats : nullptr; hu.beside = beside;
     if (two_tiles) s = launch_hist_update_tmem(hu, g.H, st);
     else s = launch_hist_update2_tc(hu, st);
     if (s != LIME_OK) return s;
-  }
-  if (side1 != nullptr) {
-    // few link rows: merge, T^j and the next layer's operands in one kernel, behind the history update that reads this layer's
-    LinkSide128Args a = *side1;
-    a.users = B; a.ell = g.ell; a.Ohat = w.Ohat; a.part_m = w.part_m; a.part_s = w.part_s; a.part_acc = w.part_acc;
-    a.chunk_start = w.chunk_start; a.WpostT = c->WpostT[layer]; a.WoT = c->WoT[layer]; a.ln = g.ln; a.eps = c->ln_eps; a.err = c->dev_err;
-    if ((s = launch_link_side_d128(a, st)) != LIME_OK) return s;
   }
   return LIME_OK;
 }
@@ -363,7 +391,10 @@ static lime_status encode_user_tc(Ctx* c, const void* hist, bool hist_normalized
     }
     return LIME_OK;
   }
-  const bool few_rows = c->tc_mode == 1 && link_side_d128_wanted(g.d, c->d_ff, g.H, g.ell, B);
+  // few link rows: the link side of layer j writes the operands of layer j + 1 while the update of layer j reads its own, so these
+  // alternate between two sets (Q2 is the attention's, complete by then)
+  const bool few_rows = few_link_rows(c, B);
+  const LinkOperands set[2] = {{w.Q2, w.K2, w.G2t, w.U2t, w.V2t, w.cQ, w.cK, 0}, {w.Q2, w.K2b, w.G2tb, w.U2tb, w.V2t, w.cQ, w.cK, 0}};
   for (int j = 0; j < g.n_layers; ++j) {
     const bool last = j == g.n_layers - 1;
     const bool raw = g.ln && j == 0 && !hist_normalized;      // rows that still need their LayerNorm want the operands' row sums
@@ -375,14 +406,15 @@ static lime_status encode_user_tc(Ctx* c, const void* hist, bool hist_normalized
       if ((j == 0 || !few_rows) &&
           (s = make_link_operands(c, j, w.That, BL, !last, w.Q2, w.K2, w.G2t, w.U2t, w.V2t, raw ? w.cQ : nullptr, raw ? w.cK : nullptr, st)) != LIME_OK)
         return s;
-      ops = LinkOperands{w.Q2, w.K2, w.G2t, w.U2t, w.V2t, w.cQ, w.cK, 0};
+      ops = set[few_rows ? j & 1 : 0];
     }
     LinkSide128Args side1{};
     if (few_rows) {
       side1.LP = w.LP; side1.lp_accumulate = j > 0; side1.need_hist = j + 1 < g.n_layers - 1;
       side1.WprepT = last ? nullptr : c->WprepT[j + 1];
       side1.link_states = (last && !c->w.cand_Wv && c->cand_heads == 1) ? link_states : nullptr;
-      side1.Q2 = w.Q2; side1.K2 = w.K2; side1.G2t = w.G2t; side1.U2t = w.U2t;
+      const LinkOperands& nx = set[(j + 1) & 1];
+      side1.Q2 = w.Q2; side1.K2 = const_cast<void*>(nx.K2); side1.G2t = const_cast<void*>(nx.G2t); side1.U2t = const_cast<void*>(nx.U2t);
     }
     LinkMlpArgs mlp{};
     mlp.LP = w.LP; mlp.lp_accumulate = j > 0;                                   // L^P = sum_j T^j  (Eq. 8)

@@ -150,6 +150,11 @@ lime_status cuda_fail(cudaError_t e, const char* where);
 //  - a kernel that allocates tensor memory calls pdl_launch_dependents() only after its allocation, so a dependent CTA
 //    that shares the SM can never hold the columns a CTA of the running kernel still waits for.
 // A kernel launched the ordinary way after such a kernel still waits for its completion, as always.
+//
+// A history update may run BESIDE the link side of its layer, launched right before it (`early`): the two read the attention's
+// result and the layer's operands and write different things.  The link-side kernels signal their dependents behind their own
+// pdl_wait(), so an update that starts finds everything up to the attention complete; it reads that past L1, and waits at its
+// end, so that whoever waits for the update has waited for the link side as well.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -159,6 +164,16 @@ __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefe
 __device__ __forceinline__ void prefetch_l2_row(const void* p, int bytes) {
   const uintptr_t a = reinterpret_cast<uintptr_t>(p);
   for (uintptr_t l = a & ~(uintptr_t)127; l < a + bytes; l += 128) prefetch_l2(reinterpret_cast<const void*>(l < a ? a : l));
+}
+#endif
+#ifdef __CUDACC__
+// First tile of block `cta` when the `n` tiles are split in order among `grid` blocks, of which the last `late` start when the others
+// are `late_by` eighths of a tile ahead (they wait for the SMs that the link side holds).
+__device__ __forceinline__ int early_first_tile(int cta, int grid, int n, int late, int late_by) {
+  const int64_t first = grid - late, share = 8 * (int64_t)n + (int64_t)late * late_by;       // share / (8 grid): tiles of an early block
+  if (share < (int64_t)grid * late_by) return cta >= first ? n : (int)(cta * (int64_t)n / first);
+  const int64_t behind = cta > first ? (cta - first) * (int64_t)grid * late_by : 0;
+  return (int)((cta * share - behind) / (8 * (int64_t)grid));
 }
 #endif
 bool pdl_enabled();      // environment LIME_PDL=0 turns the attribute off (every launch then serialises fully)
@@ -407,6 +422,9 @@ int link_attn_d256_groups(int n_chunk_upper, int H, int ell);   // groups of CTA
 lime_status launch_link_attn_tc(const LinkAttnArgs& a, cudaStream_t st);
 lime_status launch_link_attn_d128_tmem(const LinkAttnArgs& a, cudaStream_t st);   // the same for rows LayerNorm-ed already (a.ln must be 0)
 
+// An update that runs beside the link side of its layer: 1, and how many of its blocks start later and by how much (see above).
+struct BesideLinkSide { int early, late, late_by; };
+constexpr int kEarlyUsers = 1024;         // at most: their offsets are staged in shared memory, past L1
 struct HistUpdateArgs {
   const void* hist_in; void* hist_out; int64_t total;
   const void *K2, *G2t, *U2t; const float* cK; const void* WoT;   // WoT [d x f] bf16 (W_o transposed)
@@ -415,6 +433,7 @@ struct HistUpdateArgs {
   int out_ln;                           // 1: store LayerNorm(S') instead of S'
   int silu;                             // 1: SiLU(s) / ell instead of the per-head softmax (Algorithm 2)
   const float2* stats_in;               // nullable, ln only: {rstd, mean} of every row read, as left by the attention kernel
+  BesideLinkSide beside;                // k_hist_update_tmem_tc.cu only
   int* err;
 };
 bool hist_update_tmem_supported(int dtype, int d, int f, int H, int ell, int phi, int gated_mlp);     // H * ell = 128 or 256
@@ -442,6 +461,7 @@ struct LinkSide256Args {
 };
 bool link_side_d256_supported(int d, int d_ff, int H, int ell);
 lime_status launch_link_side_d256(const LinkSide256Args& a, cudaStream_t st);
+int link_side_d256_blocks(int users);
 
 // the same for d = 128 with four heads and few link rows: merge, GatedMLP and the next layer's operands (k_link_side_d128.cu)
 struct LinkSide128Args {
@@ -456,6 +476,7 @@ struct LinkSide128Args {
 };
 bool link_side_d128_wanted(int d, int d_ff, int H, int ell, int64_t users);
 lime_status launch_link_side_d128(const LinkSide128Args& a, cudaStream_t st);
+int link_side_d128_blocks(int64_t rows);
 
 struct HistUpdate256Args {
   const void* hist_in; void* hist_out; int64_t total;
@@ -467,6 +488,7 @@ struct HistUpdate256Args {
   int out_ln;                           // 1: store LayerNorm(S') instead of S'
   int silu;                             // 1: SiLU(s) / ell instead of the per-head softmax (Algorithm 2)
   float ln_eps;
+  BesideLinkSide beside;
   int* err;
 };
 bool hist_update_d256_tc_supported(int dtype, int d, int f, int H, int ell, int phi, int gated_mlp);

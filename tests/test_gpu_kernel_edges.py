@@ -397,6 +397,15 @@ def test_chunk_length_chosen_from_the_lengths(d, H, ell, lengths, phi, raw):
     _encode_against_oracle(synth.BF16, d, H, ell, 2, lengths, phi, raw, False, 6e-2, 4e-2 if phi == "silu" else 2.5e-2)
 
 
+@pytest.mark.parametrize("d,H,ell", [(128, 4, 32), (128, 4, 64), (256, 4, 32), (256, 2, 64)])
+@pytest.mark.parametrize("lengths", [[1], [129] * 2 + [0], [20] * 32, [300] * 40 + [1], [128] * 66, [140] * 150])
+@pytest.mark.parametrize("raw", [False, True])
+def test_history_update_beside_the_link_side(d, H, ell, lengths, raw):
+    """Three layers, so that the update of a layer runs beside the link side that writes the operands of the next: blocks that all find
+    an SM, blocks that start late and get fewer tiles or none, a link side of more than one wave."""
+    _encode_against_oracle(synth.BF16, d, H, ell, 3, lengths, "softmax", raw, True, 6e-2, 3e-2)
+
+
 def test_one_long_history_is_split_among_many_users():
     """One user of 4000 tokens among 99 of 100, against 100 users of 100 (d = 128): 1.46 times the time where a history is one work item
     whenever the users are many, 1.16 times split."""
