@@ -215,6 +215,29 @@ def test_three_layer_interaction_network(ell, w0, counts, form):
         assert np.all(got[~ok] == 0.0) and int(flag.item()) == total // 2
 
 
+@pytest.mark.parametrize("ell,w0", [(8, 64), (16, 512), (32, 256)])
+@pytest.mark.parametrize("total", [148 * 128, 148 * 128 + 1, 148 * 192, 148 * 192 + 1, 148 * 256 + 1, 2 * 148 * 256 + 7])
+def test_three_layer_interaction_network_of_any_number_of_candidates(ell, w0, total):
+    """128, 192 or 256 slots a block by how full the last round is: a candidate's logit is the same sums in the same order whichever it
+    is, so a large call gives the bits of the same candidates scored a thousand at a time."""
+    Bd = _lib()
+    d, V, B = 32, 500, 7
+    g = torch.Generator("cuda").manual_seed(total)
+    rand = lambda *shape: torch.randn(shape, generator=g, device="cuda").to(torch.bfloat16)
+    lime = Bd.Lime(d, 4, ell, 1, dtype=Bd.LIME_BF16)
+    lime.set_head([(Bd.to_device(w, synth.BF16), torch.from_numpy(b).cuda()) for w, b in synth.ffn_weights(5, "head", (2 * d, w0, 128, 64, 1), synth.BF16)])
+    LS, W, T = rand(B, ell, d), torch.softmax(rand(V, ell).float(), 1).to(torch.bfloat16), rand(V, d)
+    ids = torch.randint(0, V, (total,), generator=g, device="cuda", dtype=torch.int32)
+    cuts = [0, 1, 17, total // 3, total // 3, total // 2 + 5, total - 3, total]           # one user without candidates
+    score = lambda ls, i, off: lime.score_candidates_head(ls, W, T, C=0, total_cands=len(i), cand_ids=i,
+                                                          cand_off=torch.tensor(off, dtype=torch.int32, device="cuda"))
+    got = score(LS, ids, cuts)
+    for b in range(B):
+        for s in range(cuts[b], cuts[b + 1], 1000):
+            e = min(s + 1000, cuts[b + 1])
+            assert torch.equal(got[s:e], score(LS[b:b + 1], ids[s:e].contiguous(), [0, e - s]))
+
+
 @pytest.mark.parametrize("H,ell", [(2, 8), (4, 8), (2, 16)])
 @pytest.mark.parametrize("lengths", [[1], [0, 15, 100, 257, 3], [1500, 3, 700], [64] * 4, [60] * 300])
 @pytest.mark.parametrize("phi,raw,per_user", [("softmax", False, False), ("silu", False, True), ("softmax", True, True)])
