@@ -12,7 +12,10 @@
 //   warp 1    : MMA issuer   - d/16 tcgen05.mma (M=128, N=2 ell, K=16) per tile into one of two TMEM accumulators
 //   warps 2-5 : epilogue     - thread r owns item row r (TMEM lane r): row softmax in registers, bf16 row to global
 //                              (GROUP < ELL: the ELL keys are ELL / GROUP heads' keys and the softmax runs per head)
-// HBM traffic per item is the algorithmic minimum: its embedding row in, its weight row out.
+// HBM traffic per item is the algorithmic minimum: its embedding row in, its weight row out, which is what bounds it.  Rows of a
+// weight row's 64 or 128 bytes stored by a thread each reach L2 in 16-byte pieces; four lanes transposed, as pieces of 64 bytes:
+// 1,000,000 items, d = 128, back to back on the same items: 32 links 53.2 -> 52.7 us, 64 links 79.8 -> 69.2; 500,000, d = 256, 64
+// links 53.0 -> 50.0.  Programmatic launch before that: 56.2 -> 53.4, 83.5 -> 80.2, 55.2 -> 53.
 #include "lime_common.cuh"
 #include "tc_common.cuh"
 
@@ -50,6 +53,14 @@ lime_status launch_keff_split(const float* keff, int ell, int d, void* out, cuda
 __device__ __forceinline__ uint32_t pct_pack(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
+}
+
+// lanes with `upper` clear give away hi and receive into it; lanes with it set give away lo
+__device__ __forceinline__ void pct_xchg(uint4& lo, uint4& hi, bool upper, int dist) {
+  uint4 v = upper ? lo : hi;
+  v.x = __shfl_xor_sync(0xffffffffu, v.x, dist); v.y = __shfl_xor_sync(0xffffffffu, v.y, dist);
+  v.z = __shfl_xor_sync(0xffffffffu, v.z, dist); v.w = __shfl_xor_sync(0xffffffffu, v.w, dist);
+  if (upper) lo = v; else hi = v;
 }
 
 template <int ELL, int GROUP>
@@ -95,6 +106,9 @@ k_precompute_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // set-up done: the next kernel's CTAs may become resident; nothing is read or written before this wait
+  pdl_launch_dependents();
+  pdl_wait();
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -193,17 +207,29 @@ k_precompute_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__
 #pragma unroll
         for (int j = 0; j < GROUP; ++j) sc[g0 + j] *= inv;
       }
-      if (row < p.M) {
+      auto chunk = [&](int c8) -> uint4 {
+        return make_uint4(pct_pack(sc[c8 * 8 + 0], sc[c8 * 8 + 1]), pct_pack(sc[c8 * 8 + 2], sc[c8 * 8 + 3]),
+                          pct_pack(sc[c8 * 8 + 4], sc[c8 * 8 + 5]), pct_pack(sc[c8 * 8 + 6], sc[c8 * 8 + 7]));
+      };
+      if constexpr (ELL >= 32) {
+        // four chunks of 16 bytes at a time, transposed among four lanes: lane 4 j + i stores chunk i of rows 4 j .. 4 j + 3, so that a
+        // store writes whole 64-byte pieces of rows
+        uint4* dst = reinterpret_cast<uint4*>(p.out + (row - (lane & 3)) * ELL) + (lane & 3);
+#pragma unroll
+        for (int c0 = 0; c0 < ELL / 8; c0 += 4) {
+          uint4 o[4] = {chunk(c0), chunk(c0 + 1), chunk(c0 + 2), chunk(c0 + 3)};
+          pct_xchg(o[0], o[1], (lane & 1) != 0, 1);
+          pct_xchg(o[2], o[3], (lane & 1) != 0, 1);
+          pct_xchg(o[0], o[2], (lane & 2) != 0, 2);
+          pct_xchg(o[1], o[3], (lane & 2) != 0, 2);
+#pragma unroll
+          for (int m = 0; m < 4; ++m)
+            if (row - (lane & 3) + m < p.M) __stcs(dst + m * (ELL / 8) + c0, o[m]);
+        }
+      } else if (row < p.M) {
         uint4* dst = reinterpret_cast<uint4*>(p.out + row * ELL);
 #pragma unroll
-        for (int c8 = 0; c8 < ELL / 8; ++c8) {
-          uint4 o;
-          o.x = pct_pack(sc[c8 * 8 + 0], sc[c8 * 8 + 1]);
-          o.y = pct_pack(sc[c8 * 8 + 2], sc[c8 * 8 + 3]);
-          o.z = pct_pack(sc[c8 * 8 + 4], sc[c8 * 8 + 5]);
-          o.w = pct_pack(sc[c8 * 8 + 6], sc[c8 * 8 + 7]);
-          __stcs(dst + c8, o);
-        }
+        for (int c8 = 0; c8 < ELL / 8; ++c8) __stcs(dst + c8, chunk(c8));
       }
     }
   }
@@ -250,9 +276,11 @@ static lime_status launch_precompute_tc_t(const void* cand, int64_t M, int d, co
   p.n_tiles = (int)((M + PCT_TILE - 1) / PCT_TILE);
   p.stages = S; p.err = err;
   const int grid = p.n_tiles < kSMs ? p.n_tiles : kSMs;
-  LIME_CUDA(cudaFuncSetAttribute(k_precompute_tc<ELL, GROUP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  static bool smem_set[kMaxDeviceOrdinals] = {};
+  const lime_status es = ensure_dynamic_smem((const void*)k_precompute_tc<ELL, GROUP>, 232448, smem_set);      // any d
+  if (es != LIME_OK) return es;
   ProfScope _p("k_precompute_tc", st);
-  k_precompute_tc<ELL, GROUP><<<grid, PCT_THREADS, smem, st>>>(tmT, tmK, p);
+  launch_pdl(k_precompute_tc<ELL, GROUP>, dim3(grid), dim3(PCT_THREADS), smem, st, tmT, tmK, p);
   LIME_LAUNCH_CHECK("k_precompute_tc");
   return LIME_OK;
 }

@@ -62,6 +62,24 @@ def test_precompute_narrow(dtype, d, ell, M):
     assert np.abs(got - want).max() <= (1e-6 if dtype == synth.F32 else 2.0 ** -8)
 
 
+@pytest.mark.parametrize("d,ell", [(64, 16), (128, 32), (256, 64), (128, 128)])
+@pytest.mark.parametrize("M", [1, 3, 5, 127, 130, 148 * 128 + 2])
+def test_precompute_last_rows(d, ell, M):
+    """Rows leave four at a time: a last group of one to four rows, at the start and the end of a warp's 32.  The row behind the last is
+    not written; an output is rounded once (2^-9 of 1) behind keys that carry 2^-17."""
+    Bd = _lib()
+    lime = Bd.Lime(d, 1 if d <= 128 else 2, ell, 1, dtype=Bd.LIME_BF16, gated_mlp=False)
+    L, T = synth.normal_storage(1, "l", (ell, d), 1.0, synth.BF16), synth.normal_storage(1, "t", (M, d), 1.0, synth.BF16)
+    lime.set_weights(Bd.to_device(L, synth.BF16), [{}])
+    out = torch.full((M + 4, ell), -1.0, dtype=torch.bfloat16, device="cuda")
+    Bd.lime_precompute_candidate_links(lime.ctx, Bd.to_device(T, synth.BF16), out)
+    assert torch.equal(out[M:], torch.full_like(out[M:], -1.0))
+    cfg = O.OracleConfig(d=d, H=1, ell=ell, n_layers=1)
+    rows = np.unique(np.concatenate([np.arange(min(M, 300)), np.arange(max(0, M - 300), M)]))
+    want = O.precompute_candidate_links(synth.storage_to_f64(T, synth.BF16)[rows], synth.storage_to_f64(L, synth.BF16), cfg)
+    assert np.abs(Hh.to_f64(out)[rows] - want).max() <= 2.0 ** -8
+
+
 def _layer_against_oracle(dtype, d, H, ell, lengths, shared, phi, tol_max, tol_mean):
     """One XOR layer with a history update, per user against the oracle."""
     Bd = _lib()
