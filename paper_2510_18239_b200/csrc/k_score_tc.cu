@@ -20,12 +20,21 @@ namespace lime {
 constexpr int SCT_TILE = 128;
 constexpr int SCT_THREADS = 192;
 constexpr int SCT_MAX_STAGES = 8;
+// Tiles moved into L2 while the links are still encoded, HBM idle: spread evenly over all of them, so that every CTA finds some there and
+// streams the others meanwhile, and requested by the first blocks alone, which find an SM that the last link-side kernel (128 blocks at
+// most) leaves free.  64 users of 1024 tokens, with 0 / 8 / 24 / 40 MB: 8192 candidates 111.8 / 110.9 / 110.5 / 110.9 us, 24576 163.3 /
+// 161.3 / 160.1 / 160.7, 32768 186.3 / 184.7 / 184.4 / 185.2; 256 users x 512, 2048 candidates 136.0 / 135.4 / 135.5 / 136.0; 8 users, whose
+// link side is short, 32768 candidates 56.8 / 56.3 / 59.6 / 60.4.  (Each block for its own first tiles: 3 us slower; a small kernel of
+// its own ahead of the scorer: 183 for the 32768, 2 us more for the others.)
+constexpr int SCT_AHEAD_BLOCKS = 16, SCT_AHEAD_BYTES = 8000000;
 
 struct ScoreTcParams {
   float* logits;
   int B, C, d;
   int tiles_per_user, n_tiles;
   int stages;
+  int n_ahead, total;              // tiles moved into L2 before the link states exist, candidates
+  const char *T, *W;
   int* err;
 };
 
@@ -75,6 +84,15 @@ k_score_tc(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUte
   const uint32_t tmem_base = *tmem_slot;
   // set-up done: the next kernel's CTAs may become resident; nothing an earlier kernel wrote is read before this wait
   pdl_launch_dependents();
+  if (blockIdx.x < SCT_AHEAD_BLOCKS && warp == 2) {
+    for (int k = blockIdx.x * 32 + lane; k < p.n_ahead; k += SCT_AHEAD_BLOCKS * 32) {
+      const int t = (int)((int64_t)k * p.n_tiles / p.n_ahead);
+      const int64_t row0 = (int64_t)(t / p.tiles_per_user) * p.C + (t % p.tiles_per_user) * SCT_TILE;
+      const uint32_t rows = (uint32_t)min((int64_t)SCT_TILE, p.total - row0);
+      bulk_prefetch_l2(p.T + row0 * p.d * 2, rows * (uint32_t)p.d * 2);
+      bulk_prefetch_l2(p.W + row0 * ELL * 2, rows * ELL * 2);
+    }
+  }
   pdl_wait();
 
   if (warp == 0) {
@@ -237,6 +255,8 @@ static lime_status launch_score_tc_t(const ScoreArgs& a, int* err, cudaStream_t 
   p.tiles_per_user = (a.C + SCT_TILE - 1) / SCT_TILE;
   p.n_tiles = p.tiles_per_user * a.B;
   p.stages = S; p.err = err;
+  p.total = (int)a.total; p.T = (const char*)a.T; p.W = (const char*)a.W;
+  p.n_ahead = SCT_AHEAD_BYTES / (SCT_TILE * (a.d + ELL) * 2) < p.n_tiles ? SCT_AHEAD_BYTES / (SCT_TILE * (a.d + ELL) * 2) : p.n_tiles;
   int grid = p.n_tiles < kSMs ? p.n_tiles : kSMs;
   static bool smem_set[kMaxDeviceOrdinals] = {};
   const lime_status es = ensure_dynamic_smem((const void*)k_score_tc<ELL>, 227 * 1024, smem_set);      // `smem` differs by d

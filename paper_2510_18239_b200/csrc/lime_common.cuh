@@ -144,8 +144,8 @@ lime_status cuda_fail(cudaError_t e, const char* where);
 // kernel's CTAs may become resident while its predecessor still runs (as soon as every CTA of the predecessor has
 // executed pdl_launch_dependents() or exited), set up their barriers and tensor memory, and then block in pdl_wait()
 // until the predecessor has completed and its writes are visible.  Rules kept by every kernel launched this way:
-//  - nothing produced by an earlier kernel is read, and no global memory is written, before pdl_wait().  The warp-level scorer
-//    (k_score_rows.cu) does ask L2 for candidate rows before it: prefetches hold no value, and ids read that early only choose
+//  - nothing produced by an earlier kernel is read, and no global memory is written, before pdl_wait().  Two scorers (k_score_rows.cu,
+//    k_score_tc.cu) do ask L2 for candidate rows before it: prefetches hold no value, and ids read that early only choose
 //    what to prefetch, past L1, and are read again afterwards;
 //  - a kernel that allocates tensor memory calls pdl_launch_dependents() only after its allocation, so a dependent CTA
 //    that shares the SM can never hold the columns a CTA of the running kernel still waits for.
