@@ -2,7 +2,8 @@
 
 Functions carry the C entry points' names and take torch CUDA tensors (used purely as device memory) plus
 plain integers; every step of the path runs inside the library's kernels.  There is no CPU fallback: if the
-shared library is missing or a call fails, an exception is raised.
+shared library is missing or a call fails, an exception is raised.  The calls that `Lime` makes per request go
+through `_torch_binding`, the same marshalling in native code (csrc/torch_binding.cpp).
 """
 from __future__ import annotations
 
@@ -114,6 +115,23 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
 def _lib() -> ctypes.CDLL:
     """The loaded library (every call goes through here: one global read once it is loaded)."""
     return _lib_handle if _lib_handle is not None else load_library()
+
+
+_native_module = None
+
+
+def _native():
+    """The native half of this binding, joined to the loaded library.  Raises if it has not been built."""
+    global _native_module
+    if _native_module is None:
+        load_library()
+        try:
+            from . import _torch_binding
+        except ImportError as e:
+            raise RuntimeError("_torch_binding.so is missing: build it with `python -m paper_2510_18239_b200.build`") from e
+        _torch_binding.load(LIB_PATH, LimeError)
+        _native_module = _torch_binding
+    return _native_module
 
 
 def _check(status: int, where: str):
@@ -340,6 +358,7 @@ class Lime:
         self.cfg = lime_config(d, H, ell, n_layers, d_ff, dtype, phi, int(ln), int(gated_mlp), attn_scale, cand_scale, ln_eps,
                                cand_heads)
         self.ell_c = ell * (H if cand_heads == H and H > 1 else 1)      # weight columns per candidate, link-state rows
+        self._native = _native()
         self.ctx = lime_create(self.cfg)
         self.tdtype = torch_dtype(dtype)
         self._keep = []
@@ -386,48 +405,31 @@ class Lime:
         return self._ws
 
     def lengths_to_offsets(self, lengths: torch.Tensor) -> torch.Tensor:
-        off = lengths.new_empty(lengths.numel() + 1)           # int32 on the same device, as the lengths are
-        lime_lengths_to_offsets(self.ctx, lengths, off)
-        return off
+        return self._native.lengths_to_offsets(self.ctx, lengths)          # int32 on the same device, as the lengths are
 
     def gather_history(self, table: torch.Tensor, ids: torch.Tensor, flag: Optional[torch.Tensor] = None) -> torch.Tensor:
-        out = table.new_empty((ids.numel(), self.d))
-        lime_gather_history(self.ctx, table, ids, out, flag)
-        return out
+        return self._native.gather_history(self.ctx, self.d, table, ids, flag)
 
     def gather_history_normalized(self, table: torch.Tensor, ids: torch.Tensor,
                                   flag: Optional[torch.Tensor] = None) -> torch.Tensor:
-        out = table.new_empty((ids.numel(), self.d))
-        lime_gather_history_normalized(self.ctx, table, ids, out, flag)
-        return out
+        return self._native.gather_history_normalized(self.ctx, self.d, table, ids, flag)
 
     def encode_user_normalized(self, hist_normalized: torch.Tensor, off: torch.Tensor,
                                link_ctx: Optional[torch.Tensor] = None) -> torch.Tensor:
-        B = off.numel() - 1
-        ls = hist_normalized.new_empty((B, self.ell_c, self.d))
-        lime_encode_user_normalized(self.ctx, hist_normalized, off, B, link_ctx, ls, self.workspace(B, hist_normalized.shape[0]))
-        return ls
+        return self._native.encode_user_normalized(self.ctx, self.ell_c, self.d, hist_normalized, off, link_ctx,
+                                                   self.workspace(off.numel() - 1, hist_normalized.shape[0]))
 
     def precompute_candidate_links(self, cand_emb: torch.Tensor) -> torch.Tensor:
-        out = cand_emb.new_empty((cand_emb.shape[0], self.ell_c))
-        lime_precompute_candidate_links(self.ctx, cand_emb, out)
-        return out
+        return self._native.precompute_candidate_links(self.ctx, self.ell_c, cand_emb)
 
     def encode_user(self, hist: torch.Tensor, off: torch.Tensor, link_ctx: Optional[torch.Tensor] = None) -> torch.Tensor:
-        B = off.numel() - 1
-        ls = hist.new_empty((B, self.ell_c, self.d))
-        lime_encode_user(self.ctx, hist, off, B, link_ctx, ls, self.workspace(B, hist.shape[0]))
-        return ls
+        return self._native.encode_user(self.ctx, self.ell_c, self.d, hist, off, link_ctx, self.workspace(off.numel() - 1, hist.shape[0]))
 
     def score_candidates(self, link_states: torch.Tensor, cand_w: torch.Tensor, cand_emb: torch.Tensor, C: int = 0,
                          cand_off: Optional[torch.Tensor] = None, cand_ids: Optional[torch.Tensor] = None,
                          total_cands: Optional[int] = None, corpus_rows: Optional[int] = None,
                          dev_flag: Optional[torch.Tensor] = None) -> torch.Tensor:
-        B = link_states.shape[0]
-        total = total_cands if total_cands is not None else (cand_ids.numel() if cand_ids is not None else cand_emb.shape[0])
-        logits = torch.empty(total, dtype=torch.float32, device=link_states.device)
-        lime_score_candidates(self.ctx, link_states, B, cand_w, cand_emb, cand_off, C, total, cand_ids, logits, corpus_rows, dev_flag)
-        return logits
+        return self._native.score_candidates(self.ctx, link_states, cand_w, cand_emb, C, cand_off, cand_ids, total_cands, corpus_rows, dev_flag)
 
     def pack_corpus_cache(self, cand_emb: torch.Tensor, cand_w: torch.Tensor) -> torch.Tensor:
         packed = torch.empty((cand_emb.shape[0], self.cfg.d + self.ell_c), dtype=self.tdtype, device=cand_emb.device)
@@ -460,12 +462,8 @@ class Lime:
                               cand_off: Optional[torch.Tensor] = None, cand_ids: Optional[torch.Tensor] = None,
                               total_cands: Optional[int] = None, corpus_rows: Optional[int] = None,
                               dev_flag: Optional[torch.Tensor] = None) -> torch.Tensor:
-        B = link_states.shape[0]
-        total = total_cands if total_cands is not None else (cand_ids.numel() if cand_ids is not None else cand_emb.shape[0])
-        logits = torch.empty(total, dtype=torch.float32, device=link_states.device)
-        need = lime_head_workspace_bytes(self.ctx, B)
+        need = lime_head_workspace_bytes(self.ctx, link_states.shape[0])
         if self._head_ws is None or self._head_ws.numel() < need:
             self._head_ws = torch.empty(need, dtype=torch.uint8, device=link_states.device)
-        lime_score_candidates_head(self.ctx, link_states, B, cand_w, cand_emb, cand_off, C, total, cand_ids, logits,
-                                   self._head_ws, corpus_rows, dev_flag)
-        return logits
+        return self._native.score_candidates_head(self.ctx, link_states, cand_w, cand_emb, C, cand_off, cand_ids, total_cands, corpus_rows,
+                                                  dev_flag, self._head_ws)

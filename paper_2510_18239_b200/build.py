@@ -1,6 +1,7 @@
 """In-tree build of the C-ABI CUDA library (sm_100a) with nvcc.
 
-`build()` compiles every `csrc/*.cu` to an object file and links `liblime_b200.so` next to this file.
+`build()` compiles every `csrc/*.cu` to an object file and links `liblime_b200.so` next to this file, and beside it
+`_torch_binding.so`, the native half of `binding.py` (`csrc/torch_binding.cpp`, host code only).
 Objects are rebuilt only when a source or header is newer.  nvcc cross-compiles without a GPU.
 """
 from __future__ import annotations
@@ -11,12 +12,14 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "liblime_b200.so")
+BINDING = os.path.join(HERE, "_torch_binding.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -36,7 +39,28 @@ def _newest(paths) -> float:
     return max(os.path.getmtime(p) for p in paths)
 
 
+def build_binding() -> str:
+    src = os.path.join(CSRC, "torch_binding.cpp")
+    needs = [src, os.path.join(ROOT, "include", "lime.h"), __file__]
+    if os.path.exists(BINDING) and os.path.getmtime(BINDING) >= _newest(needs):
+        return BINDING
+    import torch
+    home = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    includes = [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], os.path.join(home, "include"),
+                os.path.join(home, "include", "torch", "csrc", "api", "include"), os.path.join(cuda, "include")]
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", src, "-o", BINDING]
+    cmd += [f"-I{i}" for i in includes] + [f"-L{os.path.join(home, 'lib')}", "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-ldl"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(r.stdout + r.stderr)
+        raise RuntimeError("g++ failed on " + src)
+    return BINDING
+
+
 def build(verbose: bool = False, ptxas_info: bool = False) -> str:
+    build_binding()
     os.makedirs(OBJ, exist_ok=True)
     sources = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
     headers = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h")) + [__file__]

@@ -58,3 +58,22 @@ def test_ffn_entry_points_validate_on_the_host():
     assert lib.lime_contextualize_links(None, None, 1, None, None) == 1
     assert lib.lime_head_workspace_bytes(None, 4) == 0
     assert lib.lime_score_candidates_head(None, None, 1, None, None, None, 1, 1, None, 0, None, None, None, 0, None) == 1
+
+
+def test_native_binding_refuses_what_is_no_cuda_tensor():
+    """The native half of the binding loads without a GPU and checks what it is given before anything is launched."""
+    import pytest
+    import torch
+    native = binding._native()
+    with pytest.raises(TypeError):
+        native.lengths_to_offsets(None, [1, 2])
+    with pytest.raises(TypeError):
+        native.encode_user(None, 8, 32)
+    cpu = torch.zeros((3, 32))
+    for call in (lambda: native.lengths_to_offsets(None, cpu), lambda: native.gather_history(None, 32, cpu, cpu, None),
+                 lambda: native.precompute_candidate_links(None, 8, cpu),
+                 lambda: native.score_candidates(None, cpu, cpu, cpu, 1, None, None, None, None, None)):
+        with pytest.raises(ValueError):
+            call()
+    with pytest.raises(OverflowError):
+        native.score_candidates(None, cpu, cpu, cpu, 1, None, None, 1 << 70, None, None)
