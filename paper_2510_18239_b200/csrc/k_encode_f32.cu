@@ -23,6 +23,12 @@ constexpr int EF_D = 64, EF_THREADS = 256, EF_TILE = 128;
 // with it / the generic kernels, which split by token: n = 2000 351 / 353 / 395 us, 4000 680 / 105 / 442, 32000 2985 / 466 / 886,
 // 150000 3645 / 2050 / 2035; 200000 among 399 of 50: 9817 / 2820 / 2612.
 constexpr int EF_LONG = 2048, EF_LONG_CLUSTER = 16, EF_LONG_CLUSTERS = 7;
+// From 37 users on - two blocks a user run at once up to 72, one beyond - the blocks are dealt by length instead (ef_plan), in clusters of
+// four, of which 33 run at once.  A share below 48 tokens does not pay for the exchange.  Two layers, same blocks for every user / dealt:
+// 64 users of 50..1000 113.7 / 79.1 us, 64 of 525 88.0 / 68.0, 40 of 8..1000 80.8 / 61.0, 80 of 125..1000 131.2 / 115.3, 100 of 0..500
+// 91.6 / 80.8, one of 1900 among 99 of 100 374 / 115; where there is nothing to deal the plan costs 1 to 4 us: 132 of 10..300 68.8 /
+// 72.8, 60 of 1..100 37.6 / 39.2, hence up to 116 users and from a mean of two shares on.
+constexpr int EF_PLAN_FROM = 37, EF_PLAN_CLUSTERS = 33, EF_PLAN_USERS = 116, EF_SHARE = 48;
 constexpr int EF_LD = 68;                                        // floats per row of operands read along the contraction: spreads the banks
 
 template <int H_, int ELL_>
@@ -61,6 +67,7 @@ struct EncodeF32Params {
   float* scratch;                                                // [total x d]: histories beyond shared memory
   float* out;                                                    // L^P
   int B, longer_than, skip_long;                                 // a user has to be longer than that to be a long one
+  int planned, total;                                            // 1: the blocks of a cluster are dealt to users by length (ef_plan)
   int n_layers, cluster, cap, ln, hist_ln, silu;                 // cap: history rows a block holds
   float eps, scale;                                              // scale times log2 e with the softmax
   int* err;
@@ -264,6 +271,72 @@ __device__ __forceinline__ void ef_update_tile(float* fs, float* x, int ld, int 
   }
 }
 
+// Which user this block serves, as which of how many blocks, and where they begin in the cluster: the clusters of four are dealt by
+// length, so that no share is much longer than the others.  A share length L is taken, a user gets one to four blocks of at most L
+// tokens (no fewer than EF_SHARE each), and L grows from the mean until the users fit the clusters: those of four blocks take one each,
+// those of three share theirs with one of one block, those of two go in pairs.  Every block finds the same L.  The long users of the other
+// launch, if there is one, are left out (the line as long_user_line finds it).  Warp 0 works; word: four words of shared memory.
+struct EfSlot { int b, rank, blocks, base; };
+__device__ __forceinline__ EfSlot ef_plan(const int32_t* __restrict__ off, int B, int total, int longer_than, bool skip_long, int* word) {
+  const int clusters = gridDim.x / 4, c = blockIdx.x / 4, q = blockIdx.x % 4, lane = threadIdx.x & 31;
+  if (threadIdx.x < 32) {
+    constexpr int N = (EF_PLAN_USERS + 31) / 32;
+    int len[N], most[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int b = i * 32 + lane;
+      len[i] = b < B ? off[b + 1] - off[b] : -1;
+    }
+    for (int line = longer_than; skip_long; line *= 2) {
+      int over = 0;
+#pragma unroll
+      for (int i = 0; i < N; ++i) over += len[i] > line;
+      if (__reduce_add_sync(0xffffffffu, over) <= EF_LONG_CLUSTERS || line > (1 << 29)) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) len[i] = len[i] > line ? -1 : len[i];
+        break;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) most[i] = max(1, min(4, len[i] / EF_SHARE));
+    int L = max(EF_SHARE, (total + 4 * clusters - 1) / (4 * clusters)), n1, n2, n3, n4;
+    auto blocks = [&](int i) { return len[i] < 0 ? 0 : min(most[i], 1 + (len[i] > L) + (len[i] > 2 * L) + (len[i] > 3 * L)); };
+    for (;;) {
+      int cnt = 0;                                               // users of one, two, three and four blocks, a byte each
+#pragma unroll
+      for (int i = 0; i < N; ++i) { const int k = blocks(i); cnt += k ? 1 << (8 * (k - 1)) : 0; }
+      cnt = __reduce_add_sync(0xffffffffu, cnt);
+      n1 = cnt & 255; n2 = (cnt >> 8) & 255; n3 = (cnt >> 16) & 255; n4 = (cnt >> 24) & 255;
+      const int single = max(0, n1 - n3 - 2 * (n2 & 1));
+      if (n4 + n3 + (n2 + 1) / 2 + (single + 3) / 4 <= clusters || L > (1 << 28)) break;
+      L += max(8, L / 16);
+    }
+    const int c3 = c - n4, c2 = c3 - n3, c1 = c2 - (n2 + 1) / 2;
+    int k = 1, which, rank = 0, base = q;                        // the which-th user of k blocks
+    if (c3 < 0) { k = 4; which = c; rank = q; base = 0; }
+    else if (c2 < 0) {
+      which = c3;
+      if (q < 3) { k = 3; rank = q; base = 0; }
+    } else if (c1 < 0) {
+      which = 2 * c2 + (q >> 1);
+      if (which < n2) { k = 2; rank = q & 1; base = q & 2; }
+      else which = n3 + (q & 1);
+    } else which = n3 + 2 * (n2 & 1) + 4 * c1 + q;
+    if (lane == 0) { word[0] = -1; word[1] = rank; word[2] = k; word[3] = base; }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const unsigned m = __ballot_sync(0xffffffffu, blocks(i) == k);
+      if (((m >> lane) & 1u) && __popc(m & ((1u << lane) - 1u)) == which) word[0] = i * 32 + lane;
+      which -= __popc(m);
+    }
+  }
+  __syncthreads();
+  const EfSlot s{word[0], word[1], word[2], word[3]};
+  __syncthreads();
+  return s;
+}
+
 // LONG: cluster k takes the k-th long user, and the blocks read each other's message in place (pushed, sixteen slots would not fit
 // beside the operands); without it cluster b takes user b and a long user is left out.
 template <class G, bool LONG>
@@ -272,29 +345,35 @@ k_encode_f32(const EncodeF32Params p) {
   constexpr int ELL = G::ELL, HL = G::HL, DH = G::DH, D = EF_D;
   extern __shared__ __align__(128) float fs[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int CL = LONG ? EF_LONG_CLUSTER : p.cluster, rank = blockIdx.x % CL;
+  const int CL = LONG ? EF_LONG_CLUSTER : p.cluster;
   const int c = tid & 63, kq = tid >> 6, k0 = kq * 16;           // link rows: output column, quarter of the contraction
   float* const ex = fs + G::EX;
   float* const X = ex + (LONG ? 1 : 2 * CL) * G::MSG;
   uint64_t* const bar = reinterpret_cast<uint64_t*>(fs + G::BAR);
-  const uint32_t msg_bytes = (uint32_t)(CL - 1) * G::MSG * 4;
   if (!LONG && tid == 0) {
     tc::mbar_init(bar, 1);
-    tc::mbar_arrive_expect_tx(bar, msg_bytes);
     tc::fence_barrier_init();
   }
   if (!LONG && CL > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   pdl_launch_dependents();
   pdl_wait();
   int* const word = reinterpret_cast<int*>(fs + G::MX);
-  const int b = LONG ? nth_long_user(p.off, p.B, p.longer_than, EF_LONG_CLUSTERS, blockIdx.x / CL, word) : (int)blockIdx.x / CL;
-  if (LONG && b < 0) return;                                     // the whole cluster
-  const int u0 = p.off[b], un = p.off[b + 1] - u0;
-  if (!LONG && p.skip_long && un > p.longer_than && un > long_user_line(p.off, p.B, p.longer_than, EF_LONG_CLUSTERS, word)) {
+  EfSlot me{(int)blockIdx.x / CL, (int)blockIdx.x % CL, CL, 0};
+  if (LONG) me.b = nth_long_user(p.off, p.B, p.longer_than, EF_LONG_CLUSTERS, blockIdx.x / CL, word);
+  if (LONG && me.b < 0) return;                                  // the whole cluster
+  if (!LONG && p.planned)
+    me = ef_plan(p.off, p.B, p.total, p.longer_than, p.skip_long != 0, word);
+  const int b = me.b, rank = me.rank, nb = me.blocks;
+  const int u0 = b < 0 ? 0 : p.off[b], un = b < 0 ? 0 : p.off[b + 1] - u0;
+  if (!LONG && (b < 0 || (!p.planned && p.skip_long && un > p.longer_than &&
+                          un > long_user_line(p.off, p.B, p.longer_than, EF_LONG_CLUSTERS, word)))) {
     if (CL > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     return;
   }
-  const int share = (un + CL - 1) / CL, tok0 = u0 + min(un, rank * share), n = min(un, (rank + 1) * share) - min(un, rank * share);
+  const uint32_t msg_bytes = (uint32_t)(nb - 1) * G::MSG * 4;
+  // (a peer's message that is here before the bytes are expected is counted all the same: the phase waits for this arrival)
+  if (!LONG && tid == 0) tc::mbar_arrive_expect_tx(bar, msg_bytes);
+  const int share = (un + nb - 1) / nb, tok0 = u0 + min(un, rank * share), n = min(un, (rank + 1) * share) - min(un, rank * share);
   const bool resident = share <= p.cap;
   float* const rows = resident ? X : p.scratch + (int64_t)tok0 * D;    // the block's history
   const int ld = resident ? EF_LD : D;
@@ -451,12 +530,12 @@ k_encode_f32(const EncodeF32Params p) {
     if (tid < 2 * HL) slot[HL * D + tid] = fs[G::RUN + tid];      // maxima, sums
     if (LONG) cluster_sync_all();
     else __syncthreads();
-    if (!LONG && CL > 1) {
-      if (j == 0) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // the peers run
+    if (!LONG && CL > 1 && j == 0) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // the peers run
+    if (!LONG && nb > 1) {
       const uint32_t at = (uint32_t)__cvta_generic_to_shared(slot), ba = (uint32_t)__cvta_generic_to_shared(bar);
       for (int i = tid; i < G::MSG / 4; i += EF_THREADS) {
         const float4 v = ef_ld4(slot + i * 4);
-        for (int r = 1; r < CL; ++r) ef_push(ef_peer(at + i * 16, (rank + r) % CL), v, ef_peer(ba, (rank + r) % CL));
+        for (int r = 1; r < nb; ++r) ef_push(ef_peer(at + i * 16, me.base + (rank + r) % nb), v, ef_peer(ba, me.base + (rank + r) % nb));
       }
       tc::mbar_wait(bar, (uint32_t)j & 1u, p.err, 88);
     }
@@ -469,8 +548,8 @@ k_encode_f32(const EncodeF32Params p) {
         if constexpr (LONG) return cluster_peer(static_cast<const float*>(ex), q);
         else return ex + ((j & 1) * CL + q) * G::MSG;
       };
-      for (int q = 0; q < CL; ++q) M = fmaxf(M, msg(q)[HL * D + r]);
-      for (int q = 0; q < CL; ++q) {
+      for (int q = 0; q < nb; ++q) M = fmaxf(M, msg(q)[HL * D + r]);
+      for (int q = 0; q < nb; ++q) {
         const float m = msg(q)[HL * D + r], w = m == -INFINITY ? 0.f : ef_ex2(m - M);
         S = fmaf(w, msg(q)[HL * D + HL + r], S);
         const float4 x = ef_ld4(msg(q) + i * 4);
@@ -546,15 +625,18 @@ static lime_status launch_ef(EncodeF32Params p, int B, int64_t total, cudaStream
   static_assert((G::EX + 2 * 2 * G::MSG) * 4 + 128 * EF_LD * 4 <= 232448, "two blocks a user must fit with 128 rows each");
   int cl = 1;
   while (cl < 8 && fixed_bytes(2 * cl) + 128 * kRow <= kSmem &&
-         (((int64_t)B * cl * 2 <= 144 && total / ((int64_t)B * cl * 2) >= 48) || 2 * total / ((int64_t)B * cl) > (kSmem - fixed_bytes(cl)) / kRow))
+         (((int64_t)B * cl * 2 <= 144 && total / ((int64_t)B * cl * 2) >= EF_SHARE) || 2 * total / ((int64_t)B * cl) > (kSmem - fixed_bytes(cl)) / kRow))
     cl *= 2;
-  p.cluster = cl;
   p.B = B;
   p.longer_than = EF_LONG * cl;
+  p.total = (int)total;
+  p.planned = B >= EF_PLAN_FROM && B <= EF_PLAN_USERS && total >= 2ll * EF_SHARE * B && fixed_bytes(4) + 128 * kRow <= kSmem;
+  if (p.planned) cl = 4;
+  p.cluster = cl;
   // the host knows the mean length only: room for twice the mean share, 256 rows at least, where shared memory has it
   const int64_t fixed = fixed_bytes(cl), most = (kSmem - fixed) / kRow;
   int64_t cap = 2 * total / ((int64_t)B * cl) + 1;
-  if (cap < 256) cap = 256;
+  if (cap < 256 || p.planned) cap = p.planned ? most : 256;
   if (cap > total) cap = total;
   p.cap = (int)(cap < most ? cap : most);
   auto launch = [&](void (*kernel)(EncodeF32Params), bool (&smem_set)[kMaxDeviceOrdinals], int64_t blocks, int cluster, size_t smem, const EncodeF32Params& q) -> lime_status {
@@ -592,7 +674,8 @@ static lime_status launch_ef(EncodeF32Params p, int B, int64_t total, cudaStream
     if (s != LIME_OK) return s;
   }
   static bool smem_set[kMaxDeviceOrdinals] = {};
-  return launch(k_encode_f32<G, false>, smem_set, (int64_t)B * cl, cl, (size_t)(fixed + p.cap * kRow), p);
+  const int64_t blocks = p.planned ? 4 * (B < EF_PLAN_CLUSTERS ? B : EF_PLAN_CLUSTERS) : (int64_t)B * cl;
+  return launch(k_encode_f32<G, false>, smem_set, blocks, cl, (size_t)(fixed + p.cap * kRow), p);
 }
 
 lime_status launch_encode_f32(const EncodeSmallArgs& a, int* err, cudaStream_t st) {

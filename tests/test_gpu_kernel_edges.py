@@ -429,6 +429,16 @@ def test_fp32_encode_of_long_histories(H, ell, lengths, phi, raw, per_user):
     _encode_against_oracle(synth.F32, 64, H, ell, 3, lengths, phi, raw, per_user, 1e-4, 1e-5)
 
 
+@pytest.mark.parametrize("H,ell", [(2, 8), (4, 8), (2, 16)])
+@pytest.mark.parametrize("lengths", [[1000, 900, 700, 500, 300] * 8, [0] * 30 + [600] * 20 + [1], [120] * 115 + [900], [400] * 37, [95, 96, 97] * 30,
+                                     [1400] * 40, [5000, 2100] + [144, 190] * 25 + [0], [0] * 40])
+@pytest.mark.parametrize("phi,raw,per_user", [("softmax", True, True), ("silu", False, False)])
+def test_fp32_blocks_dealt_by_length(H, ell, lengths, phi, raw, per_user):
+    """37 to 116 users: one to four blocks a user, clusters shared by users of three and one or two and two, odd ones out, empty
+    clusters and histories, shares beyond shared memory, users left to the other launch."""
+    _encode_against_oracle(synth.F32, 64, H, ell, 2, lengths, phi, raw, per_user, 1e-4, 1e-5)
+
+
 @pytest.mark.parametrize("d,H,ell", [(128, 4, 32), (128, 8, 32), (256, 8, 64)])
 @pytest.mark.parametrize("lengths", [[2000] + [20] * 80, [1025] * 2 + [512] * 70 + [0], [1024] + [30] * 70, [5000] * 3 + [513] * 7 + [40] * 60, [700] * 66])
 @pytest.mark.parametrize("phi,raw", [("softmax", False), ("silu", True)])
