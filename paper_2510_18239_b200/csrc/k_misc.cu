@@ -4,92 +4,146 @@
 namespace lime {
 
 // ----------------------------------------------------------------------------- block-wide exclusive scan
-// One block of 1024 threads walks the array in slabs of 1024 with a running carry. B is at most a few
-// thousand users per batch, so a single block is latency-optimal (one launch, no inter-block traffic).
-template <typename F>
-__device__ __forceinline__ void block_exclusive_scan(int n, int32_t* out, F value_at) {
-  __shared__ int32_t warp_tot[32];
-  __shared__ int32_t carry_s;
+// What the threads before this one hold, of two values at once, and the block's totals.  One barrier: every warp adds up the warp sums
+// itself.  `sums`: shared memory for up to 32 warps; consecutive scans alternate between two of them.
+__device__ __forceinline__ int2 block_scan2(int2 v, int2* sums, int2& total) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (threadIdx.x == 0) carry_s = 0;
-  __syncthreads();
-  for (int base = 0; base < n; base += blockDim.x) {
-    const int i = base + threadIdx.x;
-    const int32_t v = (i < n) ? value_at(i) : 0;
-    int32_t incl = v;
+  int2 incl = v;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    if (lane == 31) warp_tot[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-      int32_t w = (lane < (int)(blockDim.x >> 5)) ? warp_tot[lane] : 0;
-      int32_t wi = w;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        int32_t t = __shfl_up_sync(0xffffffffu, wi, o);
-        if (lane >= o) wi += t;
-      }
-      warp_tot[lane] = wi - w;  // exclusive prefix of warp totals
-    }
-    __syncthreads();
-    const int32_t carry = carry_s;
-    if (i < n) out[i] = carry + warp_tot[wid] + incl - v;
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry_s = carry + warp_tot[wid] + incl;  // last thread holds the slab total
-    __syncthreads();
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(0xffffffffu, incl.x, o), y = __shfl_up_sync(0xffffffffu, incl.y, o);
+    if (lane >= o) { incl.x += x; incl.y += y; }
   }
-  if (threadIdx.x == 0) out[n] = carry_s;
+  if (lane == 31) sums[wid] = incl;
+  __syncthreads();
+  const int2 w = lane < (int)(blockDim.x >> 5) ? sums[lane] : make_int2(0, 0);
+  total = make_int2(__reduce_add_sync(0xffffffffu, w.x), __reduce_add_sync(0xffffffffu, w.y));
+  return make_int2(__reduce_add_sync(0xffffffffu, lane < wid ? w.x : 0) + incl.x - v.x,
+                   __reduce_add_sync(0xffffffffu, lane < wid ? w.y : 0) + incl.y - v.y);
 }
 
 __global__ void __launch_bounds__(1024) k_offsets(const int32_t* __restrict__ len, int B, int32_t* __restrict__ off) {
+  __shared__ int2 sums[2][32];
   pdl_launch_dependents();     // simple kernel: the next one may set itself up beside it
   pdl_wait();                  // nothing is read or written before the previous kernel is complete
-  block_exclusive_scan(B, off, [&](int i) { return max(len[i], 0); });
+  int carry = 0;
+  for (int b0 = 0, k = 0; b0 < B; b0 += blockDim.x, k ^= 1) {
+    const int b = b0 + threadIdx.x;
+    int2 total;
+    const int2 before = block_scan2(make_int2(b < B ? max(len[b], 0) : 0, 0), sums[k], total);
+    if (b < B) off[b] = carry + before.x;
+    carry += total.x;
+  }
+  if (threadIdx.x == 0) off[B] = carry;
 }
 
-// Deal the (user, chunk) items of the links<-history attention to `G` groups of CTAs so that the groups' token tiles
-// come out even.  Items are sorted by size (a counting sort over their tile counts, largest first) and handed out in
+// The work lists of the XOR layers in one launch: chunks of the links<-history attention, tiles of the history update, and (group_start
+// given) the chunk items dealt to `G` groups of CTAs so that the groups' token tiles come out even.  One block, a thread per user (the
+// users of 1024 threads at a time).  Every layer waits for this kernel, so it is kept a short chain: a user's length is read once and stays
+// in a register (of the first 1024), both prefix sums are one scan, and the dealing works in shared memory up to SCAP items.  (The lengths
+// read again for each list, two scans of five barriers, the item's user looked up in global memory and two loops of one thread: 3.1 us
+// after the lookup for 256 users of 512 tokens at d = 128, 9 us for 64 users at d = 256 with 32 links; this way one request of one user
+// takes 38.0 us, 40.75 before, the 256 users 133.9, 135.7, the 64 at d = 256 225.8, 229.)
+// The dealing: items are sorted by size (a counting sort over their tile counts, largest first) and handed out in
 // rounds of G: within a round the group with the least work so far takes the largest item, the next group the next
 // one, and so on.  Ragged histories dealt round-robin leave the busiest group 16 % above the mean (1024 users of
-// 1024..4096 tokens over 37 groups); this order leaves it under 1 %.  One block; a round is one rank computation over
+// 1024..4096 tokens over 37 groups); this order leaves it under 1 %.  A round is one rank computation over
 // the G loads in shared memory and one barrier.
 // group_start[G+1], group_items[items]: the items of group j in the order it takes them.  scratch: 4 x items ints.
-__device__ void balance_groups(const int32_t* __restrict__ off, int chunk, const int32_t* __restrict__ chunk_start,
-                               const int32_t* __restrict__ chunk_user, int n_items, int G, int att_tile,
-                               int32_t* __restrict__ group_start, int32_t* __restrict__ group_items, int32_t* __restrict__ scratch) {
-  constexpr int KEYS = 256, GMAX = 160, KCAP = 16384;
+__global__ void __launch_bounds__(1024)
+k_layer_schedules(const int32_t* __restrict__ off, int B, const ChunkRule rule, int32_t* __restrict__ chunk_out,
+                  int32_t* __restrict__ chunk_start, int tile,
+                  int32_t* __restrict__ tile_start, int32_t* __restrict__ chunk_user, int32_t* __restrict__ merge_needed,
+                  int G, int att_tile, int32_t* __restrict__ group_start, int32_t* __restrict__ group_items,
+                  int32_t* __restrict__ scratch) {
+  constexpr int KEYS = 256, GMAX = 160, KCAP = 16384, SCAP = 2048;
+  __shared__ int2 sums[2][32];
   __shared__ int32_t hist[KEYS];
-  __shared__ int32_t load[GMAX], cnt[GMAX];
+  __shared__ __align__(16) int32_t load[GMAX];
+  __shared__ int32_t cnt[GMAX], first[GMAX];
   __shared__ uint8_t skey[KCAP];                   // sizes in sorted order (the first KCAP items; the rest are read from global)
-  int32_t* sorted = scratch;
-  int32_t* key_of = scratch + n_items;             // by item, then (after the sort) by sorted position
-  int32_t* group_of = scratch + 2 * (size_t)n_items;
-  int32_t* slot_of = scratch + 3 * (size_t)n_items;
-  for (int i = threadIdx.x; i < KEYS; i += blockDim.x) hist[i] = 0;
-  for (int i = threadIdx.x; i < GMAX; i += blockDim.x) { load[i] = 0; cnt[i] = 0; }
-  __syncthreads();
-  for (int i = threadIdx.x; i < n_items; i += blockDim.x) {
-    const int b = chunk_user[i];
-    const int tok = min(chunk, off[b + 1] - off[b] - (i - chunk_start[b]) * chunk);
-    const int key = min(KEYS - 1, (tok + att_tile - 1) / att_tile);
-    group_of[i] = key;                             // parked here until the scatter below
-    atomicAdd(&hist[KEYS - 1 - key], 1);           // bucket 0 holds the largest items
+  __shared__ int32_t small[3 * SCAP];
+  pdl_launch_dependents();     // simple kernel: the next one may set itself up beside it
+  const bool deal = group_start != nullptr && chunk_user != nullptr;
+  if (deal) {
+    for (int i = threadIdx.x; i < KEYS; i += blockDim.x) hist[i] = 0;
+    for (int i = threadIdx.x; i < GMAX; i += blockDim.x) { load[i] = i < G ? 0 : 0x7fffffff; cnt[i] = 0; }
   }
-  __syncthreads();
+  pdl_wait();                  // nothing is read or written before the previous kernel is complete
+  const int n_first = (int)threadIdx.x < B ? off[threadIdx.x + 1] - off[threadIdx.x] : 0;
+  auto length = [&](int b) { return b < (int)blockDim.x ? n_first : off[b + 1] - off[b]; };      // b: one of this thread's
+  int longest = 0, short_items = 0;
+  if (rule.short_tokens > 0) {
+    for (int b = threadIdx.x; b < B; b += blockDim.x) {
+      const int n = length(b);
+      longest = max(longest, n);
+      if (n > rule.short_tokens) short_items += (n + rule.short_tokens - 1) / rule.short_tokens;
+    }
+    longest = __reduce_max_sync(0xffffffffu, longest);
+    short_items = __reduce_add_sync(0xffffffffu, short_items);
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) sums[0][threadIdx.x >> 5] = make_int2(longest, short_items);
+    __syncthreads();
+    const int2 w = lane < (int)(blockDim.x >> 5) ? sums[0][lane] : make_int2(0, 0);
+    longest = __reduce_max_sync(0xffffffffu, w.x);
+    short_items = __reduce_add_sync(0xffffffffu, w.y);
+  }
+  const int chunk = longest > 2 * rule.short_tokens && short_items <= rule.short_items ? rule.short_tokens : rule.tokens;
+  // does any user's attention output need the merge step (several chunks to combine, or no history: a zero row)?
+  int merge = 0;
+  for (int b = threadIdx.x; b < B; b += blockDim.x)
+    if (length(b) <= 0 || length(b) > chunk) merge = 1;
+  merge = __syncthreads_or(merge);
   if (threadIdx.x == 0) {
-    int run = 0;
-    for (int k = 0; k < KEYS; ++k) { const int c = hist[k]; hist[k] = run; run += c; }
+    *chunk_out = chunk;
+    if (merge_needed != nullptr) *merge_needed = merge;
+  }
+  int2 carry = make_int2(0, 0);
+  int item_first = 0;                              // this thread's first item, of its first user
+  for (int b0 = 0, k = 1; b0 < B; b0 += blockDim.x, k ^= 1) {
+    const int b = b0 + threadIdx.x;
+    const int n = b < B ? max(length(b), 0) : 0;
+    const int n_chunks = (n + chunk - 1) / chunk;
+    int2 total;
+    const int2 before = block_scan2(make_int2(n_chunks, (n + tile - 1) / tile), sums[k], total);
+    const int item = carry.x + before.x;
+    if (b0 == 0) item_first = item;
+    if (b < B) { chunk_start[b] = item; tile_start[b] = carry.y + before.y; }
+    // inverse map (chunk item -> user): the attention kernel strides through the items, and one read of this table
+    // replaces a search over chunk_start per item
+    if (chunk_user != nullptr)
+      for (int i = 0; i < n_chunks; ++i) {
+        chunk_user[item + i] = b;
+        // bucket 0 holds the largest items
+        if (deal) atomicAdd(&hist[KEYS - 1 - min(KEYS - 1, (min(chunk, n - i * chunk) + att_tile - 1) / att_tile)], 1);
+      }
+    carry.x += total.x;
+    carry.y += total.y;
+  }
+  if (threadIdx.x == 0) { chunk_start[B] = carry.x; tile_start[B] = carry.y; }
+  if (!deal) return;
+  const int n_items = carry.x;
+  int32_t* const sorted = n_items <= SCAP ? small : scratch;
+  int32_t* const key_of = n_items <= SCAP ? nullptr : scratch + n_items;                 // by sorted position, from KCAP on
+  int32_t* const group_of = n_items <= SCAP ? small + SCAP : scratch + 2 * (size_t)n_items;
+  int32_t* const slot_of = n_items <= SCAP ? small + 2 * SCAP : scratch + 3 * (size_t)n_items;
+  __syncthreads();
+  {                                                // (at least KEYS threads)
+    int2 total;
+    const int mine = threadIdx.x < KEYS ? hist[threadIdx.x] : 0;
+    const int2 before = block_scan2(make_int2(mine, 0), sums[0], total);
+    if (threadIdx.x < KEYS) hist[threadIdx.x] = before.x;
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < n_items; i += blockDim.x) {
-    const int key = group_of[i];
-    const int at = atomicAdd(&hist[KEYS - 1 - key], 1);
-    sorted[at] = i;
-    key_of[at] = key;
-    if (at < KCAP) skey[at] = (uint8_t)key;
+  for (int b = threadIdx.x; b < B; b += blockDim.x) {
+    const int n = max(length(b), 0), item = b < (int)blockDim.x ? item_first : chunk_start[b];
+    for (int i = 0; i * chunk < n; ++i) {
+      const int key = min(KEYS - 1, (min(chunk, n - i * chunk) + att_tile - 1) / att_tile);
+      const int at = atomicAdd(&hist[KEYS - 1 - key], 1);
+      sorted[at] = item + i;
+      if (at < KCAP) skey[at] = (uint8_t)key;
+      else key_of[at] = key;
+    }
   }
   __syncthreads();
   for (int r0 = 0; r0 < n_items; r0 += G) {
@@ -97,9 +151,11 @@ __device__ void balance_groups(const int32_t* __restrict__ off, int chunk, const
     int rank = 0, mine = 0;
     if (j < G) {
       mine = load[j];
-      for (int o = 0; o < G; ++o) {
-        const int lo = load[o];
-        rank += (lo < mine || (lo == mine && o < j)) ? 1 : 0;
+#pragma unroll 4
+      for (int o = 0; o < G; o += 4) {             // (loads past G are the largest there is)
+        const int4 l = *reinterpret_cast<const int4*>(load + o);
+        rank += (l.x < mine || (l.x == mine && o < j)) + (l.y < mine || (l.y == mine && o + 1 < j)) +
+                (l.z < mine || (l.z == mine && o + 2 < j)) + (l.w < mine || (l.w == mine && o + 3 < j));
       }
     }
     __syncthreads();                               // every rank is taken before a load changes
@@ -112,75 +168,24 @@ __device__ void balance_groups(const int32_t* __restrict__ off, int chunk, const
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    int run = 0;
-    for (int j = 0; j < G; ++j) { group_start[j] = run; run += cnt[j]; }
-    group_start[G] = run;
+  {                                                // (at least GMAX threads)
+    int2 total;
+    const int2 before = block_scan2(make_int2((int)threadIdx.x < G ? cnt[threadIdx.x] : 0, 0), sums[1], total);
+    if ((int)threadIdx.x < G) first[threadIdx.x] = group_start[threadIdx.x] = before.x;
+    if (threadIdx.x == 0) group_start[G] = total.x;
   }
   __syncthreads();
-  for (int at = threadIdx.x; at < n_items; at += blockDim.x) group_items[group_start[group_of[at]] + slot_of[at]] = sorted[at];
+  for (int at = threadIdx.x; at < n_items; at += blockDim.x) group_items[first[group_of[at]] + slot_of[at]] = sorted[at];
 }
 
-// both work lists of the XOR layers in one launch: chunks of the links<-history attention, tiles of the history update
-__global__ void __launch_bounds__(1024)
-k_layer_schedules(const int32_t* __restrict__ off, int B, const ChunkRule rule, int32_t* __restrict__ chunk_out,
-                  int32_t* __restrict__ chunk_start, int tile,
-                  int32_t* __restrict__ tile_start, int32_t* __restrict__ chunk_user, int32_t* __restrict__ merge_needed,
-                  int G, int att_tile, int32_t* __restrict__ group_start, int32_t* __restrict__ group_items,
-                  int32_t* __restrict__ scratch) {
-  pdl_launch_dependents();     // simple kernel: the next one may set itself up beside it
-  pdl_wait();                  // nothing is read or written before the previous kernel is complete
-  int longest = 0, short_items = 0;
-  if (rule.short_tokens > 0) {
-    __shared__ int warp_longest[32], warp_items[32];           // of the block's 32 warps
-    for (int b = threadIdx.x; b < B; b += blockDim.x) {
-      const int n = off[b + 1] - off[b];
-      longest = max(longest, n);
-      if (n > rule.short_tokens) short_items += (n + rule.short_tokens - 1) / rule.short_tokens;
-    }
-    longest = __reduce_max_sync(0xffffffffu, longest);
-    short_items = __reduce_add_sync(0xffffffffu, short_items);
-    if ((threadIdx.x & 31) == 0) { warp_longest[threadIdx.x >> 5] = longest; warp_items[threadIdx.x >> 5] = short_items; }
-    __syncthreads();
-    longest = __reduce_max_sync(0xffffffffu, warp_longest[threadIdx.x & 31]);
-    short_items = __reduce_add_sync(0xffffffffu, warp_items[threadIdx.x & 31]);
-  }
-  const int chunk = longest > 2 * rule.short_tokens && short_items <= rule.short_items ? rule.short_tokens : rule.tokens;
-  // does any user's attention output need the merge step (several chunks to combine, or no history: a zero row)?
-  int merge = 0;
-  for (int b = threadIdx.x; b < B; b += blockDim.x)
-    if (off[b + 1] - off[b] <= 0 || off[b + 1] - off[b] > chunk) merge = 1;
-  merge = __syncthreads_or(merge);
-  if (threadIdx.x == 0) {
-    *chunk_out = chunk;
-    if (merge_needed != nullptr) *merge_needed = merge;
-  }
-  block_exclusive_scan(B, chunk_start, [&](int i) {
-    int n = off[i + 1] - off[i];
-    return n > 0 ? (n + chunk - 1) / chunk : 0;
-  });
-  __syncthreads();
-  block_exclusive_scan(B, tile_start, [&](int i) {
-    int n = off[i + 1] - off[i];
-    return n > 0 ? (n + tile - 1) / tile : 0;
-  });
-  // inverse map (chunk item -> user): the attention kernel strides through the items, and one read of this table
-  // replaces a search over chunk_start per item
-  __syncthreads();
-  if (chunk_user != nullptr)
-    for (int b = threadIdx.x; b < B; b += blockDim.x)
-      for (int i = chunk_start[b]; i < chunk_start[b + 1]; ++i) chunk_user[i] = b;
-  if (group_start != nullptr && chunk_user != nullptr) {
-    __syncthreads();
-    balance_groups(off, chunk, chunk_start, chunk_user, chunk_start[B], G, att_tile, group_start, group_items, scratch);
-  }
-}
+// a thread per user, 256 at least (the dealing scans its 256 buckets in one go), 1024 at most
+static int schedule_threads(int B) { return B <= 256 ? 256 : B >= 1024 ? 1024 : (B + 31) / 32 * 32; }
 
 lime_status launch_layer_schedules(const int32_t* off, int B, const ChunkRule& chunk, int32_t* chunk_out, int32_t* chunk_start, int tile, int32_t* tile_start,
                                    int32_t* chunk_user, int32_t* merge_needed, const GroupSchedule& gs, cudaStream_t st) {
   if (gs.group_start != nullptr && (gs.n_groups < 1 || gs.n_groups > 160 || gs.att_tile < 1)) return LIME_INVALID_ARG;
   ProfScope _p("k_layer_schedules", st);
-  launch_pdl(k_layer_schedules, dim3(1), dim3(1024), 0, st, off, B, chunk, chunk_out, chunk_start, tile, tile_start, chunk_user, merge_needed,
+  launch_pdl(k_layer_schedules, dim3(1), dim3(schedule_threads(B)), 0, st, off, B, chunk, chunk_out, chunk_start, tile, tile_start, chunk_user, merge_needed,
              gs.n_groups, gs.att_tile, gs.group_start, gs.group_items, gs.scratch);
   LIME_LAUNCH_CHECK("k_layer_schedules");
   return LIME_OK;
@@ -188,7 +193,7 @@ lime_status launch_layer_schedules(const int32_t* off, int B, const ChunkRule& c
 
 lime_status launch_offsets(const int32_t* len, int B, int32_t* off, cudaStream_t st) {
   ProfScope _p("k_offsets", st);
-  launch_pdl(k_offsets, dim3(1), dim3(1024), 0, st, len, B, off);
+  launch_pdl(k_offsets, dim3(1), dim3(schedule_threads(B)), 0, st, len, B, off);
   LIME_LAUNCH_CHECK("k_offsets");
   return LIME_OK;
 }
