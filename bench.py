@@ -78,6 +78,7 @@ def kernel_models(wl: synth.Workload, total_tokens: int, cand_heads: int = 1):
         "k_gemm_tc_prep": dict(flops=2.0 * BL * d * (max(n - 2, 0) * (2 * H * d + (d if d == 256 else 2 * H * f)) + (H * d if n > 1 else 0)),
                                pipe="tensor"),
         "k_link_mlp_tc": dict(flops=n * 2.0 * BL * (H * d * 2 * f + f * d), pipe="tensor"),
+        "k_link_mlp_d256_tc": dict(flops=n * 2.0 * BL * (d * d + 2 * d * f + f * d), pipe="tensor"),
         # CUDA-core path (fp32 storage and shapes the tensor-core kernels do not serve)
         "k_linear_simt_ln": dict(flops=hist_proj + link_proj, pipe="alu"),
         "k_linear_simt_glu": dict(flops=glu, pipe="alu"),

@@ -7,7 +7,7 @@
 //   links <- history scores  Q[T]_h K[S]_h^T = Q2_(h,l) . LN(S)^T    Q2_(h,l) = That_l (scale W_{Q,h} W_{K,h}^T)
 //   history <- links scores  Q[S]_h K[T]_h^T = LN(S) . K2_(h,l)^T    K2_(h,l) = That_l (scale W_{K,h} W_{Q,h}^T)
 //   GatedMLP input           O[S] W_g = P . G2,  O[S] W_u = P . U2   G2_(h,l) = That_l (W_{V,h} W_g[h rows, :])
-//   link rows                O[T] W_g = sum_h Ohat_(h,l) (W_{V,h} W_g[h rows, :])        (same folded matrices)
+//   link rows                O[T] W_g = sum_h Ohat_(h,l) (W_{V,h} W_g[h rows, :])        (same folded matrices; d = 128 only)
 // The bracketed products depend on the weights only and are formed once, here, at lime_set_weights time; `scale`
 // is the softmax scale times log2(e), so that the streaming kernels exponentiate with ex2 directly.
 #include "lime_common.cuh"
@@ -22,14 +22,14 @@ __device__ __forceinline__ float w_at(const __nv_bfloat16* W, int r, int c, int 
 //   [H*d] folded queries | [H*d] folded keys | then, with `plain_v` clear, [H*f] folded gate | [H*f] folded up;
 //   with `plain_v` set, [d] rows of W_V^T (the link values V[T] = LN(T) W_V are then formed as they stand, for the
 //   kernels that mix values head by head and apply the GatedMLP weights afterwards)
-// WpostT [2f x H*d]     (B operand of the GLU GEMM on link rows)
+// WpostT [2f x H*d]     (B operand of the GLU GEMM on link rows; nullable)
 __global__ void k_fold_weights(const __nv_bfloat16* __restrict__ Wq, const __nv_bfloat16* __restrict__ Wk,
                                const __nv_bfloat16* __restrict__ Wv, const __nv_bfloat16* __restrict__ Wg,
                                const __nv_bfloat16* __restrict__ Wu, int d, int H, int f, float scale, int plain_v,
                                __nv_bfloat16* __restrict__ WprepT, __nv_bfloat16* __restrict__ WpostT) {
   const int d_h = d / H;
   const int rows_qk = 2 * H * d;
-  const int n_prep = (rows_qk + (plain_v ? d : 2 * H * f)) * d, n_post = 2 * f * H * d;
+  const int n_prep = (rows_qk + (plain_v ? d : 2 * H * f)) * d, n_post = WpostT != nullptr ? 2 * f * H * d : 0;
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n_prep + n_post; idx += gridDim.x * blockDim.x) {
     float acc = 0.f;
     if (idx < n_prep) {

@@ -201,7 +201,7 @@ static Workspace carve(const Ctx* c, void* base, int32_t B, int64_t total) {
 // True when the whole layer runs on the tensor-core kernels (their set-up data exists for this layer).
 static bool layer_on_tensor_cores(const Ctx* c, int layer) {
   if (c->side256) return c->side_w && c->WoT[layer] && c->WguT[layer];
-  return c->tc_mode != 0 && c->WoT[layer] && c->WprepT[layer] && c->WpostT[layer] && (c->tc_mode == 1 || c->WguT[layer]);
+  return c->tc_mode != 0 && c->WoT[layer] && c->WprepT[layer] && (c->tc_mode == 1 ? c->WpostT[layer] : c->WguT[layer]);
 }
 
 // One XOR layer, tensor-core path: three link-row GEMMs around the two streaming attention kernels.
@@ -292,7 +292,7 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
   BesideLinkSide beside;
   if (c->side256) beside = beside_link_side(link_side_d256_blocks(B), 14, w.n_tile_upper, B);
   else if (side1 != nullptr) beside = beside_link_side(link_side_d128_blocks((int64_t)B * g.ell), wide ? 24 : 30, w.n_tile_upper, B);
-  else beside = beside_link_side(((int64_t)B * g.ell + 127) / 128, c->tc_mode == 2 ? 44 : wide ? 16 : 20, w.n_tile_upper, B);
+  else beside = beside_link_side(((int64_t)B * g.ell + 127) / 128, c->tc_mode == 2 ? 16 : wide ? 16 : 20, w.n_tile_upper, B);
   if ((s = c->tc_mode == 2 ? launch_link_attn_d256_tc(la, st) : launch_link_attn_tc(la, st)) != LIME_OK) return s;
   if (c->side256) {
     // merge, T^j and what follows from it - the next layer's operands included - in one kernel; `side` says what is wanted
@@ -308,8 +308,9 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
   } else {
   if ((s = launch_link_attn_merge_norm(w.chunk_start, w.merge_needed, B, g.ell, g.d, g.H, w.part_m, w.part_s, w.part_acc, w.Ohat, st)) != LIME_OK)
     return s;
-  // T^j = GatedMLP(O[T]) with W_V folded into the gate / up weights, and what the next step needs from it
+  // T^j = GatedMLP(O[T]) and what the next step needs from it
   mlp.Ohat = w.Ohat; mlp.M = (int64_t)B * g.ell; mlp.K = g.H * g.d; mlp.d = g.d; mlp.WpostT = c->WpostT[layer]; mlp.WoT = c->WoT[layer];
+  mlp.WguT = c->WguT[layer]; mlp.WvT = static_cast<const char*>(c->WprepT[layer]) + (size_t)2 * g.H * g.d * g.d * 2;     // (d = 256: k_link_prep.cu)
   mlp.ln = g.ln; mlp.ln_eps = c->ln_eps; mlp.err = c->dev_err;
   if ((s = launch_link_mlp_tc(mlp, st)) != LIME_OK) return s;
   }
@@ -694,7 +695,7 @@ lime_status lime_set_weights(lime_ctx* ctx, const lime_weights* w, void* stream)
     for (int j = 0; j < g.n_layers; ++j) {
       LIME_CUDA(need(&c->WoT[j], (size_t)g.d * c->d_ff * 2));
       LIME_CUDA(need(&c->WprepT[j], prep_rows * g.d * 2));
-      LIME_CUDA(need(&c->WpostT[j], (size_t)2 * c->d_ff * g.H * g.d * 2));
+      if (!plain_v) LIME_CUDA(need(&c->WpostT[j], (size_t)2 * c->d_ff * g.H * g.d * 2));
       if ((s = launch_transpose_bf16(w->Wo[j], c->d_ff, g.d, c->WoT[j], st)) != LIME_OK) return s;
       if (plain_v) {
         // [W_g | W_u]^T [2f x d]: the history update applies the GatedMLP weights as they stand

@@ -394,11 +394,12 @@ lime_status launch_gemm_rows_t(const void* A, int64_t M, int K, const void* Bt, 
 // GatedMLP on link rows fused with its consumers (k_link_mlp_tc.cu); d = d_ff in {128, 256}
 struct LinkMlpArgs {
   const void* Ohat; int64_t M; int K; int d;   // attention rows [M x K = H*d] bf16
-  const void* WpostT; const void* WoT;         // folded [2f x H*d] and transposed [d x f] weights, bf16
+  const void* WpostT; const void* WoT;         // folded [2f x H*d] (d = 128) and transposed [d x f] weights, bf16
+  const void *WvT, *WguT;                      // d = 256: W_V transposed [d x d], [W_g | W_u] transposed [2f x d]
   float* T_out;                                // nullable: the layer's link rows, fp32 [M x d]
   float* LP; int lp_accumulate;                // nullable running sum of Eq. 8 (0: assign, 1: add)
   void* That_next;                             // nullable: bf16 LN(T) for the next layer's link-side GEMM
-  void* link_states;                           // nullable: bf16 copy of LP after this layer
+  void* link_states;                           // nullable: bf16 copy of LP after this layer, which is then not stored
   int ln; float ln_eps;
   int* err;
 };
