@@ -12,7 +12,10 @@
 // The epilogue, one thread pair per row, writes what the rest of the layer stack needs:
 //   - T^j as fp32 (only when the caller asks for the layer's link rows)
 //   - L^P (+)= T^j, the running sum of Eq. 8
-//   - LN(T^j) as bf16, the A operand of the next layer's link-side GEMM (LayerNorm before the projections, App. C)
+//   - LN(T^j) as bf16, the A operand of the next layer's link-side GEMM (LayerNorm before the projections, App. C), or
+//   - (d = 128, the next layer is the last) that layer's folded queries Q2 = LN(T^j) . W, the only operands it needs: four or
+//     more tiles of 128 columns, formed here under the history update that runs beside this kernel, instead of a launch of
+//     the link-side GEMM between the update and the next attention (256 users x 32 links: 6.5 us)
 //   - on the last layer, the link states bf16(L^P) of Eq. 4 in its place when no candidate-side value projection follows
 // One CTA per 128 rows.  Warp 0 TMA producer, warp 1 MMA issuer, warps 2-9 epilogue (two threads per row, half of the
 // columns each; a warp may only touch the TMEM lane quarter warp_id % 4).
@@ -38,6 +41,10 @@ struct LmLayout {                                                      // d = 12
   static constexpr uint32_t WO_BYTES = 2 * LM_SUB;
   static constexpr uint32_t OFF_U = OFF_WO + WO_BYTES;                 // U [128 x 128]: 2 K-blocks
   static constexpr uint32_t OPS_END = OFF_U + 2 * LM_SUB;
+  // the queries of the next layer: LN(T) [128 x 128] behind the staged fp32 tile, a patch of 1 KB per epilogue warp, the weights of a
+  // tile [128 x 128] over W_o and over U in turn
+  static constexpr uint32_t OFF_LN = (LmOut<128>::OFF_TH + 1023) / 1024 * 1024, OFF_PATCH = OFF_LN + 2 * LM_SUB;
+  static_assert(OFF_PATCH + 8 * 1024 <= OFF_WO && WO_BYTES == 2 * LM_SUB, "beside the operands of the last contraction");
   static constexpr uint32_t OFF_EXCH = OPS_END > LmOut<128>::END ? OPS_END : LmOut<128>::END;   // [2 slots][2 halves][128] floats
   static constexpr uint32_t OFF_BAR = OFF_EXCH + 4 * 128 * 4;
   static constexpr uint32_t SMEM = OFF_BAR + 256;
@@ -64,6 +71,8 @@ struct LinkMlpParams {
   float* LP;                    // nullable: fp32 [M x d] running sum
   int lp_accumulate;            // 0: LP = T, 1: LP += T
   __nv_bfloat16* That_next;     // nullable: bf16 [M x d] = LN(T) (or T when ln == 0)
+  __nv_bfloat16* Q2;            // nullable (d = 128): [users x H*ell x d], the next layer's queries
+  int ell;
   __nv_bfloat16* link_states;   // nullable: bf16 [M x d] = LP after this layer, which is then not stored
   int ln;
   float ln_eps;
@@ -105,9 +114,10 @@ __device__ __forceinline__ void lm_glu(uint8_t* ub, uint32_t gates, uint32_t r) 
 
 // The epilogue of T = U . W_o, by the eight epilogue warps once the last contraction is done: this thread's D/2 columns of its row (TMEM
 // columns col_out on), 64 at a time.
+// With p.Q2 the rows LN(T) go to the operand at `ln_at` instead of global memory.  Returns whether every wait ended well.
 template <int D>
-__device__ __forceinline__ void lm_epilogue(const LinkMlpParams& p, uint8_t* smem, uint32_t lane_addr, uint32_t col_out, int64_t m0, int ew, int q, int half,
-                                            uint32_t r, int lane, float* exch, uint64_t* all_bar, uint64_t* pair_bar) {
+__device__ __forceinline__ bool lm_epilogue(const LinkMlpParams& p, uint8_t* smem, uint32_t lane_addr, uint32_t col_out, int64_t m0, int ew, int q, int half,
+                                            uint32_t r, int lane, float* exch, uint64_t* all_bar, uint64_t* pair_bar, uint8_t* ln_at) {
   using namespace tc;
   using Lay = LmOut<D>;
   bool ok = true;
@@ -139,7 +149,8 @@ __device__ __forceinline__ void lm_epilogue(const LinkMlpParams& p, uint8_t* sme
   }
   __syncwarp();
   if (lane == 0) mbar_arrive(all_bar);
-  if (mbar_wait(all_bar, 0, p.err, 79)) {
+  ok = mbar_wait(all_bar, 0, p.err, 79);
+  if (ok) {
     // a warp takes rows ew, ew + 8, ...; the reads of the running sum for a batch of rows are issued together
     constexpr int BATCH = 8;
     const int n_valid = (int)(p.M - m0 < 128 ? p.M - m0 : 128);
@@ -170,7 +181,7 @@ __device__ __forceinline__ void lm_epilogue(const LinkMlpParams& p, uint8_t* sme
       }
     }
   }
-  if (p.That_next) {
+  if (p.That_next || p.Q2) {
     // LN(T) for the next layer's link-side GEMM: the two halves of a row exchange their partial sums
     float mu = 0.f, rstd = 1.f;
     if (p.ln) {
@@ -183,7 +194,7 @@ __device__ __forceinline__ void lm_epilogue(const LinkMlpParams& p, uint8_t* sme
         return w;
       };
       exch[half * 128 + r] = s;
-      ok = pair_sync(77);
+      ok = ok && pair_sync(77);
       mu = (s + exch[(half ^ 1) * 128 + r]) * (1.0f / D);
       float var = 0.f;
 #pragma unroll
@@ -209,12 +220,15 @@ __device__ __forceinline__ void lm_epilogue(const LinkMlpParams& p, uint8_t* sme
         uint4 o;
         o.x = lm_pack((v[j] - mu) * rstd, (v[j + 1] - mu) * rstd); o.y = lm_pack((v[j + 2] - mu) * rstd, (v[j + 3] - mu) * rstd);
         o.z = lm_pack((v[j + 4] - mu) * rstd, (v[j + 5] - mu) * rstd); o.w = lm_pack((v[j + 6] - mu) * rstd, (v[j + 7] - mu) * rstd);
-        *reinterpret_cast<uint4*>(Th + r * TH_LD + half * (D / 2) + ch * 64 + j) = o;
+        if (p.Q2) *reinterpret_cast<uint4*>(ln_at + half * LM_SUB + lm_chunk(r, (uint32_t)(j >> 3))) = o;        // (D = 128)
+        else *reinterpret_cast<uint4*>(Th + r * TH_LD + half * (D / 2) + ch * 64 + j) = o;
       }
     }
+    if (p.Q2) return ok;
     __syncwarp();
     if (lane == 0) mbar_arrive(all_bar);
-    if (ok && mbar_wait(all_bar, 1, p.err, 80)) {
+    ok = ok && mbar_wait(all_bar, 1, p.err, 80);
+    if (ok) {
 #pragma unroll 4
       for (int i = ew; i < 128; i += 8) {
         const int64_t grow = m0 + i;
@@ -225,11 +239,12 @@ __device__ __forceinline__ void lm_epilogue(const LinkMlpParams& p, uint8_t* sme
       }
     }
   }
+  return ok;
 }
 
 __global__ void __launch_bounds__(LM_THREADS, 1)
 k_link_mlp_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-              const __grid_constant__ CUtensorMap tmWo, const LinkMlpParams p) {
+              const __grid_constant__ CUtensorMap tmWo, const __grid_constant__ CUtensorMap tmQ, const LinkMlpParams p) {
   using namespace tc;
   using Lay = LmLayout;
   constexpr int D = 128, STAGES = Lay::STAGES;
@@ -247,6 +262,11 @@ k_link_mlp_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   uint64_t* out_full = bars + 9;         // T complete
   uint64_t* pair_bar = bars + 10;        // [4], 2 warps each
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 14);
+  uint64_t* ln_ready = bars + 16;        // LN(T) in shared memory, T read (8 warps)
+  uint64_t* q_full = bars + 17;          // [2] weights of a tile of queries
+  uint64_t* q_empty = bars + 19;         // [2]
+  uint64_t* acc_full = bars + 21;        // [2] a tile of queries complete, in the columns of gate or up
+  uint64_t* acc_empty = bars + 23;       // [2] read (8 warps)
   uint64_t* all_bar = bars + 15;         // rendezvous of the 8 epilogue warps (tiles staged in shared memory)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -254,11 +274,13 @@ k_link_mlp_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-    mbar_init(wo_full, 1); mbar_init(gu_full, 1); mbar_init(u_ready, 8); mbar_init(out_full, 1);
+    mbar_init(wo_full, 1); mbar_init(gu_full, 1); mbar_init(u_ready, 8); mbar_init(out_full, 1); mbar_init(ln_ready, 8);
+    for (int i = 0; i < 2; ++i) { mbar_init(&q_full[i], 1); mbar_init(&q_empty[i], 1); mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 8); }
     for (int i = 0; i < 4; ++i) mbar_init(&pair_bar[i], 2);
     mbar_init(all_bar, 8);
     fence_barrier_init();
     prefetch_tmap(&tmA); prefetch_tmap(&tmB); prefetch_tmap(&tmWo);
+    if (p.Q2) prefetch_tmap(&tmQ);
   }
   if (warp == 1) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
   tc_fence_before();
@@ -287,9 +309,20 @@ k_link_mlp_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         tma_load_2d_hint(st + LM_SUB, &tmB, kb * 64, 0, &full[s], pol);           // gate rows
         tma_load_2d_hint(st + 2 * LM_SUB, &tmB, kb * 64, D, &full[s], pol);       // up rows
       }
+      // the next layer's query weights, a tile of 128 columns at a time, over W_o and U, once T has been formed from these
+      int nq = 0;
+      if (p.Q2 && ok) ok = mbar_wait(out_full, 0, p.err, 84);
+      for (; p.Q2 && ok && nq < p.H; ++nq) {
+        const int b = nq & 1;
+        if (!mbar_wait(&q_empty[b], ((uint32_t)(nq >> 1) & 1u) ^ 1u, p.err, 85)) { ok = false; break; }
+        mbar_arrive_expect_tx(&q_full[b], 2 * LM_SUB);
+        for (int kb = 0; kb < 2; ++kb)
+          tma_load_2d_hint(smem + (b ? Lay::OFF_U : Lay::OFF_WO) + (uint32_t)kb * LM_SUB, &tmQ, kb * 64, nq * 128, &q_full[b], pol);
+      }
       if (!ok || *(volatile int*)p.err != 0) {
         for (int j = 0; j < it && j < STAGES; ++j)
           mbar_wait_quiet(&full[(it - 1 - j) % STAGES], (uint32_t)((it - 1 - j) / STAGES) & 1u);
+        for (int j = 0; j < nq && j < 2; ++j) mbar_wait_quiet(&q_full[(nq - 1 - j) & 1], (uint32_t)((nq - 1 - j) >> 1) & 1u);
         mbar_wait_quiet(wo_full, 0);
       }
     }
@@ -321,6 +354,21 @@ k_link_mlp_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         }
         mma_commit(out_full);
       }
+      if (p.Q2 && ok) ok = mbar_wait(ln_ready, 0, p.err, 86);
+      for (int n = 0; p.Q2 && ok && n < p.H; ++n) {              // 4. the next layer's queries, over gate and up in turn
+        const int b = n & 1;
+        const uint32_t ph = (uint32_t)(n >> 1) & 1u;
+        ok = mbar_wait(&acc_empty[b], ph ^ 1u, p.err, 87) && mbar_wait(&q_full[b], ph, p.err, 88);
+        if (!ok) break;
+        tc_fence_after();
+        for (int kk = 0; kk < 8; ++kk) {
+          const uint32_t o = (uint32_t)(kk >> 2) * LM_SUB + (uint32_t)(kk & 3) * 32;
+          mma_bf16_ss(tmem_base + COL_GU + (uint32_t)b * 128, make_sdesc_k_sw128(sbase + Lay::OFF_LN + o),
+                      make_sdesc_k_sw128(sbase + (b ? Lay::OFF_U : Lay::OFF_WO) + o), idesc_128, kk != 0);
+        }
+        mma_commit(&q_empty[b]);
+        mma_commit(&acc_full[b]);
+      }
     }
   } else {
     const int ew = warp - 2;                                   // 0..7
@@ -336,8 +384,52 @@ k_link_mlp_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(u_ready);
-      if (mbar_wait(out_full, 0, p.err, 76))
-        lm_epilogue<D>(p, smem, lane_addr, COL_OUT, m0, ew, q, half, r, lane, exch, all_bar, pair_bar);
+      bool ok = mbar_wait(out_full, 0, p.err, 76);
+      if (ok) ok = lm_epilogue<D>(p, smem, lane_addr, COL_OUT, m0, ew, q, half, r, lane, exch, all_bar, pair_bar, smem + Lay::OFF_LN);
+      if (p.Q2 && ok) {
+        tc_fence_before();
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(ln_ready);
+        // rows of a tile leave as whole 128-byte lines through the warp's patch, as in k_gemm_tc.cu
+        uint8_t* patch = smem + Lay::OFF_PATCH + ew * 1024;
+        const int row = m0 + (int)r, HL = p.H * p.ell;
+        const int base_row = row < p.M ? row / p.ell * HL + row % p.ell : -1;
+        const int x7 = lane & 7, rsub = lane >> 3;
+        __nv_bfloat16* dst = p.Q2 + half * 64 + x7 * 8;
+        for (int n = 0; n < p.H; ++n) {
+          const int b = n & 1;
+          if (!mbar_wait(&acc_full[b], (uint32_t)(n >> 1) & 1u, p.err, 89)) break;
+          tc_fence_after();
+          float v[64];
+          tmem_ld_32x32(lane_addr + COL_GU + b * 128 + half * 64, *reinterpret_cast<float(*)[32]>(&v[0]));
+          tmem_ld_32x32(lane_addr + COL_GU + b * 128 + half * 64 + 32, *reinterpret_cast<float(*)[32]>(&v[32]));
+          tmem_wait_ld();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&acc_empty[b]);
+          uint4 o[8];
+#pragma unroll
+          for (int c = 0; c < 8; ++c)
+            o[c] = make_uint4(lm_pack(v[c * 8], v[c * 8 + 1]), lm_pack(v[c * 8 + 2], v[c * 8 + 3]), lm_pack(v[c * 8 + 4], v[c * 8 + 5]),
+                              lm_pack(v[c * 8 + 6], v[c * 8 + 7]));
+          const int out_row = base_row < 0 ? -1 : base_row + n * p.ell;
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            if (rsub == m) {
+#pragma unroll
+              for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(patch + x7 * 128 + ((c ^ x7) << 4)) = o[c];
+            }
+            __syncwarp();
+            const uint4 o0 = *reinterpret_cast<const uint4*>(patch + rsub * 128 + ((x7 ^ rsub) << 4));
+            const uint4 o1 = *reinterpret_cast<const uint4*>(patch + (rsub + 4) * 128 + ((x7 ^ (rsub + 4)) << 4));
+            const int r0 = __shfl_sync(0xffffffffu, out_row, m * 8 + rsub), r1 = __shfl_sync(0xffffffffu, out_row, m * 8 + rsub + 4);
+            if (r0 >= 0) *reinterpret_cast<uint4*>(dst + (int64_t)r0 * D) = o0;
+            if (r1 >= 0) *reinterpret_cast<uint4*>(dst + (int64_t)r1 * D) = o1;
+            __syncwarp();
+          }
+        }
+      }
     }
   }
 
@@ -538,7 +630,7 @@ k_link_mlp_d256_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constan
       if (lane == 0) mbar_arrive(&u_ready[hf]);
     }
     if (ok && mbar_wait(out_full, 0, p.err, 76))
-      lm_epilogue<D>(p, smem, lane_addr, COL_O, m0, ew, q, half, r, lane, exch, all_bar, pair_bar);
+      lm_epilogue<D>(p, smem, lane_addr, COL_O, m0, ew, q, half, r, lane, exch, all_bar, pair_bar, nullptr);
   }
 
   tc_fence_before();
@@ -556,14 +648,16 @@ lime_status launch_link_mlp_tc(const LinkMlpArgs& a, cudaStream_t st) {
   const uint64_t K = (uint64_t)a.K, d = (uint64_t)a.d;
   const bool wide = a.d == 256;
   if (wide && a.K != 2 * 256 && a.K != 4 * 256 && a.K != 8 * 256) return LIME_UNSUPPORTED_SHAPE;
-  CUtensorMap tmA, tmB, tmV, tmWo;
+  CUtensorMap tmA, tmB, tmV, tmWo, tmQ;
+  if (a.Q2 && (wide || a.WprepT == nullptr || a.ell < 1 || a.M * (a.K / 128) > 0x7fffffff)) return LIME_INVALID_ARG;
   if (!make_tmap_bf16_sw128(&tmA, a.Ohat, (uint64_t)a.M, K, K, 128) ||
       !make_tmap_bf16_sw128(&tmB, wide ? a.WguT : a.WpostT, 2 * d, wide ? d : K, wide ? d : K, 128) ||
-      (wide && !make_tmap_bf16_sw128(&tmV, a.WvT, d, d, d, (uint32_t)(a.d * a.d / a.K))) || !make_tmap_bf16_sw128(&tmWo, a.WoT, d, d, d, 128))
+      (wide && !make_tmap_bf16_sw128(&tmV, a.WvT, d, d, d, (uint32_t)(a.d * a.d / a.K))) || !make_tmap_bf16_sw128(&tmWo, a.WoT, d, d, d, 128) ||
+      !make_tmap_bf16_sw128(&tmQ, a.Q2 ? a.WprepT : a.WoT, a.Q2 ? K : d, d, d, 128))
     return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
   LinkMlpParams p;
   p.M = a.M; p.kblocks = a.K / 64; p.H = a.K / a.d; p.T_out = a.T_out; p.LP = a.LP; p.lp_accumulate = a.lp_accumulate;
-  p.That_next = (__nv_bfloat16*)a.That_next; p.link_states = (__nv_bfloat16*)a.link_states; p.ln = a.ln; p.ln_eps = a.ln_eps;
+  p.Q2 = (__nv_bfloat16*)a.Q2; p.ell = a.ell; p.That_next = (__nv_bfloat16*)a.That_next; p.link_states = (__nv_bfloat16*)a.link_states; p.ln = a.ln; p.ln_eps = a.ln_eps;
   p.err = a.err;
   const dim3 grid((unsigned)((a.M + 127) / 128));
   static bool smem_set[2][kMaxDeviceOrdinals] = {};
@@ -575,7 +669,7 @@ lime_status launch_link_mlp_tc(const LinkMlpArgs& a, cudaStream_t st) {
     launch_pdl(k_link_mlp_d256_tc, grid, dim3(LM_THREADS), Lm256::SMEM, st, tmA, tmV, tmB, tmWo, p);
   } else {
     ProfScope _p("k_link_mlp_tc", st);
-    launch_pdl(k_link_mlp_tc, grid, dim3(LM_THREADS), LmLayout::SMEM, st, tmA, tmB, tmWo, p);
+    launch_pdl(k_link_mlp_tc, grid, dim3(LM_THREADS), LmLayout::SMEM, st, tmA, tmB, tmWo, tmQ, p);
   }
   LIME_LAUNCH_CHECK("k_link_mlp_tc");
   return LIME_OK;

@@ -283,7 +283,8 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
   // The link side and the history update need nothing of each other: the update runs beside it (lime_common.cuh), which takes the
   // shorter of the two off the layer where SMs are free and evens out the tiles where they are not.  Eighths of a tile that a block of
   // the link side takes, by measurement (us a batch with 0 / 8 / 16 / 20 / 24 / 32 / 40, and with the update behind the link side):
-  // d = 128, three kernels: 256 users x 512, two layers 139.5 / 139.3 / 135.9 / 135.7 / 137.8 / 137.8 / 140.2, 140.3; 150 users of
+  // d = 128, three kernels (20 where the link-side GEMM follows, 32 where the queries are made along, 132.7 with 16, 133.0, 132.8, 130.4,
+  // 132.2 with 40): 256 users x 512, two layers 139.5 / 139.3 / 135.9 / 135.7 / 137.8 / 137.8 / 140.2, 140.3; 150 users of
   // 100..1500, 64 links, four layers 345.9 / 345.4 / 331.2 / 343.4 / 343.8 / 343.8 / 355.2, 351.6 (a tile of 256 stacked rows takes
   // longer); one kernel: 40 users of 100..1500 72.3 / 72.3 / 70.5 / 70.3 / 70.5 / 63.0 / 63.0, 74.3; 32 users of 2000..4000, 64 links
   // 269.8 / 268.8 / 260.4 / 260.2 / 260.5 / 261.6 / 267.8, 276.2; d = 256, 32 links: 64 users of 100..1024, three layers 244.8 / 225.4 /
@@ -292,7 +293,7 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
   BesideLinkSide beside;
   if (c->side256) beside = beside_link_side(link_side_d256_blocks(B), 14, w.n_tile_upper, B);
   else if (side1 != nullptr) beside = beside_link_side(link_side_d128_blocks((int64_t)B * g.ell), wide ? 24 : 30, w.n_tile_upper, B);
-  else beside = beside_link_side(((int64_t)B * g.ell + 127) / 128, c->tc_mode == 2 ? 16 : wide ? 16 : 20, w.n_tile_upper, B);
+  else beside = beside_link_side(((int64_t)B * g.ell + 127) / 128, mlp.Q2 ? (wide ? 20 : 32) : wide || c->tc_mode == 2 ? 16 : 20, w.n_tile_upper, B);
   if ((s = c->tc_mode == 2 ? launch_link_attn_d256_tc(la, st) : launch_link_attn_tc(la, st)) != LIME_OK) return s;
   if (c->side256) {
     // merge, T^j and what follows from it - the next layer's operands included - in one kernel; `side` says what is wanted
@@ -396,6 +397,8 @@ static lime_status encode_user_tc(Ctx* c, const void* hist, bool hist_normalized
   // alternate between two sets (Q2 is the attention's, complete by then)
   const bool few_rows = few_link_rows(c, B);
   const LinkOperands set[2] = {{w.Q2, w.K2, w.G2t, w.U2t, w.V2t, w.cQ, w.cK, 0}, {w.Q2, w.K2b, w.G2tb, w.U2tb, w.V2t, w.cQ, w.cK, 0}};
+  // the last layer needs its queries only: the GatedMLP kernel of the layer before makes them along with its rows
+  auto queries_along = [&](int j) { return c->tc_mode == 1 && !few_rows && j > 0 && j == g.n_layers - 1; };
   for (int j = 0; j < g.n_layers; ++j) {
     const bool last = j == g.n_layers - 1;
     const bool raw = g.ln && j == 0 && !hist_normalized;      // rows that still need their LayerNorm want the operands' row sums
@@ -404,7 +407,7 @@ static lime_status encode_user_tc(Ctx* c, const void* hist, bool hist_normalized
       ops = LinkOperands{c->sh_Q2, c->sh_K2, c->sh_G2t, c->sh_U2t, c->sh_V2t, c->sh_cQ, c->sh_cK, 1};
     } else {
       if (j == 0 && (s = launch_ln_rows_bf16(link_ctx, BL, g.d, g.ln, c->ln_eps, w.That, st)) != LIME_OK) return s;
-      if ((j == 0 || !few_rows) &&
+      if ((j == 0 || !(few_rows || queries_along(j))) &&
           (s = make_link_operands(c, j, w.That, BL, !last, w.Q2, w.K2, w.G2t, w.U2t, w.V2t, raw ? w.cQ : nullptr, raw ? w.cK : nullptr, st)) != LIME_OK)
         return s;
       ops = set[few_rows ? j & 1 : 0];
@@ -419,7 +422,8 @@ static lime_status encode_user_tc(Ctx* c, const void* hist, bool hist_normalized
     }
     LinkMlpArgs mlp{};
     mlp.LP = w.LP; mlp.lp_accumulate = j > 0;                                   // L^P = sum_j T^j  (Eq. 8)
-    mlp.That_next = last ? nullptr : w.That;
+    mlp.That_next = last || queries_along(j + 1) ? nullptr : w.That;
+    if (queries_along(j + 1)) { mlp.Q2 = w.Q2; mlp.WprepT = c->WprepT[j + 1]; mlp.ell = g.ell; }
     mlp.link_states = (last && !c->w.cand_Wv && c->cand_heads == 1) ? link_states : nullptr;
     s = tc_layer_core(c, j, j == 0 ? hist : w.S, off, B, total, ops, last ? nullptr : w.S, raw ? 1 : 0,
                       (g.ln && !last) ? 1 : 0, mlp, nullptr, few_rows ? &side1 : nullptr, w, st);

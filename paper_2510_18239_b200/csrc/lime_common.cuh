@@ -399,6 +399,7 @@ struct LinkMlpArgs {
   float* T_out;                                // nullable: the layer's link rows, fp32 [M x d]
   float* LP; int lp_accumulate;                // nullable running sum of Eq. 8 (0: assign, 1: add)
   void* That_next;                             // nullable: bf16 LN(T) for the next layer's link-side GEMM
+  void* Q2; const void* WprepT; int ell;       // d = 128, nullable: instead of it the next layer's queries [M / ell x K/d*ell x d]
   void* link_states;                           // nullable: bf16 copy of LP after this layer, which is then not stored
   int ln; float ln_eps;
   int* err;
