@@ -73,11 +73,11 @@ k_layer_schedules(const int32_t* __restrict__ off, int B, const ChunkRule rule, 
   const int n_first = (int)threadIdx.x < B ? off[threadIdx.x + 1] - off[threadIdx.x] : 0;
   auto length = [&](int b) { return b < (int)blockDim.x ? n_first : off[b + 1] - off[b]; };      // b: one of this thread's
   int longest = 0, short_items = 0;
-  if (rule.short_tokens > 0) {
+  if (rule.short_tokens > 0 || rule.fit_groups > 0) {
     for (int b = threadIdx.x; b < B; b += blockDim.x) {
       const int n = length(b);
       longest = max(longest, n);
-      if (n > rule.short_tokens) short_items += (n + rule.short_tokens - 1) / rule.short_tokens;
+      if (rule.short_tokens > 0 && n > rule.short_tokens) short_items += (n + rule.short_tokens - 1) / rule.short_tokens;
     }
     longest = __reduce_max_sync(0xffffffffu, longest);
     short_items = __reduce_add_sync(0xffffffffu, short_items);
@@ -88,7 +88,46 @@ k_layer_schedules(const int32_t* __restrict__ off, int B, const ChunkRule rule, 
     longest = __reduce_max_sync(0xffffffffu, w.x);
     short_items = __reduce_add_sync(0xffffffffu, w.y);
   }
-  const int chunk = longest > 2 * rule.short_tokens && short_items <= rule.short_items ? rule.short_tokens : rule.tokens;
+  const bool take_short = rule.short_tokens > 0 && longest > 2 * rule.short_tokens && short_items <= rule.short_items;
+  int chunk = take_short ? rule.short_tokens : rule.tokens;
+  if (rule.fit_groups > 0 && !take_short && longest > chunk && B <= 3 * SCAP) {
+    // Rounds of the groups over the items, each with its tiles and what an item costs besides (draining the pipeline, the way out of its
+    // accumulator, filling it again: 8800 cycles with partials to write, 3100 without, a tile of 128 tokens takes 1490): the length for
+    // which that comes out least.  A warp per length.  64 links, us with 2048 tokens (or the power of two that the total asks for) / fitted:
+    // 32 users of 32768, four layers 1646 / 1570; three layers, 10 of 30000 380 / 337, 16 of 4000..8000 191 / 167, 4 of 32768 212 / 186.
+    constexpr float OVER_PART = 5.9f, OVER_ONE = 2.1f;
+    __shared__ float best_cost[32];
+    __shared__ int best_tiles[32];
+    int tiles_all = 0;
+    for (int b = threadIdx.x; b < B; b += blockDim.x) small[b] = max(length(b), 0);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+    for (int b = lane; b < B; b += 32) tiles_all += (small[b] + 127) / 128;
+    tiles_all = __reduce_add_sync(0xffffffffu, tiles_all);
+    float cost = INFINITY;
+    int at = 0;
+    for (int t = (rule.tokens * 3 / 4 + 127) / 128 + wid; t <= 64; t += n_warps) {
+      int items = 0, ones = 0;
+      for (int b = lane; b < B; b += 32) {
+        const int k = (small[b] + t * 128 - 1) / (t * 128);
+        items += k;
+        ones += k == 1;
+      }
+      items = __reduce_add_sync(0xffffffffu, items);
+      ones = __reduce_add_sync(0xffffffffu, ones);
+      const float c = (float)((items + rule.fit_groups - 1) / rule.fit_groups) *
+                      ((float)tiles_all + OVER_PART * (float)(items - ones) + OVER_ONE * (float)ones) / (float)items;
+      if (items <= rule.fit_items && c < cost) { cost = c; at = t; }
+    }
+    if (lane == 0) { best_cost[wid] = cost; best_tiles[wid] = at; }
+    __syncthreads();
+    cost = INFINITY;
+    at = 0;
+    for (int w = 0; w < n_warps; ++w)
+      if (best_cost[w] < cost || (best_cost[w] == cost && best_tiles[w] < at)) { cost = best_cost[w]; at = best_tiles[w]; }
+    if (at > 0) chunk = at * 128;
+    __syncthreads();
+  }
   // does any user's attention output need the merge step (several chunks to combine, or no history: a zero row)?
   int merge = 0;
   for (int b = threadIdx.x; b < B; b += blockDim.x)

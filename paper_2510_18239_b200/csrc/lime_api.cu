@@ -169,8 +169,12 @@ static Workspace carve(const Ctx* c, void* base, int32_t B, int64_t total) {
   w.chunk.tokens = tc_link ? pick_chunk(total, row_blocks, many ? 2048 : 512, c->tc_mode == 2 ? 4096 : 2048) : pick_chunk(total, 1, 64);
   if (many) { w.chunk.short_tokens = 512; w.chunk.short_items = 64 / row_blocks; }
   w.chunk_dev = (int32_t*)take(4);
-  const int64_t split_items = (total + w.chunk.tokens - 1) / w.chunk.tokens;
+  // d = 128: the items go round-robin to the groups of CTAs that run at once, so k_layer_schedules fits their length to these
+  const bool fit = c->tc_mode == 1;
+  const int least = fit ? w.chunk.tokens * 3 / 4 : w.chunk.tokens;
+  const int64_t split_items = (total + least - 1) / least;
   w.n_chunk_upper = (int)((split_items > w.chunk.short_items ? split_items : w.chunk.short_items) + B);
+  if (fit) { w.chunk.fit_groups = link_attn_d256_groups(w.n_chunk_upper, g.H, g.ell); w.chunk.fit_items = w.n_chunk_upper; }
   w.n_tile_upper = (int)((total + kHistTile - 1) / kHistTile + B);
   w.chunk_user = (int32_t*)take((size_t)w.n_chunk_upper * 4);
   if (c->tc_mode == 2) {

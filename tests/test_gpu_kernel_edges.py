@@ -457,6 +457,14 @@ def test_history_update_beside_the_link_side(d, H, ell, lengths, raw):
     _encode_against_oracle(synth.BF16, d, H, ell, 3, lengths, "softmax", raw, True, 6e-2, 3e-2)
 
 
+@pytest.mark.parametrize("d,H,ell", [(128, 4, 32), (128, 4, 64)])
+@pytest.mark.parametrize("lengths", [[9000, 100], [2300] * 30 + [0], [4100, 700] * 6, [6000], [2049] * 66])
+@pytest.mark.parametrize("raw", [False, True])
+def test_chunk_length_fitted_to_the_groups(d, H, ell, lengths, raw):
+    """Histories longer than a work item: its length is what fits the CTAs that run at once, 3 to 64 tiles."""
+    _encode_against_oracle(synth.BF16, d, H, ell, 2, lengths, "softmax", raw, False, 6e-2, 2.5e-2)
+
+
 def test_one_long_history_is_split_among_many_users():
     """One user of 4000 tokens among 99 of 100, against 100 users of 100 (d = 128): 1.46 times the time where a history is one work item
     whenever the users are many, 1.16 times split."""
