@@ -23,10 +23,12 @@
 //  * d = 128, three score buffers: two groups of softmax warps take alternate tiles, one thread per row.  d = 256, two
 //    buffers: the chain of a buffer is what repeats, so all eight warps take every tile, two threads per row.
 // Measured: d = 256, 64 links (1024 users of 1024..4096 tokens) 1.51 -> 1.04 ms a launch (0.61 of the tensor peak at the
-// clock it runs at; 64-token tiles with P in shared memory and one issuing thread before); d = 128, 64 links, 32 users x
-// 32768 tokens 172 -> 128 us, bound by the exponentials (16 a cycle and SM: 1024 cycles of a tile's ~1500); 256 users x 512
-// tokens, 32 links 20 -> 16 us.  Dropped: 16 softmax warps at d = 128 (two threads per row and two groups: 200 us, the
-// polling takes the issue slots), prefetching token tiles into L2 (no change).
+// clock it runs at; 64-token tiles with P in shared memory and one issuing thread before); d = 128, 64 links, 32 users x 32768
+// tokens 172 -> 128 us and, with the items fitted to the CTAs (k_misc.cu), 110; 256 users x 512 tokens, 32 links 20 -> 16 us.
+// A tile of d = 128 takes 1490 cycles, 1024 of them the exponentials' (16 a cycle and SM), and an item 3100 to 8800 besides.
+// Dropped: 16 softmax warps at d = 128 (two threads per row and two groups: 200 us, the polling takes the issue slots),
+// prefetching token tiles into L2 (no change), a quarter to a half of the exponentials as polynomials on the FMA pipes (no
+// change to 15 % slower: the chain is what repeats, not the unit).
 #include "lime_common.cuh"
 #include "tc_common.cuh"
 

@@ -50,6 +50,9 @@ __global__ void __launch_bounds__(1024) k_offsets(const int32_t* __restrict__ le
 // 1024..4096 tokens over 37 groups); this order leaves it under 1 %.  A round is one rank computation over
 // the G loads in shared memory and one barrier.
 // group_start[G+1], group_items[items]: the items of group j in the order it takes them.  scratch: 4 x items ints.
+// FIT: the lengths of the items are fitted where some history is longer than one (rule.fit_groups); an instance of its own, because the
+// code alone, never reached, cost the batch of 256 users x 512 4.5 us.
+template <bool FIT>
 __global__ void __launch_bounds__(1024)
 k_layer_schedules(const int32_t* __restrict__ off, int B, const ChunkRule rule, int32_t* __restrict__ chunk_out,
                   int32_t* __restrict__ chunk_start, int tile,
@@ -73,11 +76,11 @@ k_layer_schedules(const int32_t* __restrict__ off, int B, const ChunkRule rule, 
   const int n_first = (int)threadIdx.x < B ? off[threadIdx.x + 1] - off[threadIdx.x] : 0;
   auto length = [&](int b) { return b < (int)blockDim.x ? n_first : off[b + 1] - off[b]; };      // b: one of this thread's
   int longest = 0, short_items = 0;
-  if (rule.short_tokens > 0 || rule.fit_groups > 0) {
+  if (rule.short_tokens > 0 || FIT) {
     for (int b = threadIdx.x; b < B; b += blockDim.x) {
       const int n = length(b);
       longest = max(longest, n);
-      if (rule.short_tokens > 0 && n > rule.short_tokens) short_items += (n + rule.short_tokens - 1) / rule.short_tokens;
+      if ((!FIT || rule.short_tokens > 0) && n > rule.short_tokens) short_items += (n + rule.short_tokens - 1) / rule.short_tokens;
     }
     longest = __reduce_max_sync(0xffffffffu, longest);
     short_items = __reduce_add_sync(0xffffffffu, short_items);
@@ -88,13 +91,13 @@ k_layer_schedules(const int32_t* __restrict__ off, int B, const ChunkRule rule, 
     longest = __reduce_max_sync(0xffffffffu, w.x);
     short_items = __reduce_add_sync(0xffffffffu, w.y);
   }
-  const bool take_short = rule.short_tokens > 0 && longest > 2 * rule.short_tokens && short_items <= rule.short_items;
+  const bool take_short = longest > 2 * rule.short_tokens && short_items <= rule.short_items && (!FIT || rule.short_tokens > 0);
   int chunk = take_short ? rule.short_tokens : rule.tokens;
-  if (rule.fit_groups > 0 && !take_short && longest > chunk && B <= 3 * SCAP) {
+  if constexpr (FIT) if (!take_short && longest > chunk && B <= 3 * SCAP) {
     // Rounds of the groups over the items, each with its tiles and what an item costs besides (draining the pipeline, the way out of its
     // accumulator, filling it again: 8800 cycles with partials to write, 3100 without, a tile of 128 tokens takes 1490): the length for
     // which that comes out least.  A warp per length.  64 links, us with 2048 tokens (or the power of two that the total asks for) / fitted:
-    // 32 users of 32768, four layers 1646 / 1570; three layers, 10 of 30000 380 / 337, 16 of 4000..8000 191 / 167, 4 of 32768 212 / 186.
+    // 32 users of 32768, four layers 1670 / 1626; three layers, 10 of 30000 383 / 354, 16 of 4000..8000 188 / 168, 4 of 32768 203 / 185.
     constexpr float OVER_PART = 5.9f, OVER_ONE = 2.1f;
     __shared__ float best_cost[32];
     __shared__ int best_tiles[32];
@@ -224,7 +227,7 @@ lime_status launch_layer_schedules(const int32_t* off, int B, const ChunkRule& c
                                    int32_t* chunk_user, int32_t* merge_needed, const GroupSchedule& gs, cudaStream_t st) {
   if (gs.group_start != nullptr && (gs.n_groups < 1 || gs.n_groups > 160 || gs.att_tile < 1)) return LIME_INVALID_ARG;
   ProfScope _p("k_layer_schedules", st);
-  launch_pdl(k_layer_schedules, dim3(1), dim3(schedule_threads(B)), 0, st, off, B, chunk, chunk_out, chunk_start, tile, tile_start, chunk_user, merge_needed,
+  launch_pdl(chunk.fit_groups > 0 ? k_layer_schedules<true> : k_layer_schedules<false>, dim3(1), dim3(schedule_threads(B)), 0, st, off, B, chunk, chunk_out, chunk_start, tile, tile_start, chunk_user, merge_needed,
              gs.n_groups, gs.att_tile, gs.group_start, gs.group_items, gs.scratch);
   LIME_LAUNCH_CHECK("k_layer_schedules");
   return LIME_OK;

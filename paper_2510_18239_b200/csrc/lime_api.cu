@@ -169,10 +169,11 @@ static Workspace carve(const Ctx* c, void* base, int32_t B, int64_t total) {
   w.chunk.tokens = tc_link ? pick_chunk(total, row_blocks, many ? 2048 : 512, c->tc_mode == 2 ? 4096 : 2048) : pick_chunk(total, 1, 64);
   if (many) { w.chunk.short_tokens = 512; w.chunk.short_items = 64 / row_blocks; }
   w.chunk_dev = (int32_t*)take(4);
-  // d = 128: the items go round-robin to the groups of CTAs that run at once, so k_layer_schedules fits their length to these
-  const bool fit = c->tc_mode == 1;
-  const int least = fit ? w.chunk.tokens * 3 / 4 : w.chunk.tokens;
-  const int64_t split_items = (total + least - 1) / least;
+  // d = 128: the items go round-robin to the groups of CTAs that run at once, so k_layer_schedules fits their length to these where the
+  // histories are half an item long on average and the items more than the groups (one user of 30000 tokens, one round, three layers
+  // with 64 links: 117.5 us, 122 fitted; 4 of 32768: 202.7, 184.8)
+  const bool fit = c->tc_mode == 1 && 2 * total >= (int64_t)w.chunk.tokens * B && total * row_blocks > (int64_t)w.chunk.tokens * kSMs;
+  const int64_t split_items = (total + w.chunk.tokens - 1) / w.chunk.tokens;
   w.n_chunk_upper = (int)((split_items > w.chunk.short_items ? split_items : w.chunk.short_items) + B);
   if (fit) { w.chunk.fit_groups = link_attn_d256_groups(w.n_chunk_upper, g.H, g.ell); w.chunk.fit_items = w.n_chunk_upper; }
   w.n_tile_upper = (int)((total + kHistTile - 1) / kHistTile + B);
@@ -287,10 +288,10 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
   // The link side and the history update need nothing of each other: the update runs beside it (lime_common.cuh), which takes the
   // shorter of the two off the layer where SMs are free and evens out the tiles where they are not.  Eighths of a tile that a block of
   // the link side takes, by measurement (us a batch with 0 / 8 / 16 / 20 / 24 / 32 / 40, and with the update behind the link side):
-  // d = 128, three kernels (20 where the link-side GEMM follows, 32 where the queries are made along, 132.7 with 16, 133.0, 132.8, 130.4,
-  // 132.2 with 40): 256 users x 512, two layers 139.5 / 139.3 / 135.9 / 135.7 / 137.8 / 137.8 / 140.2, 140.3; 150 users of
-  // 100..1500, 64 links, four layers 345.9 / 345.4 / 331.2 / 343.4 / 343.8 / 343.8 / 355.2, 351.6 (a tile of 256 stacked rows takes
-  // longer); one kernel: 40 users of 100..1500 72.3 / 72.3 / 70.5 / 70.3 / 70.5 / 63.0 / 63.0, 74.3; 32 users of 2000..4000, 64 links
+  // d = 128, the merge and the GatedMLP, a GEMM behind the update: 256 users x 512, two layers 139.5 / 139.3 / 135.9 / 135.7 / 137.8 /
+  // 137.8 / 140.2, 140.3; 150 users of 100..1500, 64 links, four layers 345.9 / 345.4 / 331.2 / 343.4 / 343.8 / 343.8 / 355.2, 351.6 (a
+  // tile of 256 stacked rows takes longer); the queries made along (mlp.Q2): 256 users x 512 136.7 with 0, 132.7 / 133.0 / 132.8 / 130.4 /
+  // 132.2 with 16 / 20 / 24 / 32 / 40; one kernel: 40 users of 100..1500 72.3 / 72.3 / 70.5 / 70.3 / 70.5 / 63.0 / 63.0, 74.3; 32 users of 2000..4000, 64 links
   // 269.8 / 268.8 / 260.4 / 260.2 / 260.5 / 261.6 / 267.8, 276.2; d = 256, 32 links: 64 users of 100..1024, three layers 244.8 / 225.4 /
   // 224.7 / 226.8 / 226.6 / 245.6 / 264.4, 245.8; 16 users 135.9 / 111.5 / 111.2 / 111.5 / 111.8 / 111.7 / 111.2, 143.5.
   const int wide = g.H * g.ell > 128;

@@ -224,7 +224,7 @@ struct GroupSchedule {
 };
 // How long the work items of the links <- history attention are: `tokens`, or `short_tokens` (0: never) where some history is over
 // twice as long as that and the histories longer than it make no more than `short_items` such chunks.
-// Where some history is longer than `tokens` and not the short ones are taken, the length of 3/4 of `tokens` to 64 tiles of 128 that fits
+// Where some history is longer than `tokens` and not the short ones are taken, the length of up to 64 tiles of 128 that fits
 // the `fit_groups` groups of CTAs best, of at most `fit_items` items (fit_groups 0: `tokens` as it is).
 struct ChunkRule { int tokens = 0, short_tokens = 0, short_items = 0, fit_groups = 0, fit_items = 0; };
 lime_status launch_layer_schedules(const int32_t* off, int B, const ChunkRule& chunk, int32_t* chunk_out, int32_t* chunk_start, int tile, int32_t* tile_start,
