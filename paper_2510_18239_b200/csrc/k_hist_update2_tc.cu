@@ -94,6 +94,7 @@ k_hist_update2_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant
   static_assert(64 % ELL == 0, "a thread owns whole heads");
   extern __shared__ __align__(1024) uint8_t smem[];
   if ((smem_u32(smem) & 1023u) != 0) {
+    pdl_wait();                                               // nobody leaves ahead of it (lime_common.cuh)
     if (threadIdx.x == 0) atomicCAS(p.err, 0, 94);
     return;
   }

@@ -114,6 +114,7 @@ k_hist_update_tmem_tc(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   constexpr int SLABS = 4 * NG;                               // slabs of a tile: halves x groups x 64 of 128 stacked rows
   extern __shared__ __align__(1024) uint8_t smem[];
   if ((smem_u32(smem) & 1023u) != 0) {                        // the swizzled tiles need a 1024-byte aligned base
+    pdl_wait();                                               // nobody leaves ahead of it (lime_common.cuh)
     if (threadIdx.x == 0) atomicCAS(p.err, 0, 98);
     return;
   }

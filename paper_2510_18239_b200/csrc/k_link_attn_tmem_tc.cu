@@ -181,6 +181,7 @@ k_link_attn_tmem_tc(const __grid_constant__ CUtensorMap tmX, const __grid_consta
   using Walk = LtItemWalk<G::STRIDED>;
   extern __shared__ __align__(1024) uint8_t smem[];
   if ((smem_u32(smem) & 1023u) != 0) {                     // the swizzled tiles need a 1024-byte aligned base
+    pdl_wait();                                               // nobody leaves ahead of it (lime_common.cuh)
     if (threadIdx.x == 0) atomicCAS(p.err, 0, 97);
     return;
   }

@@ -250,6 +250,7 @@ k_link_mlp_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   constexpr int D = 128, STAGES = Lay::STAGES;
   extern __shared__ __align__(1024) uint8_t smem[];
   if ((smem_u32(smem) & 1023u) != 0) {
+    pdl_wait();                                               // nobody leaves ahead of it (lime_common.cuh)
     if (threadIdx.x == 0) atomicCAS(p.err, 0, 93);
     return;
   }
@@ -458,6 +459,7 @@ k_link_mlp_d256_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constan
   constexpr int D = 256;
   extern __shared__ __align__(1024) uint8_t smem[];
   if ((smem_u32(smem) & 1023u) != 0) {
+    pdl_wait();                                               // nobody leaves ahead of it (lime_common.cuh)
     if (threadIdx.x == 0) atomicCAS(p.err, 0, 93);
     return;
   }

@@ -149,12 +149,21 @@ lime_status cuda_fail(cudaError_t e, const char* where);
 //    what to prefetch, past L1, and are read again afterwards;
 //  - a kernel that allocates tensor memory calls pdl_launch_dependents() only after its allocation, so a dependent CTA
 //    that shares the SM can never hold the columns a CTA of the running kernel still waits for.
+//  - no thread leaves a kernel ahead of pdl_wait(), on an error either: a kernel all of whose CTAs have left is complete although its
+//    predecessor may still run, and whoever waits for it would take that predecessor for complete too.
 // A kernel launched the ordinary way after such a kernel still waits for its completion, as always.
 //
 // A history update may run BESIDE the link side of its layer, launched right before it (`early`): the two read the attention's
-// result and the layer's operands and write different things.  The link-side kernels signal their dependents behind their own
-// pdl_wait(), so an update that starts finds everything up to the attention complete; it reads that past L1, and waits at its
-// end, so that whoever waits for the update has waited for the link side as well.
+// result and the layer's operands and write different things.  It reads what the kernels up to the attention wrote without a wait of
+// its own, and waits at its end, so that whoever waits for the update has waited for the link side as well.  The programming model
+// gives a dependent no view of anything before its own wait; that the early reads are sound rests on three things here:
+//  - order: the launch right before the update is a kernel of the link side (the merge of the partials comes ahead of that one), every
+//    thread of which signals behind its own wait.  So when the update's CTAs start, a wait for everything up to the attention has
+//    returned, which is to say those kernels are complete and their writes have been flushed to L2;
+//  - place: what it reads that early comes from L2, by TMA or by loads past L1, never through a line that L1 may have kept from before;
+//  - buffers: nothing that runs beside it writes what it reads (operands of consecutive layers alternate or are written behind it).
+// A kernel put between the attention and the update, or an exit of a link-side kernel ahead of its wait, breaks the first.
+// (tests/test_launch_order.py holds the sources against these rules.)
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
