@@ -285,7 +285,7 @@ static lime_status launch_score_gather_t(const ScoreArgs& a, int* err, cudaStrea
   ScoreGatherParams p;
   p.ids = a.cand_ids; p.logits = a.logits; p.V = (int32_t)a.corpus_rows; p.flag = a.dev_flag;
   p.B = a.B; p.C = a.C; p.d = a.d;
-  p.tiles_per_user = (a.C + SG_TILE - 1) / SG_TILE;
+  p.tiles_per_user = (int)(((int64_t)a.C + SG_TILE - 1) / SG_TILE);
   p.n_tiles = p.tiles_per_user * a.B;
   p.stages = S; p.err = err;
   const int grid = p.n_tiles < kSMs ? p.n_tiles : kSMs;

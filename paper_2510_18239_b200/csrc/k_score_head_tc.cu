@@ -317,7 +317,7 @@ static lime_status launch_score_head_tc_t(const ScoreArgs& a, const ScoreHeadArg
   ScoreHeadParams p;
   p.ids = a.cand_ids; p.flag = a.dev_flag; p.V = (int)a.corpus_rows;
   p.logits = a.logits; p.b1 = h.b1; p.w2 = h.w2; p.b2 = h.b2; p.B = a.B; p.C = a.C; p.d = a.d; p.n1 = h.n1;
-  p.tiles_per_user = (a.C + SH_TILE - 1) / SH_TILE;
+  p.tiles_per_user = (int)(((int64_t)a.C + SH_TILE - 1) / SH_TILE);
   p.n_tiles = p.tiles_per_user * a.B;
   p.stages = plan.stages; p.lsw_bufs = plan.lsw_bufs; p.terms = plan.terms; p.err = err;
   const int grid = p.n_tiles < kSMs ? p.n_tiles : kSMs;

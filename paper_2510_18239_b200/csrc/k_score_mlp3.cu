@@ -104,10 +104,11 @@ k_score_mlp3(const ScoreMlp3Params p) {
   const uint32_t ls_a = sb + lay.ls + warp * (ELL * M3_D * 2);
   bool weights_in = false;
   for (int grp = blockIdx.x * WARPS + warp; grp < ((p.n_groups + WARPS - 1) / WARPS) * WARPS; grp += gridDim.x * WARPS) {
-    const int s0 = grp * SLOTS, s1 = min(s0 + SLOTS, p.total);
-    const bool work = s0 < p.total;
-    int row = min(s0 + lane, p.total - 1);
-    bool good = lane < SLOTS && s0 + lane < p.total;
+    // slots s0 .. s0 + here - 1 (none past the last group; slot numbers go up to 2^31 - 2, so nothing is added to one ahead of a comparison)
+    const int s0 = grp < p.n_groups ? grp * SLOTS : p.total, here = min(SLOTS, p.total - s0), s1 = s0 + here;
+    const bool work = here > 0;
+    int row = lane < here ? s0 + lane : p.total - 1;
+    bool good = lane < here;
     if (p.ids != nullptr) {
       const int32_t id = __ldg(p.ids + row);
       if (good && (id < 0 || id >= p.rows) && p.flag != nullptr) atomicMin(p.flag, row);
@@ -179,8 +180,8 @@ k_score_mlp3(const ScoreMlp3Params p) {
         }
 #pragma unroll
         for (int i = 0; i < 2 * MT; ++i) {
-          const int slot = s0 + g + 8 * i;
-          if (slot >= u0 && slot < u1)
+          const int slot = g + 8 * i;
+          if (slot >= u0 - s0 && slot < u1 - s0)
 #pragma unroll
             for (int n = 0; n < 4; ++n) { o[i >> 1][n][(i & 1) * 2] = q[i >> 1][n][(i & 1) * 2]; o[i >> 1][n][(i & 1) * 2 + 1] = q[i >> 1][n][(i & 1) * 2 + 1]; }
         }
@@ -322,7 +323,7 @@ k_score_mlp3(const ScoreMlp3Params p) {
 #pragma unroll
     for (int i = 1; i < 2 * MT; ++i) mine = t == i ? v[i] : mine;
     mine += c3[M3_N2];
-    if (r < SLOTS && s0 + r < p.total) p.logits[s0 + r] = ((live >> r) & 1u) ? mine : 0.f;
+    if (r < here) p.logits[s0 + r] = ((live >> r) & 1u) ? mine : 0.f;
   }
 }
 
@@ -339,7 +340,7 @@ static lime_status launch_m3(ScoreMlp3Params p, cudaStream_t st) {
   static bool smem_set[kMaxDeviceOrdinals] = {};
   lime_status s = ensure_dynamic_smem((const void*)k_score_mlp3<ELL, MT, WARPS>, 232448, smem_set);
   if (s != LIME_OK) return s;
-  p.n_groups = (p.total + 16 * MT - 1) / (16 * MT);
+  p.n_groups = (int)(((int64_t)p.total + 16 * MT - 1) / (16 * MT));
   const int blocks = (p.n_groups + WARPS - 1) / WARPS;
   ProfScope _p("k_score_mlp3", st);
   launch_pdl(k_score_mlp3<ELL, MT, WARPS>, dim3((unsigned)(blocks < kSMs ? blocks : kSMs)), dim3(WARPS * 32), (size_t)lay.bytes, st, p);

@@ -81,8 +81,10 @@ k_score_rows(const ScoreRowsParams p) {
   // this kernel fit beside it: 100 lists of 20..1500 ids, the batch 142 -> 134 us.  The tcgen05 scorers do not gain: their CTAs
   // take a whole SM, so those that wait for one of the busy SMs start late whatever the others have prefetched)
   for (int grp = g_begin + warp; grp < min(g_end, g_begin + SR_AHEAD * SR_WARPS); grp += SR_WARPS) {
-    const int slot = grp * 16 + (lane & 15);
-    const int id = slot < p.total ? (p.ids != nullptr ? __ldcg(p.ids + slot) : slot) : -1;
+    const int s0 = grp * 16;
+    const bool in = (lane & 15) < p.total - s0;    // (not s0 + lane < total: slot numbers go up to 2^31 - 2)
+    const int slot = in ? s0 + (lane & 15) : 0;
+    const int id = in ? (p.ids != nullptr ? __ldcg(p.ids + slot) : slot) : -1;
     if (id >= 0 && id < p.rows) {
       const char* row = reinterpret_cast<const char*>(p.T + (int64_t)id * p.ldt);
       for (int o = (lane >> 4) * 128; o < D * 2; o += 256) prefetch_l2(row + o);
@@ -93,10 +95,10 @@ k_score_rows(const ScoreRowsParams p) {
   int b = -1;
   for (int grp = g_begin + warp; grp < g_end; grp += SR_WARPS) {
     const int s0 = grp * 16;
-    const int s1 = min(s0 + 16, p.total);
+    const int here = min(16, p.total - s0), s1 = s0 + here;
     // one row index per slot
-    int row = s0 + lane;
-    bool in = lane < 16 && row < s1;
+    bool in = lane < here;
+    int row = in ? s0 + lane : s0;
     if (p.ids != nullptr) {
       const int32_t id = in ? __ldg(p.ids + row) : 0;
       const bool good = id >= 0 && id < p.rows;
@@ -175,15 +177,13 @@ k_score_rows(const ScoreRowsParams p) {
         }
         // lanes t = 0, 1 keep row g + 8 t
         const float mine = t == 0 ? v[0] : v[1];
-        const int slot = s0 + g + 8 * t;
         const int u_begin = p.cand_off == nullptr ? b * p.C : __ldg(p.cand_off + b);
-        if (slot >= u_begin && slot < u_end) out = mine;
+        if (g + 8 * t >= u_begin - s0 && g + 8 * t < u_end - s0) out = mine;
       }
       if (u_end >= s1 || b + 1 >= p.B) break;
       ++b;
     }
-    const int slot = s0 + g + 8 * t;
-    if (t < 2 && slot < s1) p.logits[slot] = out;
+    if (g + 8 * t < here) p.logits[s0 + g + 8 * t] = out;       // here <= 16: threads t = 0, 1
   }
 }
 
@@ -203,9 +203,10 @@ k_score_rows_f32(const float* __restrict__ LS, const float* __restrict__ W, cons
   float4 ls[ELL][KI];
   int b = -1, loaded = -1;
   for (int grp = g_begin; grp < g_end; ++grp) {
-    const int s0 = grp * 8, s1 = min(s0 + 8, p.total), slot = s0 + g;
-    int row = min(slot, p.total - 1);
-    bool in = slot < s1;
+    const int s0 = grp * 8, here = min(8, p.total - s0), s1 = s0 + here;
+    bool in = g < here;
+    const int slot = in ? s0 + g : p.total - 1;
+    int row = slot;
     if (p.ids != nullptr) {
       const int32_t id = __ldg(p.ids + row);
       const bool good = id >= 0 && id < p.rows;
@@ -245,12 +246,12 @@ k_score_rows_f32(const float* __restrict__ LS, const float* __restrict__ W, cons
         }
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         s += __shfl_xor_sync(0xffffffffu, s, 2);
-        if (slot >= u0 && slot < u1) out = s;
+        if (g >= u0 - s0 && g < u1 - s0) out = s;
       }
       if (u1 >= s1 || b + 1 >= p.B) break;
       ++b;
     }
-    if (t == 0 && slot < s1) p.logits[slot] = out;
+    if (t == 0 && g < here) p.logits[slot] = out;
   }
 }
 

@@ -252,7 +252,7 @@ static lime_status launch_score_tc_t(const ScoreArgs& a, int* err, cudaStream_t 
     return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
   ScoreTcParams p;
   p.logits = a.logits; p.B = a.B; p.C = a.C; p.d = a.d;
-  p.tiles_per_user = (a.C + SCT_TILE - 1) / SCT_TILE;
+  p.tiles_per_user = (int)(((int64_t)a.C + SCT_TILE - 1) / SCT_TILE);
   p.n_tiles = p.tiles_per_user * a.B;
   p.stages = S; p.err = err;
   p.total = (int)a.total; p.T = (const char*)a.T; p.W = (const char*)a.W;

@@ -521,3 +521,39 @@ def test_destroy_waits_for_the_kernels_that_read_its_weight_copies():
         assert all(torch.equal(x, want) for x in got)
         del other
         lime = context(models[0])
+
+
+@pytest.mark.parametrize("kernel,dtype,d,ell,widths", [("k_score_mlp3", synth.BF16, 32, 8, (64, 128, 64)), ("k_score_rows", synth.BF16, 32, 8, ()),
+                                                       ("k_score_rows_f32", synth.F32, 64, 8, ()), ("k_score_gather_tc", synth.BF16, 64, 16, ()),
+                                                       ("k_score_head_tc", synth.BF16, 64, 32, (16,))])
+def test_as_many_candidates_as_the_call_admits(kernel, dtype, d, ell, widths):
+    """2^31 - 1 candidates of one user, the most that the entry points take: slot numbers up to the last one, which has a bad id.
+    (17 GB of ids and logits; every logit against that of its id in a short call.)"""
+    if torch.cuda.mem_get_info()[0] < 40 << 30:
+        pytest.skip("needs 40 GB of device memory")
+    Bd = _lib()
+    total, V = 2 ** 31 - 1, 1009
+    g = torch.Generator("cuda").manual_seed(3)
+    store = torch.float32 if dtype == synth.F32 else torch.bfloat16
+    rand = lambda *shape: torch.randn(shape, generator=g, device="cuda").to(store)
+    lime = Bd.Lime(d, 4, ell, 1, dtype=Bd.LIME_F32 if dtype == synth.F32 else Bd.LIME_BF16)
+    if widths:
+        lime.set_head([(Bd.to_device(w, dtype), torch.from_numpy(b).cuda()) for w, b in synth.ffn_weights(5, "head", (2 * d, *widths, 1), dtype)])
+    score = lime.score_candidates_head if widths else lime.score_candidates
+    LS, W, T = rand(1, ell, d), torch.softmax(rand(V, ell).float(), 1).to(store), rand(V, d)
+    once = torch.randperm(V, generator=g, device="cuda").to(torch.int32)
+    want = score(LS, W, T, C=V, cand_ids=once).repeat(1 << 17)
+    part, ids = once.repeat(1 << 17), torch.empty(total, dtype=torch.int32, device="cuda")
+    for s in range(0, total, len(part)):
+        ids[s:s + len(part)] = part[:min(len(part), total - s)]
+    ids[-1] = -1
+    flag = torch.full((1,), 2 ** 31 - 1, dtype=torch.int32, device="cuda")
+    Bd.lime_profile_start()
+    got = score(LS, W, T, C=total, cand_ids=ids, dev_flag=flag)
+    assert kernel.replace("_f32", "") in [name for name, _ in Bd.lime_profile_stop()[0]]
+    Bd.lime_device_status(lime.ctx)
+    assert got[-1].item() == 0.0 and flag.item() == total - 1
+    tol = 1e-4 * max(1.0, want.abs().max().item())             # fp32 sums in another order: 1e-6 of the largest terms, and as above
+    for s in range(0, total - 1, len(part)):
+        e = min(s + len(part), total - 1)
+        assert (got[s:e] - want[:e - s]).abs().max().item() <= tol, s
