@@ -50,9 +50,14 @@ __global__ void __launch_bounds__(1024) k_offsets(const int32_t* __restrict__ le
 // 1024..4096 tokens over 37 groups); this order leaves it under 1 %.  A round is one rank computation over
 // the G loads in shared memory and one barrier.
 // group_start[G+1], group_items[items]: the items of group j in the order it takes them.  scratch: 4 x items ints.
+// WALK (with the dealing): a user's items are listed by its warp's lanes together and counted in two steps.  One thread walks them
+// otherwise, 0.15 us an item: nothing for the few items that users have, 176 us for a single user of 4M tokens (977 items; 23 with WALK)
+// and 49 us of 1M (13).  An instance of its own, like FIT: where it is not needed it costs 0.5 to 1.2 us (16 users of 100..1024 tokens
+// 108.4 -> 109, 64 users 202.5 -> 203.7), so the host asks for it where the total makes more than 32 items of the ordinary length
+// (short ones, of which there are 64 at most, are left to the thread).
 // FIT: the lengths of the items are fitted where some history is longer than one (rule.fit_groups); an instance of its own, because the
 // code alone, never reached, cost the batch of 256 users x 512 4.5 us.
-template <bool FIT>
+template <bool FIT, bool WALK>
 __global__ void __launch_bounds__(1024)
 k_layer_schedules(const int32_t* __restrict__ off, int B, const ChunkRule rule, int32_t* __restrict__ chunk_out,
                   int32_t* __restrict__ chunk_start, int tile,
@@ -140,6 +145,20 @@ k_layer_schedules(const int32_t* __restrict__ off, int B, const ChunkRule rule, 
     *chunk_out = chunk;
     if (merge_needed != nullptr) *merge_needed = merge;
   }
+  // bucket 0 holds the largest items
+  auto bucket = [&](int tokens) { return KEYS - 1 - min(KEYS - 1, (tokens + att_tile - 1) / att_tile); };
+  // WALK: f(what, i, first) for the k consecutive items from `first` of every thread's user, by that thread up to OWN, else by the lanes of
+  // its warp together.  Every thread of the warp calls it.
+  constexpr int OWN = 8;
+  auto each_item = [&](int k, int first, auto f, int what) {
+    if (k <= OWN)
+      for (int i = 0; i < k; ++i) f(what, first + i, first);
+    for (unsigned many = __ballot_sync(0xffffffffu, k > OWN); many != 0; many &= many - 1) {
+      const int src = __ffs(many) - 1;
+      const int all = __shfl_sync(0xffffffffu, k, src), from = __shfl_sync(0xffffffffu, first, src), w = __shfl_sync(0xffffffffu, what, src);
+      for (int i = threadIdx.x & 31; i < all; i += 32) f(w, from + i, from);
+    }
+  };
   int2 carry = make_int2(0, 0);
   int item_first = 0;                              // this thread's first item, of its first user
   for (int b0 = 0, k = 1; b0 < B; b0 += blockDim.x, k ^= 1) {
@@ -153,12 +172,16 @@ k_layer_schedules(const int32_t* __restrict__ off, int B, const ChunkRule rule, 
     if (b < B) { chunk_start[b] = item; tile_start[b] = carry.y + before.y; }
     // inverse map (chunk item -> user): the attention kernel strides through the items, and one read of this table
     // replaces a search over chunk_start per item
-    if (chunk_user != nullptr)
+    if constexpr (WALK) {
+      each_item(n_chunks, item, [&](int user, int i, int) { chunk_user[i] = user; }, b);
+      if (n_chunks > 1) atomicAdd(&hist[bucket(chunk)], n_chunks - 1);       // full items, and the last one, which may be shorter
+      if (n_chunks > 0) atomicAdd(&hist[bucket(n - (n_chunks - 1) * chunk)], 1);
+    } else if (chunk_user != nullptr) {
       for (int i = 0; i < n_chunks; ++i) {
         chunk_user[item + i] = b;
-        // bucket 0 holds the largest items
         if (deal) atomicAdd(&hist[KEYS - 1 - min(KEYS - 1, (min(chunk, n - i * chunk) + att_tile - 1) / att_tile)], 1);
       }
+    }
     carry.x += total.x;
     carry.y += total.y;
   }
@@ -177,14 +200,29 @@ k_layer_schedules(const int32_t* __restrict__ off, int B, const ChunkRule rule, 
     if (threadIdx.x < KEYS) hist[threadIdx.x] = before.x;
   }
   __syncthreads();
-  for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    const int n = max(length(b), 0), item = b < (int)blockDim.x ? item_first : chunk_start[b];
-    for (int i = 0; i * chunk < n; ++i) {
-      const int key = min(KEYS - 1, (min(chunk, n - i * chunk) + att_tile - 1) / att_tile);
-      const int at = atomicAdd(&hist[KEYS - 1 - key], 1);
-      sorted[at] = item + i;
-      if (at < KCAP) skey[at] = (uint8_t)key;
-      else key_of[at] = key;
+  auto place = [&](int at, int item, int key) {
+    sorted[at] = item;
+    if (at < KCAP) skey[at] = (uint8_t)key;
+    else key_of[at] = key;
+  };
+  if constexpr (WALK) {
+    for (int b0 = 0; b0 < B; b0 += blockDim.x) {
+      const int b = b0 + threadIdx.x;
+      const int n = b < B ? max(length(b), 0) : 0, k = (n + chunk - 1) / chunk, item = n == 0 ? 0 : b0 == 0 ? item_first : chunk_start[b];
+      const int full = k > 1 ? atomicAdd(&hist[bucket(chunk)], k - 1) : 0;
+      each_item(k - 1, item, [&](int at, int i, int first) { place(at + i - first, i, KEYS - 1 - bucket(chunk)); }, full);
+      if (k > 0) {
+        const int in = bucket(n - (k - 1) * chunk);
+        place(atomicAdd(&hist[in], 1), item + k - 1, KEYS - 1 - in);
+      }
+    }
+  } else {
+    for (int b = threadIdx.x; b < B; b += blockDim.x) {
+      const int n = max(length(b), 0), item = b < (int)blockDim.x ? item_first : chunk_start[b];
+      for (int i = 0; i * chunk < n; ++i) {
+        const int key = min(KEYS - 1, (min(chunk, n - i * chunk) + att_tile - 1) / att_tile);
+        place(atomicAdd(&hist[KEYS - 1 - key], 1), item + i, key);
+      }
     }
   }
   __syncthreads();
@@ -227,7 +265,8 @@ lime_status launch_layer_schedules(const int32_t* off, int B, const ChunkRule& c
                                    int32_t* chunk_user, int32_t* merge_needed, const GroupSchedule& gs, cudaStream_t st) {
   if (gs.group_start != nullptr && (gs.n_groups < 1 || gs.n_groups > 160 || gs.att_tile < 1)) return LIME_INVALID_ARG;
   ProfScope _p("k_layer_schedules", st);
-  launch_pdl(chunk.fit_groups > 0 ? k_layer_schedules<true> : k_layer_schedules<false>, dim3(1), dim3(schedule_threads(B)), 0, st, off, B, chunk, chunk_out, chunk_start, tile, tile_start, chunk_user, merge_needed,
+  const auto kernel = chunk.fit_groups > 0 ? k_layer_schedules<true, false> : gs.walk ? k_layer_schedules<false, true> : k_layer_schedules<false, false>;
+  launch_pdl(kernel, dim3(1), dim3(schedule_threads(B)), 0, st, off, B, chunk, chunk_out, chunk_start, tile, tile_start, chunk_user, merge_needed,
              gs.n_groups, gs.att_tile, gs.group_start, gs.group_items, gs.scratch);
   LIME_LAUNCH_CHECK("k_layer_schedules");
   return LIME_OK;

@@ -181,6 +181,7 @@ static Workspace carve(const Ctx* c, void* base, int32_t B, int64_t total) {
   if (c->tc_mode == 2) {
     w.groups.n_groups = link_attn_d256_groups(w.n_chunk_upper, g.H, g.ell);
     w.groups.att_tile = 96;
+    w.groups.walk = split_items > 32;
     w.groups.group_start = (int32_t*)take((size_t)(w.groups.n_groups + 1) * 4);
     w.groups.group_items = (int32_t*)take((size_t)w.n_chunk_upper * 4);
     w.groups.scratch = (int32_t*)take((size_t)w.n_chunk_upper * 16);

@@ -229,6 +229,7 @@ lime_status launch_gather_ln(int dtype, const void* table, int64_t V, int d, flo
 // group_start == NULL: not wanted.  group_start[n_groups + 1], group_items[items], scratch[4 x items].
 struct GroupSchedule {
   int n_groups = 0, att_tile = 0;
+  bool walk = false;                // a single user may have many items: they are listed by its warp
   int32_t* group_start = nullptr; int32_t* group_items = nullptr; int32_t* scratch = nullptr;
 };
 // How long the work items of the links <- history attention are: `tokens`, or `short_tokens` (0: never) where some history is over

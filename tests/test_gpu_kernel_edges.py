@@ -465,6 +465,35 @@ def test_chunk_length_fitted_to_the_groups(d, H, ell, lengths, raw):
     _encode_against_oracle(synth.BF16, d, H, ell, 2, lengths, "softmax", raw, False, 6e-2, 2.5e-2)
 
 
+@pytest.mark.parametrize("lengths", [[70000, 3, 0, 513, 4608], [300] * 40 + [20480] + [4097, 4096], [9 * 512 + 1] * 20])
+def test_work_items_of_one_user_beyond_what_a_thread_walks(lengths):
+    """Eight items of a user and fewer are listed by one thread, more by its warp: 512 tokens an item, dealt to groups (d = 256)."""
+    _encode_against_oracle(synth.BF16, 256, 4, 32, 2, lengths, "softmax", False, False, 6e-2, 2.5e-2)
+
+
+def test_work_lists_of_one_user_take_no_longer_than_of_many():
+    """d = 256, a million tokens: the lists of a single user's 245 items against those of 250 users with one each.  49 us against 10 where one
+    thread walks a user's items, 12.6 where its warp does."""
+    Bd = _lib()
+    d, H, ell, total = 256, 4, 32, 1_000_000
+    lime = Bd.Lime(d, H, ell, 1, dtype=Bd.LIME_BF16)
+    g = torch.Generator("cuda").manual_seed(1)
+    rand = lambda *shape, std: (torch.randn(shape, generator=g, device="cuda") * std).to(torch.bfloat16)
+    lime.set_weights(rand(ell, d, std=1.0), [{k: rand(d, d, std=d ** -0.5) for k in ("Wq", "Wk", "Wv", "Wg", "Wu", "Wo")}])
+    hist = rand(total, d, std=1.0)
+
+    def best(lengths):
+        off = lime.lengths_to_offsets(torch.tensor(lengths, dtype=torch.int32, device="cuda"))
+        times = []
+        for _ in range(8):
+            Bd.lime_profile_start()
+            lime.encode_user_normalized(hist, off)
+            times.append(dict(Bd.lime_profile_stop()[0])["k_layer_schedules"])
+        return min(times)
+    one, many = best([total]), best([total // 250] * 250)
+    assert one <= 2.5 * many, (one, many)
+
+
 def test_one_long_history_is_split_among_many_users():
     """One user of 4000 tokens among 99 of 100, against 100 users of 100 (d = 128): 1.46 times the time where a history is one work item
     whenever the users are many, 1.16 times split."""
