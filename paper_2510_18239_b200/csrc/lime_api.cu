@@ -403,8 +403,13 @@ static lime_status encode_user_tc(Ctx* c, const void* hist, bool hist_normalized
   // alternate between two sets (Q2 is the attention's, complete by then)
   const bool few_rows = few_link_rows(c, B);
   const LinkOperands set[2] = {{w.Q2, w.K2, w.G2t, w.U2t, w.V2t, w.cQ, w.cK, 0}, {w.Q2, w.K2b, w.G2tb, w.U2tb, w.V2t, w.cQ, w.cK, 0}};
-  // the last layer needs its queries only: the GatedMLP kernel of the layer before makes them along with its rows
-  auto queries_along = [&](int j) { return c->tc_mode == 1 && !few_rows && j > 0 && j == g.n_layers - 1; };
+  // The last layer needs its queries only: the GatedMLP kernel of the layer before makes them along with its rows.  With more than 256
+  // stacked rows the update (k_hist_update2_tc.cu) does not run beside that kernel, so what it takes longer is not hidden, and a GEMM of
+  // its own is shorter while the rows are few (H * ell = 512, two layers, us with a GEMM / along: 20 users of 100..1000 tokens 80.6 / 86.4, 33
+  // 94.0 / 98.2, 100 149.7 / 150.6, 200 of 100..500 181.9 / 179.3).  More users than kEarlyUsers gain although the update waits there too
+  // (1100 users of 100..200 tokens 239.0 / 231.7).
+  const bool along = c->tc_mode == 1 && !few_rows && (g.H * g.ell <= 256 || BL > 8192);
+  auto queries_along = [&](int j) { return along && j > 0 && j == g.n_layers - 1; };
   for (int j = 0; j < g.n_layers; ++j) {
     const bool last = j == g.n_layers - 1;
     const bool raw = g.ln && j == 0 && !hist_normalized;      // rows that still need their LayerNorm want the operands' row sums

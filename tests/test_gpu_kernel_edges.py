@@ -457,6 +457,17 @@ def test_history_update_beside_the_link_side(d, H, ell, lengths, raw):
     _encode_against_oracle(synth.BF16, d, H, ell, 3, lengths, "softmax", raw, True, 6e-2, 3e-2)
 
 
+@pytest.mark.parametrize("H,ell,B,along", [(4, 32, 67, True), (8, 32, 67, True), (4, 64, 35, True), (8, 64, 35, False), (8, 64, 129, True)])
+def test_queries_of_the_last_layer(H, ell, B, along):
+    """d = 128 above 2048 link rows: formed by the GatedMLP kernel of the layer before, but for few rows with more than 256 stacked rows by a
+    GEMM of their own.  (The shared links' operands of the first layer are formed by that GEMM when the weights are set.)"""
+    Bd = _lib()
+    Bd.lime_profile_start()
+    _encode_against_oracle(synth.BF16, 128, H, ell, 2, [40, 0, 129] + [7] * (B - 3), "softmax", False, False, 6e-2, 2.5e-2)
+    names = [name for name, _ in Bd.lime_profile_stop()[0]]
+    assert "k_link_mlp_tc" in names and names.count("k_gemm_tc_prep") == (1 if along else 2), names
+
+
 @pytest.mark.parametrize("d,H,ell", [(128, 4, 32), (128, 4, 64)])
 @pytest.mark.parametrize("lengths", [[9000, 100], [2300] * 30 + [0], [4100, 700] * 6, [6000], [2049] * 66])
 @pytest.mark.parametrize("raw", [False, True])
