@@ -3,12 +3,15 @@
 Functions carry the C entry points' names and take torch CUDA tensors (used purely as device memory) plus
 plain integers; every step of the path runs inside the library's kernels.  There is no CPU fallback: if the
 shared library is missing or a call fails, an exception is raised.  The calls that `Lime` makes per request go
-through `_torch_binding`, the same marshalling in native code (csrc/torch_binding.cpp).
+through `_torch_binding`, the same marshalling in native code (csrc/torch_binding.cpp), where that has been built for
+the torch and the Python at hand, and else through `_PlainCalls`: the same kernels, 7 to 10 us of host time a call
+instead of 2 to 3.
 """
 from __future__ import annotations
 
 import ctypes
 import os
+import warnings
 from typing import Dict, Optional, Sequence
 
 import numpy as np
@@ -121,16 +124,21 @@ _native_module = None
 
 
 def _native():
-    """The native half of this binding, joined to the loaded library.  Raises if it has not been built."""
+    """The calls of a request: the native half of this binding, joined to the loaded library, or `_PlainCalls` (with a warning)."""
     global _native_module
     if _native_module is None:
         load_library()
+        from . import build
         try:
-            from . import _torch_binding
+            from . import _torch_binding as native
+            made_for = getattr(native, "made_for", "another build")
+            if made_for != build.binding_made_for():
+                raise ImportError(f"_torch_binding.so was built for {made_for}")
+            native.load(LIB_PATH, LimeError)
+            _native_module = native
         except ImportError as e:
-            raise RuntimeError("_torch_binding.so is missing: build it with `python -m paper_2510_18239_b200.build`") from e
-        _torch_binding.load(LIB_PATH, LimeError)
-        _native_module = _torch_binding
+            warnings.warn(f"{e}: calls are marshalled in Python until `python -m paper_2510_18239_b200.build` has built it")
+            _native_module = _PlainCalls
     return _native_module
 
 
@@ -143,6 +151,8 @@ def _check(status: int, where: str):
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     if t is None:
         return None
+    if not isinstance(t, torch.Tensor):
+        raise TypeError(f"expected a torch.Tensor, got {type(t).__name__}")
     if not t.is_cuda or not t.is_contiguous():
         raise ValueError("expected a contiguous CUDA tensor")
     return t.data_ptr()
@@ -345,6 +355,76 @@ def to_device(arr: np.ndarray, dtype: str, device="cuda") -> torch.Tensor:
 
 def torch_dtype(dtype: int):
     return torch.float32 if dtype == LIME_F32 else torch.bfloat16
+
+
+# ----------------------------------------------------------------------------- the calls of a request
+class _PlainCalls:
+    """What `_torch_binding` does, function by function, through the entry points above: same arguments, results and exceptions."""
+
+    @staticmethod
+    def _tensor(t):
+        if not isinstance(t, torch.Tensor):
+            raise TypeError(f"expected a torch.Tensor, got {type(t).__name__}")
+        return t
+
+    @staticmethod
+    def lengths_to_offsets(ctx, lengths):
+        off = _PlainCalls._tensor(lengths).new_empty(lengths.numel() + 1)
+        lime_lengths_to_offsets(ctx, lengths, off)
+        return off
+
+    @staticmethod
+    def _gather(call, ctx, d, table, ids, flag):
+        out = _PlainCalls._tensor(table).new_empty((_PlainCalls._tensor(ids).numel(), d))
+        call(ctx, table, ids, out, flag)
+        return out
+
+    @staticmethod
+    def gather_history(ctx, d, table, ids, flag):
+        return _PlainCalls._gather(lime_gather_history, ctx, d, table, ids, flag)
+
+    @staticmethod
+    def gather_history_normalized(ctx, d, table, ids, flag):
+        return _PlainCalls._gather(lime_gather_history_normalized, ctx, d, table, ids, flag)
+
+    @staticmethod
+    def _encode(call, ctx, ell_c, d, hist, off, link_ctx, ws):
+        B = _PlainCalls._tensor(off).numel() - 1
+        ls = _PlainCalls._tensor(hist).new_empty((B, ell_c, d))
+        call(ctx, hist, off, B, link_ctx, ls, _PlainCalls._tensor(ws))
+        return ls
+
+    @staticmethod
+    def encode_user(ctx, ell_c, d, hist, off, link_ctx, ws):
+        return _PlainCalls._encode(lime_encode_user, ctx, ell_c, d, hist, off, link_ctx, ws)
+
+    @staticmethod
+    def encode_user_normalized(ctx, ell_c, d, hist, off, link_ctx, ws):
+        return _PlainCalls._encode(lime_encode_user_normalized, ctx, ell_c, d, hist, off, link_ctx, ws)
+
+    @staticmethod
+    def precompute_candidate_links(ctx, ell_c, cand_emb):
+        out = _PlainCalls._tensor(cand_emb).new_empty((cand_emb.shape[0], ell_c))
+        lime_precompute_candidate_links(ctx, cand_emb, out)
+        return out
+
+    @staticmethod
+    def _score(call, ctx, link_states, cand_w, cand_emb, C, cand_off, cand_ids, total, rows, flag, *ws):
+        for t in (link_states, cand_w, cand_emb, *ws):
+            _PlainCalls._tensor(t)
+        if total is None:
+            total = cand_emb.shape[0] if cand_ids is None else _PlainCalls._tensor(cand_ids).numel()
+        logits = torch.empty(total, dtype=torch.float32, device=link_states.device)
+        call(ctx, link_states, link_states.shape[0], cand_w, cand_emb, cand_off, C, total, cand_ids, logits, *ws, rows, flag)
+        return logits
+
+    @staticmethod
+    def score_candidates(ctx, link_states, cand_w, cand_emb, C, cand_off, cand_ids, total, rows, flag):
+        return _PlainCalls._score(lime_score_candidates, ctx, link_states, cand_w, cand_emb, C, cand_off, cand_ids, total, rows, flag)
+
+    @staticmethod
+    def score_candidates_head(ctx, link_states, cand_w, cand_emb, C, cand_off, cand_ids, total, rows, flag, ws):
+        return _PlainCalls._score(lime_score_candidates_head, ctx, link_states, cand_w, cand_emb, C, cand_off, cand_ids, total, rows, flag, ws)
 
 
 # ----------------------------------------------------------------------------- convenience wrapper

@@ -1,8 +1,10 @@
 """In-tree build of the C-ABI CUDA library (sm_100a) with nvcc.
 
-`build()` compiles every `csrc/*.cu` to an object file and links `liblime_b200.so` next to this file, and beside it
-`_torch_binding.so`, the native half of `binding.py` (`csrc/torch_binding.cpp`, host code only).
-Objects are rebuilt only when a source or header is newer.  nvcc cross-compiles without a GPU.
+`build_library()` compiles every `csrc/*.cu` to an object file and links `liblime_b200.so` next to this file; it needs nvcc and
+nothing else.  `build_binding()` makes `_torch_binding.so` beside it, the native half of `binding.py` (`csrc/torch_binding.cpp`, host
+code only); it needs g++, torch and Python's headers.  `build()` does both, and without what the second needs the library alone:
+`binding.py` then marshals its calls in Python.  Objects are rebuilt only when a source or header is newer, the binding also when
+torch or Python have changed.  nvcc cross-compiles without a GPU.
 """
 from __future__ import annotations
 
@@ -13,6 +15,7 @@ import shutil
 import subprocess
 import sys
 import sysconfig
+from typing import Optional
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -20,6 +23,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "liblime_b200.so")
 BINDING = os.path.join(HERE, "_torch_binding.so")
+MADE_FOR = os.path.join(OBJ, "torch_binding.made_for")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -39,28 +43,47 @@ def _newest(paths) -> float:
     return max(os.path.getmtime(p) for p in paths)
 
 
-def build_binding() -> str:
-    src = os.path.join(CSRC, "torch_binding.cpp")
-    needs = [src, os.path.join(ROOT, "include", "lime.h"), __file__]
-    if os.path.exists(BINDING) and os.path.getmtime(BINDING) >= _newest(needs):
-        return BINDING
+def binding_made_for() -> str:
+    """The torch and the Python whose binary interfaces `_torch_binding.so` is compiled against."""
     import torch
+    return f"torch {torch.__version__}, {sysconfig.get_config_var('SOABI')}"
+
+
+def build_binding() -> Optional[str]:
+    """The path of the extension, or None where something that it needs is not installed (said on stderr)."""
+    src = os.path.join(CSRC, "torch_binding.cpp")
+    try:
+        made_for = binding_made_for()
+        import torch
+    except ImportError:
+        made_for = None
+    include = sysconfig.get_paths()["include"]
+    missing = [what for what, there in (("torch", made_for is not None), ("g++", shutil.which("g++") is not None),
+                                        ("Python.h", os.path.exists(os.path.join(include, "Python.h")))) if not there]
+    if missing:
+        print(f"[build] {', '.join(missing)} not found: _torch_binding.so is left out, binding.py marshals its calls in Python", file=sys.stderr)
+        return None
+    needs = [src, os.path.join(ROOT, "include", "lime.h"), __file__]
+    if os.path.exists(BINDING) and os.path.getmtime(BINDING) >= _newest(needs) and os.path.exists(MADE_FOR) and open(MADE_FOR).read() == made_for:
+        return BINDING
     home = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
-    includes = [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], os.path.join(home, "include"),
+    includes = [os.path.join(ROOT, "include"), include, os.path.join(home, "include"),
                 os.path.join(home, "include", "torch", "csrc", "api", "include"), os.path.join(cuda, "include")]
-    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f'-DLIME_MADE_FOR="{made_for}"',
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", src, "-o", BINDING]
     cmd += [f"-I{i}" for i in includes] + [f"-L{os.path.join(home, 'lib')}", "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-ldl"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         sys.stderr.write(r.stdout + r.stderr)
         raise RuntimeError("g++ failed on " + src)
+    os.makedirs(OBJ, exist_ok=True)
+    with open(MADE_FOR, "w") as f:
+        f.write(made_for)
     return BINDING
 
 
-def build(verbose: bool = False, ptxas_info: bool = False) -> str:
-    build_binding()
+def build_library(verbose: bool = False, ptxas_info: bool = False) -> str:
     os.makedirs(OBJ, exist_ok=True)
     sources = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
     headers = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h")) + [__file__]
@@ -92,6 +115,12 @@ def build(verbose: bool = False, ptxas_info: bool = False) -> str:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("link failed")
     return LIB
+
+
+def build(verbose: bool = False, ptxas_info: bool = False) -> str:
+    lib = build_library(verbose, ptxas_info)
+    build_binding()
+    return lib
 
 
 if __name__ == "__main__":

@@ -196,4 +196,8 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_torch_binding", nullptr, -1, meth
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__torch_binding(void) { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__torch_binding(void) {
+  PyObject* m = PyModule_Create(&module);
+  if (m != nullptr && PyModule_AddStringConstant(m, "made_for", LIME_MADE_FOR) < 0) Py_CLEAR(m);
+  return m;
+}

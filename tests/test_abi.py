@@ -2,6 +2,11 @@
 import ctypes
 import os
 import re
+import subprocess
+import sys
+
+import pytest
+import torch
 
 from paper_2510_18239_b200 import binding, build
 
@@ -77,3 +82,60 @@ def test_native_binding_refuses_what_is_no_cuda_tensor():
             call()
     with pytest.raises(OverflowError):
         native.score_candidates(None, cpu, cpu, cpu, 1, None, None, 1 << 70, None, None)
+
+
+def test_python_marshalling_refuses_what_is_no_cuda_tensor():
+    """The same without the native half."""
+    plain = binding._PlainCalls
+    with pytest.raises(TypeError):
+        plain.lengths_to_offsets(None, [1, 2])
+    with pytest.raises(TypeError):
+        plain.encode_user(None, 8, 32)
+    cpu = torch.zeros((3, 32))
+    for call in (lambda: plain.lengths_to_offsets(None, cpu), lambda: plain.gather_history(None, 32, cpu, cpu, None),
+                 lambda: plain.precompute_candidate_links(None, 8, cpu),
+                 lambda: plain.score_candidates(None, cpu, cpu, cpu, 1, None, None, None, None, None)):
+        with pytest.raises(ValueError):
+            call()
+
+
+def test_the_library_builds_without_what_the_binding_needs(monkeypatch, tmp_path, capsys):
+    """No g++ (or no torch, no Python.h): the C-ABI library all the same, and a word about what is left out."""
+    monkeypatch.setattr(build, "BINDING", str(tmp_path / "_torch_binding.so"))
+    monkeypatch.setattr(build, "MADE_FOR", str(tmp_path / "made_for"))
+    which = build.shutil.which
+    monkeypatch.setattr(build.shutil, "which", lambda name: None if name == "g++" else which(name))
+    assert build.build() == build.LIB and not (tmp_path / "_torch_binding.so").exists()
+    assert "g++ not found" in capsys.readouterr().err
+
+
+def test_the_binding_is_rebuilt_for_another_torch(monkeypatch, tmp_path):
+    made = []
+
+    def compiler(cmd, **kw):
+        made.append(cmd)
+        open(build.BINDING, "w").close()
+        return subprocess.CompletedProcess(cmd, 0, "", "")
+    monkeypatch.setattr(build, "BINDING", str(tmp_path / "_torch_binding.so"))
+    monkeypatch.setattr(build, "MADE_FOR", str(tmp_path / "made_for"))
+    monkeypatch.setattr(build.subprocess, "run", compiler)
+    assert build.build_binding() == build.BINDING == build.build_binding() and len(made) == 1
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    assert build.build_binding() == build.BINDING == build.build_binding() and len(made) == 2
+    assert any("torch 0.0.0" in a for a in made[1])
+
+
+@pytest.mark.parametrize("made_for", [None, "another torch"])
+def test_calls_go_through_python_without_a_fitting_extension(monkeypatch, made_for):
+    """The extension missing, or built against another torch or Python: a warning, and the calls through ctypes."""
+    monkeypatch.setattr(binding, "_native_module", None)
+    binding._native()
+    native = sys.modules["paper_2510_18239_b200._torch_binding"]
+    monkeypatch.setattr(binding, "_native_module", None)
+    if made_for is None:
+        monkeypatch.setitem(sys.modules, "paper_2510_18239_b200._torch_binding", None)
+        monkeypatch.delattr(sys.modules["paper_2510_18239_b200"], "_torch_binding", raising=False)
+    else:
+        monkeypatch.setattr(native, "made_for", made_for)
+    with pytest.warns(UserWarning, match="marshalled in Python"):
+        assert binding._native() is binding._PlainCalls

@@ -1015,3 +1015,63 @@ def test_config5_production_ragged_sampled():
     inp_len = synth.history_lengths(0, wl.B, wl.n_min, wl.n_max)
     users = [int(np.argmin(inp_len)), int(np.argmax(inp_len))]
     _sampled_parity(wl, seed=0, users=users)
+
+
+# ----------------------------------------------------------------------------- both ways of marshalling a call
+def _outcome(call):
+    try:
+        return call()
+    except Exception as e:                                     # which one, and what it says, is what is compared
+        return type(e).__name__, str(e)
+
+
+@pytest.mark.parametrize("dtype", [synth.BF16, synth.F32])
+def test_native_and_python_marshalling_make_the_same_calls(dtype):
+    """The calls of a request through `_torch_binding` and through ctypes: the same bits, and the same exceptions for the same mistakes."""
+    import paper_2510_18239_b200.binding as Bd
+    native, plain = Bd._native(), Bd._PlainCalls
+    assert native is not plain
+    d, H, ell, B, C, V = 64, 2, 8, 5, 33, 300
+    store = torch.float32 if dtype == synth.F32 else torch.bfloat16
+    g = torch.Generator("cuda").manual_seed(2)
+    rand = lambda *shape: (torch.randn(shape, generator=g, device="cuda") * d ** -0.5).to(store)
+    ints = lambda hi, n: torch.randint(0, hi, (n,), generator=g, device="cuda", dtype=torch.int32)
+    lime = Bd.Lime(d, H, ell, 2, dtype=Bd.LIME_F32 if dtype == synth.F32 else Bd.LIME_BF16)
+    lime.set_weights(rand(ell, d), [{k: rand(d, d) for k in ("Wq", "Wk", "Wv", "Wg", "Wu", "Wo")} for _ in range(2)])
+    lime.set_head([(rand(2 * d, 16), None), (rand(16, 1), None)])
+    x, table, lengths, ids = lime.ctx, rand(V, d), ints(40, B), None
+    ids, cand, flag = ints(V, int(lengths.sum())), ints(V, B * C), torch.full((1,), 7, dtype=torch.int32, device="cuda")
+    off = lime.lengths_to_offsets(lengths)
+    lists = torch.tensor([0, 1, 1, 60, 61, 90], dtype=torch.int32, device="cuda")
+    hist, ws, W = lime.gather_history(table, ids), lime.workspace(B, len(ids)), lime.precompute_candidate_links(table)
+    ls, hws = lime.encode_user(hist, off), torch.empty(1 << 20, dtype=torch.uint8, device="cuda")
+    link_ctx = torch.randn((B, ell, d), generator=g, device="cuda")
+    fresh = Bd.Lime(d, H, ell, 2, dtype=Bd.LIME_F32 if dtype == synth.F32 else Bd.LIME_BF16)       # no weights, no head
+    calls = [(name, args) for name, args in [
+        ("lengths_to_offsets", (x, lengths)), ("lengths_to_offsets", (x, lengths.cpu())), ("lengths_to_offsets", (x, lists[::2])),
+        ("lengths_to_offsets", (None, lengths)), ("lengths_to_offsets", (x, 3)),
+        ("gather_history", (x, d, table, ids, None)), ("gather_history", (x, d, table, ids, flag)), ("gather_history", (x, d, table[:, ::2], ids, None)),
+        ("gather_history", (x, d, table, ids[:0], None)), ("gather_history", (x, d, table.view(-1)[1:], ids, None)),
+        ("gather_history_normalized", (x, d, table, ids, None)), ("gather_history_normalized", (x, d, table, ids.cpu(), flag)),
+        ("encode_user", (x, ell, d, hist, off, None, ws)), ("encode_user", (x, ell, d, hist, off, link_ctx, ws)),
+        ("encode_user", (x, ell, d, hist, off, None, ws[:64])), ("encode_user", (x, ell, d, hist.t(), off, None, ws)),
+        ("encode_user", (fresh.ctx, ell, d, hist, off, None, ws)), ("encode_user", (x, ell, d, hist, off, None, None)),
+        ("encode_user_normalized", (x, ell, d, hist, off, None, ws)), ("encode_user_normalized", (x, ell, d, hist, off, link_ctx.cpu(), ws)),
+        ("precompute_candidate_links", (x, ell, table)), ("precompute_candidate_links", (x, ell, table.cpu())), ("precompute_candidate_links", (fresh.ctx, ell, table)),
+        ("score_candidates", (x, ls, W[:B * C], table[:B * C], C, None, None, None, None, None)),
+        ("score_candidates", (x, ls, W, table, C, None, cand, None, None, flag)), ("score_candidates", (x, ls, W, table, 0, lists, cand[:90].clone(), 90, V, flag)),
+        ("score_candidates", (x, ls, W, table, C + 1, None, cand, None, None, None)), ("score_candidates", (x, ls, W, table, C, None, cand, None, 0, None)),
+        ("score_candidates", (x, ls.float().cpu(), W, table, C, None, cand, None, None, None)), ("score_candidates", (x, ls, W, table, C, None, cand, -1, None, None)),
+        ("score_candidates_head", (x, ls, W, table, C, None, cand, None, None, None, hws)), ("score_candidates_head", (x, ls, W, table, 0, lists, cand[:90].clone(), 90, None, flag, hws)),
+        ("score_candidates_head", (x, ls, W, table, C, None, cand, None, None, None, hws[:256])), ("score_candidates_head", (fresh.ctx, ls, W, table, C, None, cand, None, None, None, hws)),
+    ]]
+    kinds = set()
+    for name, args in calls:
+        a, b = _outcome(lambda: getattr(native, name)(*args)), _outcome(lambda: getattr(plain, name)(*args))
+        if isinstance(a, torch.Tensor):
+            assert isinstance(b, torch.Tensor) and a.dtype == b.dtype and a.shape == b.shape and torch.equal(a, b), (name, b)
+        else:
+            assert a == b, (name, a, b)
+        kinds.add("result" if isinstance(a, torch.Tensor) else a[0])
+    assert {"result", "ValueError", "TypeError", "LimeError"} <= kinds and flag.item() == 7
+    Bd.lime_device_status(x)
