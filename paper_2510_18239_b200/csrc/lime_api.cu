@@ -251,8 +251,8 @@ static lime_status make_link_operands(Ctx* c, int layer, const void* That, int64
   return launch_gemm_prep(gp, st);
 }
 
-// How the update of `tiles` tiles at most shares the SMs with a link side of `blocks` blocks, one per SM, each of which takes as long as
-// `late_by` eighths of a tile of the update: the update's blocks that find no free SM (those of the highest index) start that much later.
+// How the update of `tiles` tiles at most shares the SMs with a link side of `blocks` blocks, one per SM: the update's blocks that find no
+// free SM (those of the highest index) start when the others are `late_by` tiles ahead.
 static BesideLinkSide beside_link_side(int64_t blocks, int late_by, int tiles, int B) {
   if (B > kEarlyUsers) return BesideLinkSide{};
   const int last = blocks > 0 ? (int)((blocks - 1) % kSMs) + 1 : 0, grid = tiles < kSMs ? tiles : kSMs;      // blocks of its last wave
@@ -287,19 +287,16 @@ static lime_status tc_layer_core(Ctx* c, int layer, const void* hist_in, const i
   const bool pass_stats = hist_ln && hist_out && two_tiles && total > 0;
   la.stats_out = pass_stats ? w.row_stats : nullptr;
   // The link side and the history update need nothing of each other: the update runs beside it (lime_common.cuh), which takes the
-  // shorter of the two off the layer where SMs are free and evens out the tiles where they are not.  Eighths of a tile that a block of
-  // the link side takes, by measurement (us a batch with 0 / 8 / 16 / 20 / 24 / 32 / 40, and with the update behind the link side):
-  // d = 128, the merge and the GatedMLP, a GEMM behind the update: 256 users x 512, two layers 139.5 / 139.3 / 135.9 / 135.7 / 137.8 /
-  // 137.8 / 140.2, 140.3; 150 users of 100..1500, 64 links, four layers 345.9 / 345.4 / 331.2 / 343.4 / 343.8 / 343.8 / 355.2, 351.6 (a
-  // tile of 256 stacked rows takes longer); the queries made along (mlp.Q2): 256 users x 512 136.7 with 0, 132.7 / 133.0 / 132.8 / 130.4 /
-  // 132.2 with 16 / 20 / 24 / 32 / 40; one kernel: 40 users of 100..1500 72.3 / 72.3 / 70.5 / 70.3 / 70.5 / 63.0 / 63.0, 74.3; 32 users of 2000..4000, 64 links
-  // 269.8 / 268.8 / 260.4 / 260.2 / 260.5 / 261.6 / 267.8, 276.2; d = 256, 32 links: 64 users of 100..1024, three layers 244.8 / 225.4 /
-  // 224.7 / 226.8 / 226.6 / 245.6 / 264.4, 245.8; 16 users 135.9 / 111.5 / 111.2 / 111.5 / 111.8 / 111.7 / 111.2, 143.5.
-  const int wide = g.H * g.ell > 128;
-  BesideLinkSide beside;
-  if (c->side256) beside = beside_link_side(link_side_d256_blocks(B), 14, w.n_tile_upper, B);
-  else if (side1 != nullptr) beside = beside_link_side(link_side_d128_blocks((int64_t)B * g.ell), wide ? 24 : 30, w.n_tile_upper, B);
-  else beside = beside_link_side(((int64_t)B * g.ell + 127) / 128, mlp.Q2 ? (wide ? 20 : 32) : wide || c->tc_mode == 2 ? 16 : 20, w.n_tile_upper, B);
+  // shorter of the two off the layer where SMs are free and evens out the tiles where they are not.  A block of the link side takes about
+  // 15 us at d = 128 and 25 at d = 256, whichever of the kernels it is: two tiles of the update (13 us each at d = 256, 7 at d = 128 with
+  // 256 stacked rows), or four where a tile is half as long (4 us, 128 stacked rows).  Whole tiles and one number a kind of tile: what a
+  // batch takes is a step function of how many tiles move, so a finer number follows the steps of the batch it was read from.  Mean gain of
+  // 27 to 33 batches of each kind over blocks that all take the same, in %, late blocks behind by 1 / 1.5 / 2 / 2.5 / 3 / 4 / 5 / 6 tiles:
+  // 128 stacked rows 1.5 / 3.5 / 4.3 / 4.9 / 5.8 / 7.0 / 6.3 / 5.8; 256 stacked rows 1.8 / 4.0 / 6.9 / 6.7 / 6.3 / 5.8 / 4.8 / 3.5; d = 256
+  // 4.2 / 5.3 / 6.2 / 5.4 / 5.7 / 3.9 / 2.3 / 1.0.
+  const int late_by = c->tc_mode == 1 && g.H * g.ell <= 128 ? 4 : 2;
+  const int64_t side_blocks = c->side256 ? link_side_d256_blocks(B) : side1 != nullptr ? link_side_d128_blocks((int64_t)B * g.ell) : ((int64_t)B * g.ell + 127) / 128;
+  const BesideLinkSide beside = beside_link_side(side_blocks, late_by, w.n_tile_upper, B);
   if ((s = c->tc_mode == 2 ? launch_link_attn_d256_tc(la, st) : launch_link_attn_tc(la, st)) != LIME_OK) return s;
   if (c->side256) {
     // merge, T^j and what follows from it - the next layer's operands included - in one kernel; `side` says what is wanted

@@ -177,12 +177,12 @@ __device__ __forceinline__ void prefetch_l2_row(const void* p, int bytes) {
 #endif
 #ifdef __CUDACC__
 // First tile of block `cta` when the `n` tiles are split in order among `grid` blocks, of which the last `late` start when the others
-// are `late_by` eighths of a tile ahead (they wait for the SMs that the link side holds).
+// are `late_by` tiles ahead (they wait for the SMs that the link side holds).
 __device__ __forceinline__ int early_first_tile(int cta, int grid, int n, int late, int late_by) {
-  const int64_t first = grid - late, share = 8 * (int64_t)n + (int64_t)late * late_by;       // share / (8 grid): tiles of an early block
+  const int64_t first = grid - late, share = n + (int64_t)late * late_by;                    // share / grid: tiles of an early block
   if (share < (int64_t)grid * late_by) return cta >= first ? n : (int)(cta * (int64_t)n / first);
   const int64_t behind = cta > first ? (cta - first) * (int64_t)grid * late_by : 0;
-  return (int)((cta * share - behind) / (8 * (int64_t)grid));
+  return (int)((cta * share - behind) / grid);
 }
 #endif
 bool pdl_enabled();      // environment LIME_PDL=0 turns the attribute off (every launch then serialises fully)

@@ -1,8 +1,12 @@
 """Kernels launched while their predecessor still runs keep the rules of lime_common.cuh: no thread leaves ahead of the wait for the
 predecessor, and the link-side kernels, beside which a history update runs, signal their dependents behind that wait."""
+import ctypes
 import glob
 import os
 import re
+import subprocess
+
+import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2510_18239_b200", "csrc")
 LINK_SIDE = {"k_link_mlp_tc", "k_link_mlp_d256_tc", "k_link_side_d128", "k_link_side_d256"}
@@ -84,3 +88,30 @@ def test_the_scan_tells_an_exit_ahead_of_the_wait():
     assert list(_events(early)) == [("exit", False), ("signal", False)]
     assert list(_events(late)) == [("exit", True), ("signal", True), ("exit", True)]
     assert list(_events(some)) == [("exit", False)]
+
+
+@pytest.fixture(scope="module")
+def first_tile(tmp_path_factory):
+    """early_first_tile of lime_common.cuh, compiled for the host as it stands there."""
+    at = tmp_path_factory.mktemp("split")
+    text = open(os.path.join(CSRC, "lime_common.cuh")).read()
+    name = "int early_first_tile(int cta, int grid, int n, int late, int late_by)"
+    (at / "split.cpp").write_text('#include <cstdint>\nextern "C" ' + name + " " + _body(text, text.index(name)))
+    subprocess.run(["g++", "-O1", "-shared", "-fPIC", str(at / "split.cpp"), "-o", str(at / "split.so")], check=True)
+    return ctypes.CDLL(str(at / "split.so")).early_first_tile
+
+
+def test_the_split_of_an_update_beside_the_link_side(first_tile):
+    """Every tile belongs to one block, whatever the grid, the late blocks and the tiles; late blocks get `late_by` tiles fewer where there
+    are enough, and nothing where the early ones are through before they start."""
+    for grid in (1, 2, 37, 147, 148):
+        for late in {0, 1, grid // 2, grid - 1, grid}:
+            for late_by in (2, 4):
+                for n in (0, 1, grid - 1, grid, 3 * grid + 1, 20 * grid + 5):
+                    first = [first_tile(c, grid, n, late, late_by) for c in range(grid + 1)]
+                    tiles = [b - a for a, b in zip(first, first[1:])]
+                    assert first[0] == 0 and first[-1] == n and min(tiles) >= 0, (grid, late, late_by, n)
+                    early, behind = tiles[:grid - late], tiles[grid - late:]
+                    if early and behind:
+                        assert max(behind) <= max(max(early) - late_by + 1, 0), (grid, late, late_by, n, tiles)
+                        assert max(early) - min(early) <= 1 and max(behind) - min(behind) <= 1
