@@ -5,8 +5,8 @@
 // About 200 k operations per candidate against 100 bytes: bound by the tensor pipe (196 KB of weights stay in shared memory).
 // The hidden layers chain through registers: a warp takes 16 or 32 candidates, forms 16 hidden units of the first layer at a
 // time (the accumulator becomes the A fragment of the second layer's k-step) and keeps the 128-wide second layer in its
-// accumulators, so no activation touches memory.  A tcgen05 version would have to send every hidden block through TMEM, the
-// register file and shared memory again, and the batches served (tens of thousands of candidates) are a single wave.
+// accumulators, so no activation touches memory.  The pipe is 66 % busy at the rate that mma.sync reaches; on tcgen05 the hidden
+// blocks would go through TMEM as A operands, as U does in the history updates (k_hist_update_tmem_tc.cu).  That form has not been built.
 // The first layer's input is not folded through the link states: O is formed per candidate (four products), so it needs no per-user
 // operand.  O and both hidden layers enter their products as a bf16 value and its bf16 remainder.  Error of the logits against
 // fp64 from the same link states (16 links, widths 512, 128, 64, four seeds): 2.0e-6 .. 5.3e-6; rounded once instead, the hidden
@@ -350,7 +350,9 @@ static lime_status launch_m3(ScoreMlp3Params p, cudaStream_t st) {
 
 // A block takes 128, 192 or 256 slots at a time: a round of the grid costs 18.4, 27.2 or 35 us (16 links, widths 512, 128, 64; the
 // whole call 23.5, 32.4 and 39.6 with one), so what counts is how full the last round is.  25,600 candidates 40.2 -> 32.4 us,
-// 12,800 39.0 -> 23.6, 45,000 74.4 -> 59.9, 200,000 211.9 -> 205.9 against 256 slots whatever their number.
+// 12,800 39.0 -> 23.6, 45,000 74.4 -> 59.9, 200,000 211.9 -> 205.9 against 256 slots whatever their number.  Other shapes take less a round,
+// in nearly the same proportion: with 8, 16 or 32 links, a first width of 64 to 512 and 1000 to 200,000 candidates the shape chosen is
+// within 2 % of the best of the three but for first widths of 64 from 120,000 candidates on (4 %).
 template <int ELL>
 static lime_status launch_m3_shape(const ScoreMlp3Params& p, cudaStream_t st) {
   auto rounds = [&](int slots) { return (double)((p.total + (int64_t)slots * kSMs - 1) / ((int64_t)slots * kSMs)); };

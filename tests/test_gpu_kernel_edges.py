@@ -457,6 +457,12 @@ def test_history_update_beside_the_link_side(d, H, ell, lengths, raw):
     _encode_against_oracle(synth.BF16, d, H, ell, 3, lengths, "softmax", raw, True, 6e-2, 3e-2)
 
 
+@pytest.mark.parametrize("d,H,ell,n_layers", [(128, 4, 32, 2), (128, 4, 64, 3), (256, 4, 32, 3), (256, 8, 64, 2)])
+def test_layers_of_more_users_than_an_early_update_serves(d, H, ell, n_layers):
+    """1025 users and more: the history updates wait for the link side again, and read the offsets from memory."""
+    _encode_against_oracle(synth.BF16, d, H, ell, n_layers, [3, 0, 129, 40] + [5, 1, 9] * 340 + [300], "softmax", False, False, 6e-2, 3e-2)
+
+
 @pytest.mark.parametrize("H,ell,B,along", [(4, 32, 67, True), (8, 32, 67, True), (4, 64, 35, True), (8, 64, 35, False), (8, 64, 129, True)])
 def test_queries_of_the_last_layer(H, ell, B, along):
     """d = 128 above 2048 link rows: formed by the GatedMLP kernel of the layer before, but for few rows with more than 256 stacked rows by a
