@@ -266,19 +266,19 @@ def launch_mode(args):
 # kernel and workload, with the hash of the kernel's source at capture time: once the source changes the figure
 # is stale and the bench reports null.
 NCU_TRAFFIC = {
-    # dense scorer: 170.0 MB read + 1.4 MB written
-    ("k_score_tc", "bf16_baseline", 256, 2048): {"bytes": 171.4e6, "source": "k_score_tc.cu", "sha": "4607381703032873"},
+    # dense scorer: 170.0 MB read + 1.0 MB written
+    ("k_score_tc", "bf16_baseline", 256, 2048): {"bytes": 171.1e6, "source": "k_score_tc.cu", "sha": "c1cbc69eeb4d8231"},
     # XOR-layer kernels: average per launch
-    ("k_link_attn_tmem_tc", "bf16_baseline", 256, 2048): {"bytes": 37.8e6, "source": "k_link_attn_tmem_tc.cu", "sha": "6410e05c815c36cb"},
-    ("k_hist_update_tmem_tc", "bf16_baseline", 256, 2048): {"bytes": 33.8e6, "source": "k_hist_update_tmem_tc.cu", "sha": "19acbb03963bab5e"},
-    # scorer by id over packed corpus records: 174.5 MB read + 4.2 MB written per launch
-    ("k_score_gather_tc", "bf16_baseline", 256, 2048): {"bytes": 178.7e6, "source": "k_score_gather_tc.cu", "sha": "d1a45f59fe51066e"},
-    # scorer through the interaction network (--head 96): 169.4 MB read + 5.0 MB written per launch
-    ("k_score_head_tc", "bf16_baseline", 256, 2048): {"bytes": 174.4e6, "source": "k_score_head_tc.cu", "sha": "345f4dcbe7ab9f5a"},
+    ("k_link_attn_tmem_tc", "bf16_baseline", 256, 2048): {"bytes": 37.8e6, "source": "k_link_attn_tmem_tc.cu", "sha": "547db7fd8d56eaad"},
+    ("k_hist_update_tmem_tc", "bf16_baseline", 256, 2048): {"bytes": 33.8e6, "source": "k_hist_update_tmem_tc.cu", "sha": "d5107b5b9a815797"},
+    # scorer by id over packed corpus records: 174.2 MB read + 3.2 MB written per launch
+    ("k_score_gather_tc", "bf16_baseline", 256, 2048): {"bytes": 177.4e6, "source": "k_score_gather_tc.cu", "sha": "b9f07adb44eef462"},
+    # scorer through the interaction network (--head 96): 169.4 MB read + 3.7 MB written per launch
+    ("k_score_head_tc", "bf16_baseline", 256, 2048): {"bytes": 173.1e6, "source": "k_score_head_tc.cu", "sha": "e5c9c1391b4a25b7"},
     # d = 256 kernels: captured on 128 users of the same model and length mix (327,680 tokens) and scaled by the tokens of
     # a launch (persistent kernels, identical tiles: traffic grows in proportion): bytes per token, average of the layers
-    ("k_link_attn_tmem_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 605.4, "source": "k_link_attn_tmem_tc.cu", "sha": "6410e05c815c36cb"},
-    ("k_hist_update_d256_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 945.4, "source": "k_hist_update_d256_tc.cu", "sha": "4b92622ae42aa190"},
+    ("k_link_attn_tmem_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 604.2, "source": "k_link_attn_tmem_tc.cu", "sha": "547db7fd8d56eaad"},
+    ("k_hist_update_d256_tc", "production_ragged", 1024, 8192): {"bytes_per_token": 943.3, "source": "k_hist_update_d256_tc.cu", "sha": "9b8468ce98c961cf"},
 }
 
 

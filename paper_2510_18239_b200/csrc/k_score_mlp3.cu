@@ -5,7 +5,7 @@
 // About 200 k operations per candidate against 100 bytes: bound by the tensor pipe (196 KB of weights stay in shared memory).
 // The hidden layers chain through registers: a warp takes 16 or 32 candidates, forms 16 hidden units of the first layer at a
 // time (the accumulator becomes the A fragment of the second layer's k-step) and keeps the 128-wide second layer in its
-// accumulators, so no activation touches memory.  The pipe is 66 % busy at the rate that mma.sync reaches; on tcgen05 the hidden
+// accumulators, so no activation touches memory.  The pipe is 60 % busy at the rate that mma.sync reaches; on tcgen05 the hidden
 // blocks would go through TMEM as A operands, as U does in the history updates (k_hist_update_tmem_tc.cu).  That form has not been built.
 // The first layer's input is not folded through the link states: O is formed per candidate (four products), so it needs no per-user
 // operand.  O and both hidden layers enter their products as a bf16 value and its bf16 remainder.  Error of the logits against
